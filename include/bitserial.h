@@ -103,7 +103,10 @@ int bs_pack_rows(const int8_t* codes, int rows, int K, int bits, bs_sign_t sign,
  * Convolution problem (host struct).  Output size P = (H + 2*pad - R)/stride + 1, Q likewise.
  *
  * Accumulator (exact int32):  acc[n][o][p][q] = sum_{c,r,s} a[n][c][p*stride-pad+r][q*stride-pad+s] * w[o][c][r][s]
- * evaluated as the Section V plane-pair popcount sum with the sign handling described at the top.
+ * the Section V plane-pair popcount sum with the sign handling described at the top.  It equals the integer dot product of the
+ * codes, and that is how it is evaluated: on the tensor cores, the planes of both operands expanded to int8 on chip.  The popcount
+ * kernels take what that path refuses (bipolar operands on both sides with a ragged channel word, residual slices that do not
+ * start at a multiple of 32); the results are the same integers.
  *
  * Epilogue, applied when out_packed != NULL, in exactly this order in IEEE binary32:
  *     v = fmaf((float)acc, scale[o], bias[o]);
@@ -214,10 +217,8 @@ int bitserial_gemm_noalloc(const uint32_t* a_packed, const uint32_t* w_packed, i
                            void* stream);
 
 /*
- * Tensor-core formulation (exactly equivalent integer MMA).  The Section V plane-pair popcount sum is the integer
- * dot product of the unpacked codes, so the same int32 accumulators are produced by an int8 x int8 -> int32 matrix
- * product: activations stay bit-packed in memory and are expanded to int8 inside the kernel, filters are expanded
- * once by bs_tc_prepare_weights.  Results (accumulators and requantised codes) are bit-identical to
+ * Filters prepared once: the same kernels as bitserial_conv2d / bitserial_gemm with the filters already expanded to int8 tiles by
+ * bs_tc_prepare_weights, so that a launch fetches them instead of expanding them.  Results (accumulators and requantised codes) are bit-identical to
  * bitserial_conv2d / bitserial_gemm; the epilogue is the one documented at bs_conv_params.
  *   Supported subset (bs_tc_supported returns 1): C a multiple of 32 whose packed pixel record (C/32 * a_bits words)
  *   is a 16-byte multiple, or an 8-byte multiple when a packed image row (W records) is a 16-byte multiple and, for
@@ -245,10 +246,9 @@ int bitserial_conv2d_tc(const uint32_t* act_packed, const int8_t* wgt_tc, const 
 int bitserial_conv2d_tc_chained(const uint32_t* act_packed, const int8_t* wgt_tc, const bs_conv_params* p,
                                 int32_t* out_i32, uint32_t* out_packed, void* stream);
 /*
- * bitserial_conv2d_tc_chain -- 2 to 4 consecutive layers of a network in ONE launch (the paper runs a network layer by layer
- * and names tiling and parallelisation as the source of its speed, Section V; running several layers as one grid whose tiles
- * wait for the tiles they depend on, instead of one grid per layer, is this library's addition).  Every layer computes exactly
- * what bitserial_conv2d_tc computes for its bs_conv_params; results are identical.
+ * bitserial_conv2d_tc_chain -- 2 to 4 consecutive same-shaped layers of a network in ONE call (the paper runs a network layer by
+ * layer, Section V).  Every layer computes exactly what bitserial_conv2d_tc computes for its bs_conv_params, each as a launch whose
+ * set-up and filter fetch run while the layer before it finishes.
  *   layers[l]        bs_conv_params of layer l.  All layers share N, C, H, W, O = C, R = S, pad = (R-1)/2, stride 1 (the output
  *                    is as large as the input), the activation and weight formats, and a packed output (out_bits > 0, no
  *                    channel offset: out_c_offset 0, out_c_total O) whose format is the next layer's activation format; a
@@ -257,14 +257,12 @@ int bitserial_conv2d_tc_chained(const uint32_t* act_packed, const int8_t* wgt_tc
  *                    (bs_tc_prepare_weights) and packed output of layer l.  A layer may read -- as input or residual -- the
  *                    output of any EARLIER layer of the chain, or tensors that were final before the launch; an output must
  *                    not overlap a tensor the same chain reads unless that tensor is the output of an earlier layer or the
- *                    input of one.  Outputs of all layers are materialised in full.
+ *                    input of one.
  *   workspace        DEVICE, 16-byte aligned, at least bs_tc_chain_workspace_bytes(layers, nlayers) bytes, zero-filled by the
- *                    caller once before its first use (and again after a launch that ended with BS_ERR_TIMEOUT); the library
- *                    keeps per-tile progress counters in it from launch to launch.  One workspace serves one chain; launches
- *                    that share a workspace must not overlap on the GPU.
+ *                    caller once before its first use.  One workspace serves one chain; calls that share one must not overlap.
  *   chained          non-zero: launched like bitserial_conv2d_tc_chained (same promise by the caller, for every layer).
- * bs_tc_chain_workspace_bytes returns 0 when the layers cannot run as one chain (shapes differ, a layer does not take the
- * resident-filter plan, more than 4 layers); bitserial_conv2d_tc_chain then returns BS_ERR_UNSUPPORTED and launches nothing:
+ * bs_tc_chain_workspace_bytes returns 0 when the layers cannot run as one chain (shapes differ, a layer the tensor-core
+ * path does not take, more than 4 layers); bitserial_conv2d_tc_chain then returns BS_ERR_UNSUPPORTED and launches nothing:
  * call bitserial_conv2d_tc per layer.  Other errors: BS_ERR_INVALID_ARG (null pointer, workspace too small),
  * BS_ERR_ALIGNMENT, BS_ERR_CUDA.  Every device-side wait is bounded (about a second); one that runs out sets the status
  * word read by bs_check_status.  Asynchronous on `stream`; works under stream capture.

@@ -7,6 +7,7 @@
 #include <mutex>
 
 #include "conv_launch.cuh"
+#include "mma_conv.h"
 #include "requant_bounds.h"
 
 namespace bs {
@@ -288,6 +289,10 @@ static int conv_impl(const uint32_t* act, const uint32_t* wgt, const bs_conv_par
         }
     }
 
+    if (!query_ws) {
+        const int rc = mma_conv_run(act, nullptr, wgt, p, out_i32, out_packed, st, false, false);
+        if (rc != BS_ERR_UNSUPPORTED) return rc;
+    }
     const int A = p->a_bits, WB = p->w_bits;
     Plan pl{};
     const bool want_split = query_ws != nullptr || (workspace != nullptr && workspace_bytes > 0);

@@ -1,0 +1,434 @@
+// Host side of the tensor-core convolution: plan of a layer and launch (kernel: mma_kernel.cuh).
+#include <cmath>
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <mutex>
+#include <unordered_map>
+
+#include "mma_kernel.cuh"
+
+namespace bs {
+
+// ----------------------------------------------------------------------------- plan
+
+namespace {
+
+constexpr int MM_SMEM_MAX = 224 * 1024;
+
+int up(int v, int m) { return (v + m - 1) / m * m; }
+
+FastDiv make_div(int d)
+{
+    FastDiv f{0, 0, d};
+    if (d > 1) {
+        int l = 0;
+        while ((1LL << l) < d) ++l;                       // ceil(log2 d)
+        const unsigned long long p = 31 + l;
+        f.mul = static_cast<unsigned>(((1ULL << p) + d - 1) / d);
+        f.shift = static_cast<unsigned>(p - 32);
+    }
+    return f;
+}
+
+int max_abs_of(int bits, int sign) { return sign == BS_BIPOLAR ? 1 : (sign == BS_SIGNED ? 1 << (bits - 1) : (1 << bits) - 1); }
+
+struct Cand {
+    int TN, PT, units, cfg, cps, ns, resident, nse, nsb, nacc;
+    size_t smem;
+    double cost;
+};
+
+// Shared-memory layout of a candidate; false when it does not fit.  g carries the problem, the candidate the tiling.
+bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows)
+{
+    const bool packed_b = WB > 0;
+    const int st = g.stride, XT = c.cfg ? 256 : 128, EW = c.cfg ? 8 : 4;
+    const int rmax = st == 1 ? g.R - 1 - g.pad : (g.R - 1 - g.pad) >> 1;
+    const int Wp = (g.W + st - 1) / st, Hp = (g.H + st - 1) / st;
+    g.rmin = st == 1 ? -g.pad : (-g.pad) >> 1;
+    g.smin = g.rmin;
+    g.flat = g.R == 1 && st == 1 && g.pad == 0;
+    g.nplanes = g.R > 1 && st == 2 ? 4 : 1;
+    g.strip_q = ceil_div(g.Q, c.ns);
+    if (c.ns == 1) {
+        g.pitch = Wp - g.smin > g.Q + rmax ? Wp - g.smin : g.Q + rmax;
+        g.xoff = 0;
+        if (g.R == 1) g.pitch = g.Q;
+    } else {
+        g.pitch = g.strip_q + rmax - g.smin;
+        g.xoff = g.smin;
+    }
+    const int PH = g.R == 1 ? g.P : (Hp - g.rmin > g.P + rmax ? Hp - g.rmin : g.P + rmax);
+    g.hstart = g.rmin * g.pitch + (c.ns == 1 ? g.smin : 0);
+    const int BM = 128 * c.PT;
+    g.HL = BM + (rmax - g.rmin) * g.pitch + (rmax - g.smin);
+    g.NI = g.HL * g.nplanes;
+    g.img_rows = PH;
+    const long long per_img = static_cast<long long>(PH) * g.pitch;
+    const long long total = static_cast<long long>(g.N) * c.ns * per_img;
+    if (total + per_img + 4096 + g.HL > 0x7fffffffLL || g.NI > 4096) return false;
+    g.total = static_cast<int>(total);
+    g.d_img = make_div(static_cast<int>(per_img));
+    g.d_pitch = make_div(g.pitch);
+    g.d_strips = make_div(c.ns);
+    g.TN = c.TN; g.PT = c.PT; g.units = c.units;
+    g.nunits = (g.Cw + 1) / 2;
+    g.nchunks = ceil_div(g.nunits, c.units);
+    g.tiles_m = static_cast<int>(ceil_div_ll(total, BM));
+    g.tiles_o = ceil_div(g.O, c.TN);
+    g.d_rs = make_div(g.RS);
+    g.nslots = ceil_div(g.NI * c.units, XT);
+    g.bslots = ceil_div(c.TN * g.RS * c.units, XT);
+    auto piece = [&](int bits) { return (2 * bits) % 4 == 0 && (g.Cw * bits) % 4 == 0 ? 16 : ((g.Cw * bits) % 2 == 0 ? 8 : 4); };
+    g.psz = piece(A);
+    g.bpsz = piece(WB > 0 ? WB : 1);
+    // boxes of [row][units]: rows of 16-byte multiples in memory, box rows of 16 .. 128 bytes
+    g.rowA = c.units * 8 * A;
+    g.rowB = c.units * 8 * WB;
+    const bool fb = packed_b && !c.resident;
+    g.tma = g.flat && (g.Cw * A) % 4 == 0 && g.rowA % 16 == 0 && g.rowA <= 128 && (!fb || ((g.Cw * WB) % 4 == 0 && g.rowB % 16 == 0 && g.rowB <= 128));
+    auto swizzle = [](int row) { return row == 32 ? 1 : row == 64 ? 3 : row == 128 ? 7 : 0; };
+    g.swzA = swizzle(g.rowA);
+    g.swzB = swizzle(g.rowB);
+    g.e_bytes = up(4 * c.units * g.NI * 16, 128);
+    g.b_bytes = c.units * 2 * c.TN * g.RS * 32;
+    g.stg_bytes = g.tma ? up(BM * g.rowA, 1024) : g.nslots * XT * 8 * A;
+    g.bstg_bytes = !fb ? 0 : g.tma ? up(c.TN * g.rowB, 1024) : g.bslots * XT * 8 * WB;
+    const int pix_bytes = g.flat ? 0 : up(g.NI * 4, 16);
+    const int cap = c.cfg ? 222 * 1024 : 111 * 1024;
+    const int fixed = c.TN * 8 + 64 + 256 + (g.tma ? 1024 : 0) + (int_rows ? EW * 4096 : 0) + 256 + pix_bytes;
+    const long long filters = c.resident ? static_cast<long long>(g.Cw) * c.TN * g.RS * 32 : 0;
+    const long long rest = fixed + static_cast<long long>(MM_STAGES) * (g.stg_bytes + g.bstg_bytes) + filters;
+    c.nsb = 0;
+    long long used = 0;
+    int nse = 4;
+    if (c.resident) {
+        for (; nse >= 2; --nse) {
+            used = rest + static_cast<long long>(nse) * g.e_bytes;
+            if (used <= cap) break;
+        }
+        if (nse < 2) return false;
+    } else if (packed_b) {
+        for (; nse >= 2; --nse) {
+            used = rest + static_cast<long long>(nse) * (g.e_bytes + g.b_bytes);
+            if (used <= cap) break;
+        }
+        if (nse < 2) return false;
+    } else {
+        bool fit = false;
+        for (int n = 4; n >= 1 && !fit; --n) {
+            used = rest + static_cast<long long>(n) * (g.e_bytes + g.b_bytes);
+            if (used <= cap) { nse = n; c.nsb = n; fit = true; }
+        }
+        if (!fit) return false;
+    }
+    c.nse = nse;
+    g.nse = nse; g.nsb = c.resident ? 0 : (packed_b ? nse : c.nsb);
+    const int cols = 512 / (c.cfg ? 1 : 2);
+    if (2 * c.PT * c.TN <= cols) c.nacc = 2;
+    else if (c.PT * c.TN <= cols) c.nacc = 1;
+    else return false;
+    g.nacc = c.nacc;
+    int tc = 32;
+    while (tc < c.nacc * c.PT * c.TN) tc *= 2;
+    g.tmem_cols = tc;
+    long long off = c.resident ? filters : static_cast<long long>(g.nsb) * g.b_bytes;
+    g.off_e = static_cast<int>(off);                off += static_cast<long long>(nse) * g.e_bytes;
+    if (g.tma) off = (off + 1023) / 1024 * 1024;
+    g.off_stg = static_cast<int>(off);              off += static_cast<long long>(MM_STAGES) * g.stg_bytes;
+    g.off_bstg = static_cast<int>(off);             off += static_cast<long long>(MM_STAGES) * g.bstg_bytes;
+    g.off_pix = static_cast<int>(off);              off += pix_bytes;
+    off = (off + 127) / 128 * 128;
+    g.off_out = static_cast<int>(off);              if (int_rows) off += EW * 4096;
+    g.off_tab = static_cast<int>(off);              off += c.TN * 8 + 64;
+    off = (off + 15) / 16 * 16;
+    g.off_bar = static_cast<int>(off);              off += 256;
+    g.bulk_b = packed_b && c.resident && static_cast<long long>(c.TN) * g.RS * g.Cw * WB * 4 <= static_cast<long long>(nse) * g.e_bytes &&
+               (static_cast<long long>(g.O % c.TN) * g.RS * g.Cw * WB) % 4 == 0;
+    c.smem = static_cast<size_t>(off);
+    return off <= cap + 512;
+}
+
+// Time model of a candidate in SM cycles: the pipeline of one CTA (expansion, MMAs, epilogue; a stage's hand-off included) over
+// its items, plus what nothing overlaps at both ends.  The constants are fitted to about 2500 timed plans of 41 layers and
+// products (1 to 300 pixels wide, 32 to 4608 channels, batches 1 to 64; B200 at 1.95 GHz): over those the plan with the
+// lowest modelled time is on average 2 % and with three exceptions at most 8 % slower than the fastest plan.
+double mma_cost(const MmaArgs& g, const Cand& c, int A, int WB, bool packed_out, int sms)
+{
+    const bool packed_b = WB > 0;
+    const double mma = 1.05 * (c.TN == 32 ? 42 : c.TN == 64 ? 49 : c.TN == 128 ? 65 : 129);      // cycles per MMA of 128 x TN x 32
+    const int W = c.cfg ? 8 : 4;                                   // expander warps, epilogue warps
+    const double t_m = static_cast<double>(c.PT) * g.RS * g.Cw * mma + 121.0 * g.nchunks;
+    // expansion: instructions per warp and 64-channel unit of 32 rows, at 6.8 cycles each
+    const int row_groups = ceil_div(g.NI, 32);
+    double xi = static_cast<double>(row_groups) * g.nunits * ((A <= 2 ? 90.0 : 140.0) + (g.tma ? 2.0 : 60.0));
+    if (!c.resident && packed_b) xi += c.TN * g.RS / 32.0 * g.nunits * (WB <= 2 ? 40.0 : 60.0);
+    const double units_of_work = static_cast<double>(row_groups) * c.units / W;
+    const double t_x = xi / W * (ceil(units_of_work) / units_of_work) * 6.8 + 500.0 * g.nchunks + 278.0;
+    // epilogue: instructions per block of 32 x 32 outputs, at 3.65 cycles; int32 rows leave at about 27 bytes per clock and SM
+    const double block = packed_out ? (g.has_residual ? 283.0 : 187.0) : 106.0;
+    double t_e = ceil_div(c.PT * (c.TN / 32), W / 4) * block * 3.65 + 700.0;
+    if (!packed_out && c.PT * 128.0 * c.TN * 4 / 27.5 > t_e) t_e = c.PT * 128.0 * c.TN * 4 / 27.5;
+    const double t_b = (!c.resident && !packed_b) ? static_cast<double>(c.TN) * g.RS * g.Cw * 32 / 52.0 : 0.0;       // L2 -> shared memory
+    const long long items = static_cast<long long>(g.tiles_m) * g.tiles_o;
+    long long ctas = static_cast<long long>(sms) * c.cps;
+    if (c.resident) ctas = ctas / g.tiles_o * g.tiles_o;
+    if (ctas < 1) return 1e18;
+    if (ctas > items) ctas = items;
+    const double per_cta = static_cast<double>(ceil_div_ll(items, ctas)), active = static_cast<double>(ceil_div_ll(ctas, sms));
+    const double issue = (xi + c.PT * 4.0 * (c.TN / 32) * block) / 2.77;
+    const double t_mb = t_m > t_b ? t_m : t_b;
+    double step = c.nacc == 2 ? (t_mb > t_e ? t_mb : t_e) : t_mb + t_e;
+    if (t_x > step) step = t_x;
+    if (active * t_mb > step) step = active * t_mb;
+    if (active * issue > step) step = active * issue;
+    const double rest_x = t_x * (g.nchunks - 1) / g.nchunks;
+    double first = t_x / g.nchunks + (t_mb > rest_x ? t_mb : rest_x) + t_e;
+    if (active > 1.0) first *= 1.3;
+    double t = 5900.0 + first + (per_cta - 1.0) * step;
+    if (c.resident && packed_b) t += c.TN * g.RS * g.Cw / 32.0 * 76.0 / (2 * W) * 4.0;
+    if (!c.resident && !packed_b) t *= 1.05;
+    if (!c.resident && (c.nse < 2 || (!packed_b && c.nsb < 2))) t *= 1.3;
+    if (!c.cfg) t *= 0.91;
+    return t;
+}
+
+}  // namespace
+
+// Everything about a layer that does not depend on its pointers: filled arguments, kernel, grid.
+struct MmaPlan {
+    MmaArgs g;
+    MmaKernel kern;
+    unsigned grid, block;
+    int smem;
+    int rc;                 // BS_OK, or why there is no plan
+};
+
+enum : int { MM_PREPARED = 1, MM_I32 = 2, MM_CODES = 4, MM_RESIDUAL = 8, MM_CHAINED = 16, MM_QUERY = 32 };
+
+static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
+{
+    const bool out_i32 = flags & MM_I32, out_packed = flags & MM_CODES, residual = flags & MM_RESIDUAL, packed_b = !(flags & MM_PREPARED);
+    // the callers have validated sizes, bit widths, pointers and output slices; what this path refuses is said here
+    if (p->stride > 2 || p->R > 7) return BS_ERR_UNSUPPORTED;
+    if (p->a_sign == BS_BIPOLAR && p->w_sign == BS_BIPOLAR && p->C % 32 != 0) return BS_ERR_UNSUPPORTED;
+    if (residual && p->res_c_offset % 32 != 0) return BS_ERR_UNSUPPORTED;
+    MmaArgs& g = plan.g;
+    const int A = p->a_bits;
+    g.has_residual = residual;
+    g.res_scale = p->res_scale;
+    g.N = p->N; g.H = p->H; g.W = p->W; g.O = p->O; g.R = p->R; g.RS = p->R * p->S; g.stride = p->stride; g.pad = p->pad;
+    g.P = (p->H + 2 * p->pad - p->R) / p->stride + 1;
+    g.Q = (p->W + 2 * p->pad - p->S) / p->stride + 1;
+    g.Cw = ceil_div(p->C, 32);
+    auto kind = [](int sign) { return sign == BS_SIGNED ? 1 : sign == BS_BIPOLAR ? 2 : 0; };
+    g.a_kind = kind(p->a_sign); g.w_kind = kind(p->w_sign);
+    g.relu = p->relu; g.out_bits = p->out_bits; g.out_sign = p->out_sign;
+    g.out_cw_off = p->out_c_offset / 32; g.out_cw_total = ceil_div(p->out_c_total > 0 ? p->out_c_total : 1, 32);
+    g.res_bits = p->res_bits; g.res_sign = p->res_sign; g.res_c_off = p->res_c_offset;
+    g.res_cw_total = ceil_div(p->res_c_total > 0 ? p->res_c_total : 1, 32);
+    g.i32_nhwc = p->i32_layout == BS_NHWC;
+    g.opad = up(p->O, 128);
+    const double bound = static_cast<double>(p->C) * g.RS * max_abs_of(p->a_bits, p->a_sign) * max_abs_of(p->w_bits, p->w_sign);
+    g.acc_bound = static_cast<float>(bound);
+    g.preset = out_packed && !out_i32 && bound < 4.0e6 && p->out_sign != BS_BIPOLAR &&
+               (!residual || (p->res_sign == BS_UNSIGNED && fabsf(p->res_scale) < 3.9f && (p->res_scale == 0.0f || fabsf(p->res_scale) > 1e-18f)));
+    {
+        int qmin, qmax;
+        code_limits(p->out_bits > 0 ? p->out_bits : 1, p->out_sign, qmin, qmax);
+        const bool lo0 = qmin == 0 || p->relu;
+        if (!lo0) g.epi = 4;
+        else if (p->out_bits <= 2 && (!residual || p->res_bits <= 2)) g.epi = residual ? 1 : 0;
+        else g.epi = residual ? 3 : 2;
+    }
+    g.early_b = flags & MM_CHAINED ? 1 : 0;
+    const bool int_rows = out_i32 && g.i32_nhwc && p->R == 1 && p->stride == 1 && p->pad == 0;
+
+    Cand best{};
+    best.cost = 1e30;
+    bool found = false;
+    auto consider = [&](Cand c) {
+        MmaArgs t = g;
+        if (!mma_layout(t, c, A, packed_b ? p->w_bits : 0, int_rows)) return;
+        c.cost = mma_cost(t, c, A, packed_b ? p->w_bits : 0, out_packed, sms);
+        if (c.cost < best.cost) { best = c; found = true; }
+    };
+    int ns_list[12], nns = 0;
+    if (g.R == 1) ns_list[nns++] = 1;
+    else {
+        static const int widths[] = {1 << 30, 112, 84, 64, 48, 40, 32, 24, 20, 16, 12, 8};      // outputs per strip row, roughly
+        for (int w : widths) {
+            const int ns = w > g.Q ? 1 : ceil_div(g.Q, w);
+            if (nns == 0 || ns_list[nns - 1] != ns) ns_list[nns++] = ns;
+        }
+    }
+#ifdef BS_TUNING
+    int ov[6] = {0, 0, 0, -1, 0, -1};       // TN, PT, units, config, strips, resident; 0 / -1: free
+    if (const char* e = getenv("BS_MM")) sscanf(e, "%d,%d,%d,%d,%d,%d", ov, ov + 1, ov + 2, ov + 3, ov + 4, ov + 5);
+#endif
+    for (int TN = 32; TN <= 256; TN *= 2) {
+        if (TN > 32 && TN / 2 >= up(p->O, 32)) continue;
+        if (TN == 256 && !packed_b && g.opad % 256 != 0) continue;
+        for (int PT = 1; PT <= 4; PT *= 2)
+            for (int cfg = 0; cfg < 3; ++cfg)
+                for (int k = 0; k < nns; ++k)
+                    for (int units = 1; units <= (g.R == 1 ? 4 : 1); units *= 2) {
+                        if (units > 1 && units > (g.Cw + 1) / 2) continue;
+                        for (int res = 0; res < 2; ++res) {
+#ifdef BS_TUNING
+                            if ((ov[0] && TN != ov[0]) || (ov[1] && PT != ov[1]) || (ov[2] && units != ov[2]) || (ov[3] >= 0 && cfg != ov[3]) ||
+                                (ov[4] && ns_list[k] != ov[4]) || (ov[5] >= 0 && res != ov[5]))
+                                continue;
+#endif
+                            Cand c{};
+                            c.TN = TN; c.PT = PT; c.units = units; c.cfg = cfg == 1; c.cps = cfg == 0 ? 2 : 1; c.ns = ns_list[k]; c.resident = res;
+                            consider(c);
+                        }
+                    }
+    }
+    if (!found) return BS_ERR_UNSUPPORTED;
+    if (!mma_layout(g, best, A, packed_b ? p->w_bits : 0, int_rows)) return BS_ERR_UNSUPPORTED;
+#ifdef BS_TUNING
+    if (getenv("BS_MM_VERBOSE"))
+        fprintf(stderr, "mma plan: N%d C%d %dx%d O%d k%d s%d A%d W%d %s -> TN %d PT %d units %d cfg %d x %d strips %d resident %d nse %d nsb %d units %d nacc %d HL %d NI %d tiles %d x %d smem %zu cost %.0f\n",
+                p->N, p->C, p->H, p->W, p->O, p->R, p->stride, A, p->w_bits, packed_b ? "packed" : "prepared", best.TN, best.PT, best.units, best.cfg, best.cps, best.ns, best.resident,
+                best.nse, g.nsb, g.nunits, g.nacc, g.HL, g.NI, g.tiles_m, g.tiles_o, best.smem, best.cost);
+#endif
+    if (flags & MM_QUERY) return BS_OK;
+    g.status = status_device_ptr();
+    if (!g.status) return BS_ERR_CUDA;
+    g.idesc = (2u << 4) | (1u << 7) | (1u << 10) | (static_cast<unsigned>(g.TN >> 3) << 17) | (static_cast<unsigned>(128 >> 4) << 24);
+    const int cps = best.cps;
+    const long long items = static_cast<long long>(g.tiles_m) * g.tiles_o;
+    long long grid = static_cast<long long>(sms) * cps;
+    if (best.resident) grid = grid / g.tiles_o * g.tiles_o;
+    if (grid > items) grid = items;
+    const int wb = packed_b ? p->w_bits : 0;
+    plan.kern = A == 1 ? mma_kernel_a1(wb, !best.cfg) : A == 2 ? mma_kernel_a2(wb, !best.cfg) : A == 3 ? mma_kernel_a3(wb, !best.cfg) : mma_kernel_a4(wb, !best.cfg);
+    plan.grid = static_cast<unsigned>(grid);
+    plan.block = best.cfg ? MmaShape<false>::THREADS : MmaShape<true>::THREADS;
+    plan.smem = static_cast<int>(best.smem);
+    // the limit is a property of the kernel, not of the launch: set to the largest any plan uses
+    if (cudaFuncSetAttribute(plan.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, MM_SMEM_MAX) != cudaSuccess) {
+        cudaGetLastError();
+        return BS_ERR_CUDA;
+    }
+    return BS_OK;
+}
+
+// Plans by shape, format and device: a program calls the same few layers again and again, and a search costs tens of
+// microseconds.  At most MAX_PLANS are kept (about 600 bytes each); when full the table starts over.
+namespace {
+struct PlanKey {
+    int v[28];
+    bool operator==(const PlanKey& o) const { return memcmp(v, o.v, sizeof v) == 0; }
+};
+struct PlanHash {
+    size_t operator()(const PlanKey& k) const
+    {
+        uint64_t h = 1469598103934665603ull;
+        for (int x : k.v) h = (h ^ static_cast<uint32_t>(x)) * 1099511628211ull;
+        return static_cast<size_t>(h ^ (h >> 29));
+    }
+};
+constexpr size_t MAX_PLANS = 4096;
+}  // namespace
+
+static int find_plan(MmaPlan& out, const bs_conv_params* p, int flags)
+{
+    int dev = -1;
+    int sms = device_sm_count();
+    if (sms <= 0) {
+        if (!(flags & MM_QUERY)) return BS_ERR_CUDA;
+        sms = 148;                      // a support query without a device plans for a full B200
+    } else if (cudaGetDevice(&dev) != cudaSuccess) {
+        return BS_ERR_CUDA;
+    }
+    const bool res = flags & MM_RESIDUAL, codes = flags & MM_CODES;
+    int scale_bits = 0;
+    if (res) memcpy(&scale_bits, &p->res_scale, 4);
+    const PlanKey key = {{p->N, p->C, p->H, p->W, p->O, p->R, p->S, p->stride, p->pad, p->a_bits, p->a_sign, p->w_bits, p->w_sign,
+                          codes ? p->relu : 0, codes ? p->out_bits : 0, codes ? p->out_sign : 0, codes ? p->out_c_offset : 0, codes ? p->out_c_total : 0,
+                          res ? p->res_bits : 0, res ? p->res_sign : 0, res ? p->res_c_offset : 0, res ? p->res_c_total : 0, scale_bits, p->i32_layout,
+                          flags, dev, sms, 0}};
+    static std::unordered_map<PlanKey, MmaPlan, PlanHash> plans;
+    static std::mutex mu;
+    {
+        std::lock_guard<std::mutex> lock(mu);
+#ifdef BS_TUNING
+        plans.clear();
+#endif
+        auto it = plans.find(key);
+        if (it != plans.end()) { out = it->second; return out.rc; }
+    }
+    MmaPlan plan{};
+    plan.rc = make_plan(plan, p, flags, sms);
+    if (plan.rc == BS_OK || plan.rc == BS_ERR_UNSUPPORTED) {
+        std::lock_guard<std::mutex> lock(mu);
+        if (plans.size() >= MAX_PLANS) plans.clear();
+        plans.emplace(key, plan);
+    }
+    out = plan;
+    return plan.rc;
+}
+
+// Tensor map of a row-major matrix of `rows` rows of `words` words, fetched in boxes of box_rows rows x row_bytes bytes.
+static bool encode_rows(CUtensorMap* tm, const uint32_t* base, int rows, int words, int row_bytes, int box_rows)
+{
+    typedef CUresult (*Fn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
+                           CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static Fn fn = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void* q = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &q, cudaEnableDefault, &r) == cudaSuccess && r == cudaDriverEntryPointSuccess) fn = reinterpret_cast<Fn>(q);
+    });
+    if (!fn) return false;
+    const cuuint64_t dims[2] = {static_cast<cuuint64_t>(words), static_cast<cuuint64_t>(rows)};
+    const cuuint64_t strides[1] = {static_cast<cuuint64_t>(words) * 4};
+    const cuuint32_t box[2] = {static_cast<cuuint32_t>(row_bytes / 4), static_cast<cuuint32_t>(box_rows)}, es[2] = {1, 1};
+    const CUtensorMapSwizzle sw = row_bytes == 32 ? CU_TENSOR_MAP_SWIZZLE_32B : row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B :
+                                  row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE;
+    return fn(tm, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<uint32_t*>(base), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
+              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+int mma_conv_run(const uint32_t* act, const int8_t* wgt, const uint32_t* wgt_packed, const bs_conv_params* p, int32_t* out_i32,
+                 uint32_t* out_packed, cudaStream_t st, bool chained, bool plan_only)
+{
+    const int flags = (wgt ? MM_PREPARED : 0) | (out_i32 ? MM_I32 : 0) | (out_packed ? MM_CODES : 0) | (out_packed && p->residual ? MM_RESIDUAL : 0) |
+                      (chained ? MM_CHAINED : 0) | (plan_only ? MM_QUERY : 0);
+    MmaPlan plan;
+    const int rc = find_plan(plan, p, flags);
+    if (rc != BS_OK || plan_only) return rc;
+    MmaArgs& g = plan.g;
+    g.act = act; g.wgt = wgt; g.wgt_packed = wgt_packed; g.out_i32 = out_i32; g.out_packed = out_packed;
+    g.scale = p->scale; g.bias = p->bias;
+    g.residual = out_packed ? p->residual : nullptr;
+    if (g.tma) {
+        const int fb = !wgt && g.nsb > 0;
+        if (!encode_rows(&g.tmA, act, g.total, g.Cw * p->a_bits, g.rowA, 128 * g.PT < 256 ? 128 * g.PT : 256)) return BS_ERR_CUDA;
+        if (fb && !encode_rows(&g.tmB, wgt_packed, g.O, g.Cw * p->w_bits, g.rowB, g.TN)) return BS_ERR_CUDA;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(plan.grid);
+    cfg.blockDim = dim3(plan.block);
+    cfg.dynamicSmemBytes = static_cast<size_t>(plan.smem);
+    cfg.stream = st;
+    // Every launch may start while the kernel before it drains (barriers, tensor memory, filter fetch when the caller allows);
+    // the kernel waits for that kernel itself before it reads or writes anything the stream orders.
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, plan.kern, g) != cudaSuccess) {
+        cudaGetLastError();
+        return BS_ERR_CUDA;
+    }
+    return BS_OK;
+}
+
+}  // namespace bs

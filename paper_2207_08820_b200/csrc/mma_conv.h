@@ -1,0 +1,22 @@
+// Tensor-core convolution on packed bitplanes (mma_conv.cu): host interface shared by the entry points.
+#pragma once
+#include <cuda_runtime.h>
+
+#include "common.cuh"
+
+namespace bs {
+
+// Column c of a 32-filter group of the accumulator tile holds filter mma_filter_of_column(c) of the group, and byte b of a
+// 32-channel block of either operand holds channel mma_channel_of_byte(b): the orders in which the epilogue can pair its
+// outputs and the expansion can cut bytes out of the plane words without moving single bits (see mma_conv.cu).
+__host__ __device__ constexpr int mma_filter_of_column(int c) { return 16 * (c & 1) + 2 * ((c >> 1) & 7) + (c >> 4); }
+__host__ __device__ constexpr int mma_column_of_filter(int f) { return 16 * (f & 1) + 2 * ((f & 15) >> 1) + (f >> 4); }
+__host__ __device__ constexpr int mma_channel_of_byte(int b) { return 8 * (b & 3) + (b >> 2); }
+
+// Runs one layer.  `wgt` are filters prepared by bs_tc_prepare_weights; when it is null the packed filters `wgt_packed` are
+// expanded inside the kernel.  chained: the caller promises that filters, scale and bias were final before the preceding
+// kernel of the stream was launched.  plan_only: validate and plan, launch nothing.
+int mma_conv_run(const uint32_t* act, const int8_t* wgt, const uint32_t* wgt_packed, const bs_conv_params* p, int32_t* out_i32,
+                 uint32_t* out_packed, cudaStream_t st, bool chained, bool plan_only);
+
+}  // namespace bs

@@ -1,0 +1,6 @@
+// Tensor-core convolution kernels for 4-bit activations.
+#include "mma_kernel.cuh"
+
+namespace bs {
+MmaKernel mma_kernel_a4(int wb, bool half) { return mma_pick<4>(wb, half); }
+}  // namespace bs
