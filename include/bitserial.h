@@ -222,8 +222,8 @@ int bitserial_gemm_noalloc(const uint32_t* a_packed, const uint32_t* w_packed, i
  * bitserial_conv2d / bitserial_gemm; the epilogue is the one documented at bs_conv_params.
  *   Supported subset (bs_tc_supported returns 1): C a multiple of 32 whose packed pixel record (C/32 * a_bits words)
  *   is a 16-byte multiple, or an 8-byte multiple when a packed image row (W records) is a 16-byte multiple and, for
- *   1x1 stride-1 layers, N*H*W is even; res_c_offset a multiple of 32; everything else as bitserial_conv2d.  Unsupported shapes return BS_ERR_UNSUPPORTED: use the
- *   popcount entry points.
+ *   1x1 stride-1 layers, N*H*W is even; res_c_offset a multiple of 32; everything else as bitserial_conv2d.  Unsupported shapes
+ *   return BS_ERR_UNSUPPORTED: use bitserial_conv2d.
  *   bs_tc_weights_bytes    bytes of the prepared int8 filter tensor (0 on bad input).
  *   bs_tc_prepare_weights  packed weights [O][R][S][Cw][w_bits] -> int8 tiles [C/32][ceil(O/128)*16][R*S][2][8][16]
  *                          (blocks of 32 channels; a_bits is accepted for forward compatibility).
@@ -271,6 +271,32 @@ size_t bs_tc_chain_workspace_bytes(const bs_conv_params* layers, int nlayers);
 int bitserial_conv2d_tc_chain(int nlayers, const uint32_t* const* act_packed, const int8_t* const* wgt_tc,
                               const bs_conv_params* layers, uint32_t* const* out_packed, void* workspace,
                               size_t workspace_bytes, int chained, void* stream);
+/*
+ * bs_sequence -- the layers of a network bound once to their tensors and run by one call (a host program that launches 20 to 50
+ * layers through its own binding spends more time on arguments than the GPU on small layers; the paper has no counterpart).
+ * bs_sequence_create validates and plans every layer; pointers, shapes and formats are those of the call and may not change while
+ * the sequence lives (the CONTENTS of the tensors may).  bs_sequence_run launches the layers in order on `stream`.
+ *   wgt_tc / wgt_packed   prepared filters, or NULL and packed filters.
+ *   chained               as in bitserial_conv2d_tc_chained, same promise.
+ *   aside                 non-zero: the layer runs on side_stream beside the layers after it, behind an event recorded before it.
+ *   join                  indices of up to four such layers (-1: none) that this layer waits for.  Every layer beside the others must
+ *                         be joined by a later one before its output is read or its tensors are reused, the last run included.
+ * A sequence belongs to the device that was current at its creation; runs of one sequence must not overlap on the host or the GPU.
+ * Works under stream capture.  Errors of create as bitserial_conv2d; it returns no sequence then.
+ */
+typedef struct bs_sequence bs_sequence;
+typedef struct {
+    const uint32_t* act_packed;
+    const int8_t* wgt_tc;
+    const uint32_t* wgt_packed;
+    uint32_t* out_packed;
+    bs_conv_params p;
+    int chained, aside;
+    int join[4];
+} bs_sequence_layer;
+int bs_sequence_create(const bs_sequence_layer* layers, int nlayers, void* side_stream, bs_sequence** sequence_out);
+int bs_sequence_run(bs_sequence* sequence, void* stream);
+void bs_sequence_destroy(bs_sequence* sequence);
 int bitserial_gemm_tc(const uint32_t* a_packed, const int8_t* w_tc, int M, int N, int K, int a_bits, bs_sign_t a_sign,
                       int w_bits, bs_sign_t w_sign, const float* scale, const float* bias, int relu, int out_bits,
                       bs_sign_t out_sign, int32_t* out_i32, uint32_t* out_packed, void* stream);

@@ -35,6 +35,12 @@ class ConvParams(ctypes.Structure):
     ]
 
 
+class SequenceLayer(ctypes.Structure):
+    """Mirror of ``bs_sequence_layer`` (include/bitserial.h)."""
+    _fields_ = [("act_packed", ctypes.c_void_p), ("wgt_tc", ctypes.c_void_p), ("wgt_packed", ctypes.c_void_p), ("out_packed", ctypes.c_void_p),
+                ("p", ConvParams), ("chained", ctypes.c_int), ("aside", ctypes.c_int), ("join", ctypes.c_int * 4)]
+
+
 def lib() -> ctypes.CDLL:
     global _lib
     if _lib is not None:
@@ -94,6 +100,12 @@ def lib() -> ctypes.CDLL:
     L.bitserial_conv2d_tc_chain.restype = i
     L.bitserial_conv2d_tc_chain.argtypes = [i, ctypes.POINTER(ctypes.c_void_p), ctypes.POINTER(ctypes.c_void_p), ctypes.POINTER(ConvParams),
                                             ctypes.POINTER(ctypes.c_void_p), vp, ctypes.c_size_t, i, vp]
+    L.bs_sequence_create.restype = i
+    L.bs_sequence_create.argtypes = [ctypes.POINTER(SequenceLayer), i, vp, ctypes.POINTER(vp)]
+    L.bs_sequence_run.restype = i
+    L.bs_sequence_run.argtypes = [vp, vp]
+    L.bs_sequence_destroy.restype = None
+    L.bs_sequence_destroy.argtypes = [vp]
     L.bitserial_gemm_tc.restype = i
     L.bitserial_gemm_tc.argtypes = [vp, vp, i, i, i, i, i, i, i, vp, vp, i, i, i, vp, vp, vp]
     L.bs_conv2d_f32.restype = i
@@ -124,6 +136,6 @@ EXPORTED = ("bs_packed_act_bytes", "bs_packed_wgt_bytes", "bs_packed_rows_bytes"
             "bitunpack_activations", "pack_weights", "bs_pack_rows", "bitserial_conv2d", "bitserial_gemm",
             "bitserial_conv2d_ws", "bitserial_gemm_ws", "bs_conv_workspace_bytes", "bs_gemm_workspace_bytes",
             "bitserial_gemm_noalloc", "bs_gemm_noalloc_max_scratch_bytes", "bs_selftest_dirty_noalloc_scratch",
-            "bs_tc_weights_bytes", "bs_tc_prepare_weights", "bs_tc_supported", "bitserial_conv2d_tc", "bitserial_conv2d_tc_chained", "bs_tc_chain_workspace_bytes", "bitserial_conv2d_tc_chain", "bitserial_gemm_tc", "bs_l2_prefetch",
+            "bs_tc_weights_bytes", "bs_tc_prepare_weights", "bs_tc_supported", "bitserial_conv2d_tc", "bitserial_conv2d_tc_chained", "bs_tc_chain_workspace_bytes", "bitserial_conv2d_tc_chain", "bitserial_gemm_tc", "bs_sequence_create", "bs_sequence_run", "bs_sequence_destroy", "bs_l2_prefetch",
             "bs_conv2d_f32", "bs_maxpool2d_f32", "bs_avgpool_codes_f32", "bs_fc_f32",
             "bs_check_status", "bs_quantiser_bounds", "bs_requant_bounds", "bs_selftest_wait_timeout", "bs_popc_rate", "bs_status_string")

@@ -245,6 +245,13 @@ def bitserial_conv2d_tc_chain(acts, wgts_tc, params, outs, workspace: torch.Tens
     _check(st, "bitserial_conv2d_tc_chain")
 
 
+def run_sequence(sequence, launches: int, stream=None) -> None:
+    """One pass of a bound sequence of layers (``bs_sequence_run``), which enqueues ``launches`` kernels."""
+    global launch_count
+    _check(lib().bs_sequence_run(sequence, _stream_ptr(stream)), "bs_sequence_run")
+    launch_count += launches - 1
+
+
 def bitserial_gemm_tc(a_packed: torch.Tensor, w_tc: torch.Tensor, N: int, K: int, w_bits: int, *, a_sign: int = UNSIGNED,
                       w_sign: int = SIGNED, scale=None, bias=None, relu: bool = False, out_bits: int = 0,
                       out_sign: int = UNSIGNED, want_i32: bool = True, out_i32: Optional[torch.Tensor] = None,

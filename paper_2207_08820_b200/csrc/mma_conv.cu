@@ -4,7 +4,9 @@
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
+#include <new>
 #include <unordered_map>
+#include <vector>
 
 #include "mma_kernel.cuh"
 
@@ -395,12 +397,12 @@ static bool encode_rows(CUtensorMap* tm, const uint32_t* base, int rows, int wor
               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-int mma_conv_run(const uint32_t* act, const int8_t* wgt, const uint32_t* wgt_packed, const bs_conv_params* p, int32_t* out_i32,
-                 uint32_t* out_packed, cudaStream_t st, bool chained, bool plan_only)
+// Plan of a layer with its pointers filled in.
+static int bind_plan(MmaPlan& plan, const uint32_t* act, const int8_t* wgt, const uint32_t* wgt_packed, const bs_conv_params* p, int32_t* out_i32,
+                     uint32_t* out_packed, bool chained, bool plan_only)
 {
     const int flags = (wgt ? MM_PREPARED : 0) | (out_i32 ? MM_I32 : 0) | (out_packed ? MM_CODES : 0) | (out_packed && p->residual ? MM_RESIDUAL : 0) |
                       (chained ? MM_CHAINED : 0) | (plan_only ? MM_QUERY : 0);
-    MmaPlan plan;
     const int rc = find_plan(plan, p, flags);
     if (rc != BS_OK || plan_only) return rc;
     MmaArgs& g = plan.g;
@@ -408,27 +410,103 @@ int mma_conv_run(const uint32_t* act, const int8_t* wgt, const uint32_t* wgt_pac
     g.scale = p->scale; g.bias = p->bias;
     g.residual = out_packed ? p->residual : nullptr;
     if (g.tma) {
-        const int fb = !wgt && g.nsb > 0;
         if (!encode_rows(&g.tmA, act, g.total, g.Cw * p->a_bits, g.rowA, 128 * g.PT < 256 ? 128 * g.PT : 256)) return BS_ERR_CUDA;
-        if (fb && !encode_rows(&g.tmB, wgt_packed, g.O, g.Cw * p->w_bits, g.rowB, g.TN)) return BS_ERR_CUDA;
+        if (!wgt && g.nsb > 0 && !encode_rows(&g.tmB, wgt_packed, g.O, g.Cw * p->w_bits, g.rowB, g.TN)) return BS_ERR_CUDA;
     }
+    return BS_OK;
+}
+
+// Every launch may start while the kernel before it drains (barriers, tensor memory, filter fetch when the caller allows); the
+// kernel waits for that kernel itself before it reads or writes anything the stream orders.
+static int launch_plan(const MmaPlan& plan, cudaStream_t st)
+{
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(plan.grid);
     cfg.blockDim = dim3(plan.block);
     cfg.dynamicSmemBytes = static_cast<size_t>(plan.smem);
     cfg.stream = st;
-    // Every launch may start while the kernel before it drains (barriers, tensor memory, filter fetch when the caller allows);
-    // the kernel waits for that kernel itself before it reads or writes anything the stream orders.
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, plan.kern, g) != cudaSuccess) {
+    if (cudaLaunchKernelEx(&cfg, plan.kern, plan.g) != cudaSuccess) {
         cudaGetLastError();
         return BS_ERR_CUDA;
     }
     return BS_OK;
 }
+
+int mma_conv_run(const uint32_t* act, const int8_t* wgt, const uint32_t* wgt_packed, const bs_conv_params* p, int32_t* out_i32,
+                 uint32_t* out_packed, cudaStream_t st, bool chained, bool plan_only)
+{
+    MmaPlan plan;
+    const int rc = bind_plan(plan, act, wgt, wgt_packed, p, out_i32, out_packed, chained, plan_only);
+    return rc != BS_OK || plan_only ? rc : launch_plan(plan, st);
+}
+
+// A bound sequence of layers: plans, pointers and tensor maps as of its creation, the events of its forks and joins.
+struct Sequence {
+    struct Step {
+        MmaPlan plan;
+        cudaEvent_t fork, done;     // set for a step that runs beside its successors
+        int join[4];                // steps beside which this one must have finished, -1: none
+    };
+    std::vector<Step> steps;
+    cudaStream_t side;
+    ~Sequence()
+    {
+        for (Step& s : steps) {
+            if (s.fork) cudaEventDestroy(s.fork);
+            if (s.done) cudaEventDestroy(s.done);
+        }
+    }
+};
+
+int mma_sequence_create(const bs_sequence_layer* layers, int n, cudaStream_t side, Sequence** out)
+{
+    Sequence* q = new (std::nothrow) Sequence;
+    if (!q) return BS_ERR_CUDA;
+    q->side = side;
+    q->steps.resize(static_cast<size_t>(n));
+    for (Sequence::Step& s : q->steps) s.fork = s.done = nullptr;
+    for (int i = 0; i < n; ++i) {
+        const bs_sequence_layer& l = layers[i];
+        Sequence::Step& s = q->steps[i];
+        // a layer beside its successors starts from an event, not from the kernel before it: no early filter fetch
+        int rc = bind_plan(s.plan, l.act_packed, l.wgt_tc, l.wgt_packed, &l.p, nullptr, l.out_packed, l.chained && !l.aside, false);
+        for (int k = 0; k < 4; ++k) {
+            s.join[k] = l.join[k];
+            if (l.join[k] >= i) rc = BS_ERR_INVALID_ARG;
+        }
+        if (rc == BS_OK && l.aside &&
+            (cudaEventCreateWithFlags(&s.fork, cudaEventDisableTiming) != cudaSuccess || cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming) != cudaSuccess)) {
+            cudaGetLastError();
+            rc = BS_ERR_CUDA;
+        }
+        if (rc != BS_OK) { delete q; return rc; }
+    }
+    *out = q;
+    return BS_OK;
+}
+
+int mma_sequence_run(Sequence* q, cudaStream_t st)
+{
+    for (Sequence::Step& s : q->steps) {
+        cudaStream_t on = st;
+        for (int k = 0; k < 4 && s.join[k] >= 0; ++k)
+            if (cudaStreamWaitEvent(st, q->steps[s.join[k]].done, 0) != cudaSuccess) { cudaGetLastError(); return BS_ERR_CUDA; }
+        if (s.fork) {
+            if (cudaEventRecord(s.fork, st) != cudaSuccess || cudaStreamWaitEvent(q->side, s.fork, 0) != cudaSuccess) { cudaGetLastError(); return BS_ERR_CUDA; }
+            on = q->side;
+        }
+        const int rc = launch_plan(s.plan, on);
+        if (rc != BS_OK) return rc;
+        if (s.done && cudaEventRecord(s.done, on) != cudaSuccess) { cudaGetLastError(); return BS_ERR_CUDA; }
+    }
+    return BS_OK;
+}
+
+void mma_sequence_destroy(Sequence* q) { delete q; }
 
 }  // namespace bs

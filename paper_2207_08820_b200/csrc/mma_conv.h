@@ -19,4 +19,10 @@ __host__ __device__ constexpr int mma_channel_of_byte(int b) { return 8 * (b & 3
 int mma_conv_run(const uint32_t* act, const int8_t* wgt, const uint32_t* wgt_packed, const bs_conv_params* p, int32_t* out_i32,
                  uint32_t* out_packed, cudaStream_t st, bool chained, bool plan_only);
 
+// A sequence of layers bound to its tensors (bs_sequence_*); the layers have been validated.
+struct Sequence;
+int mma_sequence_create(const bs_sequence_layer* layers, int n, cudaStream_t side, Sequence** out);
+int mma_sequence_run(Sequence* q, cudaStream_t st);
+void mma_sequence_destroy(Sequence* q);
+
 }  // namespace bs

@@ -42,7 +42,7 @@ static int tc_max_abs(int bits, int sign)
 }
 
 // Validation shared by the support query and the launch.  Returns BS_OK when the tensor-core path can run `p`.
-static int tc_validate(const bs_conv_params* p)
+static int tc_validate_shape(const bs_conv_params* p)
 {
     if (!p) return BS_ERR_INVALID_ARG;
     if (p->N <= 0 || p->C <= 0 || p->H <= 0 || p->W <= 0 || p->O <= 0 || p->R <= 0 || p->S <= 0) return BS_ERR_INVALID_ARG;
@@ -53,23 +53,29 @@ static int tc_validate(const bs_conv_params* p)
     if (p->stride > 2 || p->pad >= p->R) return BS_ERR_UNSUPPORTED;
     if (p->a_sign == BS_BIPOLAR && p->pad != 0) return BS_ERR_UNSUPPORTED;
     if (p->H + 2 * p->pad < p->R || p->W + 2 * p->pad < p->S) return BS_ERR_INVALID_ARG;
-    if (p->C % 32 != 0) return BS_ERR_UNSUPPORTED;
-    {
-        // packed pixel records must be 16-byte multiples, or 8-byte multiples on rows that are 16-byte multiples
-        const int fullA = ceil_div(p->C, 32) * p->a_bits;
-        const bool flat = p->R == 1 && p->stride == 1 && p->pad == 0;
-        if (fullA % 4 != 0) {
-            if (fullA % 2 != 0 || (p->W * fullA) % 4 != 0) return BS_ERR_UNSUPPORTED;
-            if (flat && (static_cast<long long>(p->N) * p->H * p->W) % 2 != 0) return BS_ERR_UNSUPPORTED;
-        }
-    }
     const long long kred = static_cast<long long>(p->C) * p->R * p->S;
     if (kred * tc_max_abs(p->a_bits, p->a_sign) * tc_max_abs(p->w_bits, p->w_sign) >= (1LL << 31)) return BS_ERR_UNSUPPORTED;
     return BS_OK;
 }
 
+// What can be run with prepared filters: channels that fill their words (the prepared tiles have no ragged block), and packed pixel
+// records of 16-byte multiples, or of 8-byte multiples on rows that are 16-byte multiples (a contract of the entry points; the
+// kernels themselves take any record).
+static int tc_validate(const bs_conv_params* p)
+{
+    const int rc = tc_validate_shape(p);
+    if (rc != BS_OK) return rc;
+    if (p->C % 32 != 0) return BS_ERR_UNSUPPORTED;
+    const int rec = p->C / 32 * p->a_bits;
+    if (rec % 4 != 0) {
+        if (rec % 2 != 0 || (p->W * rec) % 4 != 0) return BS_ERR_UNSUPPORTED;
+        if (p->R == 1 && p->stride == 1 && p->pad == 0 && (static_cast<long long>(p->N) * p->H * p->W) % 2 != 0) return BS_ERR_UNSUPPORTED;
+    }
+    return BS_OK;
+}
+
 // Output side of the validation (pointers, code formats, channel slices).
-static int tc_validate_outputs(const uint32_t* act, const int8_t* wgt, const bs_conv_params* p, const int32_t* out_i32, const uint32_t* out_packed)
+static int tc_validate_outputs(const uint32_t* act, const void* wgt, const bs_conv_params* p, const int32_t* out_i32, const uint32_t* out_packed)
 {
     if (!act || !wgt || (!out_i32 && !out_packed)) return BS_ERR_INVALID_ARG;
     if (!aligned16(act) || !aligned16(wgt) || (out_i32 && !aligned16(out_i32)) || (out_packed && !aligned16(out_packed))) return BS_ERR_ALIGNMENT;
@@ -229,3 +235,25 @@ extern "C" int bitserial_gemm_tc(const uint32_t* a_packed, const int8_t* w_tc, i
     p.out_c_offset = 0; p.out_c_total = N; p.i32_layout = BS_NHWC;
     return bs::tc_conv_impl(a_packed, w_tc, &p, out_i32, out_packed, static_cast<cudaStream_t>(stream), false);
 }
+
+extern "C" int bs_sequence_create(const bs_sequence_layer* layers, int nlayers, void* side_stream, bs_sequence** out)
+{
+    if (!layers || nlayers <= 0 || !out) return BS_ERR_INVALID_ARG;
+    for (int l = 0; l < nlayers; ++l) {
+        const bs_sequence_layer& s = layers[l];
+        if (!s.wgt_tc && !s.wgt_packed) return BS_ERR_INVALID_ARG;
+        int rc = bs::tc_validate_shape(&s.p);
+        if (rc == BS_OK && s.wgt_tc) rc = bs::tc_validate(&s.p);
+        if (rc == BS_OK) rc = bs::tc_validate_outputs(s.act_packed, s.wgt_tc ? static_cast<const void*>(s.wgt_tc) : s.wgt_packed, &s.p, nullptr, s.out_packed);
+        if (rc != BS_OK) return rc;
+        if (s.aside && !side_stream) return BS_ERR_INVALID_ARG;
+    }
+    return bs::mma_sequence_create(layers, nlayers, static_cast<cudaStream_t>(side_stream), reinterpret_cast<bs::Sequence**>(out));
+}
+
+extern "C" int bs_sequence_run(bs_sequence* sequence, void* stream)
+{
+    return sequence ? bs::mma_sequence_run(reinterpret_cast<bs::Sequence*>(sequence), static_cast<cudaStream_t>(stream)) : BS_ERR_INVALID_ARG;
+}
+
+extern "C" void bs_sequence_destroy(bs_sequence* sequence) { bs::mma_sequence_destroy(reinterpret_cast<bs::Sequence*>(sequence)); }

@@ -1,18 +1,37 @@
 """Runs a stack of quantised conv layers (``workloads.NetSpec``) through the C ABI.
 
-Host logic only: buffer planning, weight packing at set-up, one ``bitserial_conv2d`` call per layer -- or one
-``bitserial_conv2d_tc_chain`` call per run of same-shaped layers -- (residual adds and concatenations are epilogue
-arguments), optional CUDA-graph replay.
+Host logic only: buffer planning, weight packing at set-up, the layers bound once as a ``bs_sequence`` and run by one call per
+pass (residual adds and concatenations are epilogue arguments), optional CUDA-graph replay.
 """
 from __future__ import annotations
 
+import ctypes
+import weakref
 from typing import Dict, List, Optional
 
 import numpy as np
 import torch
 
 from . import api
+from ._lib import SequenceLayer, lib
 from .workloads import NetSpec
+
+
+class _Buffers(dict):
+    """Activation tensors by name; ``version`` changes when one is replaced (a bound sequence holds their addresses)."""
+    version = 0
+
+    def __setitem__(self, key, value):
+        self.version += 1
+        super().__setitem__(key, value)
+
+
+class _Sequence:
+    """A ``bs_sequence`` and the tensors it holds the addresses of."""
+
+    def __init__(self, handle: int, tensors):
+        self.handle, self.tensors = handle, tensors
+        weakref.finalize(self, lib().bs_sequence_destroy, handle).atexit = False
 
 
 class BitserialNet:
@@ -22,10 +41,9 @@ class BitserialNet:
                  engine: str = "popc", concurrent: bool = True, chains="auto"):
         """engine: "popc" = popcount kernels on the integer pipes; "tc" = tensor-core entry point for every layer it
         supports (others fall back to the popcount kernel).  concurrent: launch independent neighbouring layers on
-        two streams (see :meth:`run_layers`).  chains: with the "tc" engine, runs of consecutive same-shaped layers can go
-        through ``bitserial_conv2d_tc_chain`` (one launch per run) where the library accepts them: True = always,
-        False = never, "auto" = each such run is timed both ways at set-up and the faster form is kept (the chain wins
-        where launches dominate -- small batches -- and loses where every layer already fills the GPU)."""
+        two streams (see :meth:`schedule`).  chains: with the "tc" engine, runs of consecutive same-shaped layers can go
+        through ``bitserial_conv2d_tc_chain`` (one call per run) where the library accepts them: True = always, False and
+        "auto" = one call per layer (the launches are the same)."""
         self.net = net
         self.engine = engine
         self.act_scale = float(act_scale)
@@ -47,29 +65,25 @@ class BitserialNet:
                 w_sign=p["w_sign"],
                 scale=torch.from_numpy(p["scale"]).to(self.device),
                 bias=torch.from_numpy(p["bias"]).to(self.device)))
-        self.bufs: Dict[str, torch.Tensor] = {}
+        self.bufs: Dict[str, torch.Tensor] = _Buffers()
         for name, (C, H, W) in self.shapes.items():
             self.bufs[name] = torch.zeros(self.batch, H, W, (C + 31) // 32, net.a_bits, dtype=torch.int32, device=self.device)
-        self.units = self._plan_units(bool(chains) and engine == "tc")
+        self.units = self._plan_units(chains is True and engine == "tc")
         torch.cuda.synchronize(self.device)   # chained layers fetch filters, scale and bias ahead of stream order
-        if chains == "auto":
-            self.units = self._keep_faster_units(self.units)
         self.concurrent = concurrent
         self.side = torch.cuda.Stream(device=self.device)
         self.graph = None
         self.static_in = None
-        self.launches_per_forward = 2 + len(self.units)
+        self.launches_per_forward = 1 + len(self.layers)
+        self._sequence = self._sequence_key = None
+        self._bind()
 
     def _layer_params(self, item):
         """``bs_conv_params`` of a layer as a chain would run it, or None when its output is a slice of a wider tensor."""
         net, L = self.net, item["spec"]
         if L.dst_c_offset != 0 or self.shapes[L.dst][0] != L.O or (L.res and self.shapes[L.res][0] != L.O):
             return None
-        return api.conv_params(
-            self.bufs[L.src].shape, item["w"].shape, C=L.C, stride=L.stride, pad=L.pad, a_sign=api.UNSIGNED, w_sign=item["w_sign"],
-            scale=item["scale"], bias=item["bias"], relu=L.relu, out_bits=net.a_bits, out_sign=api.UNSIGNED,
-            residual=self.bufs[L.res] if L.res else None, res_scale=L.res_scale, res_bits=net.a_bits if L.res else 0,
-            res_sign=api.UNSIGNED)
+        return self._conv_params(item)
 
     def _plan_units(self, chains: bool) -> List[Dict]:
         """The launches of a forward pass: single layers, and runs of up to MAX_CHAIN consecutive layers that the library
@@ -110,54 +124,9 @@ class BitserialNet:
         return self.bufs[self.net.out_name]
 
     def pack_input(self, x: torch.Tensor) -> None:
-        """Quantise + bitplane-pack the fp32 input on the current stream; the filter prefetch runs beside it on the
-        side stream (a fork and a join: two parallel nodes under stream capture)."""
+        """Quantise + bitplane-pack the fp32 input on the current stream."""
         net = self.net
-        main = torch.cuda.current_stream(self.device)
-        fork = torch.cuda.Event()
-        fork.record(main)
-        self.side.wait_event(fork)
-        with torch.cuda.stream(self.side):
-            self.prefetch_filters()
-            done = torch.cuda.Event()
-            done.record(self.side)
         api.bitpack_activations(x, self.act_scale, net.a_bits, api.UNSIGNED, api.NCHW, out=self.bufs[net.in_name].view(-1))
-        main.wait_event(done)
-
-    def _time_units(self, units, reps: int = 8) -> float:
-        """Microseconds per pass of `units` launched back to back (as inside a forward pass), from a CUDA graph of `reps` passes."""
-        stream = torch.cuda.Stream(device=self.device)
-        with torch.cuda.stream(stream):
-            for u in units:
-                self.run_unit(u, chained=False)
-            stream.synchronize()
-            graph = torch.cuda.CUDAGraph()
-            with torch.cuda.graph(graph, stream=stream):
-                for _ in range(reps):
-                    for u in units:
-                        self.run_unit(u)
-            best = float("inf")
-            for _ in range(4):
-                e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-                e0.record(stream)
-                graph.replay()
-                e1.record(stream)
-                e1.synchronize()
-                best = min(best, e0.elapsed_time(e1) * 1e3 / reps)
-        return best
-
-    def _keep_faster_units(self, units):
-        out = []
-        for u in units:
-            if u["params"] is None:
-                out.append(u)
-                continue
-            singles = [dict(items=[it], params=None, workspace=None) for it in u["items"]]
-            t_chain, t_single = self._time_units([u]), self._time_units(singles)
-            u["timing_us"] = (t_chain, t_single)
-            out.extend([u] if t_chain < t_single else singles)
-        torch.cuda.synchronize(self.device)
-        return out
 
     def run_layer(self, item, chained: bool = True) -> None:
         """One conv layer through the C ABI on the current stream."""
@@ -181,13 +150,13 @@ class BitserialNet:
         api.bitserial_conv2d_tc_chain([self.bufs[it["spec"].src] for it in items], [it["w_tc"] for it in items], params,
                                       [self.bufs[it["spec"].dst] for it in items], unit["workspace"], chained=chained)
 
-    def run_layers(self) -> None:
-        """All launches in order.  With ``concurrent`` a single layer whose successor neither reads nor overwrites its
-        output (a projection shortcut beside the first conv of its block, the two 1x1 branches of a cross-stage block) is
-        launched on a side stream, so the two kernels share the GPU; events carry the dependencies, and under stream
-        capture they become the edges of the graph."""
-        main = torch.cuda.current_stream(self.device)
-        pending: Dict[str, torch.cuda.Event] = {}
+    def schedule(self):
+        """The launches in order: (unit, aside, join).  With ``concurrent`` a single layer whose successor neither reads nor
+        overwrites its output (a projection shortcut beside the first conv of its block, the two 1x1 branches of a cross-stage
+        block) runs ``aside`` on a second stream when its tiles do not fill the GPU: one wave of 128 x 128 output tiles leaves room for
+        the neighbour (batch 1 residual stack 124 -> 114 us; where both fill the GPU, sharing it costs more than it
+        hides: detection stack of batch 16 351 -> 356 us).  ``join``: positions of the launches that must be waited for first."""
+        out, pending = [], {}
         n = len(self.units)
 
         def touched(unit):
@@ -204,28 +173,87 @@ class BitserialNet:
             aside = False
             if self.concurrent and i + 1 < n and len(unit["items"]) == 1:
                 nreads, nwrites = touched(self.units[i + 1])
-                aside = (not (wnames & nreads) and not ({d for d, _ in nwrites} & reads) and not (writes & nwrites)
+                L = unit["items"][0]["spec"]
+                _, P, Q = self.shapes[L.dst]
+                small = -(-self.batch * P * Q // 128) * -(-L.O // 128) <= 148
+                aside = (small and not (wnames & nreads) and not ({d for d, _ in nwrites} & reads) and not (writes & nwrites)
                          and not (reads & set(pending)))
+            join = []
+            if aside:
+                pending.update({d: i for d in wnames})
+            else:
+                join = sorted({pending.pop(t) for t in list(reads | wnames) if t in pending})
+                if i + 1 == n:                      # the pass ends with its last launch
+                    join = sorted(set(join) | set(pending.values()))
+            out.append((unit, aside, join))
+        return out
+
+    def run_layers(self) -> None:
+        """All layers on the current stream, and on the side stream those that :meth:`schedule` puts there; under stream capture the
+        events between them become the edges of the graph."""
+        if self._bind():
+            api.run_sequence(self._sequence.handle, len(self.layers))
+            return
+        main = torch.cuda.current_stream(self.device)
+        done: Dict[int, torch.cuda.Event] = {}
+        for i, (unit, aside, join) in enumerate(self.schedule()):
             if aside:
                 fork = torch.cuda.Event()
                 fork.record(main)
                 self.side.wait_event(fork)
                 with torch.cuda.stream(self.side):
                     self.run_unit(unit, chained=False)
-                    done = torch.cuda.Event()
-                    done.record(self.side)
-                for d in wnames:
-                    pending[d] = done
+                    done[i] = torch.cuda.Event()
+                    done[i].record(self.side)
                 continue
-            for t in reads | wnames:
-                if t in pending:
-                    main.wait_event(pending.pop(t))
+            for k in join:
+                main.wait_event(done[k])
             self.run_unit(unit)
-        for ev in pending.values():
-            main.wait_event(ev)
+
+    def _bind(self) -> bool:
+        """Binds the layers to their present tensors as one sequence; False where the library does not take them as one."""
+        key = (self.bufs.version, self.concurrent, id(self.units))
+        if key == self._sequence_key:
+            return self._sequence is not None
+        self._sequence_key, self._sequence = key, None
+        steps = self.schedule()
+        at, layers = {}, []                          # position of a launch among the layers
+        for i, (unit, aside, join) in enumerate(steps):
+            for k, item in enumerate(unit["items"]):
+                if k == 0:
+                    at[i] = len(layers)
+                layers.append((item, aside, [at[j] for j in join] if k == 0 else []))
+        if any(len(j) > 4 for _, _, j in layers):
+            return False
+        arr = (SequenceLayer * len(layers))()
+        for q, (item, aside, join) in zip(arr, layers):
+            L = item["spec"]
+            q.act_packed, q.out_packed = self.bufs[L.src].data_ptr(), self.bufs[L.dst].data_ptr()
+            q.wgt_packed = item["w"].data_ptr()
+            q.wgt_tc = item["w_tc"].data_ptr() if item["w_tc"] is not None else None
+            q.p = self._conv_params(item)
+            q.chained, q.aside = 1, int(aside)
+            q.join[:] = (join + [-1] * 4)[:4]
+        handle = ctypes.c_void_p()
+        if lib().bs_sequence_create(arr, len(layers), self.side.cuda_stream, ctypes.byref(handle)) != 0:
+            return False
+        self._sequence = _Sequence(handle.value, [self.bufs[n] for n in self.shapes])
+        return True
+
+    def _conv_params(self, item):
+        net, L = self.net, item["spec"]
+        q = api.conv_params(
+            self.bufs[L.src].shape, item["w"].shape, C=L.C, stride=L.stride, pad=L.pad, a_sign=api.UNSIGNED, w_sign=item["w_sign"],
+            scale=item["scale"], bias=item["bias"], relu=L.relu, out_bits=net.a_bits, out_sign=api.UNSIGNED,
+            residual=self.bufs[L.res] if L.res else None, res_scale=L.res_scale, res_bits=net.a_bits if L.res else 0,
+            res_sign=api.UNSIGNED)
+        q.res_c_total = self.shapes[L.res][0] if L.res else L.O
+        q.out_c_offset, q.out_c_total = L.dst_c_offset, self.shapes[L.dst][0]
+        return q
 
     def prefetch_filters(self) -> None:
-        """The filters of every layer start on their way into L2 while the pack kernel and the first layers run."""
+        """A hint before a pass whose filters have left L2: they start on their way there (a separate launch; a pass does not issue it,
+        since it gains nothing while the filters are still in L2)."""
         api.l2_prefetch([item["w_tc"] if item["w_tc"] is not None else item["w"] for item in self.layers])
 
     def forward(self, x: torch.Tensor) -> torch.Tensor:
