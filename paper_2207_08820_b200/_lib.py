@@ -7,6 +7,7 @@ import os
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libbitserial_b200.so")
 _lib = None
+_native = None
 
 
 class BitserialError(RuntimeError):
@@ -39,6 +40,20 @@ class SequenceLayer(ctypes.Structure):
     """Mirror of ``bs_sequence_layer`` (include/bitserial.h)."""
     _fields_ = [("act_packed", ctypes.c_void_p), ("wgt_tc", ctypes.c_void_p), ("wgt_packed", ctypes.c_void_p), ("out_packed", ctypes.c_void_p),
                 ("p", ConvParams), ("chained", ctypes.c_int), ("aside", ctypes.c_int), ("join", ctypes.c_int * 4)]
+
+
+def native():
+    """The compiled binding (csrc/binding.cpp), linked against the library beside it."""
+    global _native
+    if _native is None:
+        lib()
+        try:
+            from . import _binding
+        except ImportError as e:
+            raise ImportError("the compiled binding is missing or stale: build it with `python -m paper_2207_08820_b200.build`.  "
+                              "There is no CPU or PyTorch fallback.") from e
+        _native = _binding
+    return _native
 
 
 def lib() -> ctypes.CDLL:

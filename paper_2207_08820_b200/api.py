@@ -11,7 +11,7 @@ from typing import Optional
 
 import torch
 
-from ._lib import BitserialError, ConvParams, lib
+from ._lib import BitserialError, ConvParams, lib, native
 
 UNSIGNED, SIGNED, BIPOLAR = 0, 1, 2
 NCHW, NHWC = 0, 1
@@ -59,19 +59,9 @@ def bitpack_activations(x: torch.Tensor, act_scale: float, a_bits: int, a_sign: 
                         layout: int = NCHW, out: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """x: float32 or int8 (codes), [N,C,H,W] (NCHW) or [N,H,W,C] (NHWC).  Returns int32 words
     viewed as [N, H, W, Cw, a_bits]."""
-    if x.dtype not in (torch.float32, torch.int8):
-        raise ValueError("x must be float32 or int8")
-    if layout == NCHW:
-        N, C, H, W = x.shape
-    else:
-        N, H, W, C = x.shape
-    Cw = (C + 31) // 32
-    if out is None:
-        out = _words(N * H * W * Cw * a_bits, x.device)
-    st = lib().bitpack_activations(_ptr(x), int(x.dtype == torch.float32), layout, N, C, H, W,
-                                   ctypes.c_float(act_scale), a_bits, a_sign, _ptr(out), _stream_ptr(stream))
+    st, out, _ = native().bitpack(x, act_scale, a_bits, a_sign, layout, out, stream)
     _check(st, "bitpack_activations")
-    return out.view(N, H, W, Cw, a_bits)
+    return out
 
 
 def bitunpack_activations(packed: torch.Tensor, C: int, a_bits: int, a_sign: int = UNSIGNED, layout: int = NCHW,
@@ -121,40 +111,12 @@ def bitserial_conv2d(act_packed: torch.Tensor, wgt_packed: torch.Tensor, *, C: i
     ``wgt_tc`` (from :func:`tc_prepare_weights`) selects the tensor-core entry point ``bitserial_conv2d_tc``;
     with ``chained`` it is ``bitserial_conv2d_tc_chained`` (set-up overlaps the preceding kernel of the stream: filters,
     scale and bias must have been final before that kernel was launched)."""
-    N, H, W, Cw, a_bits = act_packed.shape
-    O, R, S, Cw2, w_bits = wgt_packed.shape
-    if Cw != Cw2 or Cw != (C + 31) // 32:
-        raise ValueError("channel words of activations and weights disagree")
-    P = (H + 2 * pad - R) // stride + 1
-    Q = (W + 2 * pad - S) // stride + 1
-    dev = act_packed.device
-    if want_i32 and out_i32 is None:
-        shape = (N, O, P, Q) if i32_layout == NCHW else (N, P, Q, O)
-        out_i32 = torch.empty(shape, dtype=torch.int32, device=dev)
-    if out_bits > 0:
-        if out_c_total == 0:
-            out_c_total = out_c_offset + O
-        if out_packed is None:
-            out_packed = torch.zeros(N, P, Q, (out_c_total + 31) // 32, out_bits, dtype=torch.int32, device=dev)
-    p = ConvParams(N=N, C=C, H=H, W=W, O=O, R=R, S=S, stride=stride, pad=pad, a_bits=a_bits, a_sign=a_sign,
-                   w_bits=w_bits, w_sign=w_sign, scale=_ptr(scale), bias=_ptr(bias), relu=int(relu),
-                   out_bits=out_bits, out_sign=out_sign, residual=_ptr(residual), res_scale=res_scale,
-                   res_bits=res_bits, res_sign=res_sign, res_c_offset=res_c_offset,
-                   res_c_total=res_c_total if res_c_total else res_c_offset + O,
-                   out_c_offset=out_c_offset, out_c_total=out_c_total, i32_layout=i32_layout)
-    if wgt_tc is not None:
-        entry = lib().bitserial_conv2d_tc_chained if chained else lib().bitserial_conv2d_tc
-        st = entry(_ptr(act_packed), _ptr(wgt_tc), ctypes.byref(p), _ptr(out_i32),
-                   _ptr(out_packed) if out_bits > 0 else None, _stream_ptr(stream))
-    elif workspace is not None:
-        st = lib().bitserial_conv2d_ws(_ptr(act_packed), _ptr(wgt_packed), ctypes.byref(p), _ptr(out_i32),
-                                       _ptr(out_packed) if out_bits > 0 else None, _ptr(workspace),
-                                       workspace.numel() * workspace.element_size(), _stream_ptr(stream))
-    else:
-        st = lib().bitserial_conv2d(_ptr(act_packed), _ptr(wgt_packed), ctypes.byref(p), _ptr(out_i32),
-                                    _ptr(out_packed) if out_bits > 0 else None, _stream_ptr(stream))
+    st, out_i32, out_packed = native().conv2d(
+        act_packed, wgt_packed, C, stride, pad, a_sign, w_sign, scale, bias, relu, out_bits, out_sign, residual, res_scale, res_bits,
+        res_sign, res_c_offset, res_c_total, out_i32, want_i32, i32_layout, out_packed, out_c_offset, out_c_total, workspace, wgt_tc,
+        chained, stream)
     _check(st, "bitserial_conv2d")
-    return out_i32, (out_packed if out_bits > 0 else None)
+    return out_i32, out_packed
 
 
 def bitserial_gemm(a_packed: torch.Tensor, w_packed: torch.Tensor, K: int, *, a_sign: int = UNSIGNED,
@@ -164,26 +126,10 @@ def bitserial_gemm(a_packed: torch.Tensor, w_packed: torch.Tensor, K: int, *, a_
                    out_packed: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None, stream=None):
     """a_packed [M,Kw,a_bits], w_packed [N,Kw,w_bits].  Returns (out_i32 [M,N] or None, out_packed or None).
     ``workspace`` (zeroed device tensor, see :func:`gemm_workspace`) enables the reduction split (``bitserial_gemm_ws``)."""
-    M, Kw, a_bits = a_packed.shape
-    N, Kw2, w_bits = w_packed.shape
-    if Kw != Kw2 or Kw != (K + 31) // 32:
-        raise ValueError("reduction words of the operands disagree")
-    dev = a_packed.device
-    if want_i32 and out_i32 is None:
-        out_i32 = torch.empty(M, N, dtype=torch.int32, device=dev)
-    if out_bits > 0 and out_packed is None:
-        out_packed = torch.zeros(M, (N + 31) // 32, out_bits, dtype=torch.int32, device=dev)
-    if workspace is not None:
-        st = lib().bitserial_gemm_ws(_ptr(a_packed), _ptr(w_packed), M, N, K, a_bits, a_sign, w_bits, w_sign,
-                                     _ptr(scale), _ptr(bias), int(relu), out_bits, out_sign, _ptr(out_i32),
-                                     _ptr(out_packed) if out_bits > 0 else None, _ptr(workspace),
-                                     workspace.numel() * workspace.element_size(), _stream_ptr(stream))
-    else:
-        st = lib().bitserial_gemm(_ptr(a_packed), _ptr(w_packed), M, N, K, a_bits, a_sign, w_bits, w_sign,
-                                  _ptr(scale), _ptr(bias), int(relu), out_bits, out_sign, _ptr(out_i32),
-                                  _ptr(out_packed) if out_bits > 0 else None, _stream_ptr(stream))
+    st, out_i32, out_packed = native().gemm(a_packed, w_packed, -1, -1, K, a_sign, w_sign, scale, bias, relu, out_bits, out_sign,
+                                            out_i32, want_i32, out_packed, workspace, stream)
     _check(st, "bitserial_gemm")
-    return out_i32, (out_packed if out_bits > 0 else None)
+    return out_i32, out_packed
 
 
 def tc_prepare_weights(wgt_packed: torch.Tensor, C: int, w_sign: int, a_bits: int, stream=None) -> torch.Tensor:
@@ -248,7 +194,7 @@ def bitserial_conv2d_tc_chain(acts, wgts_tc, params, outs, workspace: torch.Tens
 def run_sequence(sequence, launches: int, stream=None) -> None:
     """One pass of a bound sequence of layers (``bs_sequence_run``), which enqueues ``launches`` kernels."""
     global launch_count
-    _check(lib().bs_sequence_run(sequence, _stream_ptr(stream)), "bs_sequence_run")
+    _check(native().sequence_run(sequence, stream), "bs_sequence_run")
     launch_count += launches - 1
 
 
@@ -257,16 +203,8 @@ def bitserial_gemm_tc(a_packed: torch.Tensor, w_tc: torch.Tensor, N: int, K: int
                       out_sign: int = UNSIGNED, want_i32: bool = True, out_i32: Optional[torch.Tensor] = None,
                       out_packed: Optional[torch.Tensor] = None, stream=None):
     """Tensor-core matrix product: a_packed [M,Kw,a_bits], w_tc from tc_prepare_weights on the [N,1,1,Kw,w_bits] rows."""
-    M, Kw, a_bits = a_packed.shape
-    dev = a_packed.device
-    if want_i32 and out_i32 is None:
-        out_i32 = torch.empty(M, N, dtype=torch.int32, device=dev)
-    if out_bits > 0 and out_packed is None:
-        out_packed = torch.zeros(M, (N + 31) // 32, out_bits, dtype=torch.int32, device=dev)
-    if out_bits <= 0:
-        out_packed = None
-    st = lib().bitserial_gemm_tc(_ptr(a_packed), _ptr(w_tc), M, N, K, a_bits, a_sign, w_bits, w_sign, _ptr(scale), _ptr(bias),
-                                 int(relu), out_bits, out_sign, _ptr(out_i32), _ptr(out_packed), _stream_ptr(stream))
+    st, out_i32, out_packed = native().gemm(a_packed, w_tc, N, w_bits, K, a_sign, w_sign, scale, bias, relu, out_bits, out_sign,
+                                            out_i32, want_i32, out_packed, None, stream)
     _check(st, "bitserial_gemm_tc")
     return out_i32, out_packed
 

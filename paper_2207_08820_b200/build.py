@@ -1,13 +1,15 @@
 """Builds the CUDA library in-tree: ``python -m paper_2207_08820_b200.build``.
 
 Every translation unit is compiled for sm_100a only (``-gencode arch=compute_100a,code=sm_100a``) and
-linked into ``libbitserial_b200.so`` beside this file.  Objects live in ``_build/`` (not versioned).
+linked into ``libbitserial_b200.so`` beside this file.  Objects live in ``_build/`` (not versioned).  ``_binding.so`` (host code only,
+csrc/binding.cpp) is the Python extension over it.
 """
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -15,6 +17,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libbitserial_b200.so")
+BINDING = os.path.join(HERE, "_binding.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC,
@@ -48,6 +51,22 @@ def _compile(src: str, verbose: bool) -> str:
     return obj
 
 
+def _build_binding(force: bool) -> None:
+    src = os.path.join(CSRC, "binding.cpp")
+    if not force and os.path.exists(BINDING) and os.path.getmtime(BINDING) >= max(os.path.getmtime(src), _headers_mtime()):
+        return
+    import torch
+    t = os.path.dirname(torch.__file__)
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"], "-I", os.path.join(t, "include"),
+           "-I", os.path.join(t, "include", "torch", "csrc", "api", "include"), "-I", "/usr/local/cuda/include", src, "-o", BINDING,
+           "-L", HERE, "-l:libbitserial_b200.so", "-L", os.path.join(t, "lib"), "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-ltorch",
+           "-lc10_cuda", "-lc10", "-Wl,-rpath,$ORIGIN"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError(f"g++ failed for binding.cpp:\n{res.stdout}\n{res.stderr}")
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
     stamp = os.path.join(BUILD, "flags.txt")
@@ -68,6 +87,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         res = subprocess.run(cmd, capture_output=True, text=True)
         if res.returncode != 0:
             raise RuntimeError(f"link failed:\n{res.stdout}\n{res.stderr}")
+    _build_binding(force)
     return LIB
 
 
