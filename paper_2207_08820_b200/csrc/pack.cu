@@ -7,10 +7,6 @@
 
 namespace bs {
 
-constexpr int PACK_THREADS = 256;
-constexpr int PACK_WARPS = PACK_THREADS / 32;
-constexpr int PACK_UNROLL = 8;      // NHWC: pixels in flight per warp
-
 // Quantiser of Section IV prepared for the device.  The decision
 //     code = round_half_even(clip(x / s, qmin, qmax))
 // is monotone in x, so it equals qmin + #{k : x >= bound[k]} where bound[k] is the smallest binary32 value whose
@@ -18,100 +14,11 @@ constexpr int PACK_UNROLL = 8;      // NHWC: pixels in flight per warp
 // same IEEE division, clip and rint, so the comparison form takes exactly the decision of the formula while costing
 // a few subtractions instead of a division (a binary search over the bounds for 3 and 4 bits).
 struct QuantParams {
-    float below[15];    // largest binary32 value below bound[k] (never -0): x >= bound[k]  <=>  sign bit of (below[k] - x) is set
+    float below[16];    // largest binary32 value below bound[k] (never -0): x >= bound[k]  <=>  sign bit of (below[k] - x) is set
     int bits, sign;
+    float inv, offset;  // estimate of the level, see LevelPlanes: x * inv + offset
+    int estimate;       // the scale is one for which the estimate holds
 };
-
-// Stored pattern of an int8 code as plane bits (the two's-complement low bits; bipolar: bit 0 = code > 0).
-template <int BITS>
-__device__ __forceinline__ unsigned code_pattern(int8_t x, int sign)
-{
-    if (sign == BS_BIPOLAR) return x > 0 ? 1u : 0u;
-    return static_cast<unsigned>(static_cast<int>(x)) & ((1u << BITS) - 1u);
-}
-
-// A warp copies the contiguous packed records of its tile from shared to global memory, as 128-bit stores when the
-// tile starts on a 16-byte boundary.
-__device__ __forceinline__ void store_tile_records(const uint32_t* stage, uint32_t* dst, int nwords, bool vec, int lane)
-{
-    if (vec) {
-        const int nvec = nwords / 4;
-        for (int k = lane; k < nvec; k += 32) reinterpret_cast<uint4*>(dst)[k] = reinterpret_cast<const uint4*>(stage)[k];
-        for (int k = nvec * 4 + lane; k < nwords; k += 32) dst[k] = stage[k];
-    } else {
-        for (int k = lane; k < nwords; k += 32) dst[k] = stage[k];
-    }
-}
-
-// Fallback for int8 codes in shapes the vector kernels below refuse (H*W not a multiple of 4 in NCHW, C not a multiple
-// of 32 in NHWC, bipolar codes).  One warp packs 32 consecutive pixels (flattened y*W + x) of one image, all channels,
-// with no block-wide barrier.
-//   NCHW: lane = pixel.  Every channel row is read with one coalesced request per warp, a whole 32-channel word in
-//         flight; each lane sets bit c of its own plane words from the pattern of channel c.
-//   NHWC: lane = channel.  One coalesced request per (pixel, 32-channel word); __ballot_sync over the 32 channels
-//         yields one plane word per vote.
-// The packed records of the 32 pixels are contiguous in global memory; they are parked in the warp's slice of
-// shared memory and leave through coalesced 128-bit stores.
-template <bool NHWC, int BITS>
-__global__ void __launch_bounds__(PACK_THREADS)
-bitpack_codes_kernel(const int8_t* __restrict__ x, uint32_t* __restrict__ out, int C, int HW, int Cw, long long ntiles,
-                     int tiles_per_img, int sign)
-{
-    extern __shared__ __align__(16) uint32_t pack_smem[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long tile = static_cast<long long>(blockIdx.x) * PACK_WARPS + warp;
-    if (tile >= ntiles) return;                       // whole warps leave; only __syncwarp is used below
-    const int rec = Cw * BITS;
-    uint32_t* stage = pack_smem + static_cast<size_t>(warp) * 32 * rec;      // [32 pixels][rec]
-    const long long n = tile / tiles_per_img;
-    const int hw0 = static_cast<int>(tile % tiles_per_img) * 32;
-    const int npix = min(32, HW - hw0);
-
-    if (NHWC) {
-        const int8_t* xin = x + (static_cast<size_t>(n) * HW + hw0) * C;
-        for (int cw = 0; cw < Cw; ++cw) {
-            const int c = cw * 32 + lane;
-            const bool cvalid = c < C;
-            for (int p0 = 0; p0 < 32; p0 += PACK_UNROLL) {
-                unsigned pat[PACK_UNROLL];
-#pragma unroll
-                for (int u = 0; u < PACK_UNROLL; ++u)
-                    pat[u] = (cvalid && p0 + u < npix) ? code_pattern<BITS>(xin[static_cast<size_t>(p0 + u) * C + c], sign) : 0u;
-#pragma unroll
-                for (int u = 0; u < PACK_UNROLL; ++u) {
-#pragma unroll
-                    for (int j = 0; j < BITS; ++j) {
-                        const unsigned word = __ballot_sync(0xffffffffu, (pat[u] >> j) & 1u);
-                        if (lane == j) stage[(p0 + u) * rec + cw * BITS + j] = word;
-                    }
-                }
-            }
-        }
-    } else {
-        const bool pvalid = lane < npix;
-        const int8_t* xin = x + static_cast<size_t>(n) * C * HW + hw0 + lane;
-        for (int cw = 0; cw < Cw; ++cw) {
-            uint32_t words[BITS];
-#pragma unroll
-            for (int j = 0; j < BITS; ++j) words[j] = 0u;
-            unsigned pat[32];
-#pragma unroll
-            for (int u = 0; u < 32; ++u) {
-                const int c = cw * 32 + u;
-                pat[u] = (pvalid && c < C) ? code_pattern<BITS>(xin[static_cast<size_t>(c) * HW], sign) : 0u;
-            }
-#pragma unroll
-            for (int u = 0; u < 32; ++u)
-#pragma unroll
-                for (int j = 0; j < BITS; ++j) words[j] |= ((pat[u] >> j) & 1u) << u;
-#pragma unroll
-            for (int j = 0; j < BITS; ++j) stage[lane * rec + cw * BITS + j] = words[j];
-        }
-    }
-    __syncwarp();
-    store_tile_records(stage, out + (static_cast<size_t>(n) * HW + hw0) * rec, npix * rec,
-                       (static_cast<size_t>(HW) * rec) % 4 == 0 && (32 * rec) % 4 == 0, lane);
-}
 
 // Stores the BITS plane words of one (pixel, channel word) with the widest aligned store.
 template <int BITS>
@@ -131,8 +38,8 @@ __device__ __forceinline__ void store_planes(uint32_t* dst, const uint32_t (&w)[
 //   signed zero of x yields -0.  A NaN input gives the canonical NaN (sign clear): no level reached, the lowest
 //   code, which is what clip() makes of a NaN in the formula.  +-inf behave like the comparison.
 //   2-bit codes: plane 1 = (x >= b1); plane 0 = parity of the three comparisons = sign((p0-x) ^ (p1-x) ^ (p2-x)).
-//   3- and 4-bit codes search the 7 or 15 bounds binarily: one subtraction, one sign test and one funnel shift per bit
-//   plus the selects that pick the next bound.
+//   3- and 4-bit codes: LevelPlanes below; for scales it does not take, the 7 or 15 bounds are searched binarily: one subtraction,
+//   one sign test and one funnel shift per bit plus the selects that pick the next bound.
 // One funnel shift moves a sign bit into a plane word (w = 2 w + bit); the inputs of a word are walked from position 31
 // down to 0 so that input i ends at bit i.  Per element of a 2-bit tensor: one load, three subtractions, one three-input
 // xor and two funnel shifts, which leaves the kernels waiting on HBM rather than on the issue slots.
@@ -173,6 +80,75 @@ __device__ __forceinline__ void quant_push(const QuantParams& q, float v, uint32
     }
 }
 
+// Plane words of 32 inputs, pushed from input 31 down to input 0, in the sign-bit comparison form.
+template <int BITS>
+struct SignPlanes {
+    uint32_t w[BITS];
+    const QuantParams& q;
+    __device__ __forceinline__ SignPlanes(const QuantParams& q_, const float*) : q(q_)
+    {
+#pragma unroll
+        for (int j = 0; j < BITS; ++j) w[j] = 0u;
+    }
+    __device__ __forceinline__ void push(int, float v) { quant_push<BITS>(q, v, w); }
+    __device__ __forceinline__ void finish() {}
+};
+
+// The same for 3 and 4 bits by estimate and check: k = round(x * inv + offset) with offset = -qmin - 2^-10 is the level (code - qmin) or
+// one less (x * inv is within 2^-19 of x / s for every x whose level is not clipped), and which of the two it is, the exact bound of
+// level k + 1 decides: level = k + (x >= bound[k]), one look-up in a table of 16 floats in shared memory (different entries lie in
+// different banks).  A NaN ends at level 0 (the clamp drops it, the comparison fails), infinities at the ends.
+// Adding 1.5 * 2^23 leaves k in the low mantissa bits.  The levels of inputs 4 i + g are gathered as the nibbles i of word g, so that
+// plane j is the or over g of ((word g >> j) & 0x11111111) << g: two instructions per word and plane.  About 10 instructions an
+// element against 27 of the search, which bound the kernel (64x64x56x56, 4 bits: 17.2 -> 9.9 us).
+template <int BITS>
+struct LevelPlanes {
+    uint32_t w[BITS], r[4];
+    uint32_t table;
+    float inv, offset;
+    __device__ __forceinline__ LevelPlanes(const QuantParams& q, const float* s_below)
+        : table(static_cast<uint32_t>(__cvta_generic_to_shared(s_below)) - (0x4B400000u << 2)), inv(q.inv), offset(q.offset)
+    {
+#pragma unroll
+        for (int g = 0; g < 4; ++g) r[g] = 0u;
+    }
+    __device__ __forceinline__ void push(int u, float v)
+    {
+        constexpr float top = static_cast<float>((1 << BITS) - 1);
+        const uint32_t k = __float_as_uint(fminf(fmaxf(fmaf(v, inv, offset), 0.0f), top) + 12582912.0f);
+        float below;
+        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(below) : "r"(table + (k << 2)));
+        const uint32_t over = __float_as_uint(below - v) >> 31;
+        r[u & 3] = r[u & 3] * 16u + k + over;
+    }
+    __device__ __forceinline__ void finish()
+    {
+        // the bit pattern of 1.5 * 2^23 rode along in every level
+        constexpr uint32_t carried = 0x4B400000u * 0x11111111u;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) r[g] -= carried;
+#pragma unroll
+        for (int j = 0; j < BITS; ++j) {
+            w[j] = 0u;
+#pragma unroll
+            for (int g = 0; g < 4; ++g) w[j] |= (g >= j ? r[g] << (g - j) : r[g] >> (j - g)) & (0x11111111u << g);
+        }
+    }
+};
+
+template <int BITS, bool LEVELS> struct PlanesOf { typedef SignPlanes<BITS> type; };
+template <int BITS> struct PlanesOf<BITS, true> { typedef LevelPlanes<BITS> type; };
+
+// The table of LevelPlanes; every thread of the block calls this first.
+template <bool LEVELS>
+__device__ __forceinline__ void load_levels(float* s_below, const QuantParams& q)
+{
+    if constexpr (LEVELS) {
+        if (threadIdx.x < 16) s_below[threadIdx.x] = q.below[threadIdx.x];
+        __syncthreads();
+    }
+}
+
 // Transpose of the 32 x 32 bit matrix whose row r is the word held by lane r: afterwards lane r holds column r.  Five
 // butterfly stages; stage k swaps the off-diagonal k x k blocks between lanes r and r ^ k.
 __device__ __forceinline__ uint32_t warp_transpose32(uint32_t x, int lane)
@@ -194,11 +170,13 @@ __device__ __forceinline__ uint32_t warp_transpose32(uint32_t x, int lane)
 constexpr int FAST_THREADS = 128;
 constexpr int FAST_WARPS = FAST_THREADS / 32;
 
-template <int BITS>
+template <int BITS, bool LEVELS>
 __global__ void __launch_bounds__(FAST_THREADS, 8)
 bitpack_nchw_f32_kernel(const float* __restrict__ x, uint32_t* __restrict__ out, int C, int HW, int Cw, long long nunits,
-                        int units_per_img, const QuantParams q)
+                        int units_per_img, const __grid_constant__ QuantParams q)
 {
+    __shared__ float s_below[16];
+    load_levels<LEVELS>(s_below, q);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long unit = static_cast<long long>(blockIdx.x) * FAST_WARPS + warp;
     if (unit >= nunits) return;
@@ -209,32 +187,31 @@ bitpack_nchw_f32_kernel(const float* __restrict__ x, uint32_t* __restrict__ out,
     const bool pvalid = lane < HW - hw0;
     // lanes beyond the image re-read the first pixel of the tile (always in bounds) and store nothing
     const float* xin = x + (static_cast<size_t>(n) * C + cw * 32) * HW + hw0 + (pvalid ? lane : 0);
-    uint32_t w[BITS];
-#pragma unroll
-    for (int j = 0; j < BITS; ++j) w[j] = 0u;
-    auto push = [&](float v) { quant_push<BITS>(q, v, w); };
+    typename PlanesOf<BITS, LEVELS>::type planes(q, s_below);
     const int nvalid = min(32, C - cw * 32);
+    const ptrdiff_t row = HW;
+    float v[32];
     if (nvalid == 32) {
         // a full channel word: unconditional loads, walking the channel rows downward from channel 31
-        const ptrdiff_t row = HW;
         const float* pc = xin + 31 * row;
-        float v[32];
 #pragma unroll
         for (int u = 0; u < 32; ++u) {
-            v[u] = __ldcs(pc);
+            v[31 - u] = __ldcs(pc);
             pc -= row;
         }
-#pragma unroll
-        for (int u = 0; u < 32; ++u) push(v[u]);
     } else {
         // the ragged last word: channels past C count as "no level reached"
-        for (int u = 31; u >= 0; --u) push(u < nvalid ? __ldcs(xin + static_cast<size_t>(u) * HW) : -INFINITY);
+#pragma unroll
+        for (int u = 0; u < 32; ++u) v[u] = u < nvalid ? __ldcs(xin + u * row) : -INFINITY;
     }
+#pragma unroll
+    for (int u = 31; u >= 0; --u) planes.push(u, v[u]);
+    planes.finish();
     if (!pvalid) return;
     const unsigned fl = nvalid == 32 ? 0xffffffffu : ((1u << nvalid) - 1u);
     // pattern = (qmin + count) mod 2^BITS: two's-complement codes (qmin = -2^(BITS-1)) flip the top plane only
-    if (q.sign == BS_SIGNED) w[BITS - 1] ^= fl;
-    store_planes<BITS>(out + ((static_cast<size_t>(n) * HW + hw0 + lane) * Cw + cw) * BITS, w);
+    if (q.sign == BS_SIGNED) planes.w[BITS - 1] ^= fl;
+    store_planes<BITS>(out + ((static_cast<size_t>(n) * HW + hw0 + lane) * Cw + cw) * BITS, planes.w);
 }
 
 // fp32 NHWC input, comparison form at any width.  Work unit of a warp = 32 consecutive pixels x one 32-channel word, lane
@@ -242,11 +219,13 @@ bitpack_nchw_f32_kernel(const float* __restrict__ x, uint32_t* __restrict__ out,
 // at once.  A lane shifts the plane bits of its channel into words indexed by PIXEL (pixels walked from 31 down), a
 // 32 x 32 bit transpose across the warp (five shuffles per plane) turns them into words indexed by channel held by lane
 // = pixel, and the records leave as one store per lane like in the NCHW kernel.  No votes, no shared memory.
-template <int BITS>
+template <int BITS, bool LEVELS>
 __global__ void __launch_bounds__(FAST_THREADS, 8)
 bitpack_nhwc_f32_kernel(const float* __restrict__ x, uint32_t* __restrict__ out, int C, int HW, int Cw, long long nunits,
-                        int units_per_img, const QuantParams q)
+                        int units_per_img, const __grid_constant__ QuantParams q)
 {
+    __shared__ float s_below[16];
+    load_levels<LEVELS>(s_below, q);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long unit = static_cast<long long>(blockIdx.x) * FAST_WARPS + warp;
     if (unit >= nunits) return;
@@ -259,46 +238,54 @@ bitpack_nhwc_f32_kernel(const float* __restrict__ x, uint32_t* __restrict__ out,
     const unsigned valid_word = __ballot_sync(0xffffffffu, cvalid);
     // lanes past the last channel re-read the first channel of the word (always in bounds); their words are cleared
     const float* xin = x + (static_cast<size_t>(n) * HW + hw0) * C + cw * 32 + (cvalid ? lane : 0);
-    uint32_t w[BITS];
-#pragma unroll
-    for (int j = 0; j < BITS; ++j) w[j] = 0u;
+    typename PlanesOf<BITS, LEVELS>::type planes(q, s_below);
+    const ptrdiff_t row = C;
+    float v[32];
     if (npix == 32) {
-        const ptrdiff_t row = C;
         const float* pc = xin + 31 * row;
-        float v[32];
 #pragma unroll
         for (int u = 0; u < 32; ++u) {
-            v[u] = __ldcs(pc);
+            v[31 - u] = __ldcs(pc);
             pc -= row;
         }
-#pragma unroll
-        for (int u = 0; u < 32; ++u) quant_push<BITS>(q, v[u], w);
     } else {
         // the ragged last tile of an image: pixels past the end count as "no level reached" and are not stored
-        for (int u = 31; u >= 0; --u) quant_push<BITS>(q, u < npix ? __ldcs(xin + static_cast<size_t>(u) * C) : -INFINITY, w);
+#pragma unroll
+        for (int u = 0; u < 32; ++u) v[u] = u < npix ? __ldcs(xin + u * row) : -INFINITY;
     }
 #pragma unroll
-    for (int j = 0; j < BITS; ++j) w[j] = warp_transpose32(cvalid ? w[j] : 0u, lane);
+    for (int u = 31; u >= 0; --u) planes.push(u, v[u]);
+    planes.finish();
+#pragma unroll
+    for (int j = 0; j < BITS; ++j) planes.w[j] = warp_transpose32(cvalid ? planes.w[j] : 0u, lane);
     if (lane >= npix) return;
-    if (q.sign == BS_SIGNED) w[BITS - 1] ^= valid_word;
-    store_planes<BITS>(out + ((static_cast<size_t>(n) * HW + hw0 + lane) * Cw + cw) * BITS, w);
+    if (q.sign == BS_SIGNED) planes.w[BITS - 1] ^= valid_word;
+    store_planes<BITS>(out + ((static_cast<size_t>(n) * HW + hw0 + lane) * Cw + cw) * BITS, planes.w);
 }
 
-// int8 codes, NCHW (unsigned or two's-complement codes: plane j is bit j of the byte).  At one byte per element the
-// HBM roofline leaves about five thread instructions per element, so the plane split works on four pixels at a time:
-// a lane owns four consecutive pixels and reads them as one 32-bit word per channel row (a warp = 128 pixels, 128-byte
-// requests); (r >> j) & 0x01010101 is bit j of the four codes, and a = 2 a + that, over eight channel rows from the
-// highest down, leaves in byte k of a the eight channel bits of pixel k.  A byte permute drops each finished byte into
-// the plane word of its pixel.  About 1.8 instructions per element for 2-bit codes.  Needs H*W to be a multiple of 4
-// (aligned 32-bit loads); work unit of a warp = 128 pixels x one 32-channel word.
+// Four int8 codes as plane bits: bit j of byte k is plane j of code k (the two's-complement low bits; bipolar: code > 0).
+template <int BITS>
+__device__ __forceinline__ uint32_t codes4(uint32_t r, bool bipolar)
+{
+    return BITS == 1 && bipolar ? __vcmpgts4(r, 0u) : r;
+}
+
+// int8 codes, NCHW.  At one byte per element the HBM roofline leaves about five thread instructions per element, so the plane
+// split works on four pixels at a time: a lane owns four consecutive pixels of a channel row, one 32-bit word (a warp = 128
+// pixels, 128-byte requests); (r >> j) & 0x01010101 is bit j of the four codes, and a = 2 a + that, over eight channel rows from
+// the highest down, leaves in byte k of a the eight channel bits of pixel k.  A byte permute drops each finished byte into the
+// plane word of its pixel.  About 1.8 instructions per element for 2-bit codes.  Work unit of a warp = 128 pixels x one 32-channel
+// word.  ALIGNED: H*W is a multiple of four, every row starts on a word.  Otherwise the four pixels of a lane straddle two words
+// (the second one is the next lane's first and comes from L1), joined by a funnel shift; byte loads of one pixel per lane, 32 bytes
+// a request, took 2 to 3 times as long.
 // Stores: with CW = 0 every lane writes the plane words of its pixels straight to the records (8-byte pieces of 32-byte
 // sectors, four partial writes per sector).  When the channel words of a record number CW = 1, 2 or 4, the four warps of
 // a block hold complete records of 4 / CW tiles: they park their words in shared memory as [warp][plane][pixel] (128-bit
 // stores, no bank conflicts), and after one barrier the block writes the records as whole 128-bit pieces.
-template <int BITS, int CW>
+template <int BITS, int CW, bool ALIGNED>
 __global__ void __launch_bounds__(FAST_THREADS, 8)
 bitpack_nchw_i8_kernel(const int8_t* __restrict__ x, uint32_t* __restrict__ out, int C, int HW, int Cw, long long nunits,
-                       int units_per_img)
+                       int units_per_img, long long bytes, int bipolar)
 {
     constexpr bool STAGED = CW != 0;
     __shared__ __align__(16) uint32_t stage[STAGED ? FAST_WARPS * BITS * 128 : 4];
@@ -312,17 +299,36 @@ bitpack_nchw_i8_kernel(const int8_t* __restrict__ x, uint32_t* __restrict__ out,
         const int cw = rem % Cw;
         const int hw0 = (rem / Cw) * 128;
         const int pix = hw0 + 4 * lane;
-        const bool pvalid = pix < HW;      // H*W is a multiple of 4: the four pixels of a lane are inside or outside together
-        const uint32_t* xin = reinterpret_cast<const uint32_t*>(x + (static_cast<size_t>(n) * C + cw * 32) * HW + (pvalid ? pix : hw0));
+        const bool pvalid = pix < HW;
         const int nvalid = min(32, C - cw * 32);
-        const size_t row = static_cast<size_t>(HW / 4);
         uint32_t v[32];
-        if (nvalid == 32) {
+        if constexpr (ALIGNED) {           // the four pixels of a lane are inside or outside together
+            const uint32_t* xin = reinterpret_cast<const uint32_t*>(x + (static_cast<size_t>(n) * C + cw * 32) * HW + (pvalid ? pix : hw0));
+            const size_t row = static_cast<size_t>(HW / 4);
+            if (nvalid == 32) {
 #pragma unroll
-            for (int u = 0; u < 32; ++u) v[u] = __ldcs(xin + u * row);
+                for (int u = 0; u < 32; ++u) v[u] = codes4<BITS>(__ldcs(xin + u * row), bipolar);
+            } else {
+#pragma unroll
+                for (int u = 0; u < 32; ++u) v[u] = u < nvalid ? codes4<BITS>(__ldcs(xin + u * row), bipolar) : 0u;
+            }
         } else {
+            const long long at = (n * C + cw * 32) * HW + (pvalid ? pix : hw0);
+            // only whole words inside the tensor are loaded; its last, partial word is put together from bytes
+            const long long whole = bytes >> 2;
+            uint32_t tail = 0u;
+            const long long reach = (n * C + cw * 32 + nvalid - 1) * HW + hw0 + 136;
+            if (reach > 4 * whole)
+                for (int k = 0; k < (bytes & 3); ++k) tail |= static_cast<uint32_t>(static_cast<uint8_t>(x[4 * whole + k])) << (8 * k);
+            const uint32_t* xw = reinterpret_cast<const uint32_t*>(x);
 #pragma unroll
-            for (int u = 0; u < 32; ++u) v[u] = u < nvalid ? __ldcs(xin + u * row) : 0u;
+            for (int u = 0; u < 32; ++u) {
+                const long long byte = at + static_cast<long long>(u < nvalid ? u : 0) * HW, i = byte >> 2;
+                const uint32_t lo = i < whole ? __ldg(xw + i) : tail, hi = i + 1 < whole ? __ldg(xw + i + 1) : tail;
+                v[u] = __funnelshift_r(lo, hi, static_cast<int>(byte & 3) * 8);
+            }
+#pragma unroll
+            for (int u = 0; u < 32; ++u) v[u] = u < nvalid ? codes4<BITS>(v[u], bipolar) : 0u;
         }
         uint32_t w[4][BITS];
 #pragma unroll
@@ -351,10 +357,9 @@ bitpack_nchw_i8_kernel(const int8_t* __restrict__ x, uint32_t* __restrict__ out,
             for (int j = 0; j < BITS; ++j)
                 *reinterpret_cast<uint4*>(stage + (warp * BITS + j) * 128 + 4 * lane) = make_uint4(w[0][j], w[1][j], w[2][j], w[3][j]);
         } else {
-            if (!pvalid) return;
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                store_planes<BITS>(out + ((static_cast<size_t>(n) * HW + pix + k) * Cw + cw) * BITS, w[k]);
+                if (pix + k < HW) store_planes<BITS>(out + ((static_cast<size_t>(n) * HW + pix + k) * Cw + cw) * BITS, w[k]);
         }
     }
     if constexpr (STAGED) {
@@ -422,6 +427,61 @@ bitpack_nhwc_i8_kernel(const int8_t* __restrict__ x, uint32_t* __restrict__ out,
                 w[j] |= ((((words[i] >> j) & 0x01010101u) * 0x01020408u) >> 24) << (4 * i);
         const int pix = hw0 + 32 * t + lane;
         if (pix < HW) store_planes<BITS>(out + ((static_cast<size_t>(n) * HW + pix) * Cw + cw) * BITS, w);
+    }
+}
+
+// int8 codes, NHWC, any C and any code: the whole tensor is one run of N*H*W records of C bytes, so a block takes `pix` consecutive
+// pixels (64, fewer where C is large) = one contiguous run of bytes (no image boundary), staged into shared memory by 16-byte asynchronous copies from the
+// 16-byte boundary at or below its start.  A thread then takes one (pixel, channel word): nine words of the stage from the one its
+// first byte lies in, joined by funnel shifts, and the same plane gathering as above; bits of channels past C are masked out of the
+// finished words, so what the stage holds behind the last record does not matter.  Neighbouring threads take neighbouring
+// channel words of a pixel: the packed records leave as one contiguous run.  Byte loads with votes took 10 times as long
+// (48 x 45 x 61 pixels of 50 channels, 2 bits: 18 -> 2 us).
+constexpr int RAGGED_PIX = 64, RAGGED_BYTES = 40 * 1024;
+
+template <int BITS>
+__global__ void __launch_bounds__(FAST_THREADS)
+bitpack_nhwc_ragged_i8_kernel(const int8_t* __restrict__ x, uint32_t* __restrict__ out, int C, int Cw, long long npix, int pix, int bipolar)
+{
+    extern __shared__ __align__(16) uint32_t ragged_smem[];
+    const long long p0 = static_cast<long long>(blockIdx.x) * pix;
+    const int np = static_cast<int>(npix - p0 < pix ? npix - p0 : pix);
+    const long long first = p0 * C, begin = first & ~15LL, end = first + static_cast<long long>(np) * C;
+    const int lead = static_cast<int>(first - begin), span = static_cast<int>(end - begin);
+    const int8_t* src = x + begin;
+    int8_t* stage = reinterpret_cast<int8_t*>(ragged_smem);
+    const int whole = end < npix * C ? (span + 15) / 16 : span / 16;       // 16-byte pieces inside the tensor
+    for (int i = threadIdx.x; i < whole; i += FAST_THREADS) {
+        const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(stage + 16 * i));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src + 16 * i) : "memory");
+    }
+    for (int i = 16 * whole + threadIdx.x; i < span; i += FAST_THREADS) stage[i] = src[i];
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    const int nwords = np * Cw;
+    uint32_t* dst = out + static_cast<size_t>(p0) * Cw * BITS;
+    for (int i = threadIdx.x; i < nwords; i += FAST_THREADS) {
+        const int p = i / Cw, cw = i - p * Cw;
+        const int byte = lead + p * C + cw * 32;
+        const uint32_t* q = ragged_smem + (byte >> 2);
+        const int sh = (byte & 3) * 8;
+        const int nvalid = C - cw * 32;
+        const uint32_t valid = nvalid >= 32 ? 0xffffffffu : (1u << nvalid) - 1u;
+        uint32_t w[BITS];
+#pragma unroll
+        for (int j = 0; j < BITS; ++j) w[j] = 0u;
+        uint32_t lo = q[0];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t hi = q[k + 1];
+            const uint32_t r = codes4<BITS>(__funnelshift_r(lo, hi, sh), bipolar);
+            lo = hi;
+#pragma unroll
+            for (int j = 0; j < BITS; ++j) w[j] |= ((((r >> j) & 0x01010101u) * 0x01020408u) >> 24) << (4 * k);
+        }
+#pragma unroll
+        for (int j = 0; j < BITS; ++j) w[j] &= valid;
+        store_planes<BITS>(dst + static_cast<size_t>(i) * BITS, w);
     }
 }
 
@@ -544,6 +604,16 @@ static QuantParams make_quant_params(float s, int bits, int sign)
         if (p == 0.0f) p = fabsf(p);          // drops the sign of a zero
         q.below[k] = p;
     }
+    q.below[15] = INFINITY;
+    // the estimate needs 1 / s and its products with the inputs near the bounds to be normal numbers
+    q.estimate = bits >= 3 && s > 1e-30f && s < 1e30f;
+    if (q.estimate) {
+        int qmin, qmax;
+        code_limits(bits, sign, qmin, qmax);
+        for (int k = qmax - qmin; k < 16; ++k) q.below[k] = INFINITY;     // no level above the top one
+        q.inv = 1.0f / s;
+        q.offset = static_cast<float>(-qmin) - 0x1p-10f;
+    }
     return q;
 }
 
@@ -557,22 +627,17 @@ extern "C" int bs_quantiser_bounds(float act_scale, int a_bits, bs_sign_t a_sign
     return BS_OK;
 }
 
-template <bool NHWC, int BITS>
-static int launch_bitpack_codes(const void* x, uint32_t* out, int N, int C, int HW, int sign, cudaStream_t st)
+template <int BITS>
+static int launch_bitpack_nhwc_ragged(const int8_t* x, uint32_t* out, int N, int C, int HW, int bipolar, cudaStream_t st)
 {
     const int Cw = ceil_div(C, 32);
-    const size_t smem = static_cast<size_t>(PACK_WARPS) * 32 * Cw * BITS * 4;
-    if (smem > 200 * 1024) return BS_ERR_UNSUPPORTED;
-    auto kern = bitpack_codes_kernel<NHWC, BITS>;
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
-        return BS_ERR_CUDA;
-    const int tiles_per_img = ceil_div(HW, 32);
-    const long long ntiles = static_cast<long long>(N) * tiles_per_img;
-    const long long blocks = ceil_div_ll(ntiles, PACK_WARPS);
-    if (blocks > 0x7fffffffLL) return BS_ERR_UNSUPPORTED;
-    kern<<<static_cast<unsigned>(blocks), PACK_THREADS, smem, st>>>(static_cast<const int8_t*>(x), out, C, HW, Cw, ntiles,
-                                                                  tiles_per_img, sign);
+    int pix = RAGGED_PIX;
+    while (pix > 1 && static_cast<long long>(pix) * C > RAGGED_BYTES) pix /= 2;
+    const long long npix = static_cast<long long>(N) * HW, blocks = ceil_div_ll(npix, pix);
+    // the run of bytes, the part of a piece before it, and the nine words read from the last channel word on
+    const long long smem = (static_cast<long long>(pix) * C + 15 + 15) / 16 * 16 + 64;
+    if (blocks > 0x7fffffffLL || smem > 48 * 1024) return BS_ERR_UNSUPPORTED;
+    bitpack_nhwc_ragged_i8_kernel<BITS><<<static_cast<unsigned>(blocks), FAST_THREADS, static_cast<size_t>(smem), st>>>(x, out, C, Cw, npix, pix, bipolar);
     return cudaGetLastError() == cudaSuccess ? BS_OK : BS_ERR_CUDA;
 }
 
@@ -593,54 +658,53 @@ static int launch_units(K kern, const void* x, uint32_t* out, int N, int C, int 
 }
 
 template <int BITS>
-static int launch_bitpack_nchw_i8(const void* x, uint32_t* out, int N, int C, int HW, cudaStream_t st)
+static int launch_bitpack_nchw_i8(const void* x, uint32_t* out, int N, int C, int HW, int bipolar, cudaStream_t st)
 {
+    const long long bytes = static_cast<long long>(N) * C * HW;
+    if (HW % 4 != 0) return launch_units(bitpack_nchw_i8_kernel<BITS, 0, false>, x, out, N, C, HW, 128, st, bytes, bipolar);
     switch (ceil_div(C, 32)) {      // records of 1, 2 or 4 channel words leave through the block-staged stores
-        case 1: return launch_units(bitpack_nchw_i8_kernel<BITS, 1>, x, out, N, C, HW, 128, st);
-        case 2: return launch_units(bitpack_nchw_i8_kernel<BITS, 2>, x, out, N, C, HW, 128, st);
-        case 4: return launch_units(bitpack_nchw_i8_kernel<BITS, 4>, x, out, N, C, HW, 128, st);
-        default: return launch_units(bitpack_nchw_i8_kernel<BITS, 0>, x, out, N, C, HW, 128, st);
+        case 1: return launch_units(bitpack_nchw_i8_kernel<BITS, 1, true>, x, out, N, C, HW, 128, st, bytes, bipolar);
+        case 2: return launch_units(bitpack_nchw_i8_kernel<BITS, 2, true>, x, out, N, C, HW, 128, st, bytes, bipolar);
+        case 4: return launch_units(bitpack_nchw_i8_kernel<BITS, 4, true>, x, out, N, C, HW, 128, st, bytes, bipolar);
+        default: return launch_units(bitpack_nchw_i8_kernel<BITS, 0, true>, x, out, N, C, HW, 128, st, bytes, bipolar);
     }
 }
 
+// NHWC codes: 16-byte loads straight from the records where these are whole channel words (C a multiple of 32, the planes the
+// low bits of the byte), staged through shared memory otherwise.
+template <int BITS>
+static int launch_bitpack_nhwc_i8(const void* x, uint32_t* out, int N, int C, int HW, int bipolar, cudaStream_t st)
+{
+    if (C % 32 == 0 && !bipolar) return launch_units(bitpack_nhwc_i8_kernel<BITS>, x, out, N, C, HW, 128, st);
+    return launch_bitpack_nhwc_ragged<BITS>(static_cast<const int8_t*>(x), out, N, C, HW, bipolar, st);
+}
+
 template <bool NHWC>
-static int launch_bitpack_i8(const void* x, uint32_t* out, int N, int C, int HW, int bits, cudaStream_t st)
+static int launch_bitpack_i8(const void* x, uint32_t* out, int N, int C, int HW, int bits, int bipolar, cudaStream_t st)
 {
     switch (bits) {
-        case 1: return NHWC ? launch_units(bitpack_nhwc_i8_kernel<1>, x, out, N, C, HW, 128, st) : launch_bitpack_nchw_i8<1>(x, out, N, C, HW, st);
-        case 2: return NHWC ? launch_units(bitpack_nhwc_i8_kernel<2>, x, out, N, C, HW, 128, st) : launch_bitpack_nchw_i8<2>(x, out, N, C, HW, st);
-        case 3: return NHWC ? launch_units(bitpack_nhwc_i8_kernel<3>, x, out, N, C, HW, 128, st) : launch_bitpack_nchw_i8<3>(x, out, N, C, HW, st);
-        default: return NHWC ? launch_units(bitpack_nhwc_i8_kernel<4>, x, out, N, C, HW, 128, st) : launch_bitpack_nchw_i8<4>(x, out, N, C, HW, st);
+        case 1: return NHWC ? launch_bitpack_nhwc_i8<1>(x, out, N, C, HW, bipolar, st) : launch_bitpack_nchw_i8<1>(x, out, N, C, HW, bipolar, st);
+        case 2: return NHWC ? launch_bitpack_nhwc_i8<2>(x, out, N, C, HW, bipolar, st) : launch_bitpack_nchw_i8<2>(x, out, N, C, HW, bipolar, st);
+        case 3: return NHWC ? launch_bitpack_nhwc_i8<3>(x, out, N, C, HW, bipolar, st) : launch_bitpack_nchw_i8<3>(x, out, N, C, HW, bipolar, st);
+        default: return NHWC ? launch_bitpack_nhwc_i8<4>(x, out, N, C, HW, bipolar, st) : launch_bitpack_nchw_i8<4>(x, out, N, C, HW, bipolar, st);
     }
 }
 
-// fp32 tensors: comparison-form kernels with one (32 pixels, channel word) unit per warp.
-template <bool NHWC>
-static int launch_bitpack_f32(const void* x, uint32_t* out, int N, int C, int HW, const QuantParams& q, cudaStream_t st)
+// fp32 tensors: one (32 pixels, channel word) unit per warp.
+template <int BITS, bool LEVELS>
+static int launch_f32(bool nhwc, const void* x, uint32_t* out, int N, int C, int HW, const QuantParams& q, cudaStream_t st)
+{
+    return nhwc ? launch_units(bitpack_nhwc_f32_kernel<BITS, LEVELS>, x, out, N, C, HW, 32, st, q)
+                : launch_units(bitpack_nchw_f32_kernel<BITS, LEVELS>, x, out, N, C, HW, 32, st, q);
+}
+
+static int launch_bitpack_f32(bool nhwc, const void* x, uint32_t* out, int N, int C, int HW, const QuantParams& q, cudaStream_t st)
 {
     switch (q.bits) {
-        case 1: return NHWC ? launch_units(bitpack_nhwc_f32_kernel<1>, x, out, N, C, HW, 32, st, q)
-                            : launch_units(bitpack_nchw_f32_kernel<1>, x, out, N, C, HW, 32, st, q);
-        case 2: return NHWC ? launch_units(bitpack_nhwc_f32_kernel<2>, x, out, N, C, HW, 32, st, q)
-                            : launch_units(bitpack_nchw_f32_kernel<2>, x, out, N, C, HW, 32, st, q);
-        case 3: return NHWC ? launch_units(bitpack_nhwc_f32_kernel<3>, x, out, N, C, HW, 32, st, q)
-                            : launch_units(bitpack_nchw_f32_kernel<3>, x, out, N, C, HW, 32, st, q);
-        default: return NHWC ? launch_units(bitpack_nhwc_f32_kernel<4>, x, out, N, C, HW, 32, st, q)
-                             : launch_units(bitpack_nchw_f32_kernel<4>, x, out, N, C, HW, 32, st, q);
-    }
-}
-
-// int8 codes: the vector kernels where the shape allows aligned vector loads and the planes are the low bits of the byte,
-// else the fallback.
-template <bool NHWC>
-static int launch_bitpack_codes_any(const void* x, uint32_t* out, int N, int C, int HW, int bits, int sign, cudaStream_t st)
-{
-    if (sign != BS_BIPOLAR && (NHWC ? C % 32 == 0 : HW % 4 == 0)) return launch_bitpack_i8<NHWC>(x, out, N, C, HW, bits, st);
-    switch (bits) {
-        case 1: return launch_bitpack_codes<NHWC, 1>(x, out, N, C, HW, sign, st);
-        case 2: return launch_bitpack_codes<NHWC, 2>(x, out, N, C, HW, sign, st);
-        case 3: return launch_bitpack_codes<NHWC, 3>(x, out, N, C, HW, sign, st);
-        default: return launch_bitpack_codes<NHWC, 4>(x, out, N, C, HW, sign, st);
+        case 1: return launch_f32<1, false>(nhwc, x, out, N, C, HW, q, st);
+        case 2: return launch_f32<2, false>(nhwc, x, out, N, C, HW, q, st);
+        case 3: return q.estimate ? launch_f32<3, true>(nhwc, x, out, N, C, HW, q, st) : launch_f32<3, false>(nhwc, x, out, N, C, HW, q, st);
+        default: return q.estimate ? launch_f32<4, true>(nhwc, x, out, N, C, HW, q, st) : launch_f32<4, false>(nhwc, x, out, N, C, HW, q, st);
     }
 }
 
@@ -655,12 +719,17 @@ extern "C" int bitpack_activations(const void* x, int x_is_fp32, bs_layout_t lay
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int HW = H * W;
     if (x_is_fp32) {
-        const QuantParams q = make_quant_params(act_scale, a_bits, a_sign);
-        return layout == BS_NHWC ? launch_bitpack_f32<true>(x, packed_out, N, C, HW, q, st)
-                                 : launch_bitpack_f32<false>(x, packed_out, N, C, HW, q, st);
+        // the bisection of the bounds takes several microseconds: a thread keeps the last one it made
+        static thread_local QuantParams q;
+        static thread_local float q_scale = 0.0f;
+        if (q_scale != act_scale || q.bits != a_bits || q.sign != a_sign) {
+            q = make_quant_params(act_scale, a_bits, a_sign);
+            q_scale = act_scale;
+        }
+        return launch_bitpack_f32(layout == BS_NHWC, x, packed_out, N, C, HW, q, st);
     }
-    return layout == BS_NHWC ? launch_bitpack_codes_any<true>(x, packed_out, N, C, HW, a_bits, a_sign, st)
-                             : launch_bitpack_codes_any<false>(x, packed_out, N, C, HW, a_bits, a_sign, st);
+    return layout == BS_NHWC ? launch_bitpack_i8<true>(x, packed_out, N, C, HW, a_bits, a_sign == BS_BIPOLAR, st)
+                             : launch_bitpack_i8<false>(x, packed_out, N, C, HW, a_bits, a_sign == BS_BIPOLAR, st);
 }
 
 extern "C" int bitunpack_activations(const uint32_t* packed, int N, int C, int H, int W, int a_bits, bs_sign_t a_sign,
