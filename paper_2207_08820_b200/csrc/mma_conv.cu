@@ -36,7 +36,7 @@ FastDiv make_div(int d)
 int max_abs_of(int bits, int sign) { return sign == BS_BIPOLAR ? 1 : (sign == BS_SIGNED ? 1 << (bits - 1) : (1 << bits) - 1); }
 
 struct Cand {
-    int TN, PT, units, cfg, cps, ns, resident, nse, nsb, nacc;
+    int TN, PT, units, cfg, cps, ns, resident, groups, nse, nsb, nacc;
     size_t smem;
     double cost;
 };
@@ -80,8 +80,10 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows)
     g.tiles_m = static_cast<int>(ceil_div_ll(total, BM));
     g.tiles_o = ceil_div(g.O, c.TN);
     g.d_rs = make_div(g.RS);
-    g.nslots = ceil_div(g.NI * c.units, XT);
-    g.bslots = ceil_div(c.TN * g.RS * c.units, XT);
+    g.groups = c.groups;
+    const int GT = XT / c.groups;                          // threads of an expander group
+    g.nslots = ceil_div(g.NI * c.units, GT);
+    g.bslots = ceil_div(c.TN * g.RS * c.units, GT);
     auto piece = [&](int bits) { return (2 * bits) % 4 == 0 && (g.Cw * bits) % 4 == 0 ? 16 : ((g.Cw * bits) % 2 == 0 ? 8 : 4); };
     g.psz = piece(A);
     g.bpsz = piece(WB > 0 ? WB : 1);
@@ -90,18 +92,20 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows)
     g.rowB = c.units * 8 * WB;
     const bool fb = packed_b && !c.resident;
     g.tma = g.flat && (g.Cw * A) % 4 == 0 && g.rowA % 16 == 0 && g.rowA <= 128 && (!fb || ((g.Cw * WB) % 4 == 0 && g.rowB % 16 == 0 && g.rowB <= 128));
+    g.nsp = g.tma && c.groups == 1 ? 3 : 2 * c.groups;
     auto swizzle = [](int row) { return row == 32 ? 1 : row == 64 ? 3 : row == 128 ? 7 : 0; };
     g.swzA = swizzle(g.rowA);
     g.swzB = swizzle(g.rowB);
     g.e_bytes = up(4 * c.units * g.NI * 16, 128);
     g.b_bytes = c.units * 2 * c.TN * g.RS * 32;
-    g.stg_bytes = g.tma ? up(BM * g.rowA, 1024) : g.nslots * XT * 8 * A;
-    g.bstg_bytes = !fb ? 0 : g.tma ? up(c.TN * g.rowB, 1024) : g.bslots * XT * 8 * WB;
-    const int pix_bytes = g.flat ? 0 : up(g.NI * 4, 16);
+    g.stg_bytes = g.tma ? up(BM * g.rowA, 1024) : g.nslots * GT * 8 * A;
+    g.bstg_bytes = !fb ? 0 : g.tma ? up(c.TN * g.rowB, 1024) : g.bslots * GT * 8 * WB;
+    const int rel_bytes = g.flat ? 0 : up(g.NI * 4 * (1 + (c.units == 1 ? g.nsp + c.groups : 0)), 16);      // relative rows; located pixels of each group, one table more than stages
+    const int pix_bytes = rel_bytes + (fb && !g.tma && c.units == 1 ? up(c.TN * g.RS * 4, 16) : 0);
     const int cap = c.cfg ? 222 * 1024 : 111 * 1024;
     const int fixed = c.TN * 8 + 64 + 256 + (g.tma ? 1024 : 0) + (int_rows ? EW * 4096 : 0) + 256 + pix_bytes;
     const long long filters = c.resident ? static_cast<long long>(g.Cw) * c.TN * g.RS * 32 : 0;
-    const long long rest = fixed + static_cast<long long>(MM_STAGES) * (g.stg_bytes + g.bstg_bytes) + filters;
+    const long long rest = fixed + static_cast<long long>(g.nsp) * (g.stg_bytes + g.bstg_bytes) + filters;
     c.nsb = 0;
     long long used = 0;
     int nse = 4;
@@ -125,6 +129,7 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows)
         }
         if (!fit) return false;
     }
+    if (nse < c.groups) return false;
     c.nse = nse;
     g.nse = nse; g.nsb = c.resident ? 0 : (packed_b ? nse : c.nsb);
     const int cols = 512 / (c.cfg ? 1 : 2);
@@ -138,9 +143,10 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows)
     long long off = c.resident ? filters : static_cast<long long>(g.nsb) * g.b_bytes;
     g.off_e = static_cast<int>(off);                off += static_cast<long long>(nse) * g.e_bytes;
     if (g.tma) off = (off + 1023) / 1024 * 1024;
-    g.off_stg = static_cast<int>(off);              off += static_cast<long long>(MM_STAGES) * g.stg_bytes;
-    g.off_bstg = static_cast<int>(off);             off += static_cast<long long>(MM_STAGES) * g.bstg_bytes;
-    g.off_pix = static_cast<int>(off);              off += pix_bytes;
+    g.off_stg = static_cast<int>(off);              off += static_cast<long long>(g.nsp) * g.stg_bytes;
+    g.off_bstg = static_cast<int>(off);             off += static_cast<long long>(g.nsp) * g.bstg_bytes;
+    g.off_pix = static_cast<int>(off);              g.off_brow = static_cast<int>(off) + rel_bytes;
+    off += pix_bytes;
     off = (off + 127) / 128 * 128;
     g.off_out = static_cast<int>(off);              if (int_rows) off += EW * 4096;
     g.off_tab = static_cast<int>(off);              off += c.TN * 8 + 64;
@@ -153,46 +159,47 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows)
 }
 
 // Time model of a candidate in SM cycles: the pipeline of one CTA (expansion, MMAs, epilogue; a stage's hand-off included) over
-// its items, plus what nothing overlaps at both ends.  The constants are fitted to about 2500 timed plans of 41 layers and
+// its items, plus what nothing overlaps at both ends.  The constants are fitted to about 2500 timed plans of 45 layers and
 // products (1 to 300 pixels wide, 32 to 4608 channels, batches 1 to 64; B200 at 1.95 GHz): over those the plan with the
-// lowest modelled time is on average 2 % and with three exceptions at most 8 % slower than the fastest plan.
+// lowest modelled time is on average 2 % and with two exceptions at most 8 % slower than the fastest plan.
 double mma_cost(const MmaArgs& g, const Cand& c, int A, int WB, bool packed_out, int sms)
 {
     const bool packed_b = WB > 0;
-    const double mma = 1.05 * (c.TN == 32 ? 42 : c.TN == 64 ? 49 : c.TN == 128 ? 65 : 129);      // cycles per MMA of 128 x TN x 32
+    const double mma = c.TN == 32 ? 42 : c.TN == 64 ? 49 : c.TN == 128 ? 65 : 129;      // cycles per MMA of 128 x TN x 32
     const int W = c.cfg ? 8 : 4;                                   // expander warps, epilogue warps
-    const double t_m = static_cast<double>(c.PT) * g.RS * g.Cw * mma + 121.0 * g.nchunks;
-    // expansion: instructions per warp and 64-channel unit of 32 rows, at 6.8 cycles each
+    const double t_m = static_cast<double>(c.PT) * g.RS * g.Cw * mma + 148.0 * g.nchunks;
+    // expansion: instructions per warp and 64-channel unit of 32 rows, at 5.3 cycles each; a chunk's hand-off
     const int row_groups = ceil_div(g.NI, 32);
-    double xi = static_cast<double>(row_groups) * g.nunits * ((A <= 2 ? 90.0 : 140.0) + (g.tma ? 2.0 : 60.0));
-    if (!c.resident && packed_b) xi += c.TN * g.RS / 32.0 * g.nunits * (WB <= 2 ? 40.0 : 60.0);
-    const double units_of_work = static_cast<double>(row_groups) * c.units / W;
-    const double t_x = xi / W * (ceil(units_of_work) / units_of_work) * 6.8 + 500.0 * g.nchunks + 278.0;
-    // epilogue: instructions per block of 32 x 32 outputs, at 3.65 cycles; int32 rows leave at about 27 bytes per clock and SM
-    const double block = packed_out ? (g.has_residual ? 283.0 : 187.0) : 106.0;
-    double t_e = ceil_div(c.PT * (c.TN / 32), W / 4) * block * 3.65 + 700.0;
-    if (!packed_out && c.PT * 128.0 * c.TN * 4 / 27.5 > t_e) t_e = c.PT * 128.0 * c.TN * 4 / 27.5;
-    const double t_b = (!c.resident && !packed_b) ? static_cast<double>(c.TN) * g.RS * g.Cw * 32 / 52.0 : 0.0;       // L2 -> shared memory
+    double xi = static_cast<double>(row_groups) * g.nunits * ((A <= 2 ? 102.0 : 111.0) + (g.tma ? 1.0 : 41.0));
+    if (!c.resident && packed_b) xi += c.TN * g.RS / 32.0 * g.nunits * (WB <= 2 ? 20.0 : 69.0);
+    const double units_of_work = static_cast<double>(row_groups) * c.units * c.groups / W;       // per warp of a group and chunk
+    const double chunk = xi / g.nchunks * c.groups / W * (ceil(units_of_work) / units_of_work) * 5.34 + 755.0;
+    const double t_x = chunk * g.nchunks / (1.0 + (c.groups - 1) * 0.83) + 628.0;
+    // epilogue: instructions per block of 32 x 32 outputs, at 4.6 cycles; int32 rows leave at about 30 bytes per clock and SM
+    const double block = packed_out ? (g.has_residual ? 215.0 : 138.0) : 94.0;
+    double t_e = ceil_div(c.PT * (c.TN / 32), W / 4) * block * 4.59 + 997.0;
+    if (!packed_out && c.PT * 128.0 * c.TN * 4 / 29.6 > t_e) t_e = c.PT * 128.0 * c.TN * 4 / 29.6;
+    const double t_b = (!c.resident && !packed_b) ? static_cast<double>(c.TN) * g.RS * g.Cw * 32 / 68.7 : 0.0;       // L2 -> shared memory
     const long long items = static_cast<long long>(g.tiles_m) * g.tiles_o;
     long long ctas = static_cast<long long>(sms) * c.cps;
     if (c.resident) ctas = ctas / g.tiles_o * g.tiles_o;
     if (ctas < 1) return 1e18;
     if (ctas > items) ctas = items;
     const double per_cta = static_cast<double>(ceil_div_ll(items, ctas)), active = static_cast<double>(ceil_div_ll(ctas, sms));
-    const double issue = (xi + c.PT * 4.0 * (c.TN / 32) * block) / 2.77;
+    const double issue = (xi + c.PT * 4.0 * (c.TN / 32) * block) / 3.08;
     const double t_mb = t_m > t_b ? t_m : t_b;
     double step = c.nacc == 2 ? (t_mb > t_e ? t_mb : t_e) : t_mb + t_e;
     if (t_x > step) step = t_x;
     if (active * t_mb > step) step = active * t_mb;
     if (active * issue > step) step = active * issue;
-    const double rest_x = t_x * (g.nchunks - 1) / g.nchunks;
-    double first = t_x / g.nchunks + (t_mb > rest_x ? t_mb : rest_x) + t_e;
-    if (active > 1.0) first *= 1.3;
-    double t = 5900.0 + first + (per_cta - 1.0) * step;
-    if (c.resident && packed_b) t += c.TN * g.RS * g.Cw / 32.0 * 76.0 / (2 * W) * 4.0;
-    if (!c.resident && !packed_b) t *= 1.05;
-    if (!c.resident && (c.nse < 2 || (!packed_b && c.nsb < 2))) t *= 1.3;
-    if (!c.cfg) t *= 0.91;
+    const double rest_x = t_x > chunk ? t_x - chunk : 0.0;
+    double first = chunk + (t_mb > rest_x ? t_mb : rest_x) + t_e;
+    if (active > 1.0) first *= 1.19;
+    double t = 4215.0 + first + (per_cta - 1.0) * step;
+    if (c.resident && packed_b) t += c.TN * g.RS * g.Cw / 32.0 * 122.0 / (2 * W) * 4.0;
+    if (!c.resident && !packed_b) t *= 1.07;
+    if (c.nse < 2) t *= 1.11;
+    if (!c.cfg) t *= 0.93;
     return t;
 }
 
@@ -266,8 +273,8 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
         }
     }
 #ifdef BS_TUNING
-    int ov[6] = {0, 0, 0, -1, 0, -1};       // TN, PT, units, config, strips, resident; 0 / -1: free
-    if (const char* e = getenv("BS_MM")) sscanf(e, "%d,%d,%d,%d,%d,%d", ov, ov + 1, ov + 2, ov + 3, ov + 4, ov + 5);
+    int ov[7] = {0, 0, 0, -1, 0, -1, 0};    // TN, PT, units, config, strips, resident, groups; 0 / -1: free
+    if (const char* e = getenv("BS_MM")) sscanf(e, "%d,%d,%d,%d,%d,%d,%d", ov, ov + 1, ov + 2, ov + 3, ov + 4, ov + 5, ov + 6);
 #endif
     for (int TN = 32; TN <= 256; TN *= 2) {
         if (TN > 32 && TN / 2 >= up(p->O, 32)) continue;
@@ -277,14 +284,16 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
                 for (int k = 0; k < nns; ++k)
                     for (int units = 1; units <= (g.R == 1 ? 4 : 1); units *= 2) {
                         if (units > 1 && units > (g.Cw + 1) / 2) continue;
-                        for (int res = 0; res < 2; ++res) {
+                        for (int v = 0; v < 6; ++v) {
+                            const int res = v & 1, groups = 1 << (v >> 1);
+                            if (groups > 2 && cfg != 1) continue;
 #ifdef BS_TUNING
                             if ((ov[0] && TN != ov[0]) || (ov[1] && PT != ov[1]) || (ov[2] && units != ov[2]) || (ov[3] >= 0 && cfg != ov[3]) ||
-                                (ov[4] && ns_list[k] != ov[4]) || (ov[5] >= 0 && res != ov[5]))
+                                (ov[4] && ns_list[k] != ov[4]) || (ov[5] >= 0 && res != ov[5]) || (ov[6] && groups != ov[6]))
                                 continue;
 #endif
                             Cand c{};
-                            c.TN = TN; c.PT = PT; c.units = units; c.cfg = cfg == 1; c.cps = cfg == 0 ? 2 : 1; c.ns = ns_list[k]; c.resident = res;
+                            c.TN = TN; c.PT = PT; c.units = units; c.cfg = cfg == 1; c.cps = cfg == 0 ? 2 : 1; c.ns = ns_list[k]; c.resident = res; c.groups = groups;
                             consider(c);
                         }
                     }
@@ -293,8 +302,8 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
     if (!mma_layout(g, best, A, packed_b ? p->w_bits : 0, int_rows)) return BS_ERR_UNSUPPORTED;
 #ifdef BS_TUNING
     if (getenv("BS_MM_VERBOSE"))
-        fprintf(stderr, "mma plan: N%d C%d %dx%d O%d k%d s%d A%d W%d %s -> TN %d PT %d units %d cfg %d x %d strips %d resident %d nse %d nsb %d units %d nacc %d HL %d NI %d tiles %d x %d smem %zu cost %.0f\n",
-                p->N, p->C, p->H, p->W, p->O, p->R, p->stride, A, p->w_bits, packed_b ? "packed" : "prepared", best.TN, best.PT, best.units, best.cfg, best.cps, best.ns, best.resident,
+        fprintf(stderr, "mma plan: N%d C%d %dx%d O%d k%d s%d A%d W%d %s -> TN %d PT %d units %d cfg %d x %d strips %d resident %d groups %d nse %d nsb %d units %d nacc %d HL %d NI %d tiles %d x %d smem %zu cost %.0f\n",
+                p->N, p->C, p->H, p->W, p->O, p->R, p->stride, A, p->w_bits, packed_b ? "packed" : "prepared", best.TN, best.PT, best.units, best.cfg, best.cps, best.ns, best.resident, best.groups,
                 best.nse, g.nsb, g.nunits, g.nacc, g.HL, g.NI, g.tiles_m, g.tiles_o, best.smem, best.cost);
 #endif
     if (flags & MM_QUERY) return BS_OK;

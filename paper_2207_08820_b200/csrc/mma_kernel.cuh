@@ -22,7 +22,7 @@
 
 namespace bs {
 
-constexpr int MM_STAGES = 3;         // stages of packed words in front of the expanders
+constexpr int MM_STAGES = 8;         // most stages of packed words in front of the expanders
 
 struct FastDiv { unsigned mul, shift; int d; };      // quotient of 0 <= n < 2^31 by d as umulhi(n, mul) >> shift
 
@@ -56,7 +56,8 @@ struct MmaArgs {
     int pad;
     // tiling
     int TN, PT, units, nunits, nchunks;     // filters and row tiles per item, 64-channel units per chunk / in all
-    int nse, nsb;                   // stages of the expanded-pixel ring, of the streamed-filter ring (0: filters resident)
+    int nse, nsb;                   // stages of the expanded ring; the same when filters are streamed through it, 0: filters resident
+    int groups, nsp;                // expander groups (chunk n belongs to group n mod groups), stages of packed words in all
     int tiles_m, tiles_o;
     FastDiv d_rs;
     int tma;                        // rows of pixels (and of packed, streamed filters) arrive by TMA boxes
@@ -65,7 +66,7 @@ struct MmaArgs {
     int psz, bpsz;                  // bytes per cp.async of pixels, of packed filters
     int nslots, bslots;             // (pixel, unit) and (filter row, unit) items per expander thread and chunk
     int e_bytes, b_bytes, stg_bytes, bstg_bytes;    // per stage
-    int off_e, off_stg, off_bstg, off_pix, off_tab, off_bar, off_out;
+    int off_e, off_stg, off_bstg, off_pix, off_brow, off_tab, off_bar, off_out;
     int tmem_cols, nacc;
     int preset;                     // accumulators start at the bit pattern of 1.5 * 2^23 (see the epilogue)
     int epi;                        // which instantiation of the fast requantisation
@@ -148,10 +149,10 @@ __device__ __forceinline__ void mm_mma(uint32_t d, uint32_t a_lo, uint32_t a_hi,
 {
     if (mm_elect())
         asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "setp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-            ::"r"(d), "l"((static_cast<uint64_t>(a_hi) << 32) | a_lo), "l"((static_cast<uint64_t>(b_hi) << 32) | b_lo), "r"(idesc), "r"(acc) : "memory");
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d), "l"((static_cast<uint64_t>(a_hi) << 32) | a_lo), "l"((static_cast<uint64_t>(b_hi) << 32) | b_lo), "r"(idesc), "r"(acc) : "memory");
 }
 __device__ __forceinline__ void mm_ld32(uint32_t taddr, uint32_t (&v)[32])
 {
@@ -312,6 +313,12 @@ template <int NB, int PSZ>
 __device__ __forceinline__ void stage_unit_p(uint32_t dst, uint32_t step, const uint32_t* src, const uint32_t* safe, int left)
 {
     constexpr int PW = PSZ / 4, NP = 2 * NB / PW > 0 ? 2 * NB / PW : 1;
+    if (left >= 2 * NB || left <= 0) {          // all of it, or none
+        const int bytes = left > 0 ? PSZ : 0;
+#pragma unroll
+        for (int k = 0; k < NP; ++k) mm_cp<PSZ>(dst + k * step, src + k * PW, bytes);
+        return;
+    }
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
         const int words = max(0, min(left - k * PW, PW));
@@ -400,22 +407,94 @@ __device__ __forceinline__ void issue_taps(uint32_t d, uint32_t a, uint32_t a_hi
         }
 }
 
-__device__ __forceinline__ void issue_block(const MmaArgs& g, uint32_t d, uint32_t a, uint32_t a_hi, uint32_t b, uint32_t b_hi, uint32_t acc)
+enum { TAPS_1 = 0, TAPS_3S1, TAPS_3S2, TAPS_ANY };
+
+template <int TAPS>
+__device__ __forceinline__ void issue_block(const MmaArgs& g, uint32_t d, uint32_t a, uint32_t a_hi, uint32_t b, uint32_t b_hi, uint32_t idesc, uint32_t acc,
+                                            uint32_t pitch, uint32_t HL)
 {
-    const uint32_t pitch = static_cast<uint32_t>(g.pitch), HL = static_cast<uint32_t>(g.HL);
-    if (g.R == 1) { mm_mma(d, a, a_hi, b, b_hi, g.idesc, acc); return; }
-    if (g.R == 3 && g.stride == 1) { issue_taps<3, 1>(d, a, a_hi, b, b_hi, g.idesc, acc, pitch, HL); return; }
-    if (g.R == 3 && g.pad == 1) { issue_taps<3, 2>(d, a, a_hi, b, b_hi, g.idesc, acc, pitch, HL); return; }
-    for (int r = 0; r < g.R; ++r)
-        for (int s = 0; s < g.R; ++s) {
-            const int rp = r - g.pad, sp = s - g.pad;
-            uint32_t off;
-            if (g.stride == 1) off = static_cast<uint32_t>(r * g.pitch + s);
-            else off = static_cast<uint32_t>(((rp & 1) * 2 + (sp & 1)) * g.HL + ((rp >> 1) - g.rmin) * g.pitch + (sp >> 1) - g.smin);
-            mm_mma(d, a + off, a_hi, b, b_hi, g.idesc, acc);
-            acc = 1u;
-            b += 16u;
+    if (TAPS == TAPS_1) mm_mma(d, a, a_hi, b, b_hi, idesc, acc);
+    else if (TAPS == TAPS_3S1) issue_taps<3, 1>(d, a, a_hi, b, b_hi, idesc, acc, pitch, HL);
+    else if (TAPS == TAPS_3S2) issue_taps<3, 2>(d, a, a_hi, b, b_hi, idesc, acc, pitch, HL);
+    else
+        for (int r = 0; r < g.R; ++r)
+            for (int s = 0; s < g.R; ++s) {
+                const int rp = r - g.pad, sp = s - g.pad;
+                uint32_t off;
+                if (g.stride == 1) off = static_cast<uint32_t>(r * g.pitch + s);
+                else off = static_cast<uint32_t>(((rp & 1) * 2 + (sp & 1)) * g.HL + ((rp >> 1) - g.rmin) * g.pitch + (sp >> 1) - g.smin);
+                mm_mma(d, a + off, a_hi, b, b_hi, idesc, acc);
+                acc = 1u;
+                b += 16u;
+            }
+}
+
+struct MmaIssue {
+    uint64_t *full_e, *empty_e, *full_acc, *empty_acc, *wgt_full;
+    uint32_t smem0, tmem;
+    int items;
+    bool resident;
+};
+
+// The MMA warp's walk over items and chunks.  Everything of a chunk, its commits included, goes out in one elected region.
+template <int TAPS>
+__device__ __forceinline__ void issue_items(const MmaArgs& g, const MmaIssue& m)
+{
+    const uint32_t NI16 = static_cast<uint32_t>(g.NI);
+    // K-major, no swizzle: core matrices of 8 rows x 16 bytes; leading offset = next 16 channels, stride offset = next 8 rows
+    const uint32_t a_hi = (128u >> 4) | (1u << 14), b_hi = static_cast<uint32_t>(g.RS * 16) | (1u << 14);
+    const uint32_t a_lo0 = (NI16 & 0x3FFFu) << 16, b_lo0 = (128u >> 4) << 16;
+    const uint32_t e_base = (m.smem0 + g.off_e) >> 4, w_base = m.smem0 >> 4;
+    const uint32_t blk16 = static_cast<uint32_t>(g.TN * g.RS * 2), idesc = g.idesc;
+    const uint32_t pitch = static_cast<uint32_t>(g.pitch), HL = static_cast<uint32_t>(g.HL), TN = static_cast<uint32_t>(g.TN);
+    const uint32_t e16 = static_cast<uint32_t>(g.e_bytes >> 4), b16 = static_cast<uint32_t>(g.b_bytes >> 4);
+    const int nchunks = g.nchunks, PT = g.PT, per_chunk = g.units * 2, Cw = g.Cw, nse = g.nse, nacc = g.nacc;
+    unsigned limit = 1u << 20;
+    if (m.resident) mm_wait_uniform(m.wgt_full, 0, limit);
+    MM_TRACE((threadIdx.x & 31) == 0, TR_WGT, 0);
+#ifdef BS_TRACE
+    int mseq = 0;
+#endif
+    int ie = 0, ia = 0;
+    unsigned pe = 0, pa = 0;
+    const uint32_t acc0 = g.preset ? 1u : 0u;
+    for (int it = blockIdx.x; it < m.items; it += gridDim.x) {
+        mm_wait_uniform(&m.empty_acc[ia], pa, limit);
+        const uint32_t d0 = m.tmem + static_cast<uint32_t>(ia * PT) * TN;
+        for (int c = 0; c < nchunks; ++c) {
+            const int b0 = c * per_chunk;
+            const int nb = Cw - b0 < per_chunk ? Cw - b0 : per_chunk;
+            const uint32_t wb = b_lo0 | (w_base + (m.resident ? static_cast<uint32_t>(b0) * blk16 : static_cast<uint32_t>(ie) * b16));
+            const uint32_t eb = a_lo0 | (e_base + static_cast<uint32_t>(ie) * e16);
+            mm_wait_uniform(&m.full_e[ie], pe, limit);
+            mm_fence_after();
+            MM_TRACE((threadIdx.x & 31) == 0, TR_MBEG, mseq);
+            {
+                uint32_t acc = c == 0 ? acc0 : 1u;
+                uint32_t d = d0, at = eb;
+                for (int t = 0; t < PT; ++t, d += TN, at += 128u) {
+                    uint32_t a = at, b = wb;
+                    issue_block<TAPS>(g, d, a, a_hi, b, b_hi, idesc, acc, pitch, HL);
+#pragma unroll(TAPS == TAPS_1 ? 4 : 1)
+                    for (int k = 1; k < nb; ++k) {
+                        a += 2u * NI16;
+                        b += blk16;
+                        issue_block<TAPS>(g, d, a, a_hi, b, b_hi, idesc, 1u, pitch, HL);
+                    }
+                }
+                mm_commit(&m.empty_e[ie]);
+                if (c == nchunks - 1) mm_commit(&m.full_acc[ia]);
+            }
+#ifdef BS_TRACE
+            MM_TRACE((threadIdx.x & 31) == 0, TR_MEND, mseq);
+            ++mseq;
+#endif
+            if (++ie == nse) { ie = 0; pe ^= 1u; }
         }
+        if (++ia == nacc) { ia = 0; pa ^= 1u; }
+    }
+    if (limit == 1u && (threadIdx.x & 31) == 0) atomicOr(g.status, STATUS_TIMEOUT);
+    __syncwarp();
 }
 
 // ----------------------------------------------------------------------------- epilogue
@@ -818,20 +897,19 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
     uint64_t* bars = reinterpret_cast<uint64_t*>(mm_smem + g.off_bar);
     uint64_t* full_e = bars;            // [4]
     uint64_t* empty_e = bars + 4;       // [4]
-    uint64_t* full_b = bars + 8;        // [4]
-    uint64_t* empty_b = bars + 12;      // [4]
-    uint64_t* full_acc = bars + 16;     // [2]
-    uint64_t* empty_acc = bars + 18;    // [2]
-    uint64_t* wgt_full = bars + 20;
-    uint64_t* bulk_full = bars + 21;
-    uint64_t* full_p = bars + 22;       // [MM_STAGES] packed rows landed
-    uint64_t* empty_p = bars + 25;      // [MM_STAGES] ... and expanded
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 28);
-    int* fast_ok = reinterpret_cast<int*>(bars + 29);
+    uint64_t* full_acc = bars + 8;      // [2]
+    uint64_t* empty_acc = bars + 10;    // [2]
+    uint64_t* wgt_full = bars + 12;
+    uint64_t* bulk_full = bars + 13;
+    uint64_t* full_p = bars + 14;       // [MM_STAGES] packed rows landed
+    uint64_t* empty_p = bars + 22;      // [MM_STAGES] ... and expanded
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 30);
+    int* fast_ok = reinterpret_cast<int*>(bars + 31);
 
     constexpr bool packed_b = WB > 0;
     constexpr int WBX = WB > 0 ? WB : 1;
     const bool resident = g.nsb == 0;
+    const bool stream_prepared = !resident && !packed_b;      // a stage then holds expanded pixels and the filters of the same chunk
     const int items = g.tiles_m * g.tiles_o;
     const int BM = 128 * g.PT;
 
@@ -839,15 +917,13 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
     mm_pdl_release();
     if (tid == 0) {
         for (int s = 0; s < 4; ++s) {
-            mbar_init(&full_e[s], XW);
+            mbar_init(&full_e[s], XW / g.groups + (stream_prepared ? 1 : 0));
             mbar_init(&empty_e[s], 1);
-            mbar_init(&full_b[s], 1);
-            mbar_init(&empty_b[s], 1);
         }
         for (int s = 0; s < 2; ++s) { mbar_init(&full_acc[s], 1); mbar_init(&empty_acc[s], EW); }
         mbar_init(wgt_full, packed_b ? XW + EW : 1);
         mbar_init(bulk_full, 1);
-        for (int s = 0; s < MM_STAGES; ++s) { mbar_init(&full_p[s], 1); mbar_init(&empty_p[s], XW); }
+        for (int s = 0; s < MM_STAGES; ++s) { mbar_init(&full_p[s], 1); mbar_init(&empty_p[s], XW / g.groups); }
         *fast_ok = 1;
         fence_barrier_init();
         fence_proxy_async();
@@ -860,7 +936,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
     mm_fence_before();
     __syncthreads();
     mm_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);      // uniform for the compiler, as above
     MM_TRACE(tid == 0, TR_SETUP, 0);
 
     // a CTA with resident filters keeps its filter tile; otherwise the filter tile runs fastest over the items
@@ -886,7 +962,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                     }
                 }
             }
-            const bool stream = !resident && !packed_b;
+            const bool stream = stream_prepared;
             if (stream || g.tma) {
                 int ib = 0, ip = 0;
                 unsigned pb = 0, pp = 0;
@@ -894,14 +970,14 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                     const int8_t* src = g.wgt + static_cast<size_t>(w.o) * g.TN * g.RS * 32;
                     for (int c = 0; c < g.nchunks && ok; ++c) {
                         if (stream) {
-                            ok = mm_wait(&empty_b[ib], pb ^ 1u);
+                            ok = mm_wait(&empty_e[ib], pb ^ 1u);
                             if (!ok) break;
                             const int b0 = c * g.units * 2;
                             const int nb = g.Cw - b0 < g.units * 2 ? g.Cw - b0 : g.units * 2;
-                            mbar_expect_tx(&full_b[ib], blk_bytes * nb);
+                            mbar_expect_tx(&full_e[ib], blk_bytes * nb);
                             for (int b = 0; b < nb; ++b)
-                                mm_bulk(mm_smem + static_cast<size_t>(ib) * g.b_bytes + static_cast<size_t>(b) * blk_bytes, src + (b0 + b) * blk_stride, blk_bytes, &full_b[ib]);
-                            if (++ib == g.nsb) { ib = 0; pb ^= 1u; }
+                                mm_bulk(mm_smem + static_cast<size_t>(ib) * g.b_bytes + static_cast<size_t>(b) * blk_bytes, src + (b0 + b) * blk_stride, blk_bytes, &full_e[ib]);
+                            if (++ib == g.nse) { ib = 0; pb ^= 1u; }
                         }
                         if (g.tma) {
                             if (!waited) { mm_pdl_wait(); waited = true; }
@@ -913,7 +989,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                             const int rows = BM < 256 ? BM : 256;
                             for (int r = 0; r < BM; r += rows) tma_load_2d(dst + r * g.rowA, &g.tmA, &full_p[ip], c * (g.rowA >> 2), w.m * BM + r);
                             if (fb) tma_load_2d(mm_smem + g.off_bstg + ip * g.bstg_bytes, &g.tmB, &full_p[ip], c * (g.rowB >> 2), w.o * g.TN);
-                            if (++ip == MM_STAGES) { ip = 0; pp ^= 1u; }
+                            if (++ip == g.nsp) { ip = 0; pp ^= 1u; }
                         }
                     }
                 }
@@ -923,55 +999,11 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
         __syncwarp();
     } else if (warp == WARP_MMA) {
         // ------------------------------------------------------------------ MMA issuer (all lanes in step)
-        const uint32_t NI16 = static_cast<uint32_t>(g.NI);
-        // K-major, no swizzle: core matrices of 8 rows x 16 bytes; leading offset = next 16 channels, stride offset = next 8 rows
-        const uint32_t a_hi = (128u >> 4) | (1u << 14), b_hi = static_cast<uint32_t>(g.RS * 16) | (1u << 14);
-        const uint32_t a_lo0 = (NI16 & 0x3FFFu) << 16, b_lo0 = (128u >> 4) << 16;
-        const uint32_t e_base = (smem0 + g.off_e) >> 4, w_base = smem0 >> 4;
-        const uint32_t blk16 = static_cast<uint32_t>(g.TN * g.RS * 2);
-        const bool wait_b = !resident && !packed_b;
-        unsigned limit = 1u << 20;
-        if (resident) mm_wait_uniform(wgt_full, 0, limit);
-        MM_TRACE(lane == 0, TR_WGT, 0);
-#ifdef BS_TRACE
-        int mseq = 0;
-#endif
-        int ie = 0, ib = 0, ia = 0;
-        unsigned pe = 0, pb = 0, pa = 0;
-        const uint32_t acc0 = g.preset ? 1u : 0u;
-        for (int it = blockIdx.x; it < items; it += gridDim.x) {
-            mm_wait_uniform(&empty_acc[ia], pa, limit);
-            mm_fence_after();
-            const uint32_t d0 = tmem + static_cast<uint32_t>(ia * g.PT * g.TN);
-            for (int c = 0; c < g.nchunks; ++c) {
-                mm_wait_uniform(&full_e[ie], pe, limit);
-                if (wait_b) mm_wait_uniform(&full_b[ib], pb, limit);
-                mm_fence_after();
-                MM_TRACE(lane == 0, TR_MBEG, mseq);
-                const int b0 = c * g.units * 2;
-                const int nb = g.Cw - b0 < g.units * 2 ? g.Cw - b0 : g.units * 2;
-                const uint32_t wb = w_base + (resident ? static_cast<uint32_t>(b0) * blk16 : static_cast<uint32_t>((packed_b ? ie : ib) * (g.b_bytes >> 4)));
-                const uint32_t eb = e_base + static_cast<uint32_t>(ie * (g.e_bytes >> 4));
-                for (int t = 0; t < g.PT; ++t)
-                    for (int b = 0; b < nb; ++b)
-                        issue_block(g, d0 + static_cast<uint32_t>(t * g.TN), a_lo0 | (eb + static_cast<uint32_t>(t * 128) + static_cast<uint32_t>(b) * 2u * NI16), a_hi,
-                                    b_lo0 | (wb + static_cast<uint32_t>(b) * blk16), b_hi, (c == 0 && b == 0) ? acc0 : 1u);
-                mm_commit(&empty_e[ie]);
-#ifdef BS_TRACE
-                MM_TRACE(lane == 0, TR_MEND, mseq);
-                ++mseq;
-#endif
-                if (wait_b) {
-                    mm_commit(&empty_b[ib]);
-                    if (++ib == g.nsb) { ib = 0; pb ^= 1u; }
-                }
-                if (++ie == g.nse) { ie = 0; pe ^= 1u; }
-            }
-            mm_commit(&full_acc[ia]);
-            if (++ia == g.nacc) { ia = 0; pa ^= 1u; }
-        }
-        if (limit == 1u && lane == 0) atomicOr(g.status, STATUS_TIMEOUT);
-        __syncwarp();
+        const MmaIssue m{full_e, empty_e, full_acc, empty_acc, wgt_full, smem0, tmem, items, resident};
+        if (g.R == 1) issue_items<TAPS_1>(g, m);
+        else if (g.R == 3 && g.stride == 1) issue_items<TAPS_3S1>(g, m);
+        else if (g.R == 3 && g.pad == 1) issue_items<TAPS_3S2>(g, m);
+        else issue_items<TAPS_ANY>(g, m);
     } else if (warp >= EW && warp < WARP_COPY) {
         // ------------------------------------------------------------------ expanders
         const int xt = tid - NET;
@@ -990,23 +1022,29 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
             __syncwarp();
             if (lane == 0) mm_arrive(wgt_full);
         }
-        mm_pdl_wait();
-        MM_TRACE(xt == 0, TR_PDL, 0);
+        // A chunk belongs to one group of warps.  The waits, the fence and the arrival of a chunk take several hundred cycles whatever its
+        // size; with several groups they overlap (see make_plan for how many).
+        const int G = g.groups, nx = NXT / G, xg = xt / nx, xl = xt - xg * nx;
 #ifdef BS_TRACE
         int xseq = 0;
 #endif
         if (g.tma) {
+            mm_pdl_wait();
+            MM_TRACE(xt == 0, TR_PDL, 0);
             // Flat tiles: the copy warp fetches boxes of [row][units] with TMA (a thread-by-thread copy touches one 128-byte line per
             // lane: 32 tag cycles per instruction, a thousand cycles per 256 rows of 128 channels).  Items (unit, row), row
             // fastest; the 16-byte pieces of a row are swizzled by the box so that 32 rows read without bank conflicts.
             const bool stream_b = packed_b && !resident;
             const int rowsA = BM, shA = 31 - __clz(BM), shB = 31 - __clz(g.TN);
-            int idx = 0, ip = 0;
+            int idx = xg, ip = xg;
             unsigned phase = 0, pp = 0;
             bool ok = true;
             const uint32_t g16 = static_cast<uint32_t>(g.NI) * 16u;
-            for (MmaWalk w(g); w.m < g.tiles_m && ok; w.next(g)) {
-                for (int c = 0; c < g.nchunks; ++c) {
+            int c = xg;
+            MmaWalk w(g);
+            while (c >= g.nchunks) { c -= g.nchunks; w.next(g); }
+            while (w.m < g.tiles_m) {
+                {
                     MM_TRACE(xt == 0, TR_XWAIT, xseq);
                     ok = mm_wait(&full_p[ip], pp);
                     if (ok) ok = mm_wait(&empty_e[idx], phase ^ 1u);
@@ -1015,7 +1053,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                     const int nu = g.nunits - c * g.units < g.units ? g.nunits - c * g.units : g.units;
                     const uint32_t src = smem0 + g.off_stg + static_cast<uint32_t>(ip * g.stg_bytes);
                     const uint32_t e0 = smem0 + g.off_e + static_cast<uint32_t>(idx * g.e_bytes);
-                    for (int it = xt; it < nu << shA; it += NXT) {
+                    for (int it = xl; it < nu << shA; it += nx) {
                         const int u = it >> shA, i = it & (rowsA - 1);
                         uint32_t wd[2 * A];
                         load_row_unit<A>(src, i * g.rowA + u * 8 * A, g.swzA, wd);
@@ -1024,7 +1062,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                     if (stream_b) {
                         const uint32_t bsrc = smem0 + g.off_bstg + static_cast<uint32_t>(ip * g.bstg_bytes);
                         const uint32_t bdst = smem0 + static_cast<uint32_t>(idx * g.b_bytes), blk = static_cast<uint32_t>(g.TN) * 32u;
-                        for (int it = xt; it < nu << shB; it += NXT) {
+                        for (int it = xl; it < nu << shB; it += nx) {
                             const int u = it >> shB, i = it & (g.TN - 1);
                             const int f = (i & ~31) + mma_filter_of_column(i & 31);
                             uint32_t wd[2 * WBX];
@@ -1042,20 +1080,27 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                     MM_TRACE(xt == 0, TR_XEND, xseq);
                     ++xseq;
 #endif
-                    if (++idx == g.nse) { idx = 0; phase ^= 1u; }
-                    if (++ip == MM_STAGES) { ip = 0; pp ^= 1u; }
+                    idx += G;
+                    if (idx >= g.nse) { idx -= g.nse; phase ^= 1u; }
+                    ip += G;
+                    if (ip >= g.nsp) { ip -= g.nsp; pp ^= 1u; }
+                    c += G;
+                    while (c >= g.nchunks) { c -= g.nchunks; w.next(g); }
                 }
             }
             if (!ok && lane == 0) atomicOr(g.status, STATUS_TIMEOUT);
         } else {
-        // Packed words travel through MM_STAGES stages of shared memory, one chunk (and one cp.async group) each, issued
-        // MM_STAGES - 1 chunks ahead.  A thread copies and later expands the same items, so nothing needs a barrier.
+        // Packed words travel through a group's own stages of shared memory, one chunk (and one cp.async group) each, issued as many of
+        // its chunks ahead as it has stages.  A thread copies and later expands the same items, so nothing needs a barrier.
         const bool stream_b = packed_b && !resident;
         const int rec = g.Cw * A, rows = g.TN * g.RS;
-        const uint32_t stg0 = smem0 + g.off_stg + static_cast<uint32_t>(xt * g.psz), bstg0 = smem0 + g.off_bstg + static_cast<uint32_t>(xt * g.bpsz);
-        const uint32_t step = static_cast<uint32_t>(g.nslots * NXT * g.psz), bstep = static_cast<uint32_t>(g.bslots * NXT * g.bpsz);
+        constexpr int stages = 2;
+        const uint32_t stg0 = smem0 + g.off_stg + static_cast<uint32_t>(xg * stages * g.stg_bytes + xl * g.psz);
+        const uint32_t bstg0 = smem0 + g.off_bstg + static_cast<uint32_t>(xg * stages * g.bstg_bytes + xl * g.bpsz);
+        const uint32_t step = static_cast<uint32_t>(g.nslots * nx * g.psz), bstep = static_cast<uint32_t>(g.bslots * nx * g.bpsz);
+        const uint32_t rel0 = smem0 + g.off_pix, pix0 = rel0 + static_cast<uint32_t>((1 + xg * (stages + 1)) * g.NI) * 4u, brow0 = smem0 + g.off_brow;
         // Where row i of a halo sits relative to the halo's first position: rows and columns of the position grid, parity plane.
-        // Fixed for a thread's slots, so it is found once per kernel; a tile then only adds its own origin.
+        // Found once per kernel; a tile adds its own origin.
         for (int i = xt; i < g.NI && !g.flat; i += NXT) {
             int h = i, pl = 0;
             if (g.nplanes > 1) {
@@ -1063,55 +1108,88 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                 h = i - pl * g.HL;
             }
             const int hq = fdiv(h, g.d_pitch), hr = h - hq * g.d_pitch.d;
-            asm volatile("st.shared.b32 [%0], %1;" ::"r"(smem0 + g.off_pix + static_cast<uint32_t>(i) * 4u), "r"((static_cast<uint32_t>(pl) << 30) | static_cast<uint32_t>((hq << 15) | hr)) : "memory");
+            asm volatile("st.shared.b32 [%0], %1;" ::"r"(rel0 + static_cast<uint32_t>(i) * 4u), "r"((static_cast<uint32_t>(pl) << 30) | static_cast<uint32_t>((hq << 15) | hr)) : "memory");
         }
-        if (g.units > 1 && !g.flat) asm volatile("bar.sync 3, %0;" ::"n"(NXT) : "memory");      // (unit, pixel) items read other threads' entries
-        MmaWalk iw(g);
-        int ic = 0, ibuf = 0;
-        int oy = 0, ox = 0, on = 0, ostrip = 0;              // origin of the halo being copied: row, column, image, strip
+        // Packed record of filter row i: filter of the tile in the top byte, record below it (taps and tile filters number at most 2^14).
+        if (stream_b && g.units == 1)
+            for (int i = xt; i < rows; i += NXT) {
+                int off;
+                const int f = filter_row(g, i, 1, off);
+                asm volatile("st.shared.b32 [%0], %1;" ::"r"(brow0 + static_cast<uint32_t>(i) * 4u), "r"((static_cast<uint32_t>(f) << 24) | static_cast<uint32_t>(off / g.Cw)) : "memory");
+            }
+        if (g.units > 1 || G > 1) asm volatile("bar.sync 3, %0;" ::"n"(NXT) : "memory");      // other threads' entries are read
+        MmaWalk iw(g), lw(g);
+        int ic = xg, ibuf = 0, iitem = -1, itab = 0;
+        while (ic >= g.nchunks) { ic -= g.nchunks; iw.next(g); }
+        int lc = ic, litem = -1, ltab = 0;
+        lw = iw;
+        int oy = 0, ox = 0, on = 0, ostrip = 0;              // origin of a halo: row, column, image, strip
         const int PH = g.img_rows;
+        auto origin = [&](int m) {
+            // (image, strip) and row of the first position; a halo may start above the first image
+            const int b0 = m * BM + g.hstart + g.d_img.d;
+            const int u = fdiv(b0, g.d_img), rem = b0 - u * g.d_img.d;
+            oy = fdiv(rem, g.d_pitch);
+            ox = rem - oy * g.d_pitch.d;
+            on = fdiv(u - 1 < 0 ? 0 : u - 1, g.d_strips);
+            ostrip = u - 1 - on * g.d_strips.d;
+        };
+        // input pixel of row i of the halo at the origin; -1: padding
+        auto halo_pixel = [&](int i) -> int {
+            uint32_t e;
+            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(e) : "r"(rel0 + static_cast<uint32_t>(i) * 4u));
+            int x = ox + static_cast<int>(e & 0x7FFFu), y = oy + static_cast<int>((e >> 15) & 0x7FFFu);
+            if (x >= g.d_pitch.d) { x -= g.d_pitch.d; ++y; }
+            int n = on, strip = ostrip;
+            while (y >= PH) { y -= PH; if (++strip == g.d_strips.d) { strip = 0; ++n; } }
+            const int Y = y * g.stride + static_cast<int>(e >> 31), X = (x + g.xoff + strip * g.strip_q) * g.stride + static_cast<int>((e >> 30) & 1u);
+            const bool in = n < g.N && strip >= 0 && Y < g.H && static_cast<unsigned>(X) < static_cast<unsigned>(g.W);
+            return in ? (n * g.H + Y) * g.W + X : -1;
+        };
+        auto flat_pixel = [&](int m, int i) -> int { return m * BM + i < g.total ? m * BM + i : -1; };
+        // The pixels of a thread's rows are found one chunk before their copies are issued, the first ones while the preceding kernel
+        // still runs, and kept in shared memory for all chunks of the item: about 40 instructions a row that would otherwise
+        // stand in front of every chunk's copies (a thousand cycles a chunk, more than the MMAs of 64 channels take).
+        auto locate = [&]() {
+            if (g.flat || g.units > 1) return;
+            if (lw.m < g.tiles_m && lw.it != litem) {
+                litem = lw.it;
+                origin(lw.m);
+                const uint32_t t = pix0 + static_cast<uint32_t>(ltab * g.NI) * 4u;
+                for (int i = xl; i < g.NI; i += nx) asm volatile("st.shared.b32 [%0], %1;" ::"r"(t + static_cast<uint32_t>(i) * 4u), "r"(halo_pixel(i)) : "memory");
+                if (++ltab > stages) ltab = 0;
+            }
+            lc += G;
+            while (lc >= g.nchunks) { lc -= g.nchunks; lw.next(g); }
+        };
+        uint32_t ipix = 0;
         auto issue = [&]() {
             if (iw.m < g.tiles_m) {
-                const int base = iw.m * BM + g.hstart;
-                if (!g.flat && ic == 0) {
-                    // (image, strip) and row of the first position; a halo may start above the first image
-                    const int b0 = base + g.d_img.d;
-                    const int u = fdiv(b0, g.d_img), rem = b0 - u * g.d_img.d;
-                    oy = fdiv(rem, g.d_pitch);
-                    ox = rem - oy * g.d_pitch.d;
-                    on = fdiv(u - 1 < 0 ? 0 : u - 1, g.d_strips);
-                    ostrip = u - 1 - on * g.d_strips.d;
+                if (iw.it != iitem) {
+                    iitem = iw.it;
+                    if (g.units > 1 && !g.flat) origin(iw.m);
+                    ipix = pix0 + static_cast<uint32_t>(itab * g.NI) * 4u;
+                    if (++itab > stages) itab = 0;
                 }
-                // input pixel of row i; -1: padding
-                auto halo_pixel = [&](int i) -> int {
-                    if (g.flat) return base + i < g.total ? base + i : -1;
-                    uint32_t e;
-                    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(e) : "r"(smem0 + g.off_pix + static_cast<uint32_t>(i) * 4u));
-                    int x = ox + static_cast<int>(e & 0x7FFFu), y = oy + static_cast<int>((e >> 15) & 0x7FFFu);
-                    if (x >= g.d_pitch.d) { x -= g.d_pitch.d; ++y; }
-                    int n = on, strip = ostrip;
-                    while (y >= PH) { y -= PH; if (++strip == g.d_strips.d) { strip = 0; ++n; } }
-                    const int Y = y * g.stride + static_cast<int>(e >> 31), X = (x + g.xoff + strip * g.strip_q) * g.stride + static_cast<int>((e >> 30) & 1u);
-                    const bool in = n < g.N && strip >= 0 && Y < g.H && static_cast<unsigned>(X) < static_cast<unsigned>(g.W);
-                    return in ? (n * g.H + Y) * g.W + X : -1;
-                };
                 uint32_t dst = stg0 + static_cast<uint32_t>(ibuf * g.stg_bytes);
                 if (g.units == 1) {
                     const int left = (g.Cw - 2 * ic) * A;
                     const uint32_t* src = g.act + 2 * ic * A;
-                    for (int i = xt; i < g.NI; i += NXT, dst += NXT * g.psz) {
-                        const int pixel = halo_pixel(i);
+                    for (int i = xl; i < g.NI; i += nx, dst += nx * g.psz) {
+                        int pixel;
+                        if (g.flat) pixel = flat_pixel(iw.m, i);
+                        else asm volatile("ld.shared.b32 %0, [%1];" : "=r"(pixel) : "r"(ipix + static_cast<uint32_t>(i) * 4u));
                         stage_unit<A>(g.psz, dst, step, src + static_cast<size_t>(static_cast<unsigned>(pixel < 0 ? 0 : pixel)) * rec, g.act, pixel >= 0 ? left : 0);
                     }
                 } else {
                     // items (unit, pixel), pixel fastest
-                    int u = 0, i = xt;
+                    int u = 0, i = xl;
                     while (i >= g.NI) { i -= g.NI; ++u; }
-                    for (; u < g.units; dst += NXT * g.psz) {
-                        const int pixel = halo_pixel(i), unit = ic * g.units + u;
+                    for (; u < g.units; dst += nx * g.psz) {
+                        const int pixel = g.flat ? flat_pixel(iw.m, i) : halo_pixel(i), unit = ic * g.units + u;
                         stage_unit<A>(g.psz, dst, step, g.act + static_cast<size_t>(static_cast<unsigned>(pixel < 0 ? 0 : pixel)) * rec + 2 * unit * A, g.act,
                                       pixel >= 0 ? (g.Cw - 2 * unit) * A : 0);
-                        i += NXT;
+                        i += nx;
                         while (i >= g.NI) { i -= g.NI; ++u; }
                     }
                 }
@@ -1119,30 +1197,47 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                     const uint32_t* base = g.wgt_packed + static_cast<size_t>(iw.o) * g.TN * g.RS * g.Cw * WBX;
                     const int o0 = iw.o * g.TN;
                     dst = bstg0 + static_cast<uint32_t>(ibuf * g.bstg_bytes);
-                    int u = 0, i = xt;
-                    while (i >= rows) { i -= rows; ++u; }
-                    for (; u < g.units; dst += NXT * g.bpsz) {
-                        int off;
-                        const bool live = o0 + filter_row(g, i, WBX, off) < g.O;
-                        const int unit = ic * g.units + u;
-                        stage_unit<WBX>(g.bpsz, dst, bstep, base + off + 2 * unit * WBX, g.wgt_packed, live ? (g.Cw - 2 * unit) * WBX : 0);
-                        i += NXT;
+                    if (g.units == 1) {
+                        const int left = (g.Cw - 2 * ic) * WBX;
+                        const uint32_t* src = base + 2 * ic * WBX;
+                        for (int i = xl; i < rows; i += nx, dst += nx * g.bpsz) {
+                            uint32_t e;
+                            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(e) : "r"(brow0 + static_cast<uint32_t>(i) * 4u));
+                            const bool live = o0 + static_cast<int>(e >> 24) < g.O;
+                            stage_unit<WBX>(g.bpsz, dst, bstep, src + (e & 0xFFFFFFu) * static_cast<unsigned>(g.Cw * WBX), g.wgt_packed, live ? left : 0);
+                        }
+                    } else {
+                        int u = 0, i = xl;
                         while (i >= rows) { i -= rows; ++u; }
+                        for (; u < g.units; dst += nx * g.bpsz) {
+                            int off;
+                            const bool live = o0 + filter_row(g, i, WBX, off) < g.O;
+                            const int unit = ic * g.units + u;
+                            stage_unit<WBX>(g.bpsz, dst, bstep, base + off + 2 * unit * WBX, g.wgt_packed, live ? (g.Cw - 2 * unit) * WBX : 0);
+                            i += nx;
+                            while (i >= rows) { i -= rows; ++u; }
+                        }
                     }
                 }
-                if (++ic == g.nchunks) { ic = 0; iw.next(g); }
+                ic += G;
+                while (ic >= g.nchunks) { ic -= g.nchunks; iw.next(g); }
             }
             cp_async_commit();
-            if (++ibuf == MM_STAGES) ibuf = 0;
+            if (++ibuf == stages) ibuf = 0;
         };
-        int buf = 0, idx = 0;
+        int buf = 0, idx = xg;
         unsigned phase = 0;
         bool ok = true;
-        for (int s = 0; s < MM_STAGES - 1; ++s) issue();
-        for (MmaWalk w(g); w.m < g.tiles_m; w.next(g)) {
-            for (int c = 0; c < g.nchunks; ++c) {
-                issue();
-                asm volatile("cp.async.wait_group %0;" ::"n"(MM_STAGES - 1) : "memory");
+        for (int s = 0; s <= stages; ++s) locate();
+        mm_pdl_wait();
+        MM_TRACE(xt == 0, TR_PDL, 0);
+        for (int s = 0; s < stages; ++s) issue();
+        MmaWalk w(g);
+        int c = xg;
+        while (c >= g.nchunks) { c -= g.nchunks; w.next(g); }
+        while (w.m < g.tiles_m) {
+            {
+                asm volatile("cp.async.wait_group %0;" ::"n"(stages - 1) : "memory");
                 MM_TRACE(xt == 0, TR_XWAIT, xseq);
                 if (ok) ok = mm_wait(&empty_e[idx], phase ^ 1u);
                 MM_TRACE(xt == 0, TR_XBEG, xseq);
@@ -1151,20 +1246,20 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                 uint32_t src = stg0 + static_cast<uint32_t>(buf * g.stg_bytes);
                 const uint32_t e0 = smem0 + g.off_e + static_cast<uint32_t>(idx * g.e_bytes);
                 if (g.units == 1) {
-                    uint32_t dst = e0 + static_cast<uint32_t>(xt) * 16u;
-                    for (int i = xt; i < g.NI; i += NXT, src += NXT * g.psz, dst += NXT * 16) {
+                    uint32_t dst = e0 + static_cast<uint32_t>(xl) * 16u;
+                    for (int i = xl; i < g.NI; i += nx, src += nx * g.psz, dst += nx * 16) {
                         uint32_t wd[2 * A];
                         load_unit<A>(src, step, g.psz, wd);
                         expand_unit<A>(wd, g.a_kind, dst, g16);
                     }
                 } else {
-                    int u = 0, i = xt;
+                    int u = 0, i = xl;
                     while (i >= g.NI) { i -= g.NI; ++u; }
-                    for (; u < nu; src += NXT * g.psz) {
+                    for (; u < nu; src += nx * g.psz) {
                         uint32_t wd[2 * A];
                         load_unit<A>(src, step, g.psz, wd);
                         expand_unit<A>(wd, g.a_kind, e0 + static_cast<uint32_t>(u) * 4u * g16 + static_cast<uint32_t>(i) * 16u, g16);
-                        i += NXT;
+                        i += nx;
                         while (i >= g.NI) { i -= g.NI; ++u; }
                     }
                 }
@@ -1172,9 +1267,9 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                     src = bstg0 + static_cast<uint32_t>(buf * g.bstg_bytes);
                     const uint32_t bdst = smem0 + static_cast<uint32_t>(idx * g.b_bytes), blk = static_cast<uint32_t>(rows) * 32u;
                     const bool all_live = (w.o + 1) * g.TN <= g.O;
-                    int u = 0, i = xt;
+                    int u = 0, i = xl;
                     while (i >= rows) { i -= rows; ++u; }
-                    for (; u < nu; src += NXT * g.bpsz) {
+                    for (; u < nu; src += nx * g.bpsz) {
                         uint32_t wd[2 * WBX];
                         load_unit<WBX>(src, bstep, g.bpsz, wd);
                         bool live = true;
@@ -1183,7 +1278,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                         const uint32_t d = bdst + static_cast<uint32_t>(2 * u) * blk + static_cast<uint32_t>(i >> 3) * 256u + static_cast<uint32_t>(i & 7) * 16u;
                         expand_filter_word<WBX>(wd, g.w_kind, live, d);
                         expand_filter_word<WBX>(wd + WBX, g.w_kind, live, d + blk);
-                        i += NXT;
+                        i += nx;
                         while (i >= rows) { i -= rows; ++u; }
                     }
                 }
@@ -1194,8 +1289,13 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                 MM_TRACE(xt == 0, TR_XEND, xseq);
                 ++xseq;
 #endif
-                if (++idx == g.nse) { idx = 0; phase ^= 1u; }
-                if (++buf == MM_STAGES) buf = 0;
+                issue();                       // into the stage just read
+                locate();
+                idx += G;
+                if (idx >= g.nse) { idx -= g.nse; phase ^= 1u; }
+                if (++buf == stages) buf = 0;
+                c += G;
+                while (c >= g.nchunks) { c -= g.nchunks; w.next(g); }
             }
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
