@@ -36,13 +36,13 @@ FastDiv make_div(int d)
 int max_abs_of(int bits, int sign) { return sign == BS_BIPOLAR ? 1 : (sign == BS_SIGNED ? 1 << (bits - 1) : (1 << bits) - 1); }
 
 struct Cand {
-    int TN, PT, units, cfg, cps, ns, resident, groups, nse, nsb, nacc;
+    int TN, PT, units, cfg, cps, ns, resident, groups, split, nse, nsb, nacc;
     size_t smem;
     double cost;
 };
 
 // Shared-memory layout of a candidate; false when it does not fit.  g carries the problem, the candidate the tiling.
-bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows)
+bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows, int sms)
 {
     const bool packed_b = WB > 0;
     const int st = g.stride, XT = c.cfg ? 256 : 128, EW = c.cfg ? 8 : 4;
@@ -80,6 +80,12 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows)
     g.tiles_m = static_cast<int>(ceil_div_ll(total, BM));
     g.tiles_o = ceil_div(g.O, c.TN);
     g.d_rs = make_div(g.RS);
+    // An item split over a cluster: every CTA streams its chunks, at least two of them (with one, the sums cost what it saves).  No more CTAs than two thirds of the SMs: clusters need SMs of one
+    // GPC that are free at the same time, and 128 CTAs in clusters of four already ran 20 to 50 % longer than without the split.
+    g.split = c.split;
+    g.split_log = c.split == 1 ? 0 : c.split == 2 ? 1 : c.split == 4 ? 2 : 3;
+    if (c.split > 1 && (c.resident || c.cps != 1 || g.nchunks < 2 * c.split || static_cast<long long>(g.tiles_m) * g.tiles_o * c.split * 3 > 2 * sms)) return false;
+    const int red_bytes = (c.split - 1) * 128 * c.PT * c.TN * 4;
     g.groups = c.groups;
     const int GT = XT / c.groups;                          // threads of an expander group
     g.nslots = ceil_div(g.NI * c.units, GT);
@@ -103,7 +109,7 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows)
     const int rel_bytes = g.flat ? 0 : up(g.NI * 4 * (1 + (c.units == 1 ? g.nsp + c.groups : 0)), 16);      // relative rows; located pixels of each group, one table more than stages
     const int pix_bytes = rel_bytes + (fb && !g.tma && c.units == 1 ? up(c.TN * g.RS * 4, 16) : 0);
     const int cap = c.cfg ? 222 * 1024 : 111 * 1024;
-    const int fixed = c.TN * 8 + 64 + 256 + (g.tma ? 1024 : 0) + (int_rows ? EW * 4096 : 0) + 256 + pix_bytes;
+    const int fixed = c.TN * 8 + 64 + 320 + red_bytes + (g.tma ? 1024 : 0) + (int_rows ? EW * 4096 : 0) + 256 + pix_bytes;
     const long long filters = c.resident ? static_cast<long long>(g.Cw) * c.TN * g.RS * 32 : 0;
     const long long rest = fixed + static_cast<long long>(g.nsp) * (g.stg_bytes + g.bstg_bytes) + filters;
     c.nsb = 0;
@@ -151,7 +157,8 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows)
     g.off_out = static_cast<int>(off);              if (int_rows) off += EW * 4096;
     g.off_tab = static_cast<int>(off);              off += c.TN * 8 + 64;
     off = (off + 15) / 16 * 16;
-    g.off_bar = static_cast<int>(off);              off += 256;
+    g.off_bar = static_cast<int>(off);              off += 320;
+    g.off_red = static_cast<int>(off);              off += red_bytes;
     g.bulk_b = packed_b && c.resident && static_cast<long long>(c.TN) * g.RS * g.Cw * WB * 4 <= static_cast<long long>(nse) * g.e_bytes &&
                (static_cast<long long>(g.O % c.TN) * g.RS * g.Cw * WB) % 4 == 0;
     c.smem = static_cast<size_t>(off);
@@ -167,20 +174,24 @@ double mma_cost(const MmaArgs& g, const Cand& c, int A, int WB, bool packed_out,
     const bool packed_b = WB > 0;
     const double mma = c.TN == 32 ? 42 : c.TN == 64 ? 49 : c.TN == 128 ? 65 : 129;      // cycles per MMA of 128 x TN x 32
     const int W = c.cfg ? 8 : 4;                                   // expander warps, epilogue warps
-    const double t_m = static_cast<double>(c.PT) * g.RS * g.Cw * mma + 148.0 * g.nchunks;
+    const int nchunks = ceil_div(g.nchunks, c.split);              // of one CTA
+    const double share = static_cast<double>(nchunks) / g.nchunks;
+    const double t_m = share * c.PT * g.RS * g.Cw * mma + 148.0 * nchunks;
     // expansion: instructions per warp and 64-channel unit of 32 rows, at 5.3 cycles each; a chunk's hand-off
     const int row_groups = ceil_div(g.NI, 32);
-    double xi = static_cast<double>(row_groups) * g.nunits * ((A <= 2 ? 102.0 : 111.0) + (g.tma ? 1.0 : 41.0));
-    if (!c.resident && packed_b) xi += c.TN * g.RS / 32.0 * g.nunits * (WB <= 2 ? 20.0 : 69.0);
+    double xi = share * row_groups * g.nunits * ((A <= 2 ? 102.0 : 111.0) + (g.tma ? 1.0 : 41.0));
+    if (!c.resident && packed_b) xi += share * c.TN * g.RS / 32.0 * g.nunits * (WB <= 2 ? 20.0 : 69.0);
     const double units_of_work = static_cast<double>(row_groups) * c.units * c.groups / W;       // per warp of a group and chunk
-    const double chunk = xi / g.nchunks * c.groups / W * (ceil(units_of_work) / units_of_work) * 5.34 + 755.0;
-    const double t_x = chunk * g.nchunks / (1.0 + (c.groups - 1) * 0.83) + 628.0;
+    const double chunk = xi / nchunks * c.groups / W * (ceil(units_of_work) / units_of_work) * 5.34 + 755.0;
+    const double t_x = chunk * nchunks / (1.0 + (c.groups - 1) * 0.83) + 628.0;
     // epilogue: instructions per block of 32 x 32 outputs, at 4.6 cycles; int32 rows leave at about 30 bytes per clock and SM
     const double block = packed_out ? (g.has_residual ? 215.0 : 138.0) : 94.0;
     double t_e = ceil_div(c.PT * (c.TN / 32), W / 4) * block * 4.59 + 997.0;
     if (!packed_out && c.PT * 128.0 * c.TN * 4 / 29.6 > t_e) t_e = c.PT * 128.0 * c.TN * 4 / 29.6;
-    const double t_b = (!c.resident && !packed_b) ? static_cast<double>(c.TN) * g.RS * g.Cw * 32 / 68.7 : 0.0;       // L2 -> shared memory
-    const long long items = static_cast<long long>(g.tiles_m) * g.tiles_o;
+    // sums through shared memory of the cluster
+    if (c.split > 1) t_e += 2200.0 + ceil_div(c.PT * (c.TN / 32), W / 4) * 200.0 * (c.split - 1);
+    const double t_b = (!c.resident && !packed_b) ? share * c.TN * g.RS * g.Cw * 32 / 68.7 : 0.0;       // L2 -> shared memory
+    const long long items = static_cast<long long>(g.tiles_m) * g.tiles_o * c.split;
     long long ctas = static_cast<long long>(sms) * c.cps;
     if (c.resident) ctas = ctas / g.tiles_o * g.tiles_o;
     if (ctas < 1) return 1e18;
@@ -214,7 +225,7 @@ struct MmaPlan {
     int rc;                 // BS_OK, or why there is no plan
 };
 
-enum : int { MM_PREPARED = 1, MM_I32 = 2, MM_CODES = 4, MM_RESIDUAL = 8, MM_CHAINED = 16, MM_QUERY = 32 };
+enum : int { MM_PREPARED = 1, MM_I32 = 2, MM_CODES = 4, MM_RESIDUAL = 8, MM_CHAINED = 16, MM_QUERY = 32, MM_ALONE = 64 };
 
 static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
 {
@@ -259,7 +270,7 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
     bool found = false;
     auto consider = [&](Cand c) {
         MmaArgs t = g;
-        if (!mma_layout(t, c, A, packed_b ? p->w_bits : 0, int_rows)) return;
+        if (!mma_layout(t, c, A, packed_b ? p->w_bits : 0, int_rows, sms)) return;
         c.cost = mma_cost(t, c, A, packed_b ? p->w_bits : 0, out_packed, sms);
         if (c.cost < best.cost) { best = c; found = true; }
     };
@@ -273,8 +284,8 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
         }
     }
 #ifdef BS_TUNING
-    int ov[7] = {0, 0, 0, -1, 0, -1, 0};    // TN, PT, units, config, strips, resident, groups; 0 / -1: free
-    if (const char* e = getenv("BS_MM")) sscanf(e, "%d,%d,%d,%d,%d,%d,%d", ov, ov + 1, ov + 2, ov + 3, ov + 4, ov + 5, ov + 6);
+    int ov[8] = {0, 0, 0, -1, 0, -1, 0, 0};    // TN, PT, units, config, strips, resident, groups, split; 0 / -1: free
+    if (const char* e = getenv("BS_MM")) sscanf(e, "%d,%d,%d,%d,%d,%d,%d,%d", ov, ov + 1, ov + 2, ov + 3, ov + 4, ov + 5, ov + 6, ov + 7);
 #endif
     for (int TN = 32; TN <= 256; TN *= 2) {
         if (TN > 32 && TN / 2 >= up(p->O, 32)) continue;
@@ -284,26 +295,29 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
                 for (int k = 0; k < nns; ++k)
                     for (int units = 1; units <= (g.R == 1 ? 4 : 1); units *= 2) {
                         if (units > 1 && units > (g.Cw + 1) / 2) continue;
-                        for (int v = 0; v < 6; ++v) {
-                            const int res = v & 1, groups = 1 << (v >> 1);
+                        for (int v = 0; v < 18; ++v) {
+                            const int res = v & 1, groups = 1 << ((v >> 1) % 3), split = 1 << (v / 6);
                             if (groups > 2 && cfg != 1) continue;
+                            // Splits only for calls on their own: between the layers of a stack the change to another kernel costs what
+                            // the split gains (18- and 50-layer stacks of batch 1 to 17: 2 % faster to 3 % slower).
+                            if (split > 1 && (!(flags & MM_ALONE) || res || cfg != 1 || PT > 1)) continue;
 #ifdef BS_TUNING
                             if ((ov[0] && TN != ov[0]) || (ov[1] && PT != ov[1]) || (ov[2] && units != ov[2]) || (ov[3] >= 0 && cfg != ov[3]) ||
-                                (ov[4] && ns_list[k] != ov[4]) || (ov[5] >= 0 && res != ov[5]) || (ov[6] && groups != ov[6]))
+                                (ov[4] && ns_list[k] != ov[4]) || (ov[5] >= 0 && res != ov[5]) || (ov[6] && groups != ov[6]) || (ov[7] && split != ov[7]))
                                 continue;
 #endif
                             Cand c{};
-                            c.TN = TN; c.PT = PT; c.units = units; c.cfg = cfg == 1; c.cps = cfg == 0 ? 2 : 1; c.ns = ns_list[k]; c.resident = res; c.groups = groups;
+                            c.TN = TN; c.PT = PT; c.units = units; c.cfg = cfg == 1; c.cps = cfg == 0 ? 2 : 1; c.ns = ns_list[k]; c.resident = res; c.groups = groups; c.split = split;
                             consider(c);
                         }
                     }
     }
     if (!found) return BS_ERR_UNSUPPORTED;
-    if (!mma_layout(g, best, A, packed_b ? p->w_bits : 0, int_rows)) return BS_ERR_UNSUPPORTED;
+    if (!mma_layout(g, best, A, packed_b ? p->w_bits : 0, int_rows, sms)) return BS_ERR_UNSUPPORTED;
 #ifdef BS_TUNING
     if (getenv("BS_MM_VERBOSE"))
-        fprintf(stderr, "mma plan: N%d C%d %dx%d O%d k%d s%d A%d W%d %s -> TN %d PT %d units %d cfg %d x %d strips %d resident %d groups %d nse %d nsb %d units %d nacc %d HL %d NI %d tiles %d x %d smem %zu cost %.0f\n",
-                p->N, p->C, p->H, p->W, p->O, p->R, p->stride, A, p->w_bits, packed_b ? "packed" : "prepared", best.TN, best.PT, best.units, best.cfg, best.cps, best.ns, best.resident, best.groups,
+        fprintf(stderr, "mma plan: N%d C%d %dx%d O%d k%d s%d A%d W%d %s -> TN %d PT %d units %d cfg %d x %d strips %d resident %d groups %d split %d nse %d nsb %d units %d nacc %d HL %d NI %d tiles %d x %d smem %zu cost %.0f\n",
+                p->N, p->C, p->H, p->W, p->O, p->R, p->stride, A, p->w_bits, packed_b ? "packed" : "prepared", best.TN, best.PT, best.units, best.cfg, best.cps, best.ns, best.resident, best.groups, best.split,
                 best.nse, g.nsb, g.nunits, g.nacc, g.HL, g.NI, g.tiles_m, g.tiles_o, best.smem, best.cost);
 #endif
     if (flags & MM_QUERY) return BS_OK;
@@ -314,9 +328,11 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
     const long long items = static_cast<long long>(g.tiles_m) * g.tiles_o;
     long long grid = static_cast<long long>(sms) * cps;
     if (best.resident) grid = grid / g.tiles_o * g.tiles_o;
-    if (grid > items) grid = items;
+    if (best.split > 1) grid = items * best.split;
+    else if (grid > items) grid = items;
     const int wb = packed_b ? p->w_bits : 0;
-    plan.kern = A == 1 ? mma_kernel_a1(wb, !best.cfg) : A == 2 ? mma_kernel_a2(wb, !best.cfg) : A == 3 ? mma_kernel_a3(wb, !best.cfg) : mma_kernel_a4(wb, !best.cfg);
+    const bool half = !best.cfg, split = best.split > 1;
+    plan.kern = A == 1 ? mma_kernel_a1(wb, half, split) : A == 2 ? mma_kernel_a2(wb, half, split) : A == 3 ? mma_kernel_a3(wb, half, split) : mma_kernel_a4(wb, half, split);
     plan.grid = static_cast<unsigned>(grid);
     plan.block = best.cfg ? MmaShape<false>::THREADS : MmaShape<true>::THREADS;
     plan.smem = static_cast<int>(best.smem);
@@ -408,10 +424,10 @@ static bool encode_rows(CUtensorMap* tm, const uint32_t* base, int rows, int wor
 
 // Plan of a layer with its pointers filled in.
 static int bind_plan(MmaPlan& plan, const uint32_t* act, const int8_t* wgt, const uint32_t* wgt_packed, const bs_conv_params* p, int32_t* out_i32,
-                     uint32_t* out_packed, bool chained, bool plan_only)
+                     uint32_t* out_packed, bool chained, bool plan_only, bool alone)
 {
     const int flags = (wgt ? MM_PREPARED : 0) | (out_i32 ? MM_I32 : 0) | (out_packed ? MM_CODES : 0) | (out_packed && p->residual ? MM_RESIDUAL : 0) |
-                      (chained ? MM_CHAINED : 0) | (plan_only ? MM_QUERY : 0);
+                      (chained ? MM_CHAINED : 0) | (plan_only ? MM_QUERY : 0) | (alone && !chained ? MM_ALONE : 0);
     const int rc = find_plan(plan, p, flags);
     if (rc != BS_OK || plan_only) return rc;
     MmaArgs& g = plan.g;
@@ -434,11 +450,14 @@ static int launch_plan(const MmaPlan& plan, cudaStream_t st)
     cfg.blockDim = dim3(plan.block);
     cfg.dynamicSmemBytes = static_cast<size_t>(plan.smem);
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = static_cast<unsigned>(plan.g.split);
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = plan.g.split > 1 ? 2 : 1;
     if (cudaLaunchKernelEx(&cfg, plan.kern, plan.g) != cudaSuccess) {
         cudaGetLastError();
         return BS_ERR_CUDA;
@@ -450,7 +469,7 @@ int mma_conv_run(const uint32_t* act, const int8_t* wgt, const uint32_t* wgt_pac
                  uint32_t* out_packed, cudaStream_t st, bool chained, bool plan_only)
 {
     MmaPlan plan;
-    const int rc = bind_plan(plan, act, wgt, wgt_packed, p, out_i32, out_packed, chained, plan_only);
+    const int rc = bind_plan(plan, act, wgt, wgt_packed, p, out_i32, out_packed, chained, plan_only, true);
     return rc != BS_OK || plan_only ? rc : launch_plan(plan, st);
 }
 
@@ -483,7 +502,7 @@ int mma_sequence_create(const bs_sequence_layer* layers, int n, cudaStream_t sid
         const bs_sequence_layer& l = layers[i];
         Sequence::Step& s = q->steps[i];
         // a layer beside its successors starts from an event, not from the kernel before it: no early filter fetch
-        int rc = bind_plan(s.plan, l.act_packed, l.wgt_tc, l.wgt_packed, &l.p, nullptr, l.out_packed, l.chained && !l.aside, false);
+        int rc = bind_plan(s.plan, l.act_packed, l.wgt_tc, l.wgt_packed, &l.p, nullptr, l.out_packed, l.chained && !l.aside, false, false);
         for (int k = 0; k < 4; ++k) {
             s.join[k] = l.join[k];
             if (l.join[k] >= i) rc = BS_ERR_INVALID_ARG;

@@ -2,7 +2,7 @@
 #include "mma_kernel.cuh"
 
 namespace bs {
-MmaKernel mma_kernel_a2(int wb, bool half) { return mma_pick<2>(wb, half); }
+MmaKernel mma_kernel_a2(int wb, bool half, bool split) { return mma_pick<2>(wb, half, split); }
 }  // namespace bs
 
 #ifdef BS_TRACE

@@ -2,5 +2,5 @@
 #include "mma_kernel.cuh"
 
 namespace bs {
-MmaKernel mma_kernel_a4(int wb, bool half) { return mma_pick<4>(wb, half); }
+MmaKernel mma_kernel_a4(int wb, bool half, bool split) { return mma_pick<4>(wb, half, split); }
 }  // namespace bs

@@ -57,6 +57,7 @@ struct MmaArgs {
     // tiling
     int TN, PT, units, nunits, nchunks;     // filters and row tiles per item, 64-channel units per chunk / in all
     int nse, nsb;                   // stages of the expanded ring; the same when filters are streamed through it, 0: filters resident
+    int split, split_log;           // CTAs (a cluster) that share the chunks of an item
     int groups, nsp;                // expander groups (chunk n belongs to group n mod groups), stages of packed words in all
     int tiles_m, tiles_o;
     FastDiv d_rs;
@@ -66,7 +67,7 @@ struct MmaArgs {
     int psz, bpsz;                  // bytes per cp.async of pixels, of packed filters
     int nslots, bslots;             // (pixel, unit) and (filter row, unit) items per expander thread and chunk
     int e_bytes, b_bytes, stg_bytes, bstg_bytes;    // per stage
-    int off_e, off_stg, off_bstg, off_pix, off_brow, off_tab, off_bar, off_out;
+    int off_e, off_stg, off_bstg, off_pix, off_brow, off_tab, off_bar, off_out, off_red;
     int tmem_cols, nacc;
     int preset;                     // accumulators start at the bit pattern of 1.5 * 2^23 (see the epilogue)
     int epi;                        // which instantiation of the fast requantisation
@@ -176,6 +177,12 @@ __device__ __forceinline__ void mm_ld16(uint32_t taddr, uint32_t (&v)[16])
         : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ void mm_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// Values loaded from tensor memory may be touched only after the wait: arithmetic on them must not move above it.
+__device__ __forceinline__ void mm_landed(uint32_t (&v)[16])
+{
+    asm volatile("" : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+                      "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]));
+}
 __device__ __forceinline__ void mm_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void mm_st8(uint32_t taddr, uint32_t x)
 {
@@ -202,6 +209,38 @@ __device__ __forceinline__ void mm_cp(uint32_t dst, const void* src, int bytes) 
 __device__ __forceinline__ void mm_sts(uint32_t dst, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
 {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ void mm_st16(uint32_t taddr, const uint32_t* v)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+                 ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
+                   "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]) : "memory");
+}
+__device__ __forceinline__ void mm_cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Shared-memory address `addr` of this CTA in the CTA of rank 0 of the cluster.
+__device__ __forceinline__ uint32_t mm_leader(uint32_t addr)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(addr));
+    return r;
+}
+// Bounded wait for arrivals of other CTAs of the cluster.
+__device__ __forceinline__ bool mm_wait_cluster(uint64_t* bar, unsigned parity)
+{
+    const uint32_t addr = smem_u32(bar);
+    for (unsigned it = 0; it < (1u << 20); ++it) {
+        unsigned ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok) : "r"(addr), "r"(parity) : "memory");
+        if (ok) return true;
+    }
+    return false;
 }
 typedef unsigned long long u64;
 __device__ __forceinline__ u64 f2_pack(uint32_t lo, uint32_t hi) { u64 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi)); return r; }
@@ -429,6 +468,18 @@ __device__ __forceinline__ void issue_block(const MmaArgs& g, uint32_t d, uint32
             }
 }
 
+// Chunks of this CTA: all of them, or its share of an item split over a cluster.
+struct MmaChunks {
+    int beg, n, rank;
+    __device__ __forceinline__ MmaChunks(const MmaArgs& g, bool split) : beg(0), n(g.nchunks), rank(0)
+    {
+        if (!split) return;
+        rank = blockIdx.x & (g.split - 1);
+        beg = (rank * g.nchunks) >> g.split_log;
+        n = (((rank + 1) * g.nchunks) >> g.split_log) - beg;
+    }
+};
+
 struct MmaIssue {
     uint64_t *full_e, *empty_e, *full_acc, *empty_acc, *wgt_full;
     uint32_t smem0, tmem;
@@ -437,18 +488,21 @@ struct MmaIssue {
 };
 
 // The MMA warp's walk over items and chunks.  Everything of a chunk, its commits included, goes out in one elected region.
-template <int TAPS>
+template <int TAPS, bool SPLIT>
 __device__ __forceinline__ void issue_items(const MmaArgs& g, const MmaIssue& m)
 {
     const uint32_t NI16 = static_cast<uint32_t>(g.NI);
     // K-major, no swizzle: core matrices of 8 rows x 16 bytes; leading offset = next 16 channels, stride offset = next 8 rows
     const uint32_t a_hi = (128u >> 4) | (1u << 14), b_hi = static_cast<uint32_t>(g.RS * 16) | (1u << 14);
     const uint32_t a_lo0 = (NI16 & 0x3FFFu) << 16, b_lo0 = (128u >> 4) << 16;
-    const uint32_t e_base = (m.smem0 + g.off_e) >> 4, w_base = m.smem0 >> 4;
+    // descriptors take the offset within the CTA; in a cluster the upper bits of a shared address name the CTA
+    const uint32_t smem_off = m.smem0 & 0x3FFFFu, e_base = (smem_off + g.off_e) >> 4, w_base = smem_off >> 4;
     const uint32_t blk16 = static_cast<uint32_t>(g.TN * g.RS * 2), idesc = g.idesc;
     const uint32_t pitch = static_cast<uint32_t>(g.pitch), HL = static_cast<uint32_t>(g.HL), TN = static_cast<uint32_t>(g.TN);
     const uint32_t e16 = static_cast<uint32_t>(g.e_bytes >> 4), b16 = static_cast<uint32_t>(g.b_bytes >> 4);
-    const int nchunks = g.nchunks, PT = g.PT, per_chunk = g.units * 2, Cw = g.Cw, nse = g.nse, nacc = g.nacc;
+    const MmaChunks range(g, SPLIT);
+    const int log = SPLIT ? g.split_log : 0;
+    const int nchunks = range.n, PT = g.PT, per_chunk = g.units * 2, Cw = g.Cw, nse = g.nse, nacc = g.nacc;
     unsigned limit = 1u << 20;
     if (m.resident) mm_wait_uniform(m.wgt_full, 0, limit);
     MM_TRACE((threadIdx.x & 31) == 0, TR_WGT, 0);
@@ -458,11 +512,11 @@ __device__ __forceinline__ void issue_items(const MmaArgs& g, const MmaIssue& m)
     int ie = 0, ia = 0;
     unsigned pe = 0, pa = 0;
     const uint32_t acc0 = g.preset ? 1u : 0u;
-    for (int it = blockIdx.x; it < m.items; it += gridDim.x) {
+    for (int it = blockIdx.x >> log; it < m.items; it += gridDim.x >> log) {
         mm_wait_uniform(&m.empty_acc[ia], pa, limit);
         const uint32_t d0 = m.tmem + static_cast<uint32_t>(ia * PT) * TN;
         for (int c = 0; c < nchunks; ++c) {
-            const int b0 = c * per_chunk;
+            const int b0 = (range.beg + c) * per_chunk;
             const int nb = Cw - b0 < per_chunk ? Cw - b0 : per_chunk;
             const uint32_t wb = b_lo0 | (w_base + (m.resident ? static_cast<uint32_t>(b0) * blk16 : static_cast<uint32_t>(ie) * b16));
             const uint32_t eb = a_lo0 | (e_base + static_cast<uint32_t>(ie) * e16);
@@ -577,16 +631,17 @@ static __device__ __noinline__ void requant32_formula(const MmaArgs& g, const ui
 
 // Work items of a CTA: item = pixel tile * tiles_o + filter tile, walked without divisions.
 struct MmaWalk {
-    int it, m, o, dm, dn;
-    __device__ __forceinline__ MmaWalk(const MmaArgs& g)
+    int it, m, o, dm, dn, log;       // log: of the CTAs that share an item
+    __device__ __forceinline__ MmaWalk(const MmaArgs& g, int log_) : log(log_)
     {
-        it = blockIdx.x;
+        it = blockIdx.x >> log;
         m = it / g.tiles_o; o = it - m * g.tiles_o;
-        dm = gridDim.x / g.tiles_o; dn = gridDim.x - dm * g.tiles_o;
+        const int n = gridDim.x >> log;
+        dm = n / g.tiles_o; dn = n - dm * g.tiles_o;
     }
     __device__ __forceinline__ void next(const MmaArgs& g)
     {
-        it += gridDim.x; m += dm; o += dn;
+        it += gridDim.x >> log; m += dm; o += dn;
         if (o >= g.tiles_o) { o -= g.tiles_o; ++m; }
     }
 };
@@ -649,7 +704,57 @@ struct MmaEpi {
     int row0;                // tile row of this thread
     int set;                 // 0 or 1: which of the two warps of a lane quadrant
     int tid, lane, warp;
+    uint64_t* red_full;      // the partial sums of the other CTAs of a split item have arrived
 };
+
+// Split items.  CTAs of rank 1 and up send their accumulators to the shared memory of rank 0 ([rank - 1][column][row], so a warp
+// stores 128 contiguous bytes), which adds them to its own in tensor memory and goes on as if it had done all the chunks.
+template <int EW>
+__device__ __forceinline__ bool send_partials(const MmaArgs& g, const MmaEpi& e, int rank)
+{
+    if (!mm_wait(&e.full_acc[0], 0)) return false;
+    mm_fence_after();
+    const uint32_t bias = g.preset ? MM_PRESET : 0u;
+    const int columns = g.PT * g.TN;
+    const uint32_t dst = mm_leader(smem_u32(e.smem + g.off_red)) + static_cast<uint32_t>(((rank - 1) * columns * 128 + e.row0) * 4);
+    for (int c0 = e.set * 32; c0 < columns; c0 += EW / 4 * 32)
+        for (int h = 0; h < 32; h += 16) {
+            uint32_t v[16];
+            mm_ld16(e.acc + static_cast<uint32_t>(c0 + h), v);
+            mm_ld_wait();
+            mm_landed(v);
+#pragma unroll
+            for (int c = 0; c < 16; ++c)
+                asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(dst + static_cast<uint32_t>((c0 + h + c) * 512)), "r"(v[c] - bias) : "memory");
+        }
+    __syncwarp();
+    if (e.lane == 0) asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(mm_leader(smem_u32(e.red_full))) : "memory");
+    return true;
+}
+template <int EW>
+__device__ __forceinline__ bool merge_partials(const MmaArgs& g, const MmaEpi& e)
+{
+    if (!mm_wait_cluster(e.red_full, 0)) return false;
+    const int columns = g.PT * g.TN;
+    const uint32_t src = smem_u32(e.smem + g.off_red) + static_cast<uint32_t>(e.row0 * 4);
+    for (int c0 = e.set * 32; c0 < columns; c0 += EW / 4 * 32)
+        for (int h = 0; h < 32; h += 16) {
+            uint32_t v[16];
+            mm_ld16(e.acc + static_cast<uint32_t>(c0 + h), v);
+            mm_ld_wait();
+            mm_landed(v);
+            for (int r = 0; r < g.split - 1; ++r)
+#pragma unroll
+                for (int c = 0; c < 16; ++c) {
+                    uint32_t x;
+                    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(x) : "r"(src + static_cast<uint32_t>((r * columns + c0 + h + c) * 512)));
+                    v[c] += x;
+                }
+            mm_st16(e.acc + static_cast<uint32_t>(c0 + h), v);
+        }
+    mm_st_wait();
+    return true;
+}
 
 __device__ __forceinline__ void store_codes(const MmaArgs& g, int pix, int ob, uint32_t (&ow)[4])
 {
@@ -711,7 +816,7 @@ static __device__ __noinline__ void epilogue_item_formula(const MmaArgs& g, uint
 
 // Codes out, fast form.  One warp's accumulators arrive 16 columns at a time; the next 16 are on their way from tensor memory
 // while the current ones are computed, and the residual words of a group are fetched one group ahead.
-template <int OBC, int RESC, bool LO0, int EW, bool PING>
+template <int OBC, int RESC, bool LO0, int EW, bool SPLIT, bool PING>
 __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e)
 {
     constexpr int STEP = EW / 4;
@@ -724,7 +829,7 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
     int tab_o = -1, ia = 0;
     unsigned pa = 0;
     bool ok = true, fast = false, waited = !g.early_b;
-    for (MmaWalk w(g); w.m < g.tiles_m; w.next(g)) {
+    for (MmaWalk w(g, SPLIT ? g.split_log : 0); w.m < g.tiles_m; w.next(g)) {
         const int o0 = w.o * g.TN;
         if (w.o != tab_o) {
             if (tab_o >= 0) asm volatile("bar.sync 2, %0;" ::"n"(EW * 32) : "memory");     // every warp is done with the old table
@@ -743,6 +848,7 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
         if (RESC && t < g.PT && px.valid && o0 + cc * 32 < g.O) load_residual(g, px.pix, o0 + cc * 32, rn);
         if (ok) ok = mm_wait(&e.full_acc[ia], pa);    // after a wait that ran out the walk goes on without waiting, so the named barriers stay matched
         mm_fence_after();
+        if (SPLIT && ok) ok = merge_partials<EW>(g, e);
         MM_TRACE(e.tid == 0, TR_EBEG, (w.it - static_cast<int>(blockIdx.x)) / static_cast<int>(gridDim.x));
         const uint32_t acc = e.acc + static_cast<uint32_t>(ia * g.PT * g.TN);
         if (!fast) {
@@ -761,6 +867,7 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
             for (int j = 0; j < 4; ++j) rw[j] = rn[j];
             if (!PING) mm_ld16(col, A);
             mm_ld_wait();
+            mm_landed(A);
             if (PING) mm_ld16(col + 16, B);
             mm_st8(col, MM_PRESET);
             mm_st8(col + 8, MM_PRESET);
@@ -784,6 +891,7 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
             }
             requant16<OBC, RESC, LO0>(A, tab, rtab, z[0], z[2], lo2, hi2, Wa);
             mm_ld_wait();
+            if (PING) mm_landed(B); else mm_landed(A);
             if (PING && t < g.PT) mm_ld16(acc + static_cast<uint32_t>(t * g.TN + cc * 32), A);
             mm_st8(col + 16, MM_PRESET);
             mm_st8(col + 24, MM_PRESET);
@@ -812,7 +920,7 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
 }
 
 // int32 accumulators out (and codes through the formula where both are asked for or the fast form does not apply).
-template <int EW>
+template <int EW, bool SPLIT>
 __device__ __forceinline__ bool epilogue_general(const MmaArgs& g, const MmaEpi& e)
 {
     const int groups = g.TN >> 5;
@@ -820,10 +928,11 @@ __device__ __forceinline__ bool epilogue_general(const MmaArgs& g, const MmaEpi&
     unsigned pa = 0;
     bool ok = true;
     mm_pdl_wait();
-    for (MmaWalk w(g); w.m < g.tiles_m; w.next(g)) {
+    for (MmaWalk w(g, SPLIT ? g.split_log : 0); w.m < g.tiles_m; w.next(g)) {
         const int o0 = w.o * g.TN, base = w.m * 128 * g.PT + e.row0;
         if (ok) ok = mm_wait(&e.full_acc[ia], pa);
         mm_fence_after();
+        if (SPLIT && ok) ok = merge_partials<EW>(g, e);
         MM_TRACE(e.tid == 0, TR_EBEG, (w.it - static_cast<int>(blockIdx.x)) / static_cast<int>(gridDim.x));
         const uint32_t acc = e.acc + static_cast<uint32_t>(ia * g.PT * g.TN);
         int t = 0, cc = e.set;
@@ -886,7 +995,8 @@ struct MmaShape {
     static constexpr int EW = HALF ? 4 : 8, XW = HALF ? 4 : 8, THREADS = (EW + XW + 2) * 32, CPS = HALF ? 2 : 1;
 };
 
-template <int A, int WB, bool HALF>
+// SPLIT: an item belongs to a cluster of CTAs, each with a share of its chunks.
+template <int A, int WB, bool HALF, bool SPLIT>
 __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) bitserial_mma_kernel(const __grid_constant__ MmaArgs g)
 {
     extern __shared__ __align__(1024) unsigned char mm_smem[];
@@ -905,6 +1015,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
     uint64_t* empty_p = bars + 22;      // [MM_STAGES] ... and expanded
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 30);
     int* fast_ok = reinterpret_cast<int*>(bars + 31);
+    uint64_t* red_full = bars + 32;     // partial sums of a split item
 
     constexpr bool packed_b = WB > 0;
     constexpr int WBX = WB > 0 ? WB : 1;
@@ -923,6 +1034,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
         for (int s = 0; s < 2; ++s) { mbar_init(&full_acc[s], 1); mbar_init(&empty_acc[s], EW); }
         mbar_init(wgt_full, packed_b ? XW + EW : 1);
         mbar_init(bulk_full, 1);
+        if (SPLIT) mbar_init(red_full, (g.split - 1) * EW);
         for (int s = 0; s < MM_STAGES; ++s) { mbar_init(&full_p[s], 1); mbar_init(&empty_p[s], XW / g.groups); }
         *fast_ok = 1;
         fence_barrier_init();
@@ -936,6 +1048,9 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
     mm_fence_before();
     __syncthreads();
     mm_fence_after();
+    if (SPLIT) mm_cluster_sync();      // the barriers of rank 0 are initialised
+    const MmaChunks range(g, SPLIT);
+    const int walk_log = SPLIT ? g.split_log : 0;
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);      // uniform for the compiler, as above
     MM_TRACE(tid == 0, TR_SETUP, 0);
 
@@ -966,9 +1081,9 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
             if (stream || g.tma) {
                 int ib = 0, ip = 0;
                 unsigned pb = 0, pp = 0;
-                for (MmaWalk w(g); w.m < g.tiles_m && ok; w.next(g)) {
+                for (MmaWalk w(g, walk_log); w.m < g.tiles_m && ok; w.next(g)) {
                     const int8_t* src = g.wgt + static_cast<size_t>(w.o) * g.TN * g.RS * 32;
-                    for (int c = 0; c < g.nchunks && ok; ++c) {
+                    for (int c = range.beg; c < range.beg + range.n && ok; ++c) {
                         if (stream) {
                             ok = mm_wait(&empty_e[ib], pb ^ 1u);
                             if (!ok) break;
@@ -1000,10 +1115,10 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
     } else if (warp == WARP_MMA) {
         // ------------------------------------------------------------------ MMA issuer (all lanes in step)
         const MmaIssue m{full_e, empty_e, full_acc, empty_acc, wgt_full, smem0, tmem, items, resident};
-        if (g.R == 1) issue_items<TAPS_1>(g, m);
-        else if (g.R == 3 && g.stride == 1) issue_items<TAPS_3S1>(g, m);
-        else if (g.R == 3 && g.pad == 1) issue_items<TAPS_3S2>(g, m);
-        else issue_items<TAPS_ANY>(g, m);
+        if (g.R == 1) issue_items<TAPS_1, SPLIT>(g, m);
+        else if (g.R == 3 && g.stride == 1) issue_items<TAPS_3S1, SPLIT>(g, m);
+        else if (g.R == 3 && g.pad == 1) issue_items<TAPS_3S2, SPLIT>(g, m);
+        else issue_items<TAPS_ANY, SPLIT>(g, m);
     } else if (warp >= EW && warp < WARP_COPY) {
         // ------------------------------------------------------------------ expanders
         const int xt = tid - NET;
@@ -1041,8 +1156,8 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
             bool ok = true;
             const uint32_t g16 = static_cast<uint32_t>(g.NI) * 16u;
             int c = xg;
-            MmaWalk w(g);
-            while (c >= g.nchunks) { c -= g.nchunks; w.next(g); }
+            MmaWalk w(g, walk_log);
+            while (c >= range.n) { c -= range.n; w.next(g); }
             while (w.m < g.tiles_m) {
                 {
                     MM_TRACE(xt == 0, TR_XWAIT, xseq);
@@ -1050,7 +1165,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                     if (ok) ok = mm_wait(&empty_e[idx], phase ^ 1u);
                     if (!ok) break;
                     MM_TRACE(xt == 0, TR_XBEG, xseq);
-                    const int nu = g.nunits - c * g.units < g.units ? g.nunits - c * g.units : g.units;
+                    const int nu = min(g.units, g.nunits - (range.beg + c) * g.units);
                     const uint32_t src = smem0 + g.off_stg + static_cast<uint32_t>(ip * g.stg_bytes);
                     const uint32_t e0 = smem0 + g.off_e + static_cast<uint32_t>(idx * g.e_bytes);
                     for (int it = xl; it < nu << shA; it += nx) {
@@ -1085,7 +1200,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                     ip += G;
                     if (ip >= g.nsp) { ip -= g.nsp; pp ^= 1u; }
                     c += G;
-                    while (c >= g.nchunks) { c -= g.nchunks; w.next(g); }
+                    while (c >= range.n) { c -= range.n; w.next(g); }
                 }
             }
             if (!ok && lane == 0) atomicOr(g.status, STATUS_TIMEOUT);
@@ -1118,11 +1233,11 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                 asm volatile("st.shared.b32 [%0], %1;" ::"r"(brow0 + static_cast<uint32_t>(i) * 4u), "r"((static_cast<uint32_t>(f) << 24) | static_cast<uint32_t>(off / g.Cw)) : "memory");
             }
         if (g.units > 1 || G > 1) asm volatile("bar.sync 3, %0;" ::"n"(NXT) : "memory");      // other threads' entries are read
-        MmaWalk iw(g), lw(g);
+        MmaWalk iw(g, walk_log);
         int ic = xg, ibuf = 0, iitem = -1, itab = 0;
-        while (ic >= g.nchunks) { ic -= g.nchunks; iw.next(g); }
+        while (ic >= range.n) { ic -= range.n; iw.next(g); }
         int lc = ic, litem = -1, ltab = 0;
-        lw = iw;
+        MmaWalk lw = iw;
         int oy = 0, ox = 0, on = 0, ostrip = 0;              // origin of a halo: row, column, image, strip
         const int PH = g.img_rows;
         auto origin = [&](int m) {
@@ -1160,7 +1275,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                 if (++ltab > stages) ltab = 0;
             }
             lc += G;
-            while (lc >= g.nchunks) { lc -= g.nchunks; lw.next(g); }
+            while (lc >= range.n) { lc -= range.n; lw.next(g); }
         };
         uint32_t ipix = 0;
         auto issue = [&]() {
@@ -1172,9 +1287,10 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                     if (++itab > stages) itab = 0;
                 }
                 uint32_t dst = stg0 + static_cast<uint32_t>(ibuf * g.stg_bytes);
+                const int chunk = range.beg + ic;
                 if (g.units == 1) {
-                    const int left = (g.Cw - 2 * ic) * A;
-                    const uint32_t* src = g.act + 2 * ic * A;
+                    const int left = (g.Cw - 2 * chunk) * A;
+                    const uint32_t* src = g.act + 2 * chunk * A;
                     for (int i = xl; i < g.NI; i += nx, dst += nx * g.psz) {
                         int pixel;
                         if (g.flat) pixel = flat_pixel(iw.m, i);
@@ -1186,7 +1302,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                     int u = 0, i = xl;
                     while (i >= g.NI) { i -= g.NI; ++u; }
                     for (; u < g.units; dst += nx * g.psz) {
-                        const int pixel = g.flat ? flat_pixel(iw.m, i) : halo_pixel(i), unit = ic * g.units + u;
+                        const int pixel = g.flat ? flat_pixel(iw.m, i) : halo_pixel(i), unit = chunk * g.units + u;
                         stage_unit<A>(g.psz, dst, step, g.act + static_cast<size_t>(static_cast<unsigned>(pixel < 0 ? 0 : pixel)) * rec + 2 * unit * A, g.act,
                                       pixel >= 0 ? (g.Cw - 2 * unit) * A : 0);
                         i += nx;
@@ -1198,8 +1314,8 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                     const int o0 = iw.o * g.TN;
                     dst = bstg0 + static_cast<uint32_t>(ibuf * g.bstg_bytes);
                     if (g.units == 1) {
-                        const int left = (g.Cw - 2 * ic) * WBX;
-                        const uint32_t* src = base + 2 * ic * WBX;
+                        const int left = (g.Cw - 2 * chunk) * WBX;
+                        const uint32_t* src = base + 2 * chunk * WBX;
                         for (int i = xl; i < rows; i += nx, dst += nx * g.bpsz) {
                             uint32_t e;
                             asm volatile("ld.shared.b32 %0, [%1];" : "=r"(e) : "r"(brow0 + static_cast<uint32_t>(i) * 4u));
@@ -1212,7 +1328,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                         for (; u < g.units; dst += nx * g.bpsz) {
                             int off;
                             const bool live = o0 + filter_row(g, i, WBX, off) < g.O;
-                            const int unit = ic * g.units + u;
+                            const int unit = chunk * g.units + u;
                             stage_unit<WBX>(g.bpsz, dst, bstep, base + off + 2 * unit * WBX, g.wgt_packed, live ? (g.Cw - 2 * unit) * WBX : 0);
                             i += nx;
                             while (i >= rows) { i -= rows; ++u; }
@@ -1220,7 +1336,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                     }
                 }
                 ic += G;
-                while (ic >= g.nchunks) { ic -= g.nchunks; iw.next(g); }
+                while (ic >= range.n) { ic -= range.n; iw.next(g); }
             }
             cp_async_commit();
             if (++ibuf == stages) ibuf = 0;
@@ -1232,16 +1348,16 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
         mm_pdl_wait();
         MM_TRACE(xt == 0, TR_PDL, 0);
         for (int s = 0; s < stages; ++s) issue();
-        MmaWalk w(g);
+        MmaWalk w(g, walk_log);
         int c = xg;
-        while (c >= g.nchunks) { c -= g.nchunks; w.next(g); }
+        while (c >= range.n) { c -= range.n; w.next(g); }
         while (w.m < g.tiles_m) {
             {
                 asm volatile("cp.async.wait_group %0;" ::"n"(stages - 1) : "memory");
                 MM_TRACE(xt == 0, TR_XWAIT, xseq);
                 if (ok) ok = mm_wait(&empty_e[idx], phase ^ 1u);
                 MM_TRACE(xt == 0, TR_XBEG, xseq);
-                const int nu = g.nunits - c * g.units < g.units ? g.nunits - c * g.units : g.units;
+                const int nu = min(g.units, g.nunits - (range.beg + c) * g.units);
                 const uint32_t g16 = static_cast<uint32_t>(g.NI) * 16u;
                 uint32_t src = stg0 + static_cast<uint32_t>(buf * g.stg_bytes);
                 const uint32_t e0 = smem0 + g.off_e + static_cast<uint32_t>(idx * g.e_bytes);
@@ -1295,7 +1411,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                 if (idx >= g.nse) { idx -= g.nse; phase ^= 1u; }
                 if (++buf == stages) buf = 0;
                 c += G;
-                while (c >= g.nchunks) { c -= g.nchunks; w.next(g); }
+                while (c >= range.n) { c -= range.n; w.next(g); }
             }
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -1331,18 +1447,20 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
         MmaEpi e;
         e.smem = mm_smem; e.full_acc = full_acc; e.empty_acc = empty_acc; e.fast_ok = fast_ok;
         e.acc = tmem + lane_addr; e.row0 = quad * 32 + lane; e.set = set;
-        e.tid = tid; e.lane = lane; e.warp = warp;
+        e.tid = tid; e.lane = lane; e.warp = warp; e.red_full = red_full;
         bool ok;
-        if (!g.preset) ok = epilogue_general<EW>(g, e);
-        else if (g.epi == 0) ok = epilogue_codes<2, 0, true, EW, true>(g, e);
-        else if (g.epi == 1) ok = epilogue_codes<2, 2, true, EW, true>(g, e);
-        else if (g.epi == 2) ok = epilogue_codes<4, 0, true, EW, true>(g, e);
-        else if (g.epi == 3) ok = epilogue_codes<4, 4, true, EW, true>(g, e);
-        else ok = epilogue_codes<4, 4, false, EW, true>(g, e);
+        if (SPLIT && range.rank > 0) ok = send_partials<EW>(g, e, range.rank);
+        else if (!g.preset) ok = epilogue_general<EW, SPLIT>(g, e);
+        else if (g.epi == 0) ok = epilogue_codes<2, 0, true, EW, SPLIT, true>(g, e);
+        else if (g.epi == 1) ok = epilogue_codes<2, 2, true, EW, SPLIT, true>(g, e);
+        else if (g.epi == 2) ok = epilogue_codes<4, 0, true, EW, SPLIT, true>(g, e);
+        else if (g.epi == 3) ok = epilogue_codes<4, 4, true, EW, SPLIT, true>(g, e);
+        else ok = epilogue_codes<4, 4, false, EW, SPLIT, true>(g, e);
         if (!ok && lane == 0) atomicOr(g.status, STATUS_TIMEOUT);
     }
     mm_fence_before();
     __syncthreads();
+    if (SPLIT) mm_cluster_sync();      // shared memory of rank 0 stays until everything sent has arrived
     MM_TRACE(tid == 0, TR_END, 0);
     if (warp == WARP_MMA) {
         mm_fence_after();
@@ -1353,21 +1471,26 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
 typedef void (*MmaKernel)(MmaArgs);
 
 // The instantiations for A activation bits, one translation unit each (mma_inst_a*.cu): filters prepared (wb = 0) or packed in wb
-// bits, half an SM or a whole one per CTA.
-MmaKernel mma_kernel_a1(int wb, bool half);
-MmaKernel mma_kernel_a2(int wb, bool half);
-MmaKernel mma_kernel_a3(int wb, bool half);
-MmaKernel mma_kernel_a4(int wb, bool half);
+// bits, half an SM or a whole one per CTA, a whole one with the item split over a cluster.
+MmaKernel mma_kernel_a1(int wb, bool half, bool split);
+MmaKernel mma_kernel_a2(int wb, bool half, bool split);
+MmaKernel mma_kernel_a3(int wb, bool half, bool split);
+MmaKernel mma_kernel_a4(int wb, bool half, bool split);
 
+template <int A, int WB>
+MmaKernel mma_pick_shape(bool half, bool split)
+{
+    return split ? bitserial_mma_kernel<A, WB, false, true> : half ? bitserial_mma_kernel<A, WB, true, false> : bitserial_mma_kernel<A, WB, false, false>;
+}
 template <int A>
-MmaKernel mma_pick(int wb, bool half)
+MmaKernel mma_pick(int wb, bool half, bool split)
 {
     switch (wb) {
-        case 0: return half ? bitserial_mma_kernel<A, 0, true> : bitserial_mma_kernel<A, 0, false>;
-        case 1: return half ? bitserial_mma_kernel<A, 1, true> : bitserial_mma_kernel<A, 1, false>;
-        case 2: return half ? bitserial_mma_kernel<A, 2, true> : bitserial_mma_kernel<A, 2, false>;
-        case 3: return half ? bitserial_mma_kernel<A, 3, true> : bitserial_mma_kernel<A, 3, false>;
-        default: return half ? bitserial_mma_kernel<A, 4, true> : bitserial_mma_kernel<A, 4, false>;
+        case 0: return mma_pick_shape<A, 0>(half, split);
+        case 1: return mma_pick_shape<A, 1>(half, split);
+        case 2: return mma_pick_shape<A, 2>(half, split);
+        case 3: return mma_pick_shape<A, 3>(half, split);
+        default: return mma_pick_shape<A, 4>(half, split);
     }
 }
 
