@@ -300,7 +300,9 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
                             if (groups > 2 && cfg != 1) continue;
                             // Splits only for calls on their own: between the layers of a stack the change to another kernel costs what
                             // the split gains (18- and 50-layer stacks of batch 1 to 17: 2 % faster to 3 % slower).
-                            if (split > 1 && (!(flags & MM_ALONE) || res || cfg != 1 || PT > 1)) continue;
+                            // 32 filters wide: wider tiles expand more filters per CTA, and 32 without a split then beats them
+                            // (3734 x 70 x 2944: 13.7 us; 128 wide and split: 19.9; 3000 x 64 x 4096: 32 wide 13.9, split 11.1).
+                            if (split > 1 && (!(flags & MM_ALONE) || res || cfg != 1 || PT > 1 || TN > 32)) continue;
 #ifdef BS_TUNING
                             if ((ov[0] && TN != ov[0]) || (ov[1] && PT != ov[1]) || (ov[2] && units != ov[2]) || (ov[3] >= 0 && cfg != ov[3]) ||
                                 (ov[4] && ns_list[k] != ov[4]) || (ov[5] >= 0 && res != ov[5]) || (ov[6] && groups != ov[6]) || (ov[7] && split != ov[7]))
