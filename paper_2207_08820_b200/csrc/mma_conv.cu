@@ -182,7 +182,7 @@ double mma_cost(const MmaArgs& g, const Cand& c, int A, int WB, bool packed_out,
     double xi = share * row_groups * g.nunits * ((A <= 2 ? 102.0 : 111.0) + (g.tma ? 1.0 : 41.0));
     if (!c.resident && packed_b) xi += share * c.TN * g.RS / 32.0 * g.nunits * (WB <= 2 ? 20.0 : 69.0);
     const double units_of_work = static_cast<double>(row_groups) * c.units * c.groups / W;       // per warp of a group and chunk
-    const double chunk = xi / nchunks * c.groups / W * (ceil(units_of_work) / units_of_work) * 5.34 + 755.0;
+    const double chunk = xi / nchunks * c.groups / W * (ceil(units_of_work) / units_of_work) * 5.34 + 629.0;
     const double t_x = chunk * nchunks / (1.0 + (c.groups - 1) * 0.83) + 628.0;
     // epilogue: instructions per block of 32 x 32 outputs, at 4.6 cycles; int32 rows leave at about 30 bytes per clock and SM
     const double block = packed_out ? (g.has_residual ? 215.0 : 138.0) : 94.0;
