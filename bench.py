@@ -37,8 +37,6 @@ from paper_2207_08820_b200 import workloads as wl  # noqa: E402
 ACT_SCALE = 0.25
 METRIC = "bitserial_conv_effective_gops"
 UNIT = "GOPS"
-POPC_PER_CLK_PER_SM = 16          # population count throughput per SM per clock (CUDA programming guide, arithmetic table)
-POPC_PER_WORDOP = 2.0 / 3.0       # executed by the kernel's 3:2 carry-save adder: three popc32(AND) word operations cost two counts
 
 
 def make_net(name: str, batch: int, hw: int = 0):
@@ -65,10 +63,10 @@ def wordops_per_image(net) -> int:
     return total
 
 
-def layer_roofline(net, engine: str, peaks: dict, popc_peak: float):
+def layer_roofline(net, engine: str, peaks: dict):
     """Per layer: algorithmic work, minimum bytes, and the roofline time max(t_compute, t_hbm) on both tensor denominators.
     Returns (rows, sums).  Minimum bytes of a layer: packed input once + filters (int8 tiles on the tensor-core engine, packed
-    planes on the popcount engine) + residual + packed output."""
+    planes otherwise) + residual + packed output.  Both engines run the same tensor-core kernel."""
     shapes = net.tensor_shapes()
     hbm = peaks["hbm_gbs"] * 1e9
     int8_burst = 2.0 * peaks["bf16_tflops"] * 1e12
@@ -85,12 +83,9 @@ def layer_roofline(net, engine: str, peaks: dict, popc_peak: float):
         res_bytes = out_bytes if L.res else 0
         nbytes = act_bytes + wgt_bytes + out_bytes + res_bytes
         t_hbm = nbytes / hbm
-        if engine == "tc":
-            tb, ts = 2.0 * macs / int8_burst, 2.0 * macs / int8_sust
-        else:
-            tb = ts = wops / popc_peak
+        tb, ts = 2.0 * macs / int8_burst, 2.0 * macs / int8_sust
         rows.append({"name": L.name, "macs": macs, "wordops": wops, "bytes": nbytes, "t_hbm": t_hbm, "t_compute_burst": tb,
-                     "t_compute_sustained": ts, "bound": "hbm" if t_hbm > tb else ("tensor" if engine == "tc" else "alu")})
+                     "t_compute_sustained": ts, "bound": "hbm" if t_hbm > tb else "tensor"})
     sums = {"roofline_s_burst": sum(max(r["t_hbm"], r["t_compute_burst"]) for r in rows),
             "roofline_s_sustained": sum(max(r["t_hbm"], r["t_compute_sustained"]) for r in rows),
             "bytes": sum(r["bytes"] for r in rows), "hbm_bound_layers": sum(r["bound"] == "hbm" for r in rows)}
@@ -104,7 +99,7 @@ def captured_traffic(net_name: str, batch: int):
     import hashlib
     import re
     path = os.path.join(ROOT, "profiles", f"bitserial_conv_tc_kernels_{net_name}_dram_traffic.md")
-    src = os.path.join(ROOT, "paper_2207_08820_b200", "csrc", "tc_conv.cu")
+    src = os.path.join(ROOT, "paper_2207_08820_b200", "csrc", "mma_kernel.cuh")
     if not (os.path.exists(path) and os.path.exists(src)):
         return None, None
     text = open(path).read()
@@ -234,8 +229,7 @@ class LaunchTimer:
 
 def sweep_peaks(torch):
     peaks, peak_kind = measured_peaks()
-    sms = torch.cuda.get_device_properties(0).multi_processor_count
-    return {"popc": POPC_PER_CLK_PER_SM * sms * peaks["sm_max_mhz"] * 1e6, "int8_burst": 2.0 * peaks["bf16_tflops"] * 1e12,
+    return {"int8_burst": 2.0 * peaks["bf16_tflops"] * 1e12,
             "int8_sustained": 2.0 * peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"]) * 1e12,
             "hbm": peaks["hbm_gbs"] * 1e9, "kind": peak_kind}
 
@@ -260,8 +254,7 @@ def measure_bitwidth_sweep(torch, api, timed, pk):
         ms, best = timed(lambda: api.bitserial_conv2d(xp, wp, **kw))                   # packed output only
         row = {"w_bits": wb, "a_bits": ab, "pairs": wb * ab, "ms": ms, "ms_best": best, "ms_with_int32_out": ms_acc,
                "gops": 2.0 * macs / ms / 1e6, "Tword_ops_per_s": wops / ms / 1e9,
-               "frac_popc_algorithmic": wops / (ms * 1e-3) / pk["popc"],
-               "frac_popc_executed": wops * POPC_PER_WORDOP / (ms * 1e-3) / pk["popc"]}
+               "frac_int8_burst": 2.0 * macs / (ms * 1e-3) / pk["int8_burst"]}
         if api.tc_supported(c["N"], c["C"], c["H"], c["W"], c["O"], 3, 1, 1, ab, c["a_sign"], wb, c["w_sign"]):
             wt = api.tc_prepare_weights(wp, c["C"], c["w_sign"], ab)
             tms, _ = timed(lambda: api.bitserial_conv2d(xp, wp, wgt_tc=wt, **kw))
@@ -288,11 +281,10 @@ def measure_gemm_sweep(torch, api, timed, pk):
             macs = M * M * K
             wops = macs // 32 * c["a_bits"] * c["w_bits"]
             nbytes = (a_p.numel() + w_p.numel() + out.numel()) * 4
-            t_popc, t_hbm = wops * POPC_PER_WORDOP / pk["popc"], nbytes / pk["hbm"]       # executed counts (3:2 carry-save adder)
+            t_alu, t_hbm = 2.0 * macs / pk["int8_burst"], nbytes / pk["hbm"]
             row = {"M": M, "N": M, "K": K, "ms": ms, "ms_best": best, "gops": 2.0 * macs / ms / 1e6,
                    "Tword_ops_per_s": wops / ms / 1e9, "GB_per_s": nbytes / ms / 1e6,
-                   "bound": "alu" if t_popc >= t_hbm else "hbm", "frac": max(t_popc, t_hbm) / (ms * 1e-3),
-                   "frac_algorithmic": max(wops / pk["popc"], t_hbm) / (ms * 1e-3)}
+                   "bound": "tensor" if t_alu >= t_hbm else "hbm", "frac": max(t_alu, t_hbm) / (ms * 1e-3)}
             wt = api.tc_prepare_weights(w_p.view(M, 1, 1, -1, c["w_bits"]), K, c["w_sign"], c["a_bits"])
             tms, _ = timed(lambda: api.bitserial_gemm_tc(a_p, wt, M, K, c["w_bits"], a_sign=c["a_sign"], w_sign=c["w_sign"], out_i32=out))
             t_tc, t_hbm_tc = 2.0 * macs / pk["int8_burst"], (a_p.numel() * 4 + wt.numel() + out.numel() * 4) / pk["hbm"]
@@ -330,10 +322,10 @@ def run_sweep(args):
         "metric": METRIC, "value": tot_ops / tot_ms / 1e6, "unit": UNIT, "n_gpus": 1, "steps": steps, "warmup": args.warmup,
         "ms_per_step": tot_ms, "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "int32",
         "data": "synthetic",
-        "config": {"workload": name, "engine": "popc", "l2": "flushed before every launch (256 MB write, then read back)",
+        "config": {"workload": name, "engine": "popc (packed filters)", "l2": "flushed before every launch (256 MB write, then read back)",
                    "launch": "one eager launch per case, CUDA events around it (launch latency included)"},
         "sweep": rows,
-        "peaks": {"popc_word_ops_per_s": pk["popc"], "int8_ops_per_s_burst": pk["int8_burst"], "int8_ops_per_s_sustained": pk["int8_sustained"],
+        "peaks": {"int8_ops_per_s_burst": pk["int8_burst"], "int8_ops_per_s_sustained": pk["int8_sustained"],
                   "hbm_bytes_per_s": pk["hbm"], "kind": pk["kind"]},
         "gpu_launches": timed.launches, "clocks": clocks.summary()}))
 
@@ -345,8 +337,8 @@ def measure_other_configs(torch, api, stream, args):
       gemm_sweep / bitwidth_sweep   as the stand-alone sweeps, fewer repetitions;
       detection_backbone            the detection-shaped stack at batch 16 on the tensor-core engine: conv time per pass under a
                                     CUDA graph, images/s, and sum(roofline time) / measured time over its layers;
-      layer_chains   the residual stack's conv layers at batch 16 and 64, one launch per layer against runs of same-shaped
-                     layers as one launch (bitserial_conv2d_tc_chain), and how many launches the runner's set-up timing keeps;
+      layer_chains   the residual stack's conv layers at batch 16 and 64, one call per layer against runs of same-shaped
+                     layers as one call (bitserial_conv2d_tc_chain; the launches are the same), and how many calls the default makes;
       pack_large     the pack kernels on inputs larger than L2 (fp32 NCHW and NHWC, 2 and 3 bits)."""
     from paper_2207_08820_b200.net import BitserialNet
     dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
@@ -399,16 +391,16 @@ def measure_other_configs(torch, api, stream, args):
     out["single_layer"] = {"workload": "conv3x3_n1_c64_o64_hw56_w2a2 (warm L2, 20 launches per CUDA graph)",
                            "popc_us": t_popc * 1e3, "tc_us": t_tc * 1e3, "popc_gops": 2.0 * macs1 / t_popc / 1e6, "tc_gops": 2.0 * macs1 / t_tc / 1e6,
                            "launch_floor_us": {"popc": f_popc * 1e3, "tc": f_tc * 1e3, "what": "one-tile launch (1x1 conv on an 8x8 image), same method"},
-                           "roofline_us": {"popc_executed": macs1 // 32 * 4 * POPC_PER_WORDOP / pk["popc"] * 1e6, "tensor_burst": 2.0 * macs1 / pk["int8_burst"] * 1e6},
+                           "roofline_us": {"tensor_burst": 2.0 * macs1 / pk["int8_burst"] * 1e6},
                            "bound": "launch latency: the layer's arithmetic is shorter than one launch"}
     # ---- sweeps
     timed = LaunchTimer(torch, 2, 5)
     rows, _, _ = measure_gemm_sweep(torch, api, timed, pk)
     out["gemm_sweep"] = [{k: (round(v, 5) if isinstance(v, float) else v) for k, v in r.items()
-                          if k in ("M", "K", "ms", "bound", "frac", "frac_algorithmic", "tc_ms", "tc_bound", "tc_frac")} for r in rows]
+                          if k in ("M", "K", "ms", "bound", "frac", "tc_ms", "tc_bound", "tc_frac")} for r in rows]
     rows, _, _ = measure_bitwidth_sweep(torch, api, timed, pk)
     out["bitwidth_sweep"] = [{k: (round(v, 5) if isinstance(v, float) else v) for k, v in r.items()
-                              if k in ("w_bits", "a_bits", "pairs", "ms", "Tword_ops_per_s", "frac_popc_algorithmic", "frac_popc_executed", "tc_ms",
+                              if k in ("w_bits", "a_bits", "pairs", "ms", "Tword_ops_per_s", "frac_int8_burst", "tc_ms",
                                        "tc_frac_int8_burst")} for r in rows]
     launches += timed.launches
     # ---- pack kernels on inputs larger than L2
@@ -434,7 +426,7 @@ def measure_other_configs(torch, api, stream, args):
         stream.synchronize()
         t_pack = graph_time(lambda: runner.pack_input(x), reps=1, rounds=5)
         t_conv = graph_time(runner.run_layers, reps=1, rounds=8)
-    _, sums = layer_roofline(net, "tc", peaks, pk["popc"])
+    _, sums = layer_roofline(net, "tc", peaks)
     macs = net.macs_per_image() * net.batch
     launches += 0
     out["detection_backbone"] = {"workload": f"{net.name}_batch{net.batch}_w2a2 (warm L2, one CUDA graph per pass)", "layers": len(net.layers),
@@ -681,46 +673,31 @@ def run_ours(args):
 
     if rank == 0:
         macs = net.macs_per_image() * net.batch
-        wops = wordops_per_image(net) * net.batch
         gops = 2.0 * macs * world / (t_step * 1e-3) / 1e9
         peaks, peak_kind = measured_peaks()
-        sms = torch.cuda.get_device_properties(local).multi_processor_count
-        popc_peak = POPC_PER_CLK_PER_SM * sms * peaks["sm_max_mhz"] * 1e6          # counts/s at the maximum SM clock
-        popc_measured = api.bs_popc_rate(4096)
         # dense int8 = 2 x bf16 (nominal ratio); the conv kernels are timed 17 us at a time inside a millisecond step at the
         # maximum clock, so the burst figure is the denominator of `frac`; the sustained one is printed beside it
         int8_burst = 2.0 * peaks["bf16_tflops"]
         int8_sustained = 2.0 * peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"])
 
-        def popc_roofline(t_ms):
-            a = wops / (t_ms * 1e-3)
-            _, sums = layer_roofline(net, "popc", peaks, popc_peak / POPC_PER_WORDOP)
-            return {"bound": "alu", "kernel": "bitserial_conv_kernel", "achieved": a * POPC_PER_WORDOP / 1e12, "peak": popc_peak / 1e12,
-                    "unit": "Tpopc/s", "frac": a * POPC_PER_WORDOP / popc_peak, "traffic": None,
-                    "peak_source": f"{POPC_PER_CLK_PER_SM} popc/clk/SM x {sms} SMs x {peaks['sm_max_mhz']:.0f} MHz ({peak_kind} clock); achieved = population "
-                                   "counts EXECUTED per second: the 3:2 carry-save adder executes 2 counts per 3 popc32(AND) word operations of the plane-pair sum",
-                    "frac_algorithmic": a / popc_peak, "achieved_algorithmic_Twordop_s": a / 1e12,
-                    "frac_per_layer_roofline": sums["roofline_s_burst"] / (t_ms * 1e-3), "hbm_bound_layers": sums["hbm_bound_layers"],
-                    "popc_pipe_measured": popc_measured / 1e12, "launches_per_step": len(net.layers),
-                    "avg_launch_ms": t_ms / len(net.layers)}
-
         tc_traffic, tc_traffic_src = captured_traffic(net.name, net.batch)
 
-        def tensor_roofline(t_ms):
+        def tensor_roofline(t_ms, engine):
             a = 2.0 * macs / (t_ms * 1e-3) / 1e12
-            rows, sums = layer_roofline(net, "tc", peaks, popc_peak)
-            return {"bound": "tensor", "kernel": "bitserial_conv_tc_persistent_kernel", "achieved": a, "peak": int8_burst,
+            _, sums = layer_roofline(net, engine, peaks)
+            traffic = tc_traffic if engine == "tc" else None
+            return {"bound": "tensor", "kernel": "bitserial_mma_kernel", "achieved": a, "peak": int8_burst,
                     "unit": "TOP/s", "frac": a / int8_burst, "peak_burst": int8_burst, "peak_sustained": int8_sustained,
                     "frac_sustained": a / int8_sustained,
                     # per layer max(t_tensor, t_hbm), summed over the stack, over the measured conv time
                     "frac_per_layer_roofline": sums["roofline_s_burst"] / (t_ms * 1e-3),
                     "frac_per_layer_roofline_sustained": sums["roofline_s_sustained"] / (t_ms * 1e-3),
                     "hbm_bound_layers": sums["hbm_bound_layers"], "algorithmic_bytes_per_launch": sums["bytes"] / len(net.layers),
-                    "traffic": tc_traffic / len(net.layers) if tc_traffic else None, "traffic_source": tc_traffic_src,
+                    "traffic": traffic / len(net.layers) if traffic else None, "traffic_source": tc_traffic_src if engine == "tc" else None,
                     "peak_source": f"2 x {peak_kind} bf16 cuBLAS TFLOP/s (nominal int8:bf16 ratio); burst figure (kernels of ~17 us inside a short step at the maximum clock)",
                     "launches_per_step": len(net.layers), "avg_launch_ms": t_ms / len(net.layers)}
 
-        roof = tensor_roofline(t_conv) if args.engine == "tc" else popc_roofline(t_conv)
+        roof = tensor_roofline(t_conv, args.engine)
         in_bytes = x_host.numel() * 4
         pack_bytes = in_bytes + in_buf.numel() * 4
         line = {
@@ -746,16 +723,15 @@ def run_ours(args):
         line["config"]["engine"] = args.engine
         line["config"]["conv_launches_per_step"] = len(runner.units)
         if t_conv_other is not None:
-            alt = popc_roofline(t_conv_other) if other == "popc" else tensor_roofline(t_conv_other)
+            alt = tensor_roofline(t_conv_other, other)
             alt["engine"] = other
             alt["conv_ms"] = t_conv_other
             line["other_engine"] = alt
-        popc_frac = (roof if args.engine == "popc" else line.get("other_engine", {})).get("frac")
-        tc_frac = (roof if args.engine == "tc" else line.get("other_engine", {})).get("frac")
+        fracs = {args.engine: roof["frac"], **({other: line["other_engine"]["frac"]} if t_conv_other is not None else {})}
         line["target_0p60_of_roofline"] = {
-            "popcount_kernel_frac_executed": popc_frac, "tensor_core_kernel_frac": tc_frac,
-            "statement": "the bit-serial (popcount) conv kernel is measured against the popc-pipe peak on executed counts; the tensor-core "
-                         "formulation, adopted because it is faster in absolute time, is measured against the int8 tensor peak and does not reach 0.60 of it"}
+            "packed_filters_frac": fracs.get("popc"), "prepared_filters_frac": fracs.get("tc"),
+            "statement": "both engines evaluate the plane-pair sum as an integer matrix product on the tensor cores (packed filters expanded on chip, or "
+                         "prepared once) and are measured against the int8 tensor peak; neither reaches 0.60 of it over the whole stack"}
         if configs is not None:
             line["configs"] = configs
             line["gpu_launches"] += config_launches
@@ -796,9 +772,8 @@ def main():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-configs", action="store_true", help="leave out the compact measurements of the other workloads")
     ap.add_argument("--engine", default="tc", choices=["popc", "tc"],
-                    help="popc: popcount kernels on the integer pipes; tc: exact int8 tensor-core formulation")
-    ap.add_argument("--chains", default="auto", choices=["auto", "on", "off"], help="runs of same-shaped layers as one launch: timed at set-up and "
-                    "kept where faster (auto), always, or never; --eager implies off")
+                    help="popc: packed filters, expanded on chip; tc: filters prepared as int8 tiles once (the same tensor-core kernel)")
+    ap.add_argument("--chains", default="auto", choices=["auto", "on", "off"], help="runs of same-shaped layers as one call (on) or one call per layer; the launches are the same")
     ap.add_argument("--eager", action="store_true", help="plain stream launches instead of CUDA graphs (for per-launch profiling)")
     args = ap.parse_args()
     if args.workload in ("bitwidth_sweep", "gemm_sweep"):

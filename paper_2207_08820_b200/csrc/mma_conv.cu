@@ -168,7 +168,7 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows, int sms)
 // Time model of a candidate in SM cycles: the pipeline of one CTA (expansion, MMAs, epilogue; a stage's hand-off included) over
 // its items, plus what nothing overlaps at both ends.  The constants are fitted to about 2500 timed plans of 45 layers and
 // products (1 to 300 pixels wide, 32 to 4608 channels, batches 1 to 64; B200 at 1.95 GHz): over those the plan with the
-// lowest modelled time is on average 2 % and with two exceptions at most 8 % slower than the fastest plan.
+// lowest modelled time is on average 2 to 3 % and at most 16 % slower than the fastest plan.
 double mma_cost(const MmaArgs& g, const Cand& c, int A, int WB, bool packed_out, int sms)
 {
     const bool packed_b = WB > 0;
