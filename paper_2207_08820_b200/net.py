@@ -39,8 +39,8 @@ class BitserialNet:
 
     def __init__(self, net: NetSpec, params: Dict[str, Dict], act_scale: float, device="cuda", batch: Optional[int] = None,
                  engine: str = "popc", concurrent: bool = True, chains="auto"):
-        """engine: "popc" = popcount kernels on the integer pipes; "tc" = tensor-core entry point for every layer it
-        supports (others fall back to the popcount kernel).  concurrent: launch independent neighbouring layers on
+        """engine: "popc" = packed filters, expanded on chip; "tc" = filters prepared as int8 tiles once for every layer that
+        supports it (others keep packed filters).  concurrent: launch independent neighbouring layers on
         two streams (see :meth:`schedule`).  chains: with the "tc" engine, runs of consecutive same-shaped layers can go
         through ``bitserial_conv2d_tc_chain`` (one call per run) where the library accepts them: True = always, False and
         "auto" = one call per layer (the launches are the same)."""
