@@ -258,7 +258,8 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
         int qmin, qmax;
         code_limits(p->out_bits > 0 ? p->out_bits : 1, p->out_sign, qmin, qmax);
         const bool lo0 = qmin == 0 || p->relu;
-        if (!lo0) g.epi = 4;
+        // the forms with a residual read its words and a table of multipliers that is written only where there is one
+        if (!lo0) g.epi = residual ? 5 : 4;
         else if (p->out_bits <= 2 && (!residual || p->res_bits <= 2)) g.epi = residual ? 1 : 0;
         else g.epi = residual ? 3 : 2;
     }

@@ -70,7 +70,7 @@ struct MmaArgs {
     int off_e, off_stg, off_bstg, off_pix, off_brow, off_tab, off_bar, off_out, off_red;
     int tmem_cols, nacc;
     int preset;                     // accumulators start at the bit pattern of 1.5 * 2^23 (see the epilogue)
-    int epi;                        // which instantiation of the fast requantisation
+    int epi;                        // which instantiation of the fast requantisation: odd ones read a residual and its multipliers
     int early_b;                    // filters may be read before the preceding kernel has finished
     int opad;
     unsigned idesc;
@@ -1455,6 +1455,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
         else if (g.epi == 1) ok = epilogue_codes<2, 2, true, EW, SPLIT, true>(g, e);
         else if (g.epi == 2) ok = epilogue_codes<4, 0, true, EW, SPLIT, true>(g, e);
         else if (g.epi == 3) ok = epilogue_codes<4, 4, true, EW, SPLIT, true>(g, e);
+        else if (g.epi == 4) ok = epilogue_codes<4, 0, false, EW, SPLIT, true>(g, e);
         else ok = epilogue_codes<4, 4, false, EW, SPLIT, true>(g, e);
         if (!ok && lane == 0) atomicOr(g.status, STATUS_TIMEOUT);
     }
