@@ -375,13 +375,18 @@ static int find_plan(MmaPlan& out, const bs_conv_params* p, int flags)
     } else if (cudaGetDevice(&dev) != cudaSuccess) {
         return BS_ERR_CUDA;
     }
-    const bool res = flags & MM_RESIDUAL, codes = flags & MM_CODES;
+    // What a caller leaves in fields that its outputs do not depend on reaches neither the key nor the plan: without codes the epilogue's,
+    // without a residual the residual's.
+    bs_conv_params q = *p;
+    if (!(flags & MM_CODES)) q.relu = q.out_bits = q.out_sign = q.out_c_offset = q.out_c_total = 0;
+    if (!(flags & MM_RESIDUAL)) {
+        q.res_bits = q.res_sign = q.res_c_offset = q.res_c_total = 0;
+        q.res_scale = 0.0f;
+    }
     int scale_bits = 0;
-    if (res) memcpy(&scale_bits, &p->res_scale, 4);
-    const PlanKey key = {{p->N, p->C, p->H, p->W, p->O, p->R, p->S, p->stride, p->pad, p->a_bits, p->a_sign, p->w_bits, p->w_sign,
-                          codes ? p->relu : 0, codes ? p->out_bits : 0, codes ? p->out_sign : 0, codes ? p->out_c_offset : 0, codes ? p->out_c_total : 0,
-                          res ? p->res_bits : 0, res ? p->res_sign : 0, res ? p->res_c_offset : 0, res ? p->res_c_total : 0, scale_bits, p->i32_layout,
-                          flags, dev, sms, 0}};
+    memcpy(&scale_bits, &q.res_scale, 4);
+    const PlanKey key = {{q.N, q.C, q.H, q.W, q.O, q.R, q.S, q.stride, q.pad, q.a_bits, q.a_sign, q.w_bits, q.w_sign, q.relu, q.out_bits, q.out_sign,
+                          q.out_c_offset, q.out_c_total, q.res_bits, q.res_sign, q.res_c_offset, q.res_c_total, scale_bits, q.i32_layout, flags, dev, sms, 0}};
     static std::unordered_map<PlanKey, MmaPlan, PlanHash> plans;
     static std::mutex mu;
     {
@@ -393,7 +398,7 @@ static int find_plan(MmaPlan& out, const bs_conv_params* p, int flags)
         if (it != plans.end()) { out = it->second; return out.rc; }
     }
     MmaPlan plan{};
-    plan.rc = make_plan(plan, p, flags, sms);
+    plan.rc = make_plan(plan, &q, flags, sms);
     if (plan.rc == BS_OK || plan.rc == BS_ERR_UNSUPPORTED) {
         std::lock_guard<std::mutex> lock(mu);
         if (plans.size() >= MAX_PLANS) plans.clear();

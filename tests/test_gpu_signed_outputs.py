@@ -1,6 +1,7 @@
 """Signed output codes without ReLU and without a residual, each layer directly behind a launch that fills most of the shared memory of every
 SM with prepared filters of -1 (0xFF bytes, NaN as floats): what a kernel reads there without having written it shows in its codes.
-The epilogue takes the oracle's binary32 operations in its order, so the codes must be equal."""
+The epilogue takes the oracle's binary32 operations in its order, so the codes must be equal.  And layers without a residual whose other
+residual fields hold something: a null pointer means none, whatever they say, in this call and in later ones of the shape."""
 import numpy as np
 import pytest
 
@@ -57,4 +58,26 @@ def test_signed_codes_without_residual(fillers, layer, prepared):
         fill()
         _, got = api.bitserial_conv2d(xa, wp, C=C, stride=stride, pad=k // 2, w_sign=w_sign, scale=sc, bias=bi, out_bits=out, out_sign=api.SIGNED, wgt_tc=wt)
         assert np.array_equal(words(got), want)
+    api.bs_check_status()
+
+
+@pytest.mark.parametrize("relu,out_sign", [(False, api.SIGNED), (True, api.SIGNED), (True, api.UNSIGNED)])
+@pytest.mark.parametrize("prepared", [False, True])
+def test_residual_fields_without_a_residual(relu, out_sign, prepared):
+    out, hw = 3, 13 + 2 * prepared + 4 * relu + 8 * out_sign       # a shape that no call has been planned for
+    rng = np.random.default_rng(hw)
+    x, f = wl.rand_codes(rng, (2, 64, hw, hw), 2, 0), wl.rand_codes(rng, (64, 64, 3, 3), 2, 1)
+    acc = oracle.conv2d_i32(x, f, 1, 1)
+    scale = np.full(64, 4 / float(acc.std()), np.float32)
+    bias = (-scale * acc.mean(axis=(0, 2, 3)) + np.float32(0.25)).astype(np.float32)
+    want = oracle.pack_activations(oracle.requantize(acc, scale, bias, relu, out, out_sign), out, out_sign)
+    res = wl.rand_codes(rng, (2, 64, hw, hw), 2, 0)
+    want_res = oracle.pack_activations(oracle.requantize(acc, scale, bias, relu, out, out_sign, res=res, res_scale=0.5), out, out_sign)
+    xa, wp, rp = api.bitpack_activations(dev(x), 1.0, 2), api.pack_weights(dev(f), 2, 1), api.bitpack_activations(dev(res), 1.0, 2)
+    kw = dict(C=64, pad=1, scale=dev(scale), bias=dev(bias), relu=relu, out_bits=out, out_sign=out_sign,
+              wgt_tc=api.tc_prepare_weights(wp, 64, 1, 2) if prepared else None)
+    left = dict(res_scale=0.5, res_bits=2, res_sign=api.UNSIGNED, res_c_offset=32, res_c_total=96)
+    for fields, residual, codes in ((left, None, want), ({}, None, want), (dict(left, res_c_offset=0, res_c_total=64), rp, want_res), (left, None, want)):
+        _, got = api.bitserial_conv2d(xa, wp, residual=residual, **fields, **kw)
+        assert np.array_equal(words(got), codes)
     api.bs_check_status()
