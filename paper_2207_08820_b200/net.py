@@ -13,25 +13,29 @@ import numpy as np
 import torch
 
 from . import api
-from ._lib import SequenceLayer, lib
+from ._lib import SequenceLayer, lib, native
 from .workloads import NetSpec
 
 
-class _Buffers(dict):
-    """Activation tensors by name; ``version`` changes when one is replaced (a bound sequence holds their addresses)."""
-    version = 0
-
-    def __setitem__(self, key, value):
-        self.version += 1
-        super().__setitem__(key, value)
-
-
 class _Sequence:
-    """A ``bs_sequence`` and the tensors it holds the addresses of."""
+    """The launches of a pass bound to what they read and write.  ``handle``: the ``bs_sequence``, None where the library does not take the
+    layers as one.  ``dicts`` name the tensors and settings of the layers; ``values`` are what was found there, kept alive because a sequence
+    and the graphs captured from it hold the tensors' ``addresses``."""
 
-    def __init__(self, handle: int, tensors):
-        self.handle, self.tensors = handle, tensors
+    def __init__(self, units, concurrent, dicts):
+        self.units, self.concurrent = units, concurrent
+        self.dicts = tuple(dicts)
+        self.values = tuple(v for d in self.dicts for v in d.values())
+        self.addresses = tuple(v.data_ptr() if isinstance(v, torch.Tensor) else None for v in self.values)
+        self.handle = None
+
+    def own(self, handle: int) -> None:
+        self.handle = handle
         weakref.finalize(self, lib().bs_sequence_destroy, handle).atexit = False
+
+    def current(self, units, concurrent) -> bool:
+        """Whether nothing was replaced since: the dicts hold the same objects, the tensors are where they were."""
+        return units is self.units and concurrent == self.concurrent and native().unchanged(self.dicts, self.values, self.addresses)
 
 
 class BitserialNet:
@@ -65,7 +69,7 @@ class BitserialNet:
                 w_sign=p["w_sign"],
                 scale=torch.from_numpy(p["scale"]).to(self.device),
                 bias=torch.from_numpy(p["bias"]).to(self.device)))
-        self.bufs: Dict[str, torch.Tensor] = _Buffers()
+        self.bufs: Dict[str, torch.Tensor] = {}
         for name, (C, H, W) in self.shapes.items():
             self.bufs[name] = torch.zeros(self.batch, H, W, (C + 31) // 32, net.a_bits, dtype=torch.int32, device=self.device)
         self.units = self._plan_units(chains is True and engine == "tc")
@@ -75,7 +79,8 @@ class BitserialNet:
         self.graph = None
         self.static_in = None
         self.launches_per_forward = 1 + len(self.layers)
-        self._sequence = self._sequence_key = None
+        self._sequence: Optional[_Sequence] = None
+        self._captured: Optional[_Sequence] = None      # what the graph was captured from
         self._bind()
 
     def _layer_params(self, item):
@@ -211,11 +216,15 @@ class BitserialNet:
             self.run_unit(unit)
 
     def _bind(self) -> bool:
-        """Binds the layers to their present tensors as one sequence; False where the library does not take them as one."""
-        key = (self.bufs.version, self.concurrent, id(self.units))
-        if key == self._sequence_key:
-            return self._sequence is not None
-        self._sequence_key, self._sequence = key, None
+        """Binds the layers as one sequence to the tensors and settings they have now, again when one was replaced; False where the library does
+        not take them as one."""
+        q = self._sequence
+        if q is not None and q.current(self.units, self.concurrent):
+            return q.handle is not None
+        items = [item for unit in self.units for item in unit["items"]]
+        self._sequence = _Sequence(self.units, self.concurrent, [self.bufs, *items, *(vars(item["spec"]) for item in items)])
+        if q is not None and not torch.cuda.is_current_stream_capturing():
+            torch.cuda.synchronize(self.device)     # as at set-up: what replaced a filter, scale or bias has to be final
         steps = self.schedule()
         at, layers = {}, []                          # position of a launch among the layers
         for i, (unit, aside, join) in enumerate(steps):
@@ -228,16 +237,15 @@ class BitserialNet:
         arr = (SequenceLayer * len(layers))()
         for q, (item, aside, join) in zip(arr, layers):
             L = item["spec"]
-            q.act_packed, q.out_packed = self.bufs[L.src].data_ptr(), self.bufs[L.dst].data_ptr()
-            q.wgt_packed = item["w"].data_ptr()
-            q.wgt_tc = item["w_tc"].data_ptr() if item["w_tc"] is not None else None
+            q.act_packed, q.out_packed = api._ptr(self.bufs[L.src]), api._ptr(self.bufs[L.dst])
+            q.wgt_packed, q.wgt_tc = api._ptr(item["w"]), api._ptr(item["w_tc"])
             q.p = self._conv_params(item)
             q.chained, q.aside = 1, int(aside)
             q.join[:] = (join + [-1] * 4)[:4]
         handle = ctypes.c_void_p()
         if lib().bs_sequence_create(arr, len(layers), self.side.cuda_stream, ctypes.byref(handle)) != 0:
             return False
-        self._sequence = _Sequence(handle.value, [self.bufs[n] for n in self.shapes])
+        self._sequence.own(handle.value)
         return True
 
     def _conv_params(self, item):
@@ -261,13 +269,15 @@ class BitserialNet:
         return self._run(x)
 
     def capture(self, x: torch.Tensor) -> None:
-        """Record one forward pass into a CUDA graph replayed by :meth:`replay` (input copied into a static buffer)."""
+        """Record one forward pass into a CUDA graph replayed by :meth:`replay` (input copied into a static buffer).  The graph keeps the
+        tensors it was captured with; entries replaced later take effect in :meth:`forward` and in the next capture."""
         self.static_in = x.clone()
         self._run(self.static_in)            # warm-up outside capture: plans, descriptors, module loading
         torch.cuda.synchronize()
         self.graph = torch.cuda.CUDAGraph()
         with torch.cuda.graph(self.graph):
             self._run(self.static_in)
+        self._captured = self._sequence
 
     def replay(self, x: Optional[torch.Tensor] = None) -> torch.Tensor:
         if x is not None:

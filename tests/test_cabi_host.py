@@ -170,3 +170,28 @@ def test_product_never_imports_oracle():
             if f.endswith((".py", ".cu", ".cuh", ".h")):
                 text = open(os.path.join(dirpath, f)).read()
                 assert "import oracle" not in text and "from oracle" not in text and "bitserial_oracle" not in text, f
+
+
+def test_binding_sees_replaced_entries(L):
+    """What a bound run of layers asks before each pass, on host tensors: the same objects in the same order, tensors where they were."""
+    import torch
+    from paper_2207_08820_b200._lib import native
+    d = [dict(a=torch.zeros(4), b=None, c=3), {}, dict(a=torch.zeros(4), s="x")]
+    values = tuple(v for e in d for v in e.values())
+    args = tuple(d), values, tuple(v.data_ptr() if isinstance(v, torch.Tensor) else None for v in values)
+    same = lambda: native().unchanged(*args)
+    assert same()
+    for change, back in ((lambda: d[0].update(a=torch.zeros(4)), lambda: d[0].update(a=values[0])),
+                         (lambda: d[0].update(b=0), lambda: d[0].update(b=None)),
+                         (lambda: d[2].update(t=1), lambda: d[2].pop("t")),
+                         (lambda: d[1].update(t=1), lambda: d[1].clear()),
+                         (lambda: d[2].pop("s"), lambda: d[2].update(s=values[4]))):
+        change()
+        assert not same()
+        back()
+        assert same()
+    values[3].data = torch.ones(4)              # the same tensor, elsewhere
+    assert not same()
+    for wrong in ((1,) + args[1:], args[:2] + (args[2][:-1],), ((1,),) + args[1:]):
+        with pytest.raises(ValueError):
+            native().unchanged(*wrong)

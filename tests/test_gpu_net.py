@@ -104,3 +104,70 @@ def test_resnet50_body_full_batch_sampled():
 def test_detection_backbone_352px_input():
     """The paper's 352 px detection input: first packed tensor 176 px, widths 176 / 88 / 44 / 22 / 11."""
     compare_stack(wl.detection_backbone(1, hw=176), 1, seed=4000, engine="tc")
+
+
+@pytest.mark.parametrize("engine", ["popc", "tc"])
+def test_replaced_entries_take_effect(engine):
+    """Filters, scales, biases and settings of a layer may be replaced between passes: the next pass uses the new ones, a captured graph
+    goes on with those it was captured with.  (The replaced tensors are kept here, so nothing stale is ever freed memory.)"""
+    spec = lambda: wl.resnet18_body(2, 28)
+    a, b = (BitserialNet(spec(), wl.network_params(wl.resnet18_body(2, 28), seed), ACT_SCALE, batch=2, engine=engine) for seed in (3000, 3100))
+    x = dev(wl.network_input(a.net, 3000, ACT_SCALE, batch=2))
+    a.capture(x)
+    before, want = a.forward(x).clone(), b.forward(x).clone()
+    assert not torch.equal(before, want)
+    kept = [dict(item) for item in a.layers]
+    for mine, theirs in zip(a.layers, b.layers):
+        mine.update({k: theirs[k] for k in ("w", "w_tc", "scale", "bias")})      # all at once, past __setitem__
+    assert torch.equal(a.forward(x), want)
+    assert torch.equal(a.replay(x), before)
+    del kept
+    # a tensor whose storage moved, and a setting of a layer
+    last, other = a.layers[-1], b.layers[-1]
+    old_bias, last["bias"].data = last["bias"].data, last["bias"] + 1.0
+    last["spec"].res_scale = 0.25
+    other["bias"], other["spec"].res_scale = old_bias + 1.0, 0.25
+    want = b.forward(x).clone()
+    assert torch.equal(a.forward(x), want)
+    fresh = wl.network_params(wl.resnet18_body(2, 28), 3100)
+    fresh[last["spec"].name]["bias"] = fresh[last["spec"].name]["bias"] + np.float32(1.0)
+    net = spec()
+    net.layers[-1].res_scale = 0.25
+    assert torch.equal(BitserialNet(net, fresh, ACT_SCALE, batch=2, engine=engine).forward(x), want)
+    api.bs_check_status()
+
+
+def test_bound_tensors_stay_alive():
+    """What a bound run of layers or a captured graph holds the addresses of is not freed when its entry is replaced."""
+    import weakref
+    net = wl.resnet18_body(1, 28)
+    runner = BitserialNet(net, wl.network_params(net, 3000), ACT_SCALE, batch=1, engine="tc")
+    x = dev(wl.network_input(net, 3000, ACT_SCALE, batch=1))
+    runner.capture(x)
+    want = runner.replay(x).clone()
+    refs = []
+    for item in runner.layers:
+        for key in ("w", "w_tc", "scale", "bias"):
+            refs.append(weakref.ref(item[key]))
+            item[key] = item[key].clone()
+    assert torch.equal(runner.forward(x), want) and torch.equal(runner.replay(x), want)
+    assert all(r() is not None for r in refs)              # the graph's
+    runner.capture(x)
+    runner.forward(x)
+    assert all(r() is None for r in refs)                  # nobody's any more
+    api.bs_check_status()
+
+
+def test_bound_run_checks_its_tensors():
+    net = wl.resnet18_body(1, 28)
+    runner = BitserialNet(net, wl.network_params(net, 3000), ACT_SCALE, batch=1, engine="tc")
+    x = dev(wl.network_input(net, 3000, ACT_SCALE, batch=1))
+    want = runner.forward(x).clone()
+    item = runner.layers[3]
+    for key, wrong in (("scale", item["scale"].cpu()), ("w_tc", item["w_tc"].cpu()), ("bias", torch.zeros(2 * item["bias"].numel(), device="cuda")[::2])):
+        right, item[key] = item[key], wrong
+        with pytest.raises(ValueError):
+            runner.forward(x)
+        item[key] = right
+        assert torch.equal(runner.forward(x), want)
+    api.bs_check_status()
