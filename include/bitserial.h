@@ -170,7 +170,10 @@ int bitserial_gemm(const uint32_t* a_packed, const uint32_t* w_packed, int M, in
  *                    first call and every call leaves it zero again, so one cudaMemset at allocation suffices.
  *                    Calls that share a workspace must not overlap on the GPU (use one stream, or one workspace
  *                    per stream).  A NULL or too small workspace falls back to the unsplit kernel.
- *   bs_*_workspace_bytes  bytes the planner wants for this shape on the CURRENT device (0: no split would be used).
+ *                    Only the popcount kernels split this way: a call that the tensor-core kernel takes (see bs_conv_params)
+ *                    neither reads nor writes the workspace.
+ *   bs_*_workspace_bytes  bytes the popcount planner wants for this shape on the CURRENT device (0: it would not split), whichever
+ *                    kernel the call then runs.
  *                    Plans depend on the multiprocessor count, which is looked up per device: ask with the device
  *                    current on which the call will run.  No launch.
  */
@@ -198,11 +201,12 @@ int bitserial_gemm_ws(const uint32_t* a_packed, const uint32_t* w_packed, int M,
  *   Arguments, outputs and results are exactly those of bitserial_gemm (bit-identical).
  *   Limit: shapes whose split plan needs more than the built-in scratch (roughly M*N above 400 thousand outputs
  *   when the planner splits) return BS_ERR_UNSUPPORTED and launch nothing; use bitserial_gemm or bitserial_gemm_ws.
- *   Shapes the planner does not split run the ordinary kernel and touch no scratch.
+ *   The limit counts the popcount kernels' plan of the shape, whichever kernel the call then runs.  Only calls that run those
+ *   kernels with a split touch the scratch; what the tensor-core kernel takes (see bs_conv_params) is one launch.
  *   First call on a device: looks up the device address of the built-in array (once per device, with that device
  *   current).  Make that first call before starting any stream capture.
  *   Sharing: all calls on a device use the same array, which keeps the previous call's contents.  A call that ran to
- *   completion leaves the part it used zero again (the last block of a tile restores it), so the clearing each call
+ *   completion leaves the part it used zero again (the last block of a tile restores it), so the clearing a split call
  *   does on `stream` before its kernel is a guard against a predecessor that did NOT complete normally (one that ended
  *   with BS_ERR_TIMEOUT) and against a caller that wrote to the array.  Two calls that overlap on the GPU (different
  *   streams without ordering) race on the array and give wrong results; serialise them.

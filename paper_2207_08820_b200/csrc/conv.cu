@@ -251,9 +251,10 @@ static int max_abs_code(int bits, int sign)
 }
 
 // `query_ws` != NULL: validate, plan with the reduction split allowed, report the workspace it wants, launch nothing.
+// clear_ws: zero the part of the workspace that a split uses before its kernel (calls the tensor cores take use none of it).
 static int conv_impl(const uint32_t* act, const uint32_t* wgt, const bs_conv_params* p, int32_t* out_i32,
                      uint32_t* out_packed, void* workspace, size_t workspace_bytes, cudaStream_t st,
-                     size_t* query_ws = nullptr)
+                     size_t* query_ws = nullptr, bool clear_ws = false)
 {
     if (!p) return BS_ERR_INVALID_ARG;
     if (!query_ws && (!act || !wgt || (!out_i32 && !out_packed))) return BS_ERR_INVALID_ARG;
@@ -368,6 +369,7 @@ static int conv_impl(const uint32_t* act, const uint32_t* wgt, const bs_conv_par
         if (!encode_map(&g.tmW, wgt, 3, dims, strides, box)) g.tma_w = 0;
     }
 
+    if (clear_ws && pl.ksplit > 1 && cudaMemsetAsync(workspace, 0, pl.ws_bytes, st) != cudaSuccess) { cudaGetLastError(); return BS_ERR_CUDA; }
     const unsigned grid = static_cast<unsigned>(tiles), block = static_cast<unsigned>(pl.NT);
     typedef int (*LaunchFn)(int, int, const ConvArgs&, unsigned, unsigned, size_t, cudaStream_t);
     static const LaunchFn table[4][3] = {{launch_conv_a1_f2, launch_conv_a1_f4, launch_conv_a1_f8},
@@ -494,16 +496,14 @@ extern "C" int bitserial_gemm_noalloc(const uint32_t* a_packed, const uint32_t* 
     int st = bs::conv_impl(nullptr, nullptr, &p, nullptr, nullptr, nullptr, 0, nullptr, &need);
     if (st != BS_OK) return st;
     if (need > BS_STATIC_SCRATCH_BYTES) return BS_ERR_UNSUPPORTED;   // beyond the built-in scratch: use bitserial_gemm_ws
-    cudaStream_t cs = static_cast<cudaStream_t>(stream);
     void* scratch = nullptr;
     if (need > 0) {
         scratch = bs::static_scratch_ptr(&st);
         if (!scratch) return st;
-        // Partial sums and arrival counters must start at zero.  A call that completed leaves them zero again, so this
-        // clearing is defensive: it covers a predecessor that gave up on a bounded wait (BS_ERR_TIMEOUT) half-way.
-        if (cudaMemsetAsync(scratch, 0, need, cs) != cudaSuccess) { cudaGetLastError(); return BS_ERR_CUDA; }
     }
-    return bs::conv_impl(a_packed, w_packed, &p, out_i32, out_packed, scratch, need, cs);
+    // Partial sums and arrival counters must start at zero.  A call that completed leaves them zero again, so clearing them is
+    // defensive: it covers a predecessor that gave up on a bounded wait (BS_ERR_TIMEOUT) half-way.
+    return bs::conv_impl(a_packed, w_packed, &p, out_i32, out_packed, scratch, need, static_cast<cudaStream_t>(stream), nullptr, true);
 }
 
 // Test aid: fills the built-in scratch with a byte value, standing in for a predecessor that did not finish cleanly,
