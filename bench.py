@@ -337,8 +337,8 @@ def measure_other_configs(torch, api, stream, args):
       gemm_sweep / bitwidth_sweep   as the stand-alone sweeps, fewer repetitions;
       detection_backbone            the detection-shaped stack at batch 16 on the tensor-core engine: conv time per pass under a
                                     CUDA graph, images/s, and sum(roofline time) / measured time over its layers;
-      layer_chains   the residual stack's conv layers at batch 16 and 64, one call per layer against runs of same-shaped
-                     layers as one call (bitserial_conv2d_tc_chain; the launches are the same), and how many calls the default makes;
+      layer_chains   the residual stack's conv layers at batch 16 and 64, the bound sequence (one call) against a call per unit, runs of
+                     same-shaped layers among them as one (bitserial_conv2d_tc_chain); the launches are the same;
       pack_large     the pack kernels on inputs larger than L2 (fp32 NCHW and NHWC, 2 and 3 bits)."""
     from paper_2207_08820_b200.net import BitserialNet
     dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
@@ -436,23 +436,20 @@ def measure_other_configs(torch, api, stream, args):
                                  "hbm_bound_layers": sums["hbm_bound_layers"],
                                  "pack_frac_hbm": (x.numel() * 4 + runner.bufs[net.in_name].numel() * 4) / (t_pack * 1e-3) / pk["hbm"]}
     del runner, x
-    # ---- runs of same-shaped layers as one launch (bitserial_conv2d_tc_chain) against one launch per layer
+    # ---- the bound sequence against calls of bitserial_conv2d_tc_chain (runs of same-shaped layers) and of single layers
     chain_rows = []
     for b in (16, 64):
         cnet, cseed = make_net("resnet18_body", b)
         cparams = wl.network_params(cnet, cseed)
-        row = {"workload": f"resnet18_body_batch{b}_w2a2, conv layers only (warm L2, one CUDA graph per pass)"}
-        for key, mode in (("per_layer", False), ("chains", True)):
-            r = BitserialNet(cnet, cparams, ACT_SCALE, batch=b, engine="tc", chains=mode)
+        r = BitserialNet(cnet, cparams, ACT_SCALE, batch=b, engine="tc", chains=True)
+        row = {"workload": f"resnet18_body_batch{b}_w2a2, conv layers only (warm L2, one CUDA graph per pass)", "launches": len(r.layers)}
+        for key, fn, calls in (("sequence", r.run_layers, 1), ("chains", r.run_units, len(r.units))):
             with torch.cuda.stream(stream):
-                r.run_layers()
+                fn()
                 stream.synchronize()
-                row[key + "_ms"] = graph_time(r.run_layers, reps=1, rounds=8)
-            row[key + "_launches"] = len(r.units)
-            del r
-        auto = BitserialNet(cnet, cparams, ACT_SCALE, batch=b, engine="tc", chains="auto")
-        row["auto_keeps_launches"] = len(auto.units)
-        del auto
+                row[key + "_ms"] = graph_time(fn, reps=1, rounds=8)
+            row[key + "_calls"] = calls
+        del r
         chain_rows.append(row)
     out["layer_chains"] = chain_rows
     # ---- the whole mixed-precision classifier: floating-point stem and head around the headline stack
@@ -502,8 +499,7 @@ def run_ours(args):
     params = wl.network_params(net, seed)
     x_host = torch.from_numpy(wl.network_input(net, replicas.rank_seed(seed, rank), ACT_SCALE)).pin_memory()
     x_dev = x_host.cuda()
-    chains = False if args.eager or args.chains == "off" else (True if args.chains == "on" else "auto")
-    runner = BitserialNet(net, params, ACT_SCALE, batch=net.batch, engine=args.engine, chains=chains)
+    runner = BitserialNet(net, params, ACT_SCALE, batch=net.batch, engine=args.engine, chains=args.chains == "on")
 
     stream = torch.cuda.Stream()
     with torch.cuda.stream(stream):
@@ -515,8 +511,7 @@ def run_ours(args):
         def run_pack():
             runner.pack_input(x_dev)
 
-        def run_convs():
-            runner.run_layers()
+        run_convs = runner.run_units if args.chains == "on" else runner.run_layers
 
         if args.eager:
             replay_pack, replay_conv = run_pack, run_convs
@@ -721,7 +716,8 @@ def run_ours(args):
             "clocks": clocks.summary(),
         }
         line["config"]["engine"] = args.engine
-        line["config"]["conv_launches_per_step"] = len(runner.units)
+        line["config"]["conv_launches_per_step"] = len(net.layers)
+        line["config"]["conv_calls_per_step"] = len(runner.units) if args.chains == "on" else 1
         if t_conv_other is not None:
             alt = tensor_roofline(t_conv_other, other)
             alt["engine"] = other
@@ -773,7 +769,7 @@ def main():
     ap.add_argument("--no-configs", action="store_true", help="leave out the compact measurements of the other workloads")
     ap.add_argument("--engine", default="tc", choices=["popc", "tc"],
                     help="popc: packed filters, expanded on chip; tc: filters prepared as int8 tiles once (the same tensor-core kernel)")
-    ap.add_argument("--chains", default="auto", choices=["auto", "on", "off"], help="runs of same-shaped layers as one call (on) or one call per layer; the launches are the same")
+    ap.add_argument("--chains", default="auto", choices=["auto", "on", "off"], help="on: runs of same-shaped layers as one call each instead of the bound sequence; the launches are the same")
     ap.add_argument("--eager", action="store_true", help="plain stream launches instead of CUDA graphs (for per-launch profiling)")
     args = ap.parse_args()
     if args.workload in ("bitwidth_sweep", "gemm_sweep"):

@@ -264,6 +264,7 @@ int bitserial_conv2d_tc_chained(const uint32_t* act_packed, const int8_t* wgt_tc
  *                    input of one.
  *   workspace        DEVICE, 16-byte aligned, at least bs_tc_chain_workspace_bytes(layers, nlayers) bytes, zero-filled by the
  *                    caller once before its first use.  One workspace serves one chain; calls that share one must not overlap.
+ *                    (Part of the call; the kernels it launches at present leave the workspace alone.)
  *   chained          non-zero: launched like bitserial_conv2d_tc_chained (same promise by the caller, for every layer).
  * bs_tc_chain_workspace_bytes returns 0 when the layers cannot run as one chain (shapes differ, a layer the tensor-core
  * path does not take, more than 4 layers); bitserial_conv2d_tc_chain then returns BS_ERR_UNSUPPORTED and launches nothing:

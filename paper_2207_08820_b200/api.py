@@ -16,7 +16,7 @@ from ._lib import BitserialError, ConvParams, lib, native
 UNSIGNED, SIGNED, BIPOLAR = 0, 1, 2
 NCHW, NHWC = 0, 1
 
-launch_count = 0   # kernels enqueued through this binding (every entry point below launches exactly one)
+launch_count = 0   # kernels enqueued through this binding (one by every entry point below but chains and sequences of layers)
 
 
 def _stream_ptr(stream: Optional[torch.cuda.Stream]) -> int:
@@ -174,21 +174,22 @@ def _params_array(params):
 
 
 def tc_chain_workspace_bytes(params) -> int:
-    """Bytes of the (zero-filled) workspace ``bitserial_conv2d_tc_chain`` needs for these layers; 0 when they cannot run as
-    one launch."""
+    """Bytes of the workspace ``bitserial_conv2d_tc_chain`` asks for with these layers; 0 when they cannot run as one chain."""
     return int(lib().bs_tc_chain_workspace_bytes(_params_array(params), len(params)))
 
 
 def bitserial_conv2d_tc_chain(acts, wgts_tc, params, outs, workspace: torch.Tensor, chained: bool = False, stream=None) -> None:
-    """Several same-shaped layers in one launch (``bitserial_conv2d_tc_chain``): per layer the packed input, the prepared
+    """Several same-shaped layers in one call, a launch each (``bitserial_conv2d_tc_chain``): per layer the packed input, the prepared
     filters, the :func:`conv_params` and the packed output tensor.  ``workspace``: device tensor of
-    :func:`tc_chain_workspace_bytes` bytes, zero-filled once before its first use."""
+    :func:`tc_chain_workspace_bytes` bytes."""
+    global launch_count
     n = len(params)
     vp = ctypes.c_void_p * n
     st = lib().bitserial_conv2d_tc_chain(n, vp(*[_ptr(t) for t in acts]), vp(*[_ptr(t) for t in wgts_tc]), _params_array(params),
                                          vp(*[_ptr(t) for t in outs]), _ptr(workspace), workspace.numel() * workspace.element_size(),
                                          int(chained), _stream_ptr(stream))
     _check(st, "bitserial_conv2d_tc_chain")
+    launch_count += n - 1
 
 
 def run_sequence(sequence, launches: int, stream=None) -> None:

@@ -127,7 +127,8 @@ static bool tc_chain_ok(int n, const bs_conv_params* params)
     return mma_conv_run(nullptr, reinterpret_cast<const int8_t*>(16), nullptr, p0, nullptr, nullptr, nullptr, false, true) == BS_OK;
 }
 
-// 16 x 8 output tiles of one layer: what the size of a chain's workspace is counted in.
+// The layers of a chain are launches of their own and use no workspace.  The call still asks for one, of the size callers were always told: a
+// word for every 16 x 8 output tile of every layer.
 static long long tc_chain_tiles(const bs_conv_params* p)
 {
     if (p->R == 1) return ceil_div_ll(static_cast<long long>(p->N) * p->H * p->W, 128);

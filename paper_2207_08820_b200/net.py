@@ -45,9 +45,9 @@ class BitserialNet:
                  engine: str = "popc", concurrent: bool = True, chains="auto"):
         """engine: "popc" = packed filters, expanded on chip; "tc" = filters prepared as int8 tiles once for every layer that
         supports it (others keep packed filters).  concurrent: launch independent neighbouring layers on
-        two streams (see :meth:`schedule`).  chains: with the "tc" engine, runs of consecutive same-shaped layers can go
-        through ``bitserial_conv2d_tc_chain`` (one call per run) where the library accepts them: True = always, False and
-        "auto" = one call per layer (the launches are the same)."""
+        two streams (see :meth:`schedule`).  chains: True groups, with the "tc" engine, runs of consecutive same-shaped layers that the
+        library accepts into units which :meth:`run_units` issues as one ``bitserial_conv2d_tc_chain`` call each; False and "auto" = a unit per
+        layer.  A pass is one call of a bound sequence whatever the units are; the launches are the same on either way."""
         self.net = net
         self.engine = engine
         self.act_scale = float(act_scale)
@@ -91,8 +91,8 @@ class BitserialNet:
         return self._conv_params(item)
 
     def _plan_units(self, chains: bool) -> List[Dict]:
-        """The launches of a forward pass: single layers, and runs of up to MAX_CHAIN consecutive layers that the library
-        accepts as one chain (same shape, resident-filter plan) and whose inputs come from outside the run or from an
+        """The calls of :meth:`run_units`: single layers, and runs of up to MAX_CHAIN consecutive layers that the library
+        accepts as one chain (same shape) and whose inputs come from outside the run or from an
         earlier layer of it.  Longest run first, greedily from the front."""
         units, i, n = [], 0, len(self.layers)
         while i < n:
@@ -146,7 +146,7 @@ class BitserialNet:
             wgt_tc=item["w_tc"], chained=chained and item["w_tc"] is not None)
 
     def run_unit(self, unit, chained: bool = True) -> None:
-        """One launch on the current stream: a layer, or a chain of layers."""
+        """One call on the current stream: a layer, or a chain of layers."""
         if unit["params"] is None:
             self.run_layer(unit["items"][0], chained=chained)
             return
@@ -156,7 +156,7 @@ class BitserialNet:
                                       [self.bufs[it["spec"].dst] for it in items], unit["workspace"], chained=chained)
 
     def schedule(self):
-        """The launches in order: (unit, aside, join).  With ``concurrent`` a single layer whose successor neither reads nor
+        """The calls in order: (unit, aside, join).  With ``concurrent`` a single layer whose successor neither reads nor
         overwrites its output (a projection shortcut beside the first conv of its block, the two 1x1 branches of a cross-stage
         block) runs ``aside`` on a second stream when its tiles do not fill the GPU: one wave of 128 x 128 output tiles leaves room for
         the neighbour (batch 1 residual stack 124 -> 114 us; where both fill the GPU, sharing it costs more than it
@@ -198,7 +198,11 @@ class BitserialNet:
         events between them become the edges of the graph."""
         if self._bind():
             api.run_sequence(self._sequence.handle, len(self.layers))
-            return
+        else:
+            self.run_units()
+
+    def run_units(self) -> None:
+        """The same launches one call per unit: what :meth:`run_layers` does where the library does not take the layers as one sequence."""
         main = torch.cuda.current_stream(self.device)
         done: Dict[int, torch.cuda.Event] = {}
         for i, (unit, aside, join) in enumerate(self.schedule()):

@@ -1,4 +1,4 @@
-"""GPU parity of ``bitserial_conv2d_tc_chain`` (several same-shaped layers in one launch): every layer's packed output against
+"""GPU parity of ``bitserial_conv2d_tc_chain`` (several same-shaped layers in one call): every layer's packed output against
 the oracle run layer by layer on the same seeded inputs (direct integer convolution + requantisation), word for word; repeated
 launches on one workspace, CUDA-graph replay, guard words around every output, and the shapes the entry point must refuse."""
 import ctypes
@@ -87,7 +87,7 @@ SHAPES = [
     # seed, N, C, H, W, k, layers
     (11, 3, 64, 24, 24, 3, 4),
     (12, 5, 128, 14, 14, 3, 3),
-    (13, 8, 64, 56, 56, 3, 4),       # 224 pixel tiles per layer over several hundred CTAs: tiles really wait for other CTAs
+    (13, 8, 64, 56, 56, 3, 4),       # 224 pixel tiles per layer over several hundred CTAs
     (14, 2, 64, 20, 12, 5, 2),
     (15, 4, 64, 16, 16, 1, 2),       # 1x1: flat pixel tiles
     (16, 1, 32, 40, 40, 3, 2),
@@ -110,8 +110,7 @@ def test_chain_matches_oracle(seed, N, C, H, W, k, nlayers):
 
 @pytest.mark.parametrize("a_bits", [1, 3, 4])
 def test_chain_other_activation_widths(a_bits):
-    """The 1-, 3- and 4-bit instantiations of the chain kernel (3- and 4-bit outputs take the formula epilogue, 4-bit records are
-    twice as long): same comparison with the oracle, layer by layer."""
+    """1-, 3- and 4-bit activations and outputs (4-bit records are twice as long): same comparison with the oracle, layer by layer."""
     x, layers, want = make_chain(30 + a_bits, 3, 64, 24, 24, 3, 3, a_bits=a_bits)
     assert len(np.unique(want[-1])) >= min(3, 1 << a_bits)
     g = ChainOnGpu(x, layers, 3, a_bits=a_bits)
@@ -122,8 +121,8 @@ def test_chain_other_activation_widths(a_bits):
 
 
 def test_chain_repeated_launches_and_graph_replay():
-    """The progress counters live on from launch to launch: three launches in a row, then a captured graph replayed three
-    times, with the outputs wiped in between; every run must reproduce the oracle."""
+    """Three calls in a row, then a captured graph replayed three times, with the outputs wiped in between; every run must reproduce the
+    oracle."""
     x, layers, want = make_chain(21, 4, 64, 28, 28, 3, 4)
     g = ChainOnGpu(x, layers, 3)
     assert g.nbytes > 0
@@ -199,6 +198,7 @@ def test_chain_refuses_what_it_cannot_run():
 
 
 def test_net_runner_uses_chains_and_fewer_launches():
+    """With chains a runner has fewer units: calls of ``run_units``, among them chains, with the launches of the bound sequence that a pass runs."""
     net = wl.resnet18_body(4)
     params = wl.network_params(net, 3000)
     runner = BitserialNet(net, params, 0.25, batch=4, engine="tc", chains=True)
@@ -213,7 +213,23 @@ def test_net_runner_uses_chains_and_fewer_launches():
     assert torch.equal(a, b)
     for name in net.tensor_shapes():
         assert torch.equal(runner.bufs[name], plain.bufs[name]), name
-    # "auto" keeps, per run of layers, whichever form it timed faster: any mix of the two, same results
+    for units, calls in ((runner, len(runner.units)), (plain, 19)):
+        for name in net.tensor_shapes():
+            if name != net.in_name:
+                units.bufs[name].fill_(-1)
+        made, entered = [], api.launch_count
+        run_unit = units.run_unit
+        units.run_unit = lambda unit, chained=True: (made.append(unit), run_unit(unit, chained=chained))
+        units.run_units()
+        api.bs_check_status()
+        assert len(made) == calls and api.launch_count - entered == 19
+        assert any(len(u["items"]) >= 3 for u in made) == (calls < 19)
+        assert torch.equal(units.bufs[net.out_name], b)
+        # a pass of layers that the library does not take as one sequence goes the same way
+        units._bind = lambda: False
+        units.bufs[net.out_name].fill_(-1)
+        assert torch.equal(units.forward(x), b) and len(made) == 2 * calls
+    # "auto": a unit per layer
     auto = BitserialNet(net, params, 0.25, batch=4, engine="tc", chains="auto")
     assert len(runner.units) <= len(auto.units) <= 19
     assert torch.equal(auto.forward(x), b)
