@@ -43,7 +43,7 @@ struct MmaArgs {
     int a_kind, w_kind;         // 0 unsigned, 1 two's complement, 2 bipolar
     int relu, out_bits, out_sign, out_cw_off, out_cw_total;
     int res_bits, res_sign, res_c_off, res_cw_total;
-    int i32_nhwc, acc_small;
+    int i32_nhwc;
     float acc_bound;                // largest possible |accumulator|
     // position numbering
     int flat;                       // positions are the pixels themselves (1x1, stride 1)
@@ -816,7 +816,7 @@ static __device__ __noinline__ void epilogue_item_formula(const MmaArgs& g, uint
 
 // Codes out, fast form.  One warp's accumulators arrive 16 columns at a time; the next 16 are on their way from tensor memory
 // while the current ones are computed, and the residual words of a group are fetched one group ahead.
-template <int OBC, int RESC, bool LO0, int EW, bool SPLIT, bool PING>
+template <int OBC, int RESC, bool LO0, int EW, bool SPLIT>
 __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e)
 {
     constexpr int STEP = EW / 4;
@@ -856,7 +856,7 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
             t = g.PT;
         }
         uint32_t A[16], B[16];
-        if (PING && t < g.PT) mm_ld16(acc + static_cast<uint32_t>(t * g.TN + cc * 32), A);
+        if (t < g.PT) mm_ld16(acc + static_cast<uint32_t>(t * g.TN + cc * 32), A);
         while (t < g.PT) {
             const int ob = o0 + cc * 32, pix = px.pix;
             const bool live = px.valid && ob < g.O;
@@ -865,10 +865,9 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
             uint32_t rw[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) rw[j] = rn[j];
-            if (!PING) mm_ld16(col, A);
             mm_ld_wait();
             mm_landed(A);
-            if (PING) mm_ld16(col + 16, B);
+            mm_ld16(col + 16, B);
             mm_st8(col, MM_PRESET);
             mm_st8(col + 8, MM_PRESET);
             // the next group's place and residual
@@ -891,11 +890,11 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
             }
             requant16<OBC, RESC, LO0>(A, tab, rtab, z[0], z[2], lo2, hi2, Wa);
             mm_ld_wait();
-            if (PING) mm_landed(B); else mm_landed(A);
-            if (PING && t < g.PT) mm_ld16(acc + static_cast<uint32_t>(t * g.TN + cc * 32), A);
+            mm_landed(B);
+            if (t < g.PT) mm_ld16(acc + static_cast<uint32_t>(t * g.TN + cc * 32), A);
             mm_st8(col + 16, MM_PRESET);
             mm_st8(col + 24, MM_PRESET);
-            requant16<OBC, RESC, LO0>(PING ? B : A, tab + 128u, rtab, z[1], z[3], lo2, hi2, Wb);
+            requant16<OBC, RESC, LO0>(B, tab + 128u, rtab, z[1], z[3], lo2, hi2, Wb);
             uint32_t ow[4] = {0, 0, 0, 0};
             if (OBC == 2) {
                 ow[0] = (Wa[0] & 0x55555555u) | ((Wb[0] << 1) & 0xAAAAAAAAu);
@@ -1451,12 +1450,12 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
         bool ok;
         if (SPLIT && range.rank > 0) ok = send_partials<EW>(g, e, range.rank);
         else if (!g.preset) ok = epilogue_general<EW, SPLIT>(g, e);
-        else if (g.epi == 0) ok = epilogue_codes<2, 0, true, EW, SPLIT, true>(g, e);
-        else if (g.epi == 1) ok = epilogue_codes<2, 2, true, EW, SPLIT, true>(g, e);
-        else if (g.epi == 2) ok = epilogue_codes<4, 0, true, EW, SPLIT, true>(g, e);
-        else if (g.epi == 3) ok = epilogue_codes<4, 4, true, EW, SPLIT, true>(g, e);
-        else if (g.epi == 4) ok = epilogue_codes<4, 0, false, EW, SPLIT, true>(g, e);
-        else ok = epilogue_codes<4, 4, false, EW, SPLIT, true>(g, e);
+        else if (g.epi == 0) ok = epilogue_codes<2, 0, true, EW, SPLIT>(g, e);
+        else if (g.epi == 1) ok = epilogue_codes<2, 2, true, EW, SPLIT>(g, e);
+        else if (g.epi == 2) ok = epilogue_codes<4, 0, true, EW, SPLIT>(g, e);
+        else if (g.epi == 3) ok = epilogue_codes<4, 4, true, EW, SPLIT>(g, e);
+        else if (g.epi == 4) ok = epilogue_codes<4, 0, false, EW, SPLIT>(g, e);
+        else ok = epilogue_codes<4, 4, false, EW, SPLIT>(g, e);
         if (!ok && lane == 0) atomicOr(g.status, STATUS_TIMEOUT);
     }
     mm_fence_before();

@@ -171,3 +171,15 @@ def test_bound_run_checks_its_tensors():
         item[key] = right
         assert torch.equal(runner.forward(x), want)
     api.bs_check_status()
+
+
+def test_prefetched_filters():
+    """The hint changes nothing that a pass computes."""
+    net = wl.resnet18_body(1, 28)
+    runner = BitserialNet(net, wl.network_params(net, 3000), ACT_SCALE, batch=1, engine="tc")
+    x = dev(wl.network_input(net, 3000, ACT_SCALE, batch=1))
+    want = runner.forward(x).clone()
+    runner.bufs[net.out_name].fill_(-1)
+    runner.prefetch_filters()
+    assert torch.equal(runner.forward(x), want)
+    api.bs_check_status()
