@@ -1,5 +1,5 @@
-"""Seeded random-shape sweep: shapes, bit-widths, signs, strides and pads drawn within the library's limits, on the
-popcount entry point and, where the shape is supported, on the tensor-core entry point.  Accumulators bit-exact against
+"""Seeded random-shape sweep: shapes, bit-widths, signs, strides and pads drawn within the library's limits, on the entry point that
+takes packed filters and, where the shape is supported, on the one that takes prepared filters (the same kernel but for what it refuses).  Accumulators bit-exact against
 the oracle's direct integer convolution / matrix product, requantised codes equal to the oracle's epilogue and plane
 split (tolerance: at most 1e-4 of codes off by one level; zero expected)."""
 import numpy as np
@@ -40,7 +40,7 @@ def test_random_conv_shape(index):
     want = oracle.conv2d_i32(c["x"], c["w"], d["stride"], d["pad"])
     codes = oracle.requantize(want, c["scale"], c["bias"], True, d["out_bits"], 0)
     want_packed = oracle.pack_activations(codes, d["out_bits"], 0)
-    acc, packed = gpu_conv(c)                      # popcount entry point, guard words around both outputs
+    acc, packed = gpu_conv(c)                      # packed filters, guard words around both outputs
     assert np.array_equal(acc, want), d
     assert np.array_equal(packed, want_packed), d
     if api.tc_supported(d["N"], d["C"], d["H"], d["W"], d["O"], d["k"], d["stride"], d["pad"], d["a_bits"], d["a_sign"],

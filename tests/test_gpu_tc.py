@@ -1,13 +1,13 @@
-"""GPU parity for the tensor-core entry points: int32 accumulators bit-exact against the oracle's direct integer
+"""GPU parity for the entry points that take prepared filters: int32 accumulators bit-exact against the oracle's direct integer
 convolution, requantised codes equal to the oracle's epilogue (tolerance: at most 1e-4 of codes off by one level;
-zero expected), and identical to the popcount entry points."""
+zero expected)."""
 import numpy as np
 import pytest
 import torch
 
 import oracle
 from paper_2207_08820_b200 import api, workloads as wl
-from gpu_util import Guarded, conv_out_shapes, dev, words
+from gpu_util import Guarded, conv_out_shapes, dev, gpu_conv, words
 
 pytestmark = pytest.mark.gpu
 
@@ -121,15 +121,19 @@ def test_tc_residual_matches_oracle_and_popcount_path():
     assert np.array_equal(acc, want)
     codes = oracle.requantize(want, c["scale"], c["bias"], True, 2, 0, res=res, res_scale=0.5)
     assert np.array_equal(packed, oracle.pack_activations(codes, 2, 0))
+    # the same residual eight channels into a wider tensor: inside a word, so the popcount kernels take the layer
+    wider = np.concatenate([wl.rand_codes(rng, (2, 8, 12, 12), 2, 0), res], axis=1)
+    acc_popc, packed_popc = gpu_conv(c, residual=(wider, 2, 0), res_scale=0.5, res_c_offset=8)
+    assert np.array_equal(acc_popc, acc) and np.array_equal(packed_popc, packed)
 
 
 @pytest.mark.parametrize("kind", ["extreme_positive", "mixed_sign"])
 @pytest.mark.parametrize("with_res", [False, True])
 @pytest.mark.parametrize("out", [(2, 0), (2, 1), (1, 0), (1, 2)])
 def test_tc_epilogue_scale_bias_corner_cases(kind, with_res, out):
-    """Per-filter scales and biases at the corners of the comparison epilogue: tiny and huge positive scales with
-    biases that push every threshold out of the accumulator range (integer thresholds saturate), and filters with
-    zero or negative scale (the kernel must fall back to the floating-point comparison)."""
+    """Per-filter scales and biases at the corners of the fast requantisation: tiny and huge positive scales with
+    biases that push every level out of the accumulators' range (the formula takes over, one output at a time), and filters with
+    zero or negative scale."""
     out_bits, out_sign = out
     c = wl.single_conv_case(seed=31, N=2, C=64, H=13, W=13, O=96, calibrated=True)
     rng = np.random.default_rng(5)
@@ -157,7 +161,7 @@ def test_tc_epilogue_scale_bias_corner_cases(kind, with_res, out):
 @pytest.mark.parametrize("out_bits,out_sign", [(3, 0), (4, 0), (3, 1), (4, 1)])
 @pytest.mark.parametrize("with_res", [False, True])
 def test_tc_wide_output_codes(out_bits, out_sign, with_res):
-    """3- and 4-bit outputs take the formula epilogue (no comparison form); with a 3-bit signed residual on top."""
+    """3- and 4-bit outputs: the fast requantisation of wide codes, signed and unsigned; the formula with a 3-bit signed residual on top."""
     c = wl.single_conv_case(seed=77, N=2, C=64, H=11, W=13, O=72, calibrated=True)
     rng = np.random.default_rng(9)
     scale = (c["scale"] * (2 ** (out_bits - 2))).astype(np.float32)
@@ -194,8 +198,7 @@ def test_tc_gemm(M, N, K):
 def test_tc_gemm_4096_sampled(M, N, K):
     """The largest shapes of the matrix-product sweep on the tensor-core entry point: the oracle evaluates sampled rows
     and columns; row and column sums of the whole product are checked against sums formed from the operands (a property
-    that holds at any size); the requantised output is compared on the sampled rows.  K = 4608 and 3200 stage the packed
-    rows in segments; 4000 x 4608 x 3200 has a last pixel tile of 32 rows and a last segment of 56 of 72 words."""
+    that holds at any size); the requantised output is compared on the sampled rows.  4000 rows end inside a tile."""
     c = wl.gemm_case(M, N, K, seed=wl.gemm_sweep_seed(M, K) if M == 4096 else 2100 + K)
     scale, bias = wl.calibrated_scale_bias(c["w"], 2, 0, 2)
     ap = api.bs_pack_rows(dev(c["a"]), 2, 0)
