@@ -8,7 +8,7 @@ namespace bs {
 
 // Column c of a 32-filter group of the accumulator tile holds filter mma_filter_of_column(c) of the group, and byte b of a
 // 32-channel block of either operand holds channel mma_channel_of_byte(b): the orders in which the epilogue can pair its
-// outputs and the expansion can cut bytes out of the plane words without moving single bits (see mma_conv.cu).
+// outputs and the expansion can cut bytes out of the plane words without moving single bits (see mma_kernel.cuh).
 __host__ __device__ constexpr int mma_filter_of_column(int c) { return 16 * (c & 1) + 2 * ((c >> 1) & 7) + (c >> 4); }
 __host__ __device__ constexpr int mma_column_of_filter(int f) { return 16 * (f & 1) + 2 * ((f & 15) >> 1) + (f >> 4); }
 __host__ __device__ constexpr int mma_channel_of_byte(int b) { return 8 * (b & 3) + (b >> 2); }

@@ -487,7 +487,8 @@ struct MmaIssue {
     bool resident;
 };
 
-// The MMA warp's walk over items and chunks.  Everything of a chunk, its commits included, goes out in one elected region.
+// The MMA warp's walk over items and chunks, in uniform code; every MMA and every commit elects its thread by itself (one elected region
+// for a whole chunk was slower: its descriptors move through vector registers, 100 cycles per MMA against 85 to 90).
 template <int TAPS, bool SPLIT>
 __device__ __forceinline__ void issue_items(const MmaArgs& g, const MmaIssue& m)
 {

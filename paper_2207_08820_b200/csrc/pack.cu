@@ -100,7 +100,7 @@ struct SignPlanes {
 // different banks).  A NaN ends at level 0 (the clamp drops it, the comparison fails), infinities at the ends.
 // Adding 1.5 * 2^23 leaves k in the low mantissa bits.  The levels of inputs 4 i + g are gathered as the nibbles i of word g, so that
 // plane j is the or over g of ((word g >> j) & 0x11111111) << g: two instructions per word and plane.  About 10 instructions an
-// element against 27 of the search, which bound the kernel (64x64x56x56, 4 bits: 17.2 -> 9.9 us).
+// element against 27 of the search, which bound the kernel (64x64x56x56, 4 bits, NCHW: 17.2 -> 12.5 us).
 template <int BITS>
 struct LevelPlanes {
     uint32_t w[BITS], r[4];
@@ -440,7 +440,7 @@ bitpack_nhwc_i8_kernel(const int8_t* __restrict__ x_in, uint32_t* __restrict__ o
 // first byte lies in, joined by funnel shifts, and the same plane gathering as above; bits of channels past C are masked out of the
 // finished words, so what the stage holds behind the last record does not matter.  Neighbouring threads take neighbouring
 // channel words of a pixel: the packed records leave as one contiguous run.  Byte loads with votes took 10 times as long
-// (48 x 45 x 61 pixels of 50 channels, 2 bits: 18 -> 2 us).
+// (48 x 45 x 61 pixels of 50 channels, 2 bits: 18.2 -> 3.9 us a call).
 constexpr int RAGGED_PIX = 64, RAGGED_BYTES = 40 * 1024;
 
 template <int BITS>
@@ -632,8 +632,10 @@ extern "C" int bs_quantiser_bounds(float act_scale, int a_bits, bs_sign_t a_sign
     return BS_OK;
 }
 
-// NHWC codes of more channels than this start behind the kernel before, not beside its end: with all blocks begun at once the long
-// strides took longer (20 x 14 x 14 x 512: 4.1 -> 5.3 us a call; 64 x 56 x 56 x 64 gains, 6.2 -> 4.7).
+// NHWC codes of more channels than this start behind the kernel before, not beside its end.  Up to 128 channels the early start is
+// faster at every size measured (14 x 14 pixels, 2 bits, back to back; 8 M codes of 64 channels: 6.1 -> 4.4 us a call, of 128: 7.1 -> 5.8;
+// 0.5 M: 3.7 -> 3.5).  Above, most sizes gain as much (8 M of 256: 8.2 -> 6.2, of 384: 7.0 -> 6.0), but some lose, and not the same ones for
+// neighbouring widths (8 M of 300: 6.2 -> 7.3; 4 M of 384: 6.2 -> 6.6, of 512: 6.2 -> 7.2): the line stands where none does.
 constexpr int NHWC_DEPENDENT_C = 128;
 
 template <int BITS>
