@@ -47,6 +47,7 @@ def native():
     global _native
     if _native is None:
         lib()
+        import torch  # noqa: F401  (the binding's libraries are found through it)
         try:
             from . import _binding
         except ImportError as e:

@@ -195,3 +195,8 @@ def test_binding_sees_replaced_entries(L):
     for wrong in ((1,) + args[1:], args[:2] + (args[2][:-1],), ((1,),) + args[1:]):
         with pytest.raises(ValueError):
             native().unchanged(*wrong)
+
+
+def test_binding_loads_before_anything_else(L):
+    """In a process that has not imported torch, and whose build found everything up to date."""
+    subprocess.run([sys.executable, "-c", "from paper_2207_08820_b200 import _lib; _lib.native()"], cwd=ROOT, check=True)
