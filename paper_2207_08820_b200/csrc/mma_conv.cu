@@ -70,6 +70,8 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows, int sms)
     const long long per_img = static_cast<long long>(PH) * g.pitch;
     const long long total = static_cast<long long>(g.N) * c.ns * per_img;
     if (total + per_img + 4096 + g.HL > 0x7fffffffLL || g.NI > 4096) return false;
+    // the kernel counts input pixels (stride 2: up to four times the positions) and the words of a packed filter tile in 32 bits
+    if (static_cast<long long>(g.N) * g.H * g.W > 0x7fffffffLL || (packed_b && static_cast<long long>(c.TN) * g.RS * g.Cw * WB > 0x7fffffffLL)) return false;
     g.total = static_cast<int>(total);
     g.d_img = make_div(static_cast<int>(per_img));
     g.d_pitch = make_div(g.pitch);

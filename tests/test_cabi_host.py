@@ -200,3 +200,12 @@ def test_binding_sees_replaced_entries(L):
 def test_binding_loads_before_anything_else(L):
     """In a process that has not imported torch, and whose build found everything up to date."""
     subprocess.run([sys.executable, "-c", "from paper_2207_08820_b200 import _lib; _lib.native()"], cwd=ROOT, check=True)
+
+
+def test_planner_refuses_more_input_pixels_than_it_can_count(L):
+    """Stride 2 has a quarter as many outputs as input pixels, whose number has to fit 31 bits too."""
+    from paper_2207_08820_b200 import api
+    for k in (1, 3):
+        supported = lambda N, stride: api.tc_supported(N, 32, 6000, 6000, 32, k, stride, k // 2, 4, api.UNSIGNED, 2, api.SIGNED)
+        assert supported(59, 2) and supported(58, 1)                 # 2.12e9 pixels
+        assert not supported(60, 2) and not supported(60, 1)         # 2.16e9
