@@ -107,7 +107,8 @@ def bitserial_conv2d(act_packed: torch.Tensor, wgt_packed: torch.Tensor, *, C: i
                      stream=None):
     """act_packed [N,H,W,Cw,a_bits], wgt_packed [O,R,S,Cw,w_bits].  Returns (out_i32 or None, out_packed or None).
     A packed output is produced when ``out_bits`` > 0 (allocated here unless ``out_packed`` is given).
-    ``workspace`` (zeroed device tensor, see :func:`conv_workspace`) enables the reduction split (``bitserial_conv2d_ws``).
+    ``workspace`` (zeroed device tensor, see :func:`conv_workspace`) lets the popcount kernels split the reduction
+    (``bitserial_conv2d_ws``; the tensor-core kernel leaves it alone).
     ``wgt_tc`` (from :func:`tc_prepare_weights`) selects the tensor-core entry point ``bitserial_conv2d_tc``;
     with ``chained`` it is ``bitserial_conv2d_tc_chained`` (set-up overlaps the preceding kernel of the stream: filters,
     scale and bias must have been final before that kernel was launched)."""
@@ -125,7 +126,8 @@ def bitserial_gemm(a_packed: torch.Tensor, w_packed: torch.Tensor, K: int, *, a_
                    out_i32: Optional[torch.Tensor] = None, want_i32: bool = True,
                    out_packed: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None, stream=None):
     """a_packed [M,Kw,a_bits], w_packed [N,Kw,w_bits].  Returns (out_i32 [M,N] or None, out_packed or None).
-    ``workspace`` (zeroed device tensor, see :func:`gemm_workspace`) enables the reduction split (``bitserial_gemm_ws``)."""
+    ``workspace`` (zeroed device tensor, see :func:`gemm_workspace`) lets the popcount kernels split the reduction
+    (``bitserial_gemm_ws``; the tensor-core kernel leaves it alone)."""
     st, out_i32, out_packed = native().gemm(a_packed, w_packed, -1, -1, K, a_sign, w_sign, scale, bias, relu, out_bits, out_sign,
                                             out_i32, want_i32, out_packed, workspace, stream)
     _check(st, "bitserial_gemm")
@@ -211,14 +213,14 @@ def bitserial_gemm_tc(a_packed: torch.Tensor, w_tc: torch.Tensor, N: int, K: int
 
 
 def gemm_workspace(M: int, N: int, K: int, a_bits: int, a_sign: int, w_bits: int, w_sign: int, device="cuda"):
-    """Zeroed workspace for the reduction split of this matrix product, or None when the planner would not split."""
+    """Zeroed workspace for the reduction split of this matrix product, or None when the popcount planner would not split."""
     nbytes = lib().bs_gemm_workspace_bytes(M, N, K, a_bits, a_sign, w_bits, w_sign)
     return torch.zeros((nbytes + 3) // 4, dtype=torch.int32, device=device) if nbytes else None
 
 
 def conv_workspace(N: int, C: int, H: int, W: int, O: int, k: int, stride: int, pad: int, a_bits: int, a_sign: int,
                    w_bits: int, w_sign: int, device="cuda"):
-    """Zeroed workspace for the reduction split of this convolution, or None when the planner would not split."""
+    """Zeroed workspace for the reduction split of this convolution, or None when the popcount planner would not split."""
     p = ConvParams(N=N, C=C, H=H, W=W, O=O, R=k, S=k, stride=stride, pad=pad, a_bits=a_bits, a_sign=a_sign,
                    w_bits=w_bits, w_sign=w_sign)
     nbytes = lib().bs_conv_workspace_bytes(ctypes.byref(p))
