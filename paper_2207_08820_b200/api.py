@@ -15,6 +15,7 @@ from ._lib import BitserialError, ConvParams, lib, native
 
 UNSIGNED, SIGNED, BIPOLAR = 0, 1, 2
 NCHW, NHWC = 0, 1
+ERR_UNSUPPORTED = 2
 
 launch_count = 0   # kernels enqueued through this binding (one by every entry point below but chains and sequences of layers)
 
@@ -249,6 +250,25 @@ def maxpool2d_f32(x: torch.Tensor, k: int, stride: int, pad: int, out: Optional[
         out = torch.empty(N, C, P, Q, dtype=torch.float32, device=x.device)
     _check(lib().bs_maxpool2d_f32(_ptr(x), N, C, H, W, k, stride, pad, _ptr(out), _stream_ptr(stream)), "bs_maxpool2d_f32")
     return out
+
+
+def stem_codes_f32(x: torch.Tensor, w: torch.Tensor, bias: Optional[torch.Tensor], act_scale: float, a_bits: int, out: torch.Tensor,
+                   stream=None) -> bool:
+    """Stem convolution (stride 2, pad 3) with ReLU, 3x3 stride-2 max pooling and quantise + pack in one call (``bs_stem_codes_f32``): images to the
+    packed codes of :func:`conv2d_f32`, :func:`maxpool2d_f32` and :func:`bitpack_activations`.  False where the library has no such kernel for
+    the shape: nothing was launched."""
+    N, C, H, W = x.shape
+    O, C2, R, S = w.shape
+    if C != C2 or x.dtype != torch.float32 or w.dtype != torch.float32:
+        raise ValueError("float32 tensors with matching channels expected")
+    P, Q = (H - 1) // 2 + 1, (W - 1) // 2 + 1
+    if out.numel() != packed_act_words(N, O, (P - 1) // 2 + 1, (Q - 1) // 2 + 1, a_bits):
+        raise ValueError("output of another size")
+    st = lib().bs_stem_codes_f32(_ptr(x), _ptr(w), _ptr(bias), N, C, H, W, O, R, S, 2, 3, act_scale, a_bits, _ptr(out), _stream_ptr(stream))
+    if st == ERR_UNSUPPORTED:
+        return False
+    _check(st, "bs_stem_codes_f32")
+    return True
 
 
 def avgpool_codes_f32(packed: torch.Tensor, C: int, a_sign: int, inv: float, out: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:

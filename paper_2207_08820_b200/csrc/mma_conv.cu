@@ -20,19 +20,6 @@ constexpr int MM_SMEM_MAX = 224 * 1024;
 
 int up(int v, int m) { return (v + m - 1) / m * m; }
 
-FastDiv make_div(int d)
-{
-    FastDiv f{0, 0, d};
-    if (d > 1) {
-        int l = 0;
-        while ((1LL << l) < d) ++l;                       // ceil(log2 d)
-        const unsigned long long p = 31 + l;
-        f.mul = static_cast<unsigned>(((1ULL << p) + d - 1) / d);
-        f.shift = static_cast<unsigned>(p - 32);
-    }
-    return f;
-}
-
 int max_abs_of(int bits, int sign) { return sign == BS_BIPOLAR ? 1 : (sign == BS_SIGNED ? 1 << (bits - 1) : (1 << bits) - 1); }
 
 struct Cand {

@@ -25,6 +25,18 @@ namespace bs {
 constexpr int MM_STAGES = 8;         // most stages of packed words in front of the expanders
 
 struct FastDiv { unsigned mul, shift; int d; };      // quotient of 0 <= n < 2^31 by d as umulhi(n, mul) >> shift
+inline FastDiv make_div(int d)
+{
+    FastDiv f{0, 0, d};
+    if (d > 1) {
+        int l = 0;
+        while ((1LL << l) < d) ++l;                       // ceil(log2 d)
+        const unsigned long long p = 31 + l;
+        f.mul = static_cast<unsigned>(((1ULL << p) + d - 1) / d);
+        f.shift = static_cast<unsigned>(p - 32);
+    }
+    return f;
+}
 
 struct MmaArgs {
     CUtensorMap tmA, tmB;           // flat tiles with aligned rows: packed pixels (words, rows), packed filters (words, filters)

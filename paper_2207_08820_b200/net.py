@@ -302,9 +302,9 @@ class BitserialNet:
 
 
 class BitserialFullNet:
-    """The whole mixed-precision classifier of ``workloads.FullNetSpec`` through the C ABI: floating-point stem
-    (``bs_conv2d_f32`` + ``bs_maxpool2d_f32``), quantise + pack, the quantised body (:class:`BitserialNet`), floating-point head
-    (``bs_avgpool_codes_f32`` + ``bs_fc_f32``).  Host logic only."""
+    """The whole mixed-precision classifier of ``workloads.FullNetSpec`` through the C ABI: floating-point stem and quantiser (one kernel,
+    ``bs_stem_codes_f32``, or ``bs_conv2d_f32`` + ``bs_maxpool2d_f32`` + quantise and pack for shapes it does not take), the quantised body
+    (:class:`BitserialNet`), floating-point head (``bs_avgpool_codes_f32`` + ``bs_fc_f32``).  Host logic only."""
 
     def __init__(self, net, params: Dict[str, Dict], device="cuda", batch: Optional[int] = None, engine: str = "tc"):
         self.net = net
@@ -316,17 +316,45 @@ class BitserialFullNet:
         self.fc_w, self.fc_b = to(params["fc"]["w"]), to(params["fc"]["bias"])
         h1 = (net.hw + 2 * 3 - 7) // 2 + 1
         h2 = (h1 + 2 - 3) // 2 + 1
-        self.stem_conv = torch.empty(self.batch, 64, h1, h1, dtype=torch.float32, device=self.device)
-        self.stem_pool = torch.empty(self.batch, 64, h2, h2, dtype=torch.float32, device=self.device)
+        self._stem_conv = torch.empty(self.batch, 64, h1, h1, dtype=torch.float32, device=self.device)
+        self._stem_pool = torch.empty(self.batch, 64, h2, h2, dtype=torch.float32, device=self.device)
+        self._fused_images: Optional[torch.Tensor] = None      # images of the last pass, where it made no float tensors of the stem
         C, H, W = net.body.tensor_shapes()[net.body.out_name]
         self.pooled = torch.empty(self.batch, C, dtype=torch.float32, device=self.device)
         self.logits = torch.empty(self.batch, net.classes, dtype=torch.float32, device=self.device)
         self.inv = float(np.float32(np.float32(net.body_act_scale) / np.float32(H * W)))
-        self.launches_per_forward = 4 + self.body.launches_per_forward
+        self.launches_per_forward = 2 + self.body.launches_per_forward      # two more where the stem runs as layers of its own
 
     def run_stem(self, images: torch.Tensor) -> None:
-        api.conv2d_f32(images, self.stem_w, self.stem_b, stride=2, pad=3, relu=True, out=self.stem_conv)
-        api.maxpool2d_f32(self.stem_conv, 3, 2, 1, out=self.stem_pool)
+        """The stem as layers of its own: images to ``stem_conv`` and ``stem_pool``."""
+        self._fused_images = None
+        api.conv2d_f32(images, self.stem_w, self.stem_b, stride=2, pad=3, relu=True, out=self._stem_conv)
+        api.maxpool2d_f32(self._stem_conv, 3, 2, 1, out=self._stem_pool)
+
+    def run_front(self, images: torch.Tensor) -> None:
+        """Images to the body's packed input."""
+        body = self.body
+        if tuple(images.shape) == (self.batch, 3, self.net.hw, self.net.hw) and api.stem_codes_f32(
+                images, self.stem_w, self.stem_b, body.act_scale, body.net.a_bits, body.bufs[body.net.in_name]):
+            self._fused_images = images
+        else:
+            self.run_stem(images)
+            body.pack_input(self._stem_pool)
+
+    @property
+    def stem_conv(self) -> torch.Tensor:
+        """Float output of the stem convolution.  A pass through the fused kernel does not make it: for inspection it is then evaluated from the
+        images of that pass, as they are now."""
+        if self._fused_images is not None:
+            self.run_stem(self._fused_images)
+        return self._stem_conv
+
+    @property
+    def stem_pool(self) -> torch.Tensor:
+        """Float output of the stem's pooling, like :attr:`stem_conv`."""
+        if self._fused_images is not None:
+            self.run_stem(self._fused_images)
+        return self._stem_pool
 
     def run_head(self) -> None:
         body = self.net.body
@@ -335,8 +363,7 @@ class BitserialFullNet:
 
     def forward(self, images: torch.Tensor) -> torch.Tensor:
         """images: float32 [batch, 3, hw, hw] on the device.  Returns the logits [batch, classes]."""
-        self.run_stem(images)
-        self.body.pack_input(self.stem_pool)
+        self.run_front(images)
         self.body.run_layers()
         self.run_head()
         return self.logits

@@ -1,0 +1,123 @@
+"""The fused stem (``bs_stem_codes_f32``: convolution, ReLU, pooling, quantiser) against the oracle and against the separate layers: the codes
+are equal, whatever the images, filters and scale, since outputs near a bound of the quantiser take the layers' own arithmetic."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2207_08820_b200 import api, workloads as wl
+from paper_2207_08820_b200.net import BitserialFullNet
+from gpu_util import Guarded, dev
+
+pytestmark = pytest.mark.gpu
+
+
+def inputs(N, H, W, seed=0, bias=0.1):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    x = torch.randn(N, 3, H, W, generator=g, device="cuda")
+    w = torch.randn(64, 3, 7, 7, generator=g, device="cuda") / math.sqrt(147.0)
+    return x, w, torch.randn(64, generator=g, device="cuda") * bias
+
+
+def compare(x, w, b, scale=0.25):
+    pool = api.maxpool2d_f32(api.conv2d_f32(x, w, b, 2, 3, True), 3, 2, 1)
+    want = api.bitpack_activations(pool, scale, 2)
+    guard = Guarded()
+    out = guard.empty(tuple(want.shape), fill=-1)
+    assert api.stem_codes_f32(x, w, b, scale, 2, out)
+    api.bs_check_status()
+    guard.check()
+    assert torch.equal(out, want)
+
+
+# one pixel pair, one pooled row, odd heights, widths whose rows end inside a tile or a slab, runs that cross images, the widest rows
+@pytest.mark.parametrize("N,H,W", [(5, 1, 2), (2, 8, 8), (1, 7, 34), (2, 37, 46), (3, 64, 64), (149, 20, 24), (9, 75, 126), (2, 224, 224), (1, 90, 254), (2, 256, 256), (1, 50, 278)])
+def test_sizes(N, H, W):
+    compare(*inputs(N, H, W, seed=H))
+    x, w, _ = inputs(N, H, W, seed=H + 1)
+    compare(x, w, None)
+
+
+def test_against_oracle():
+    x, w, b = inputs(2, 58, 66, seed=5)
+    pool = oracle.maxpool2d_f32(oracle.conv2d_f32(x.cpu().numpy(), w.cpu().numpy(), b.cpu().numpy(), 2, 3, True), 3, 2, 1)
+    codes = oracle.quantize(pool, 0.25, 2, api.UNSIGNED)
+    out = torch.empty(2, 15, 17, 2, 2, dtype=torch.int32, device="cuda")
+    assert api.stem_codes_f32(x, w, b, 0.25, 2, out)
+    assert np.array_equal(api.bitunpack_activations(out, 64, 2).cpu().numpy(), codes)
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), -float("inf"), 3e38, 1e30, 2.0 ** 20, 1e6, 1e-30, 1e-42])
+def test_single_values(value):
+    x, w, b = inputs(2, 64, 64, seed=9)
+    x[1, 2, 31, 17] = value
+    compare(x, w, b)
+
+
+@pytest.mark.parametrize("case", ["zero", "constant", "on the bounds", "small images", "large images", "zero filters", "one large filter", "large bias",
+                                  "bad filters", "cancelling", "denormal"])
+def test_values(case):
+    x, w, b = inputs(2, 66, 70, seed=11)
+    if case == "zero":
+        x.zero_()
+    elif case == "constant":
+        x.fill_(0.37)
+    elif case == "on the bounds":        # half of the outputs are the bias, which is a bound or its neighbour: all undecided
+        x[:, :, :40] = 0.0
+        b.copy_(torch.tensor([0.125, 0.375, 0.625, 0.12500001], device="cuda").repeat(16))
+    elif case == "small images":
+        x *= 1e-25
+        w *= 1e25
+    elif case == "large images":
+        x *= 255.0
+    elif case == "zero filters":
+        w.zero_()
+    elif case == "one large filter":
+        w[7] *= 1e6
+    elif case == "large bias":
+        b *= 1e4
+    elif case == "bad filters":
+        w[3, 1, 2, 2], w[40, 0, 0, 0], b[7], b[9] = float("inf"), float("nan"), float("inf"), float("nan")
+    elif case == "cancelling":           # the order of the chain decides
+        w.fill_(1.0)
+        x[:, 0], x[:, 2] = 3e5, -3e5
+    else:
+        x *= 1e-42
+    compare(x, w, b)
+
+
+@pytest.mark.parametrize("scale", [1e-20, 0.01, 0.25, 0.6, 1.5, 37.0, 1e20])
+def test_scales(scale):
+    compare(*inputs(2, 64, 64, seed=13), scale=scale)
+
+
+@pytest.mark.parametrize("C,O,k,W,bits", [(4, 64, 7, 64, 2), (3, 32, 7, 64, 2), (3, 64, 5, 64, 2), (3, 64, 7, 63, 2), (3, 64, 7, 64, 3), (3, 64, 7, 400, 2)])
+def test_other_shapes_are_refused(C, O, k, W, bits):
+    x, w = torch.zeros(1, C, 64, W, device="cuda"), torch.zeros(O, C, k, k, device="cuda")
+    q = (W - 1) // 2 + 1
+    out = torch.full((1, 16, (q - 1) // 2 + 1, (O + 31) // 32, bits), -1, dtype=torch.int32, device="cuda")
+    assert not api.stem_codes_f32(x, w, None, 0.25, bits, out)
+    assert bool((out == -1).all())
+
+
+@pytest.mark.parametrize("hw", [32, 64, 284])
+def test_classifier_front(hw):
+    """Both ways of the classifier's front, the float tensors of the stem, and filters replaced between passes."""
+    net = wl.resnet18_full(batch=2, hw=hw)
+    params = wl.full_network_params(net, 8300)
+    images = dev(wl.full_network_input(net, 8300))
+    runner = BitserialFullNet(net, params, batch=2)
+    logits = runner.forward(images).clone()
+    packed = runner.body.bufs[net.body.in_name].clone()
+    conv, pool = runner.stem_conv.clone(), runner.stem_pool.clone()
+    runner.run_stem(images)
+    assert torch.equal(conv, runner.stem_conv) and torch.equal(pool, runner.stem_pool)
+    runner.body.pack_input(runner.stem_pool)
+    assert torch.equal(packed, runner.body.bufs[net.body.in_name])
+    runner.stem_w.mul_(-1.0)
+    assert not torch.equal(runner.forward(images), logits)
+    runner.stem_w = -runner.stem_w
+    assert torch.equal(runner.forward(images), logits)
+    api.bs_check_status()
