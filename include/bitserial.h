@@ -221,16 +221,17 @@ int bitserial_gemm_noalloc(const uint32_t* a_packed, const uint32_t* w_packed, i
                            void* stream);
 
 /*
- * Filters prepared once: the same kernels as bitserial_conv2d / bitserial_gemm with the filters already expanded to int8 tiles by
+ * Filters prepared once: the same kernels as bitserial_conv2d / bitserial_gemm with the filters already expanded to operand tiles by
  * bs_tc_prepare_weights, so that a launch fetches them instead of expanding them.  Results (accumulators and requantised codes) are bit-identical to
  * bitserial_conv2d / bitserial_gemm; the epilogue is the one documented at bs_conv_params.
  *   Supported subset (bs_tc_supported returns 1): C a multiple of 32 whose packed pixel record (C/32 * a_bits words)
  *   is a 16-byte multiple, or an 8-byte multiple when a packed image row (W records) is a 16-byte multiple and, for
  *   1x1 stride-1 layers, N*H*W is even; res_c_offset a multiple of 32; everything else as bitserial_conv2d.  Unsupported shapes
  *   return BS_ERR_UNSUPPORTED: use bitserial_conv2d.
- *   bs_tc_weights_bytes    bytes of the prepared int8 filter tensor (0 on bad input).
- *   bs_tc_prepare_weights  packed weights [O][R][S][Cw][w_bits] -> int8 tiles [C/32][ceil(O/128)*16][R*S][2][8][16]
- *                          (blocks of 32 channels; a_bits is accepted for forward compatibility).
+ *   bs_tc_weights_bytes    bytes of the prepared filter tensor (0 on bad input).
+ *   bs_tc_prepare_weights  packed weights [O][R][S][Cw][w_bits] -> tiles for layers of a_bits activation bits: nibbles
+ *                          [ceil(C/64)][ceil(O/128)*16][R*S][2][8][16 bytes] where a_bits and w_bits are at most 2 (the first half of the
+ *                          tensor or so), int8 [C/32][ceil(O/128)*16][R*S][2][8][16] otherwise.  Use them with layers of the same widths.
  */
 size_t bs_tc_weights_bytes(int O, int C, int R, int S);
 int bs_tc_prepare_weights(const uint32_t* wgt_packed, int O, int C, int R, int S, int w_bits, bs_sign_t w_sign,

@@ -65,6 +65,8 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows, int sms)
     g.d_strips = make_div(c.ns);
     g.TN = c.TN; g.PT = c.PT; g.units = c.units;
     g.nunits = (g.Cw + 1) / 2;
+    g.nblk = g.f4 ? g.nunits : g.Cw;
+    const int bpu = g.f4 ? 1 : 2;                          // K steps of a unit
     g.nchunks = ceil_div(g.nunits, c.units);
     g.tiles_m = static_cast<int>(ceil_div_ll(total, BM));
     g.tiles_o = ceil_div(g.O, c.TN);
@@ -91,15 +93,16 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows, int sms)
     auto swizzle = [](int row) { return row == 32 ? 1 : row == 64 ? 3 : row == 128 ? 7 : 0; };
     g.swzA = swizzle(g.rowA);
     g.swzB = swizzle(g.rowB);
-    g.e_bytes = up(4 * c.units * g.NI * 16, 128);
-    g.b_bytes = c.units * 2 * c.TN * g.RS * 32;
-    g.stg_bytes = g.tma ? up(BM * g.rowA, 1024) : g.nslots * GT * 8 * A;
+    g.one_word = g.f4 && g.Cw == 1 && !g.tma;
+    g.e_bytes = up((g.one_word ? 1 : 2 * bpu) * c.units * g.NI * 16, 128);
+    g.b_bytes = c.units * bpu * c.TN * g.RS * 32;
+    g.stg_bytes = g.tma ? up(BM * g.rowA, 1024) : g.nslots * GT * (g.one_word ? 4 : 8) * A;
     g.bstg_bytes = !fb ? 0 : g.tma ? up(c.TN * g.rowB, 1024) : g.bslots * GT * 8 * WB;
     const int rel_bytes = g.flat ? 0 : up(g.NI * 4 * (1 + (c.units == 1 ? g.nsp + c.groups : 0)), 16);      // relative rows; located pixels of each group, one table more than stages
     const int pix_bytes = rel_bytes + (fb && !g.tma && c.units == 1 ? up(c.TN * g.RS * 4, 16) : 0);
     const int cap = c.cfg ? 222 * 1024 : 111 * 1024;
     const int fixed = c.TN * 8 + 64 + 320 + red_bytes + (g.tma ? 1024 : 0) + (int_rows ? EW * 4096 : 0) + 256 + pix_bytes;
-    const long long filters = c.resident ? static_cast<long long>(g.Cw) * c.TN * g.RS * 32 : 0;
+    const long long filters = c.resident ? static_cast<long long>(g.nblk) * c.TN * g.RS * 32 : 0;
     const long long rest = fixed + static_cast<long long>(g.nsp) * (g.stg_bytes + g.bstg_bytes) + filters;
     c.nsb = 0;
     long long used = 0;
@@ -127,13 +130,14 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows, int sms)
     if (nse < c.groups) return false;
     c.nse = nse;
     g.nse = nse; g.nsb = c.resident ? 0 : (packed_b ? nse : c.nsb);
-    const int cols = 512 / (c.cfg ? 1 : 2);
+    const int sf = g.f4 ? MM_SF_COLS : 0, cols = 512 / (c.cfg ? 1 : 2) - sf;
     if (2 * c.PT * c.TN <= cols) c.nacc = 2;
     else if (c.PT * c.TN <= cols) c.nacc = 1;
     else return false;
     g.nacc = c.nacc;
     int tc = 32;
-    while (tc < c.nacc * c.PT * c.TN) tc *= 2;
+    g.sf_col = c.nacc * c.PT * c.TN;
+    while (tc < g.sf_col + sf) tc *= 2;
     g.tmem_cols = tc;
     long long off = c.resident ? filters : static_cast<long long>(g.nsb) * g.b_bytes;
     g.off_e = static_cast<int>(off);                off += static_cast<long long>(nse) * g.e_bytes;
@@ -155,38 +159,51 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows, int sms)
 }
 
 // Time model of a candidate in SM cycles: the pipeline of one CTA (expansion, MMAs, epilogue; a stage's hand-off included) over
-// its items, plus what nothing overlaps at both ends.  The constants are fitted to about 2500 timed plans of 45 layers and
-// products (1 to 300 pixels wide, 32 to 4608 channels, batches 1 to 64; B200 at 1.95 GHz): over those the plan with the
-// lowest modelled time is on average 2 to 3 % and at most 16 % slower than the fastest plan.
+// its items, plus what nothing overlaps at both ends.  The constants are fitted to timed plans (B200 at 1.95 GHz): int8 to about 2500 of
+// 45 layers and products (1 to 300 pixels wide, 32 to 4608 channels, batches 1 to 64), the plan with the lowest modelled time being on
+// average 2 to 3 % and at most 16 % slower than the fastest; nibbles to 8300 of 49, on average 1.4 % and at most 19 % slower (with the
+// constants of int8: 4.5 % and 91 %, most of it from filters staged piece by piece, which cost twice what was assumed).
+struct MmaFit {
+    double mma_chunk;                       // cycles per chunk beside its MMAs
+    double unit, one_word, flat, staged;    // expansion, instructions per warp and 64-channel unit of 32 rows: arithmetic, of 32 channels only, copies by TMA, by thread
+    double filt_flat, filt_staged;          // packed filters streamed, instructions per 32 rows and unit
+    double x_cpi, x_chunk, x_group, x_once; // cycles per such instruction, per chunk; share by which a further group overlaps; once
+    double e_res, e_codes, e_i32, e_cpi, e_once;        // epilogue, instructions per block of 32 x 32 outputs; cycles per instruction; per item
+    double l2;                              // bytes per cycle of streamed prepared filters
+    double ipc, two_first, start, filt_resident, streamed, one_stage, half;
+};
+constexpr MmaFit FIT_INT8 = {148, 102, 102, 1, 41, 20, 20, 5.34, 629, 0.83, 628, 215, 138, 94, 4.59, 997, 68.7, 3.08, 1.19, 4215, 122, 1.07, 1.11, 0.93};
+constexpr MmaFit FIT_NIBBLES = {280, 64.5, 41.6, 1, 80, 52, 129, 5.64, 513, 0.79, 693, 265, 120, 94, 4.2, 960, 68.3, 1.45, 1.21, 3208, 211, 1.05, 0.98, 0.905};
+
 double mma_cost(const MmaArgs& g, const Cand& c, int A, int WB, bool packed_out, int sms)
 {
+    const MmaFit& k = g.f4 ? FIT_NIBBLES : FIT_INT8;
     const bool packed_b = WB > 0;
-    const double mma = c.TN == 32 ? 42 : c.TN == 64 ? 49 : c.TN == 128 ? 65 : 129;      // cycles per MMA of 128 x TN x 32
+    const double mma = c.TN == 32 ? 42 : c.TN == 64 ? 49 : c.TN == 128 ? 65 : 129;      // cycles per MMA of 128 x TN x (32 int8 or 64 nibbles)
     const int W = c.cfg ? 8 : 4;                                   // expander warps, epilogue warps
     const int nchunks = ceil_div(g.nchunks, c.split);              // of one CTA
     const double share = static_cast<double>(nchunks) / g.nchunks;
-    const double t_m = share * c.PT * g.RS * g.Cw * mma + 148.0 * nchunks;
-    // expansion: instructions per warp and 64-channel unit of 32 rows, at 5.3 cycles each; a chunk's hand-off
+    const double t_m = share * c.PT * g.RS * g.nblk * mma + k.mma_chunk * nchunks;
     const int row_groups = ceil_div(g.NI, 32);
-    double xi = share * row_groups * g.nunits * ((A <= 2 ? 102.0 : 111.0) + (g.tma ? 1.0 : 41.0));
-    if (!c.resident && packed_b) xi += share * c.TN * g.RS / 32.0 * g.nunits * (WB <= 2 ? 20.0 : 69.0);
+    double xi = share * row_groups * g.nunits * ((g.one_word ? k.one_word : A <= 2 ? k.unit : k.unit + 9.0) + (g.tma ? k.flat : k.staged));
+    if (!c.resident && packed_b) xi += share * c.TN * g.RS / 32.0 * g.nunits * (WB <= 2 ? (g.tma ? k.filt_flat : k.filt_staged) : 69.0);
     const double units_of_work = static_cast<double>(row_groups) * c.units * c.groups / W;       // per warp of a group and chunk
-    const double chunk = xi / nchunks * c.groups / W * (ceil(units_of_work) / units_of_work) * 5.34 + 629.0;
-    const double t_x = chunk * nchunks / (1.0 + (c.groups - 1) * 0.83) + 628.0;
-    // epilogue: instructions per block of 32 x 32 outputs, at 4.6 cycles; int32 rows leave at about 30 bytes per clock and SM
-    const double block = packed_out ? (g.has_residual ? 215.0 : 138.0) : 94.0;
-    double t_e = ceil_div(c.PT * (c.TN / 32), W / 4) * block * 4.59 + 997.0;
+    const double chunk = xi / nchunks * c.groups / W * (ceil(units_of_work) / units_of_work) * k.x_cpi + k.x_chunk;
+    const double t_x = chunk * nchunks / (1.0 + (c.groups - 1) * k.x_group) + k.x_once;
+    // int32 rows leave at about 30 bytes per clock and SM
+    const double block = packed_out ? (g.has_residual ? k.e_res : k.e_codes) : k.e_i32;
+    double t_e = ceil_div(c.PT * (c.TN / 32), W / 4) * block * k.e_cpi + k.e_once;
     if (!packed_out && c.PT * 128.0 * c.TN * 4 / 29.6 > t_e) t_e = c.PT * 128.0 * c.TN * 4 / 29.6;
     // sums through shared memory of the cluster
     if (c.split > 1) t_e += 2200.0 + ceil_div(c.PT * (c.TN / 32), W / 4) * 200.0 * (c.split - 1);
-    const double t_b = (!c.resident && !packed_b) ? share * c.TN * g.RS * g.Cw * 32 / 68.7 : 0.0;       // L2 -> shared memory
+    const double t_b = (!c.resident && !packed_b) ? share * c.TN * g.RS * g.nblk * 32 / k.l2 : 0.0;       // L2 -> shared memory
     const long long items = static_cast<long long>(g.tiles_m) * g.tiles_o * c.split;
     long long ctas = static_cast<long long>(sms) * c.cps;
     if (c.resident) ctas = ctas / g.tiles_o * g.tiles_o;
     if (ctas < 1) return 1e18;
     if (ctas > items) ctas = items;
     const double per_cta = static_cast<double>(ceil_div_ll(items, ctas)), active = static_cast<double>(ceil_div_ll(ctas, sms));
-    const double issue = (xi + c.PT * 4.0 * (c.TN / 32) * block) / 3.08;
+    const double issue = (xi + c.PT * 4.0 * (c.TN / 32) * block) / k.ipc;
     const double t_mb = t_m > t_b ? t_m : t_b;
     double step = c.nacc == 2 ? (t_mb > t_e ? t_mb : t_e) : t_mb + t_e;
     if (t_x > step) step = t_x;
@@ -194,12 +211,12 @@ double mma_cost(const MmaArgs& g, const Cand& c, int A, int WB, bool packed_out,
     if (active * issue > step) step = active * issue;
     const double rest_x = t_x > chunk ? t_x - chunk : 0.0;
     double first = chunk + (t_mb > rest_x ? t_mb : rest_x) + t_e;
-    if (active > 1.0) first *= 1.19;
-    double t = 4215.0 + first + (per_cta - 1.0) * step;
-    if (c.resident && packed_b) t += c.TN * g.RS * g.Cw / 32.0 * 122.0 / (2 * W) * 4.0;
-    if (!c.resident && !packed_b) t *= 1.07;
-    if (c.nse < 2) t *= 1.11;
-    if (!c.cfg) t *= 0.93;
+    if (active > 1.0) first *= k.two_first;
+    double t = k.start + first + (per_cta - 1.0) * step;
+    if (c.resident && packed_b) t += c.TN * g.RS * (g.f4 ? 2 * g.nblk : g.Cw) / 32.0 * k.filt_resident / (2 * W) * 4.0;
+    if (!c.resident && !packed_b) t *= k.streamed;
+    if (c.nse < 2) t *= k.one_stage;
+    if (!c.cfg) t *= k.half;
     return t;
 }
 
@@ -239,6 +256,7 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
     g.res_cw_total = ceil_div(p->res_c_total > 0 ? p->res_c_total : 1, 32);
     g.i32_nhwc = p->i32_layout == BS_NHWC;
     g.opad = up(p->O, 128);
+    g.f4 = mma_nibbles(p->C, g.RS, p->a_bits, p->w_bits);
     const double bound = static_cast<double>(p->C) * g.RS * max_abs_of(p->a_bits, p->a_sign) * max_abs_of(p->w_bits, p->w_sign);
     g.acc_bound = static_cast<float>(bound);
     g.preset = out_packed && !out_i32 && bound < 4.0e6 && p->out_sign != BS_BIPOLAR &&
@@ -315,7 +333,8 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
     if (flags & MM_QUERY) return BS_OK;
     g.status = status_device_ptr();
     if (!g.status) return BS_ERR_CUDA;
-    g.idesc = (2u << 4) | (1u << 7) | (1u << 10) | (static_cast<unsigned>(g.TN >> 3) << 17) | (static_cast<unsigned>(128 >> 4) << 24);
+    // int32 += int8 x int8, or float += e2m1 x e2m1 with ue8m0 scale factors; TN columns, 128 rows
+    g.idesc = (g.f4 ? (1u << 7) | (1u << 10) | (1u << 23) : (2u << 4) | (1u << 7) | (1u << 10)) | (static_cast<unsigned>(g.TN >> 3) << 17) | (static_cast<unsigned>(128 >> 4) << 24);
     const int cps = best.cps;
     const long long items = static_cast<long long>(g.tiles_m) * g.tiles_o;
     long long grid = static_cast<long long>(sms) * cps;
@@ -324,7 +343,7 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
     else if (grid > items) grid = items;
     const int wb = packed_b ? p->w_bits : 0;
     const bool half = !best.cfg, split = best.split > 1;
-    plan.kern = A == 1 ? mma_kernel_a1(wb, half, split) : A == 2 ? mma_kernel_a2(wb, half, split) : A == 3 ? mma_kernel_a3(wb, half, split) : mma_kernel_a4(wb, half, split);
+    plan.kern = g.f4 ? (A == 1 ? mma_kernel_f1(wb, half, split) : mma_kernel_f2(wb, half, split)) : A == 1 ? mma_kernel_a1(wb, half, split) : A == 2 ? mma_kernel_a2(wb, half, split) : A == 3 ? mma_kernel_a3(wb, half, split) : mma_kernel_a4(wb, half, split);
     plan.grid = static_cast<unsigned>(grid);
     plan.block = best.cfg ? MmaShape<false>::THREADS : MmaShape<true>::THREADS;
     plan.smem = static_cast<int>(best.smem);

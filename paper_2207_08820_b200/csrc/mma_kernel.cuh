@@ -15,6 +15,11 @@
 // 421 tiles (512 with rectangular ones).  Wide images are cut into strips so that the halo of a tile stays short.
 // Stride 2 keeps one such plane per parity of row and column.
 //
+// Codes of one and two bits on both sides run as tcgen05.mma kind::mxf4 (F4): two-bit codes are the small e2m1 floats 0, 0.5, 1, 1.5 with a
+// sign, so a nibble holds the code (sign and magnitude), scale factors of 2 in both operands make the products whole numbers, and
+// the sums stay exact in binary32 (below 2^22 by the plan; whole numbers up to 30188 and beyond compared).  A K = 64 step takes as long
+// and reads as many bytes as a K = 32 step of kind::i8, so operands, filter traffic and MMA time are all half as large.
+//
 // Every wait on an mbarrier is bounded; a wait that runs out sets the device status word and the CTA drains.
 #pragma once
 #include "conv_kernel.cuh"
@@ -81,7 +86,10 @@ struct MmaArgs {
     int e_bytes, b_bytes, stg_bytes, bstg_bytes;    // per stage
     int off_e, off_stg, off_bstg, off_pix, off_brow, off_tab, off_bar, off_out, off_red;
     int tmem_cols, nacc;
-    int preset;                     // accumulators start at the bit pattern of 1.5 * 2^23 (see the epilogue)
+    int f4;                         // kind::mxf4: operands of nibbles, float accumulators
+    int nblk, sf_col;               // K steps of all channels per tap; column of the scale factors
+    int one_word;                   // a unit has one channel word (32 channels in all): the second half of a K step meets zero filters
+    int preset;                     // the fast requantisation applies; integer accumulators then start at the bit pattern of 1.5 * 2^23 (see the epilogue)
     int epi;                        // which instantiation of the fast requantisation: odd ones read a residual and its multipliers
     int early_b;                    // filters may be read before the preceding kernel has finished
     int opad;
@@ -166,6 +174,15 @@ __device__ __forceinline__ void mm_mma(uint32_t d, uint32_t a_lo, uint32_t a_hi,
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(d), "l"((static_cast<uint64_t>(a_hi) << 32) | a_lo), "l"((static_cast<uint64_t>(b_hi) << 32) | b_lo), "r"(idesc), "r"(acc) : "memory");
+}
+__device__ __forceinline__ void mm_mma4(uint32_t d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, uint32_t idesc, uint32_t acc, uint32_t sf)
+{
+    if (mm_elect())
+        asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], %1, %2, %3, [%5], [%5], p;\n\t}"
+        ::"r"(d), "l"((static_cast<uint64_t>(a_hi) << 32) | a_lo), "l"((static_cast<uint64_t>(b_hi) << 32) | b_lo), "r"(idesc), "r"(acc), "r"(sf) : "memory");
 }
 __device__ __forceinline__ void mm_ld32(uint32_t taddr, uint32_t (&v)[32])
 {
@@ -306,10 +323,46 @@ __device__ __forceinline__ void expand_word(const uint32_t* p, int kind, uint32_
     }
 }
 
-// Two channel words (one 64-channel unit) of a staged row -> four 16-byte rows of the operand, `g16` bytes apart.
+// 32 codes of one or two planes -> 32 nibbles, nibble j of word m = channel 4 j + m, sign and magnitude (magnitude in halves).  NB = 2: 10
+// operations, and half the bytes.
 template <int NB>
-__device__ __forceinline__ void expand_unit(const uint32_t (&w)[2 * NB], int kind, uint32_t dst, uint32_t g16)
+__device__ __forceinline__ void expand_nibbles(const uint32_t* p, int kind, uint32_t (&o)[4])
 {
+    if (NB == 1) {
+#pragma unroll
+        for (int m = 0; m < 4; ++m) o[m] = (p[0] >> m) & 0x11111111u;
+        if (kind == 1) {            // the only plane weighs -1
+#pragma unroll
+            for (int m = 0; m < 4; ++m) o[m] *= 9u;
+        } else if (kind == 2) {
+#pragma unroll
+            for (int m = 0; m < 4; ++m) o[m] = 0x99999999u ^ (o[m] << 3);
+        }
+    } else {
+        const uint32_t p1 = p[NB > 1 ? 1 : 0];
+        const uint32_t e = (p[0] & 0x55555555u) | ((p1 << 1) & 0xAAAAAAAAu), d = ((p[0] >> 1) & 0x55555555u) | (p1 & 0xAAAAAAAAu);
+        o[0] = e & 0x33333333u; o[1] = d & 0x33333333u; o[2] = (e >> 2) & 0x33333333u; o[3] = (d >> 2) & 0x33333333u;
+        if (kind == 1) {            // 2 -> -2, 3 -> -1
+#pragma unroll
+            for (int m = 0; m < 4; ++m) o[m] = ((o[m] << 2) & 0x88888888u) | (o[m] & 0x11111111u) | (o[m] & ~(o[m] << 1) & 0x22222222u);
+        }
+    }
+}
+
+// Two channel words (one 64-channel unit) of a staged row -> four 16-byte rows of the operand (two of nibbles), `g16` bytes apart.  one: the
+// second word does not exist.
+template <int NB, bool F4>
+__device__ __forceinline__ void expand_unit(const uint32_t (&w)[2 * NB], int kind, uint32_t dst, uint32_t g16, bool one)
+{
+    if constexpr (F4) {
+        uint32_t n[4];
+        expand_nibbles<NB>(w, kind, n);
+        mm_sts(dst, n[0], n[1], n[2], n[3]);
+        if (one) return;
+        expand_nibbles<NB>(w + NB, kind, n);
+        mm_sts(dst + g16, n[0], n[1], n[2], n[3]);
+        return;
+    }
     uint32_t o[8];
     expand_word<NB>(w, kind, o);
     mm_sts(dst, o[0], o[1], o[2], o[3]);
@@ -321,19 +374,22 @@ __device__ __forceinline__ void expand_unit(const uint32_t (&w)[2 * NB], int kin
 
 // Staged pieces of one unit: piece k of a thread's slot sits `step` bytes after piece k - 1.
 template <int NB>
-__device__ __forceinline__ void load_unit(uint32_t src, uint32_t step, int psz, uint32_t (&w)[2 * NB])
+__device__ __forceinline__ void load_unit(uint32_t src, uint32_t step, int psz, uint32_t (&w)[2 * NB], bool one = false)
 {
     if (psz == 16 && (2 * NB) % 4 == 0) {
 #pragma unroll
         for (int k = 0; k < 2 * NB / 4; ++k)
+            if (!one || k < NB / 4)
             asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w[(4 * k) % (2 * NB)]), "=r"(w[(4 * k + 1) % (2 * NB)]), "=r"(w[(4 * k + 2) % (2 * NB)]),
                          "=r"(w[(4 * k + 3) % (2 * NB)]) : "r"(src + k * step));
     } else if (psz == 8) {
 #pragma unroll
-        for (int k = 0; k < NB; ++k) asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(w[2 * k]), "=r"(w[2 * k + 1]) : "r"(src + k * step));
+        for (int k = 0; k < NB; ++k)
+            if (!one || 2 * k < NB) asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(w[2 * k]), "=r"(w[2 * k + 1]) : "r"(src + k * step));
     } else {
 #pragma unroll
-        for (int k = 0; k < 2 * NB; ++k) asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w[k]) : "r"(src + k * step));
+        for (int k = 0; k < 2 * NB; ++k)
+            if (!one || k < NB) asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w[k]) : "r"(src + k * step));
     }
 }
 
@@ -361,9 +417,14 @@ __device__ __forceinline__ void load_row_unit(uint32_t stage, int off, int mask,
 
 // cp.async of one unit (two channel words, NB planes each) of a packed row; `left` words of it exist, the rest is zero.
 template <int NB, int PSZ>
-__device__ __forceinline__ void stage_unit_p(uint32_t dst, uint32_t step, const uint32_t* src, const uint32_t* safe, int left)
+__device__ __forceinline__ void stage_unit_p(uint32_t dst, uint32_t step, const uint32_t* src, const uint32_t* safe, int left, bool one)
 {
     constexpr int PW = PSZ / 4, NP = 2 * NB / PW > 0 ? 2 * NB / PW : 1;
+    if (one) {                                  // one channel word: all of it, or none
+#pragma unroll
+        for (int k = 0; k < (NP + 1) / 2; ++k) mm_cp<PSZ>(dst + k * step, src + k * PW, left > 0 ? PSZ : 0);
+        return;
+    }
     if (left >= 2 * NB || left <= 0) {          // all of it, or none
         const int bytes = left > 0 ? PSZ : 0;
 #pragma unroll
@@ -377,11 +438,11 @@ __device__ __forceinline__ void stage_unit_p(uint32_t dst, uint32_t step, const 
     }
 }
 template <int NB>
-__device__ __forceinline__ void stage_unit(int psz, uint32_t dst, uint32_t step, const uint32_t* src, const uint32_t* safe, int left)
+__device__ __forceinline__ void stage_unit(int psz, uint32_t dst, uint32_t step, const uint32_t* src, const uint32_t* safe, int left, bool one = false)
 {
-    if (psz == 16) stage_unit_p<NB, 16>(dst, step, src, safe, left);
-    else if (psz == 8) stage_unit_p<NB, 8>(dst, step, src, safe, left);
-    else stage_unit_p<NB, 4>(dst, step, src, safe, left);
+    if (psz == 16) stage_unit_p<NB, 16>(dst, step, src, safe, left, one);
+    else if (psz == 8) stage_unit_p<NB, 8>(dst, step, src, safe, left, one);
+    else stage_unit_p<NB, 4>(dst, step, src, safe, left, one);
 }
 
 // ----------------------------------------------------------------------------- filters expanded in the kernel
@@ -397,10 +458,17 @@ __device__ __forceinline__ int filter_row(const MmaArgs& g, int i, int WB, int& 
     return f;
 }
 
-// One channel word of a filter row -> its two 16-byte core-matrix rows; rows past the last filter are zero.
-template <int WB>
+// One channel word of a filter row -> its two 16-byte core-matrix rows (one of nibbles); rows past the last filter are zero.
+template <int WB, bool F4>
 __device__ __forceinline__ void expand_filter_word(const uint32_t* w, int kind, bool live, uint32_t dst)
 {
+    if constexpr (F4) {
+        uint32_t n[4];
+        expand_nibbles<WB>(w, kind, n);
+        const uint32_t keep = live ? 0xffffffffu : 0u;
+        mm_sts(dst, n[0] & keep, n[1] & keep, n[2] & keep, n[3] & keep);
+        return;
+    }
     uint32_t o[8];
     expand_word<WB>(w, kind, o);
     if (kind == 2 && !live) {            // a bipolar row must not turn missing bits into -1
@@ -411,12 +479,13 @@ __device__ __forceinline__ void expand_filter_word(const uint32_t* w, int kind, 
     mm_sts(dst + 128u, o[4], o[5], o[6], o[7]);
 }
 
-// `base`: packed records of the tile's filters, in shared memory (bulk copy) or global.
-template <int WB>
+// `base`: packed records of the tile's filters, in shared memory (bulk copy) or global.  Nibbles: a K step is two channel words, the second
+// of an odd number zero.
+template <int WB, bool F4>
 __device__ __forceinline__ void expand_filters_resident(const MmaArgs& g, uint32_t b_base, const uint32_t* base, int o0, int t, int nt)
 {
     constexpr int BATCH = 4;                // loads in flight per thread
-    const int rows = g.TN * g.RS, total = rows * g.Cw;
+    const int rows = g.TN * g.RS, total = rows * (F4 ? 2 * g.nblk : g.Cw);
     const uint32_t blk = static_cast<uint32_t>(rows) * 32u;
     int i = t, cw = 0;
     while (i >= rows) { i -= rows; ++cw; }
@@ -427,7 +496,7 @@ __device__ __forceinline__ void expand_filters_resident(const MmaArgs& g, uint32
         for (int b = 0; b < BATCH; ++b) {
             int off = 0;
             live[b] = cw < g.Cw && o0 + filter_row(g, i, WB, off) < g.O;
-            dst[b] = b_base + cw * blk + static_cast<uint32_t>(i >> 3) * 256u + static_cast<uint32_t>(i & 7) * 16u;
+            dst[b] = b_base + (F4 ? (cw >> 1) * blk + (cw & 1) * 128u : cw * blk) + static_cast<uint32_t>(i >> 3) * 256u + static_cast<uint32_t>(i & 7) * 16u;
 #pragma unroll
             for (int k = 0; k < WB; ++k) w[b][k] = live[b] ? base[off + cw * WB + k] : 0u;
             i += nt;
@@ -435,7 +504,7 @@ __device__ __forceinline__ void expand_filters_resident(const MmaArgs& g, uint32
         }
 #pragma unroll
         for (int b = 0; b < BATCH; ++b)
-            if (j0 + b * nt < total) expand_filter_word<WB>(w[b], g.w_kind, live[b], dst[b]);
+            if (j0 + b * nt < total) expand_filter_word<WB, F4>(w[b], g.w_kind, live[b], dst[b]);
     }
 }
 
@@ -443,9 +512,16 @@ __device__ __forceinline__ void expand_filters_resident(const MmaArgs& g, uint32
 
 // Fixed kernel sizes: the taps are unrolled, nothing but additions on uniform registers between the MMAs.
 // a, b: descriptor words of the block's operands; PITCH and plane offsets in 16-byte units.
-template <int R, int ST>
+template <bool F4>
+__device__ __forceinline__ void issue_mma(uint32_t d, uint32_t a, uint32_t a_hi, uint32_t b, uint32_t b_hi, uint32_t idesc, uint32_t acc, uint32_t sf)
+{
+    if constexpr (F4) mm_mma4(d, a, a_hi, b, b_hi, idesc, acc, sf);
+    else mm_mma(d, a, a_hi, b, b_hi, idesc, acc);
+}
+
+template <int R, int ST, bool F4>
 __device__ __forceinline__ void issue_taps(uint32_t d, uint32_t a, uint32_t a_hi, uint32_t b, uint32_t b_hi, uint32_t idesc, uint32_t acc, uint32_t pitch,
-                                           uint32_t HL)
+                                           uint32_t HL, uint32_t sf)
 {
 #pragma unroll
     for (int r = 0; r < R; ++r)
@@ -454,19 +530,19 @@ __device__ __forceinline__ void issue_taps(uint32_t d, uint32_t a, uint32_t a_hi
             // 3x3, pad 1, stride 2: taps -1, 0, 1 -> parity 1, 0, 1, shift -1, 0, 0
             const uint32_t off = ST == 1 ? r * pitch + s
                                          : ((r != 1 ? 2u : 0u) + (s != 1 ? 1u : 0u)) * HL + (r > 0 ? pitch : 0u) + (s > 0 ? 1u : 0u);
-            mm_mma(d, a + off, a_hi, b + static_cast<uint32_t>(r * R + s) * 16u, b_hi, idesc, (r == 0 && s == 0) ? acc : 1u);
+            issue_mma<F4>(d, a + off, a_hi, b + static_cast<uint32_t>(r * R + s) * 16u, b_hi, idesc, (r == 0 && s == 0) ? acc : 1u, sf);
         }
 }
 
 enum { TAPS_1 = 0, TAPS_3S1, TAPS_3S2, TAPS_ANY };
 
-template <int TAPS>
+template <int TAPS, bool F4>
 __device__ __forceinline__ void issue_block(const MmaArgs& g, uint32_t d, uint32_t a, uint32_t a_hi, uint32_t b, uint32_t b_hi, uint32_t idesc, uint32_t acc,
-                                            uint32_t pitch, uint32_t HL)
+                                            uint32_t pitch, uint32_t HL, uint32_t sf)
 {
-    if (TAPS == TAPS_1) mm_mma(d, a, a_hi, b, b_hi, idesc, acc);
-    else if (TAPS == TAPS_3S1) issue_taps<3, 1>(d, a, a_hi, b, b_hi, idesc, acc, pitch, HL);
-    else if (TAPS == TAPS_3S2) issue_taps<3, 2>(d, a, a_hi, b, b_hi, idesc, acc, pitch, HL);
+    if (TAPS == TAPS_1) issue_mma<F4>(d, a, a_hi, b, b_hi, idesc, acc, sf);
+    else if (TAPS == TAPS_3S1) issue_taps<3, 1, F4>(d, a, a_hi, b, b_hi, idesc, acc, pitch, HL, sf);
+    else if (TAPS == TAPS_3S2) issue_taps<3, 2, F4>(d, a, a_hi, b, b_hi, idesc, acc, pitch, HL, sf);
     else
         for (int r = 0; r < g.R; ++r)
             for (int s = 0; s < g.R; ++s) {
@@ -474,7 +550,7 @@ __device__ __forceinline__ void issue_block(const MmaArgs& g, uint32_t d, uint32
                 uint32_t off;
                 if (g.stride == 1) off = static_cast<uint32_t>(r * g.pitch + s);
                 else off = static_cast<uint32_t>(((rp & 1) * 2 + (sp & 1)) * g.HL + ((rp >> 1) - g.rmin) * g.pitch + (sp >> 1) - g.smin);
-                mm_mma(d, a + off, a_hi, b, b_hi, idesc, acc);
+                issue_mma<F4>(d, a + off, a_hi, b, b_hi, idesc, acc, sf);
                 acc = 1u;
                 b += 16u;
             }
@@ -501,13 +577,14 @@ struct MmaIssue {
 
 // The MMA warp's walk over items and chunks, in uniform code; every MMA and every commit elects its thread by itself (one elected region
 // for a whole chunk was slower: its descriptors move through vector registers, 100 cycles per MMA against 85 to 90).
-template <int TAPS, bool SPLIT>
+template <int TAPS, bool SPLIT, bool F4>
 __device__ __forceinline__ void issue_items(const MmaArgs& g, const MmaIssue& m)
 {
     const uint32_t NI16 = static_cast<uint32_t>(g.NI);
     // K-major, no swizzle: core matrices of 8 rows x 16 bytes; leading offset = next 16 channels, stride offset = next 8 rows
     const uint32_t a_hi = (128u >> 4) | (1u << 14), b_hi = static_cast<uint32_t>(g.RS * 16) | (1u << 14);
-    const uint32_t a_lo0 = (NI16 & 0x3FFFu) << 16, b_lo0 = (128u >> 4) << 16;
+    // (32 channels as nibbles: the second half of the step reads the first again, against zeros)
+    const uint32_t a_lo0 = F4 && g.one_word ? 0u : (NI16 & 0x3FFFu) << 16, b_lo0 = (128u >> 4) << 16;
     // descriptors take the offset within the CTA; in a cluster the upper bits of a shared address name the CTA
     const uint32_t smem_off = m.smem0 & 0x3FFFFu, e_base = (smem_off + g.off_e) >> 4, w_base = smem_off >> 4;
     const uint32_t blk16 = static_cast<uint32_t>(g.TN * g.RS * 2), idesc = g.idesc;
@@ -515,7 +592,8 @@ __device__ __forceinline__ void issue_items(const MmaArgs& g, const MmaIssue& m)
     const uint32_t e16 = static_cast<uint32_t>(g.e_bytes >> 4), b16 = static_cast<uint32_t>(g.b_bytes >> 4);
     const MmaChunks range(g, SPLIT);
     const int log = SPLIT ? g.split_log : 0;
-    const int nchunks = range.n, PT = g.PT, per_chunk = g.units * 2, Cw = g.Cw, nse = g.nse, nacc = g.nacc;
+    const int nchunks = range.n, PT = g.PT, per_chunk = F4 ? g.units : g.units * 2, blocks = g.nblk, nse = g.nse, nacc = g.nacc;
+    const uint32_t sf = m.tmem + static_cast<uint32_t>(g.sf_col);
     unsigned limit = 1u << 20;
     if (m.resident) mm_wait_uniform(m.wgt_full, 0, limit);
     MM_TRACE((threadIdx.x & 31) == 0, TR_WGT, 0);
@@ -524,13 +602,13 @@ __device__ __forceinline__ void issue_items(const MmaArgs& g, const MmaIssue& m)
 #endif
     int ie = 0, ia = 0;
     unsigned pe = 0, pa = 0;
-    const uint32_t acc0 = g.preset ? 1u : 0u;
+    const uint32_t acc0 = !F4 && g.preset ? 1u : 0u;
     for (int it = blockIdx.x >> log; it < m.items; it += gridDim.x >> log) {
         mm_wait_uniform(&m.empty_acc[ia], pa, limit);
         const uint32_t d0 = m.tmem + static_cast<uint32_t>(ia * PT) * TN;
         for (int c = 0; c < nchunks; ++c) {
             const int b0 = (range.beg + c) * per_chunk;
-            const int nb = Cw - b0 < per_chunk ? Cw - b0 : per_chunk;
+            const int nb = blocks - b0 < per_chunk ? blocks - b0 : per_chunk;
             const uint32_t wb = b_lo0 | (w_base + (m.resident ? static_cast<uint32_t>(b0) * blk16 : static_cast<uint32_t>(ie) * b16));
             const uint32_t eb = a_lo0 | (e_base + static_cast<uint32_t>(ie) * e16);
             mm_wait_uniform(&m.full_e[ie], pe, limit);
@@ -541,12 +619,12 @@ __device__ __forceinline__ void issue_items(const MmaArgs& g, const MmaIssue& m)
                 uint32_t d = d0, at = eb;
                 for (int t = 0; t < PT; ++t, d += TN, at += 128u) {
                     uint32_t a = at, b = wb;
-                    issue_block<TAPS>(g, d, a, a_hi, b, b_hi, idesc, acc, pitch, HL);
+                    issue_block<TAPS, F4>(g, d, a, a_hi, b, b_hi, idesc, acc, pitch, HL, sf);
 #pragma unroll(TAPS == TAPS_1 ? 4 : 1)
                     for (int k = 1; k < nb; ++k) {
                         a += 2u * NI16;
                         b += blk16;
-                        issue_block<TAPS>(g, d, a, a_hi, b, b_hi, idesc, 1u, pitch, HL);
+                        issue_block<TAPS, F4>(g, d, a, a_hi, b, b_hi, idesc, 1u, pitch, HL, sf);
                     }
                 }
                 mm_commit(&m.empty_e[ie]);
@@ -566,10 +644,11 @@ __device__ __forceinline__ void issue_items(const MmaArgs& g, const MmaIssue& m)
 
 // ----------------------------------------------------------------------------- epilogue
 
+constexpr int MM_SF_COLS = 32;                  // columns that hold scale factors (eight bytes a row and column of the operands need at most 16)
 constexpr uint32_t MM_PRESET = 0x4B400000u;      // 1.5 * 2^23: an accumulator that starts here IS the float 12582912 + acc
 
 // Fast requantisation of 16 accumulators of one pixel = half a group of 32 filters (codes of 1..4 bits, residual codes unsigned).
-//   acc -> float: the accumulators start at the bit pattern of 1.5 * 2^23, so one subtraction converts (|acc| < 2^22).
+//   acc -> float: integer accumulators start at the bit pattern of 1.5 * 2^23, so one subtraction converts (|acc| < 2^22); those of F4 are floats.
 //   t = fmaf(acc, scale, bias) and fmaf(res_scale, res, t) in the formula's order, two outputs per instruction (f32x2), all
 //   scaled by 2^-24: an exact change of the exponents (the caller's table check keeps every value in the normal range).
 //   rint: adding 0.75 (one ulp = 2^-24) leaves the rounded level in the low mantissa bits; two outputs are clamped as a pair
@@ -580,7 +659,7 @@ constexpr uint32_t MM_PRESET = 0x4B400000u;      // 1.5 * 2^23: an accumulator t
 // one word (4 i' and two words for wider codes), and a few operations per group de-interleave the words of both halves into
 // planes.  About 4 instructions per output, a quarter of them loads and integer ALU; the threshold-table form it replaces
 // took 8 (12 with a residual).
-template <int OBC, int RESC, bool LO0>
+template <int OBC, int RESC, bool LO0, bool F4>
 __device__ __forceinline__ void requant16(const uint32_t (&v)[16], uint32_t tab, uint32_t rtab, uint32_t z0, uint32_t z1, uint32_t lo2, uint32_t hi2,
                                           uint32_t (&W)[2])
 {
@@ -591,7 +670,8 @@ __device__ __forceinline__ void requant16(const uint32_t (&v)[16], uint32_t tab,
     for (int i = 0; i < 8; ++i) {
         u64 s2, b2;
         asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(s2), "=l"(b2) : "r"(tab + i * 16));
-        u64 t = f2_fma(f2_add(f2_pack(v[2 * i], v[2 * i + 1]), unbias), s2, b2);
+        const u64 acc = f2_pack(v[2 * i], v[2 * i + 1]);
+        u64 t = f2_fma(F4 ? acc : f2_add(acc, unbias), s2, b2);
         if (RESC) {
             u64 rmul;
             asm volatile("ld.shared.b64 %0, [%1];" : "=l"(rmul) : "r"(rtab + (RESC == 2 ? i : (i >> 1) * 2) * 8));
@@ -722,12 +802,18 @@ struct MmaEpi {
 
 // Split items.  CTAs of rank 1 and up send their accumulators to the shared memory of rank 0 ([rank - 1][column][row], so a warp
 // stores 128 contiguous bytes), which adds them to its own in tensor memory and goes on as if it had done all the chunks.
-template <int EW>
+// Whole number of an accumulator.
+__device__ __forceinline__ uint32_t acc_int(bool f4, uint32_t v, uint32_t bias)
+{
+    return f4 ? __float_as_uint(__uint_as_float(v) + 12582912.0f) - MM_PRESET : v - bias;
+}
+
+template <int EW, bool F4>
 __device__ __forceinline__ bool send_partials(const MmaArgs& g, const MmaEpi& e, int rank)
 {
     if (!mm_wait(&e.full_acc[0], 0)) return false;
     mm_fence_after();
-    const uint32_t bias = g.preset ? MM_PRESET : 0u;
+    const uint32_t bias = !F4 && g.preset ? MM_PRESET : 0u;
     const int columns = g.PT * g.TN;
     const uint32_t dst = mm_leader(smem_u32(e.smem + g.off_red)) + static_cast<uint32_t>(((rank - 1) * columns * 128 + e.row0) * 4);
     for (int c0 = e.set * 32; c0 < columns; c0 += EW / 4 * 32)
@@ -744,7 +830,7 @@ __device__ __forceinline__ bool send_partials(const MmaArgs& g, const MmaEpi& e,
     if (e.lane == 0) asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(mm_leader(smem_u32(e.red_full))) : "memory");
     return true;
 }
-template <int EW>
+template <int EW, bool F4>
 __device__ __forceinline__ bool merge_partials(const MmaArgs& g, const MmaEpi& e)
 {
     if (!mm_wait_cluster(e.red_full, 0)) return false;
@@ -761,7 +847,7 @@ __device__ __forceinline__ bool merge_partials(const MmaArgs& g, const MmaEpi& e
                 for (int c = 0; c < 16; ++c) {
                     uint32_t x;
                     asm volatile("ld.shared.b32 %0, [%1];" : "=r"(x) : "r"(src + static_cast<uint32_t>((r * columns + c0 + h + c) * 512)));
-                    v[c] += x;
+                    v[c] = F4 ? __float_as_uint(__uint_as_float(v[c]) + __uint_as_float(x)) : v[c] + x;
                 }
             mm_st16(e.acc + static_cast<uint32_t>(c0 + h), v);
         }
@@ -807,7 +893,7 @@ static __device__ __noinline__ void epilogue_formula(const MmaArgs& g, uint32_t 
     mm_ld32(addr, v);
     mm_ld_wait();
     if (live) {
-        for (int c = 0; c < 32; ++c) v[c] -= bias;
+        for (int c = 0; c < 32; ++c) v[c] = acc_int(g.f4, v[c], bias);
         if (g.residual) load_residual(g, pix, ob, rw);
         requant32_formula(g, v, ob, rw, ow);
         store_codes(g, pix, ob, ow);
@@ -823,13 +909,14 @@ static __device__ __noinline__ void epilogue_item_formula(const MmaArgs& g, uint
         const MmaPixel px = mma_pixel(g, base + t * 128);
         const uint32_t col = acc + static_cast<uint32_t>(t * g.TN + cc * 32);
         epilogue_formula(g, col, px.valid && o0 + cc * 32 < g.O, px.pix, o0 + cc * 32, MM_PRESET);
-        for (int c = 0; c < 32; c += 8) mm_st8(col + c, MM_PRESET);
+        if (!g.f4)
+            for (int c = 0; c < 32; c += 8) mm_st8(col + c, MM_PRESET);
     }
 }
 
 // Codes out, fast form.  One warp's accumulators arrive 16 columns at a time; the next 16 are on their way from tensor memory
 // while the current ones are computed, and the residual words of a group are fetched one group ahead.
-template <int OBC, int RESC, bool LO0, int EW, bool SPLIT>
+template <int OBC, int RESC, bool LO0, int EW, bool SPLIT, bool F4>
 __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e)
 {
     constexpr int STEP = EW / 4;
@@ -861,7 +948,7 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
         if (RESC && t < g.PT && px.valid && o0 + cc * 32 < g.O) load_residual(g, px.pix, o0 + cc * 32, rn);
         if (ok) ok = mm_wait(&e.full_acc[ia], pa);    // after a wait that ran out the walk goes on without waiting, so the named barriers stay matched
         mm_fence_after();
-        if (SPLIT && ok) ok = merge_partials<EW>(g, e);
+        if (SPLIT && ok) ok = merge_partials<EW, F4>(g, e);
         MM_TRACE(e.tid == 0, TR_EBEG, (w.it - static_cast<int>(blockIdx.x)) / static_cast<int>(gridDim.x));
         const uint32_t acc = e.acc + static_cast<uint32_t>(ia * g.PT * g.TN);
         if (!fast) {
@@ -881,8 +968,7 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
             mm_ld_wait();
             mm_landed(A);
             mm_ld16(col + 16, B);
-            mm_st8(col, MM_PRESET);
-            mm_st8(col + 8, MM_PRESET);
+            if (!F4) { mm_st8(col, MM_PRESET); mm_st8(col + 8, MM_PRESET); }
             // the next group's place and residual
             cc += STEP;
             const int t_old = t;
@@ -901,13 +987,12 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
                 z[2] = ((p >> 2) & 0x33333333u) | (r & 0xCCCCCCCCu);          // 2, 6, .. (half 0, odd pairs)
                 z[3] = ((q >> 2) & 0x33333333u) | (s & 0xCCCCCCCCu);
             }
-            requant16<OBC, RESC, LO0>(A, tab, rtab, z[0], z[2], lo2, hi2, Wa);
+            requant16<OBC, RESC, LO0, F4>(A, tab, rtab, z[0], z[2], lo2, hi2, Wa);
             mm_ld_wait();
             mm_landed(B);
             if (t < g.PT) mm_ld16(acc + static_cast<uint32_t>(t * g.TN + cc * 32), A);
-            mm_st8(col + 16, MM_PRESET);
-            mm_st8(col + 24, MM_PRESET);
-            requant16<OBC, RESC, LO0>(B, tab + 128u, rtab, z[1], z[3], lo2, hi2, Wb);
+            if (!F4) { mm_st8(col + 16, MM_PRESET); mm_st8(col + 24, MM_PRESET); }
+            requant16<OBC, RESC, LO0, F4>(B, tab + 128u, rtab, z[1], z[3], lo2, hi2, Wb);
             uint32_t ow[4] = {0, 0, 0, 0};
             if (OBC == 2) {
                 ow[0] = (Wa[0] & 0x55555555u) | ((Wb[0] << 1) & 0xAAAAAAAAu);
@@ -920,7 +1005,7 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
             }
             if (live) store_codes(g, pix, ob, ow);
         }
-        mm_st_wait();
+        if (!F4) mm_st_wait();
         mm_fence_before();
         __syncwarp();
         if (e.lane == 0) mm_arrive(&e.empty_acc[ia]);
@@ -932,7 +1017,7 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
 }
 
 // int32 accumulators out (and codes through the formula where both are asked for or the fast form does not apply).
-template <int EW, bool SPLIT>
+template <int EW, bool SPLIT, bool F4>
 __device__ __forceinline__ bool epilogue_general(const MmaArgs& g, const MmaEpi& e)
 {
     const int groups = g.TN >> 5;
@@ -944,7 +1029,7 @@ __device__ __forceinline__ bool epilogue_general(const MmaArgs& g, const MmaEpi&
         const int o0 = w.o * g.TN, base = w.m * 128 * g.PT + e.row0;
         if (ok) ok = mm_wait(&e.full_acc[ia], pa);
         mm_fence_after();
-        if (SPLIT && ok) ok = merge_partials<EW>(g, e);
+        if (SPLIT && ok) ok = merge_partials<EW, F4>(g, e);
         MM_TRACE(e.tid == 0, TR_EBEG, (w.it - static_cast<int>(blockIdx.x)) / static_cast<int>(gridDim.x));
         const uint32_t acc = e.acc + static_cast<uint32_t>(ia * g.PT * g.TN);
         int t = 0, cc = e.set;
@@ -958,6 +1043,9 @@ __device__ __forceinline__ bool epilogue_general(const MmaArgs& g, const MmaEpi&
                 uint32_t v[32];
                 mm_ld32(col, v);
                 mm_ld_wait();
+                if (F4)
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) v[c] = acc_int(true, v[c], 0u);
                 if (g.flat && g.i32_nhwc && (g.O & 3) == 0 && g.O - ob >= 32) {
                     // the 32 x 32 block of the warp goes through 4 KB of shared memory so that a store writes whole lines
                     uint4* sw = reinterpret_cast<uint4*>(e.smem + g.off_out + e.warp * 4096);
@@ -1007,8 +1095,8 @@ struct MmaShape {
     static constexpr int EW = HALF ? 4 : 8, XW = HALF ? 4 : 8, THREADS = (EW + XW + 2) * 32, CPS = HALF ? 2 : 1;
 };
 
-// SPLIT: an item belongs to a cluster of CTAs, each with a share of its chunks.
-template <int A, int WB, bool HALF, bool SPLIT>
+// SPLIT: an item belongs to a cluster of CTAs, each with a share of its chunks.  F4: nibbles (A and WB at most 2).
+template <int A, int WB, bool HALF, bool SPLIT, bool F4>
 __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) bitserial_mma_kernel(const __grid_constant__ MmaArgs g)
 {
     extern __shared__ __align__(1024) unsigned char mm_smem[];
@@ -1084,8 +1172,8 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                         mm_bulk(mm_smem + g.off_e, g.wgt_packed + static_cast<size_t>(o0) * g.RS * g.Cw * WBX, static_cast<unsigned>(words) * 4u, bulk_full);
                     } else {
                         const int8_t* src = g.wgt + static_cast<size_t>(o0) * g.RS * 32;
-                        mbar_expect_tx(wgt_full, blk_bytes * g.Cw);
-                        for (int b = 0; b < g.Cw; ++b) mm_bulk(mm_smem + static_cast<size_t>(b) * blk_bytes, src + b * blk_stride, blk_bytes, wgt_full);
+                        mbar_expect_tx(wgt_full, blk_bytes * g.nblk);
+                        for (int b = 0; b < g.nblk; ++b) mm_bulk(mm_smem + static_cast<size_t>(b) * blk_bytes, src + b * blk_stride, blk_bytes, wgt_full);
                     }
                 }
             }
@@ -1099,8 +1187,8 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                         if (stream) {
                             ok = mm_wait(&empty_e[ib], pb ^ 1u);
                             if (!ok) break;
-                            const int b0 = c * g.units * 2;
-                            const int nb = g.Cw - b0 < g.units * 2 ? g.Cw - b0 : g.units * 2;
+                            const int step = F4 ? g.units : g.units * 2, b0 = c * step;
+                            const int nb = g.nblk - b0 < step ? g.nblk - b0 : step;
                             mbar_expect_tx(&full_e[ib], blk_bytes * nb);
                             for (int b = 0; b < nb; ++b)
                                 mm_bulk(mm_smem + static_cast<size_t>(ib) * g.b_bytes + static_cast<size_t>(b) * blk_bytes, src + (b0 + b) * blk_stride, blk_bytes, &full_e[ib]);
@@ -1127,10 +1215,10 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
     } else if (warp == WARP_MMA) {
         // ------------------------------------------------------------------ MMA issuer (all lanes in step)
         const MmaIssue m{full_e, empty_e, full_acc, empty_acc, wgt_full, smem0, tmem, items, resident};
-        if (g.R == 1) issue_items<TAPS_1, SPLIT>(g, m);
-        else if (g.R == 3 && g.stride == 1) issue_items<TAPS_3S1, SPLIT>(g, m);
-        else if (g.R == 3 && g.pad == 1) issue_items<TAPS_3S2, SPLIT>(g, m);
-        else issue_items<TAPS_ANY, SPLIT>(g, m);
+        if (g.R == 1) issue_items<TAPS_1, SPLIT, F4>(g, m);
+        else if (g.R == 3 && g.stride == 1) issue_items<TAPS_3S1, SPLIT, F4>(g, m);
+        else if (g.R == 3 && g.pad == 1) issue_items<TAPS_3S2, SPLIT, F4>(g, m);
+        else issue_items<TAPS_ANY, SPLIT, F4>(g, m);
     } else if (warp >= EW && warp < WARP_COPY) {
         // ------------------------------------------------------------------ expanders
         const int xt = tid - NET;
@@ -1142,7 +1230,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                 if (!mm_wait(bulk_full, 0)) atomicOr(g.status, STATUS_TIMEOUT);
                 src = reinterpret_cast<const uint32_t*>(mm_smem + g.off_e);
             }
-            expand_filters_resident<WBX>(g, smem0, src, o0, tid, NXT + NET);
+            expand_filters_resident<WBX, F4>(g, smem0, src, o0, tid, NXT + NET);
             fence_proxy_async();
             // the parked tile has been read: the ring may be filled once every warp is here
             asm volatile("bar.sync 4, %0;" ::"n"(NXT + NET) : "memory");
@@ -1184,7 +1272,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                         const int u = it >> shA, i = it & (rowsA - 1);
                         uint32_t wd[2 * A];
                         load_row_unit<A>(src, i * g.rowA + u * 8 * A, g.swzA, wd);
-                        expand_unit<A>(wd, g.a_kind, e0 + static_cast<uint32_t>(u) * 4u * g16 + static_cast<uint32_t>(i) * 16u, g16);
+                        expand_unit<A, F4>(wd, g.a_kind, e0 + static_cast<uint32_t>(u) * (F4 ? 2u : 4u) * g16 + static_cast<uint32_t>(i) * 16u, g16, false);
                     }
                     if (stream_b) {
                         const uint32_t bsrc = smem0 + g.off_bstg + static_cast<uint32_t>(ip * g.bstg_bytes);
@@ -1194,10 +1282,10 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                             const int f = (i & ~31) + mma_filter_of_column(i & 31);
                             uint32_t wd[2 * WBX];
                             load_row_unit<WBX>(bsrc, f * g.rowB + u * 8 * WBX, g.swzB, wd);
-                            const bool live = w.o * g.TN + f < g.O;
-                            const uint32_t d = bdst + static_cast<uint32_t>(2 * u) * blk + static_cast<uint32_t>(i >> 3) * 256u + static_cast<uint32_t>(i & 7) * 16u;
-                            expand_filter_word<WBX>(wd, g.w_kind, live, d);
-                            expand_filter_word<WBX>(wd + WBX, g.w_kind, live, d + blk);
+                            const bool live = w.o * g.TN + f < g.O, both = 2 * ((range.beg + c) * g.units + u) + 1 < g.Cw;
+                            const uint32_t d = bdst + static_cast<uint32_t>(F4 ? u : 2 * u) * blk + static_cast<uint32_t>(i >> 3) * 256u + static_cast<uint32_t>(i & 7) * 16u;
+                            expand_filter_word<WBX, F4>(wd, g.w_kind, live, d);
+                            expand_filter_word<WBX, F4>(wd + WBX, g.w_kind, live && both, d + (F4 ? 128u : blk));
                         }
                     }
                     fence_proxy_async();
@@ -1307,7 +1395,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                         int pixel;
                         if (g.flat) pixel = flat_pixel(iw.m, i);
                         else asm volatile("ld.shared.b32 %0, [%1];" : "=r"(pixel) : "r"(ipix + static_cast<uint32_t>(i) * 4u));
-                        stage_unit<A>(g.psz, dst, step, src + static_cast<size_t>(static_cast<unsigned>(pixel < 0 ? 0 : pixel)) * rec, g.act, pixel >= 0 ? left : 0);
+                        stage_unit<A>(g.psz, dst, step, src + static_cast<size_t>(static_cast<unsigned>(pixel < 0 ? 0 : pixel)) * rec, g.act, pixel >= 0 ? left : 0, F4 && g.one_word);
                     }
                 } else {
                     // items (unit, pixel), pixel fastest
@@ -1377,8 +1465,8 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                     uint32_t dst = e0 + static_cast<uint32_t>(xl) * 16u;
                     for (int i = xl; i < g.NI; i += nx, src += nx * g.psz, dst += nx * 16) {
                         uint32_t wd[2 * A];
-                        load_unit<A>(src, step, g.psz, wd);
-                        expand_unit<A>(wd, g.a_kind, dst, g16);
+                        load_unit<A>(src, step, g.psz, wd, F4 && g.one_word);
+                        expand_unit<A, F4>(wd, g.a_kind, dst, g16, F4 && g.one_word);
                     }
                 } else {
                     int u = 0, i = xl;
@@ -1386,7 +1474,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                     for (; u < nu; src += nx * g.psz) {
                         uint32_t wd[2 * A];
                         load_unit<A>(src, step, g.psz, wd);
-                        expand_unit<A>(wd, g.a_kind, e0 + static_cast<uint32_t>(u) * 4u * g16 + static_cast<uint32_t>(i) * 16u, g16);
+                        expand_unit<A, F4>(wd, g.a_kind, e0 + static_cast<uint32_t>(u) * (F4 ? 2u : 4u) * g16 + static_cast<uint32_t>(i) * 16u, g16, false);
                         i += nx;
                         while (i >= g.NI) { i -= g.NI; ++u; }
                     }
@@ -1403,9 +1491,10 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                         bool live = true;
                         int off;
                         if (!all_live) live = w.o * g.TN + filter_row(g, i, WBX, off) < g.O;
-                        const uint32_t d = bdst + static_cast<uint32_t>(2 * u) * blk + static_cast<uint32_t>(i >> 3) * 256u + static_cast<uint32_t>(i & 7) * 16u;
-                        expand_filter_word<WBX>(wd, g.w_kind, live, d);
-                        expand_filter_word<WBX>(wd + WBX, g.w_kind, live, d + blk);
+                        const bool both = 2 * ((range.beg + c) * g.units + u) + 1 < g.Cw;
+                        const uint32_t d = bdst + static_cast<uint32_t>(F4 ? u : 2 * u) * blk + static_cast<uint32_t>(i >> 3) * 256u + static_cast<uint32_t>(i & 7) * 16u;
+                        expand_filter_word<WBX, F4>(wd, g.w_kind, live, d);
+                        expand_filter_word<WBX, F4>(wd + WBX, g.w_kind, live && both, d + (F4 ? 128u : blk));
                         i += nx;
                         while (i >= rows) { i -= rows; ++u; }
                     }
@@ -1433,7 +1522,10 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
         // ------------------------------------------------------------------ epilogue
         const int quad = warp & 3, set = warp >> 2;
         const uint32_t lane_addr = static_cast<uint32_t>(quad * 32) << 16;
-        if (g.preset) {
+        if (F4) {           // scale factors of 2 for every row, column and block
+            for (int c = set * 8; c < MM_SF_COLS; c += 8 * (EW / 4)) mm_st8(tmem + lane_addr + static_cast<uint32_t>(g.sf_col + c), 0x80808080u);
+            mm_st_wait();
+        } else if (g.preset) {
             for (int c = set * 8; c < g.tmem_cols; c += 8 * (EW / 4)) mm_st8(tmem + lane_addr + static_cast<uint32_t>(c), MM_PRESET);
             mm_st_wait();
         }
@@ -1448,7 +1540,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                 if (!mm_wait(bulk_full, 0)) atomicOr(g.status, STATUS_TIMEOUT);
                 src = reinterpret_cast<const uint32_t*>(mm_smem + g.off_e);
             }
-            expand_filters_resident<WBX>(g, smem0, src, o0, tid, NXT + NET);
+            expand_filters_resident<WBX, F4>(g, smem0, src, o0, tid, NXT + NET);
             fence_proxy_async();
             // the parked tile has been read: the ring may be filled once every warp is here
             asm volatile("bar.sync 4, %0;" ::"n"(NXT + NET) : "memory");
@@ -1461,14 +1553,14 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
         e.acc = tmem + lane_addr; e.row0 = quad * 32 + lane; e.set = set;
         e.tid = tid; e.lane = lane; e.warp = warp; e.red_full = red_full;
         bool ok;
-        if (SPLIT && range.rank > 0) ok = send_partials<EW>(g, e, range.rank);
-        else if (!g.preset) ok = epilogue_general<EW, SPLIT>(g, e);
-        else if (g.epi == 0) ok = epilogue_codes<2, 0, true, EW, SPLIT>(g, e);
-        else if (g.epi == 1) ok = epilogue_codes<2, 2, true, EW, SPLIT>(g, e);
-        else if (g.epi == 2) ok = epilogue_codes<4, 0, true, EW, SPLIT>(g, e);
-        else if (g.epi == 3) ok = epilogue_codes<4, 4, true, EW, SPLIT>(g, e);
-        else if (g.epi == 4) ok = epilogue_codes<4, 0, false, EW, SPLIT>(g, e);
-        else ok = epilogue_codes<4, 4, false, EW, SPLIT>(g, e);
+        if (SPLIT && range.rank > 0) ok = send_partials<EW, F4>(g, e, range.rank);
+        else if (!g.preset) ok = epilogue_general<EW, SPLIT, F4>(g, e);
+        else if (g.epi == 0) ok = epilogue_codes<2, 0, true, EW, SPLIT, F4>(g, e);
+        else if (g.epi == 1) ok = epilogue_codes<2, 2, true, EW, SPLIT, F4>(g, e);
+        else if (g.epi == 2) ok = epilogue_codes<4, 0, true, EW, SPLIT, F4>(g, e);
+        else if (g.epi == 3) ok = epilogue_codes<4, 4, true, EW, SPLIT, F4>(g, e);
+        else if (g.epi == 4) ok = epilogue_codes<4, 0, false, EW, SPLIT, F4>(g, e);
+        else ok = epilogue_codes<4, 4, false, EW, SPLIT, F4>(g, e);
         if (!ok && lane == 0) atomicOr(g.status, STATUS_TIMEOUT);
     }
     mm_fence_before();
@@ -1483,28 +1575,35 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
 
 typedef void (*MmaKernel)(MmaArgs);
 
-// The instantiations for A activation bits, one translation unit each (mma_inst_a*.cu): filters prepared (wb = 0) or packed in wb
-// bits, half an SM or a whole one per CTA, a whole one with the item split over a cluster.
+// The instantiations for A activation bits, a translation unit each (mma_inst_a*.cu; nibbles: mma_inst_f*.cu): filters prepared (wb = 0)
+// or packed in wb bits, half an SM or a whole one per CTA, a whole one with the item split over a cluster.
 MmaKernel mma_kernel_a1(int wb, bool half, bool split);
 MmaKernel mma_kernel_a2(int wb, bool half, bool split);
 MmaKernel mma_kernel_a3(int wb, bool half, bool split);
 MmaKernel mma_kernel_a4(int wb, bool half, bool split);
+MmaKernel mma_kernel_f1(int wb, bool half, bool split);
+MmaKernel mma_kernel_f2(int wb, bool half, bool split);
 
-template <int A, int WB>
+template <int A, int WB, bool F4>
 MmaKernel mma_pick_shape(bool half, bool split)
 {
-    return split ? bitserial_mma_kernel<A, WB, false, true> : half ? bitserial_mma_kernel<A, WB, true, false> : bitserial_mma_kernel<A, WB, false, false>;
+    return split ? bitserial_mma_kernel<A, WB, false, true, F4> : half ? bitserial_mma_kernel<A, WB, true, false, F4> : bitserial_mma_kernel<A, WB, false, false, F4>;
 }
 template <int A>
 MmaKernel mma_pick(int wb, bool half, bool split)
 {
     switch (wb) {
-        case 0: return mma_pick_shape<A, 0>(half, split);
-        case 1: return mma_pick_shape<A, 1>(half, split);
-        case 2: return mma_pick_shape<A, 2>(half, split);
-        case 3: return mma_pick_shape<A, 3>(half, split);
-        default: return mma_pick_shape<A, 4>(half, split);
+        case 0: return mma_pick_shape<A, 0, false>(half, split);
+        case 1: return mma_pick_shape<A, 1, false>(half, split);
+        case 2: return mma_pick_shape<A, 2, false>(half, split);
+        case 3: return mma_pick_shape<A, 3, false>(half, split);
+        default: return mma_pick_shape<A, 4, false>(half, split);
     }
+}
+template <int A>
+MmaKernel mma_pick_nibbles(int wb, bool half, bool split)
+{
+    return wb == 0 ? mma_pick_shape<A, 0, true>(half, split) : wb == 1 ? mma_pick_shape<A, 1, true>(half, split) : mma_pick_shape<A, 2, true>(half, split);
 }
 
 }  // namespace bs

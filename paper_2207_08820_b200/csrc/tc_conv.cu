@@ -5,10 +5,10 @@
 namespace bs {
 
 // One thread per 16-byte vector of the prepared filter layout [C/32][O/8][tap][2][8 filters][16 channels], the core matrices of
-// the B operand block by block.  Within a group of 32 filters the rows, and within a block of 32 channels the bytes, stand in
-// the orders of mma_conv.h.
+// the B operand block by block; nibbles: [ceil(C/64)][O/8][tap][2][8 filters][32 channels], sign and magnitude.  Within a group of 32 filters
+// the rows, and within a block of 32 channels the bytes, stand in the orders of mma_conv.h; nibble j of word m is channel 4 j + m.
 __global__ void tc_prepare_weights_kernel(const uint32_t* __restrict__ packed, int8_t* __restrict__ out, long long nvec, int O, int RS, int Cw,
-                                          int WB, int sign, int opad8)
+                                          int WB, int sign, int opad8, bool nibbles)
 {
     const long long idx = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (idx >= nvec) return;
@@ -21,7 +21,18 @@ __global__ void tc_prepare_weights_kernel(const uint32_t* __restrict__ packed, i
     const int col = og * 8 + row;
     const int o = (col & ~31) + mma_filter_of_column(col & 31);
     uint32_t vals[4] = {0, 0, 0, 0};
-    if (o < O) {
+    if (nibbles) {
+        const int cw = blk * 2 + half;
+        if (o < O && cw < Cw) {
+            const uint32_t* w = packed + ((static_cast<size_t>(o) * RS + tap) * Cw + cw) * WB;
+            for (int ch = 0; ch < 32; ++ch) {
+                unsigned pat = 0;
+                for (int i = 0; i < WB; ++i) pat |= ((w[i] >> ch) & 1u) << i;
+                const int v = pattern_value(pat, WB, sign);
+                vals[ch & 3] |= static_cast<uint32_t>(v < 0 ? 8 - v : v) << (4 * (ch >> 2));
+            }
+        }
+    } else if (o < O) {
         const uint32_t* w = packed + ((static_cast<size_t>(o) * RS + tap) * Cw + blk) * WB;
         for (int b = 0; b < 16; ++b) {
             const int ch = mma_channel_of_byte(half * 16 + b);
@@ -184,11 +195,12 @@ extern "C" int bs_tc_prepare_weights(const uint32_t* wgt_packed, int O, int C, i
     if (!bs::aligned16(wgt_packed) || !bs::aligned16(out)) return BS_ERR_ALIGNMENT;
     if (C % 32 != 0) return BS_ERR_UNSUPPORTED;
     const int opad8 = (O + 127) / 128 * 16;
-    const long long nvec = static_cast<long long>(C / 32) * opad8 * R * S * 2 * 8;
+    const bool nibbles = bs::mma_nibbles(C, R * S, a_bits, w_bits);
+    const long long nvec = static_cast<long long>(nibbles ? (C / 32 + 1) / 2 : C / 32) * opad8 * R * S * 2 * 8;
     const long long blocks = (nvec + 255) / 256;
     if (blocks > 0x7fffffffLL) return BS_ERR_UNSUPPORTED;
     bs::tc_prepare_weights_kernel<<<static_cast<unsigned>(blocks), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        wgt_packed, out, nvec, O, R * S, C / 32, w_bits, w_sign, opad8);
+        wgt_packed, out, nvec, O, R * S, C / 32, w_bits, w_sign, opad8, nibbles);
     return cudaGetLastError() == cudaSuccess ? BS_OK : BS_ERR_CUDA;
 }
 
