@@ -1016,6 +1016,179 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
     return ok;
 }
 
+// Nibbles, codes of at most two bits; items of two or four row tiles: two row tiles at a time (NT), so that the scales and biases of 32 filters are
+// read once for both.  An LDS.128 costs four wavefronts of shared memory even when all lanes read the same address, and 16 of them for every
+// 32 x 32 outputs (24 with the residual's multipliers, which are shifts here) took more of its bandwidth than the MMAs' operands.  Eight
+// columns of each tile are computed while the next eight are on their way.
+// conv2_x of 64 images: 14.1 -> 13.5 us without, 16.4 -> 15.1 us with a residual.  (Fragments of 16 x 256 bits, whose lanes need the
+// constants of 8 filters only, made it 16.1 and 19.7: trading codes for plane words between lanes costs more than the loads.)
+__device__ __forceinline__ void mm_ld8(uint32_t taddr, uint32_t (&v)[8])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void mm_landed8(uint32_t (&v)[8])
+{
+    asm volatile("" : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]));
+}
+// Eight columns of two tiles: codes of pair i at bits 2 i of either half of W.  z: residual codes of the pairs from bit 0 of either half on.
+template <bool RES, int NT>
+__device__ __forceinline__ void requant8(const uint32_t (&v)[NT][8], uint32_t tab, const uint32_t (&z)[NT], u64 rmul, u64 rmul4, uint32_t hi2, uint32_t (&W)[NT])
+{
+    const u64 magic = f2_pack(0x3F400000u, 0x3F400000u);
+    uint32_t k[NT][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        u64 s2, b2;
+        asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(s2), "=l"(b2) : "r"(tab + i * 16));
+#pragma unroll
+        for (int j = 0; j < NT; ++j) {
+            u64 t = f2_fma(f2_pack(v[j][2 * i], v[j][2 * i + 1]), s2, b2);
+            if (RES) {
+                const uint32_t c = i < 2 ? z[j] : z[j] >> 4, m = i & 1 ? 12u : 3u;
+                t = f2_fma(f2_pack(c & m, (c >> 16) & m), i & 1 ? rmul4 : rmul, t);
+            }
+            uint32_t lo, hi;
+            f2_split(f2_add(t, magic), lo, hi);
+            k[j][i] = __vimin_s16x2_relu(__byte_perm(lo, hi, 0x5410), hi2);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < NT; ++j) W[j] = (k[j][0] + (k[j][1] << 2)) + ((k[j][2] + (k[j][3] << 2)) << 4);
+}
+template <bool RES, int NT, int EW, bool SPLIT>
+__device__ __forceinline__ bool epilogue_tiles(const MmaArgs& g, const MmaEpi& e)
+{
+    constexpr int STEP = EW / 4;
+    const uint32_t tab0 = smem_u32(e.smem + g.off_tab);
+    int qmin, qmax;
+    code_limits(g.out_bits, g.out_sign, qmin, qmax);
+    const uint32_t hi2 = (static_cast<uint32_t>(qmax) & 0xFFFFu) * 0x10001u;
+    // a residual code in the low bits of a word is the denormal code * 2^-149; everything is scaled by 2^-24
+    const uint32_t rm = __float_as_uint(g.res_scale * __uint_as_float(252u << 23)), rm4 = __float_as_uint(g.res_scale * __uint_as_float(250u << 23));
+    const u64 rmul = f2_pack(rm, rm), rmul4 = f2_pack(rm4, rm4);
+    const int groups = g.TN >> 5;
+    int tab_o = -1, ia = 0;
+    unsigned pa = 0;
+    bool ok = true, fast = false, waited = !g.early_b;
+    for (MmaWalk w(g, SPLIT ? g.split_log : 0); w.m < g.tiles_m; w.next(g)) {
+        const int o0 = w.o * g.TN;
+        if (w.o != tab_o) {
+            if (tab_o >= 0) asm volatile("bar.sync 2, %0;" ::"n"(EW * 32) : "memory");     // every warp is done with the old table
+            epilogue_tables(g, reinterpret_cast<float4*>(e.smem + g.off_tab), reinterpret_cast<float2*>(e.smem + g.off_tab + g.TN * 8), e.fast_ok, o0,
+                            e.tid, EW * 32);
+            asm volatile("bar.sync 2, %0;" ::"n"(EW * 32) : "memory");
+            fast = *reinterpret_cast<volatile int*>(e.fast_ok) != 0;
+            tab_o = w.o;
+        }
+        if (!waited) { mm_pdl_wait(); waited = true; }
+        const int base = w.m * 128 * g.PT + e.row0;
+        // units (NT tiles, group), group fastest
+        int t = 0, cc = e.set;
+        while (cc >= groups) { cc -= groups; t += NT; }
+        int pix[NT];
+        auto pixels = [&]() {
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+                const MmaPixel px = mma_pixel(g, base + (t + j) * 128);
+                pix[j] = px.valid ? px.pix : -1;
+            }
+        };
+        uint32_t rn[NT][4];
+        auto residual = [&](int ob) {
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) rn[j][k] = 0;
+                if (RES && pix[j] >= 0 && ob < g.O) load_residual(g, pix[j], ob, rn[j]);
+            }
+        };
+        if (t < g.PT) {
+            pixels();
+            residual(o0 + cc * 32);
+        }
+        if (ok) ok = mm_wait(&e.full_acc[ia], pa);    // after a wait that ran out the walk goes on without waiting, so the named barriers stay matched
+        mm_fence_after();
+        if (SPLIT && ok) ok = merge_partials<EW, true>(g, e);
+        MM_TRACE(e.tid == 0, TR_EBEG, (w.it - static_cast<int>(blockIdx.x)) / static_cast<int>(gridDim.x));
+        const uint32_t acc = e.acc + static_cast<uint32_t>(ia * g.PT * g.TN), TN = static_cast<uint32_t>(g.TN);
+        if (!fast) {
+            epilogue_item_formula(g, acc, base, o0, e.set, STEP);
+            t = g.PT;
+        }
+        uint32_t v[2][NT][8];           // [buffer][tile]
+        uint32_t col = acc + static_cast<uint32_t>(t * g.TN + cc * 32);
+        if (t < g.PT)
+#pragma unroll
+            for (int j = 0; j < NT; ++j) mm_ld8(col + j * TN, v[0][j]);
+        while (t < g.PT) {
+            const int ob = o0 + cc * 32;
+            const uint32_t tab = tab0 + static_cast<uint32_t>(cc) * 256u;
+            int to[NT];
+            uint32_t z[2][NT];                             // [half of the filters][tile]
+#pragma unroll
+            for (int j = 0; j < NT; ++j) { to[j] = pix[j]; z[0][j] = z[1][j] = 0u; }
+            if (RES)
+#pragma unroll
+                for (int j = 0; j < NT; ++j) {
+                    z[0][j] = (rn[j][0] & 0x55555555u) | ((rn[j][1] << 1) & 0xAAAAAAAAu);
+                    z[1][j] = ((rn[j][0] >> 1) & 0x55555555u) | (rn[j][1] & 0xAAAAAAAAu);
+                }
+            // the next unit's place and residual
+            cc += STEP;
+            const int t_old = t;
+            while (cc >= groups) { cc -= groups; t += NT; }
+            const bool more = t < g.PT;
+            if (more) {
+                if (t != t_old) pixels();
+                residual(o0 + cc * 32);
+            }
+            const uint32_t next = acc + static_cast<uint32_t>(t * g.TN + cc * 32);
+            uint32_t H[2][NT];                             // [half][tile]
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                mm_ld_wait();
+#pragma unroll
+                for (int j = 0; j < NT; ++j) mm_landed8(v[p & 1][j]);
+                if (p < 3 || more) {
+                    const uint32_t from = p < 3 ? col + 8u * (p + 1) : next;
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) mm_ld8(from + j * TN, v[(p & 1) ^ 1][j]);
+                }
+                uint32_t zp[NT], W[NT];
+#pragma unroll
+                for (int j = 0; j < NT; ++j) zp[j] = z[p >> 1][j] >> (8 * (p & 1));
+                requant8<RES, NT>(v[p & 1], tab + 64u * p, zp, rmul, rmul4, hi2, W);
+#pragma unroll
+                for (int j = 0; j < NT; ++j) H[p >> 1][j] = p & 1 ? H[p >> 1][j] + (W[j] << 8) : W[j];
+            }
+            col = next;
+#pragma unroll
+            for (int j = 0; j < NT; ++j)
+                if (to[j] >= 0 && ob < g.O) {
+                    uint32_t ow[4] = {(H[0][j] & 0x55555555u) | ((H[1][j] << 1) & 0xAAAAAAAAu), ((H[0][j] >> 1) & 0x55555555u) | (H[1][j] & 0xAAAAAAAAu), 0u, 0u};
+                    store_codes(g, to[j], ob, ow);
+                }
+        }
+        mm_fence_before();
+        __syncwarp();
+        if (e.lane == 0) mm_arrive(&e.empty_acc[ia]);
+        MM_TRACE(e.tid == 0, TR_EEND, (w.it - static_cast<int>(blockIdx.x)) / static_cast<int>(gridDim.x));
+        if (++ia == g.nacc) { ia = 0; pa ^= 1u; }
+    }
+    if (!waited) mm_pdl_wait();
+    return ok;
+}
+
+// Codes of at most two bits from zero on, residual codes of at most two bits.
+template <bool RES, int EW, bool SPLIT, bool F4>
+__device__ __forceinline__ bool epilogue_two_bits(const MmaArgs& g, const MmaEpi& e)
+{
+    if constexpr (!F4) return epilogue_codes<2, RES ? 2 : 0, true, EW, SPLIT, false>(g, e);
+    else if constexpr (SPLIT) return epilogue_tiles<RES, 1, EW, true>(g, e);       // one row tile
+    else return g.PT > 1 ? epilogue_tiles<RES, 2, EW, false>(g, e) : epilogue_tiles<RES, 1, EW, false>(g, e);
+}
+
 // int32 accumulators out (and codes through the formula where both are asked for or the fast form does not apply).
 template <int EW, bool SPLIT, bool F4>
 __device__ __forceinline__ bool epilogue_general(const MmaArgs& g, const MmaEpi& e)
@@ -1555,8 +1728,8 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
         bool ok;
         if (SPLIT && range.rank > 0) ok = send_partials<EW, F4>(g, e, range.rank);
         else if (!g.preset) ok = epilogue_general<EW, SPLIT, F4>(g, e);
-        else if (g.epi == 0) ok = epilogue_codes<2, 0, true, EW, SPLIT, F4>(g, e);
-        else if (g.epi == 1) ok = epilogue_codes<2, 2, true, EW, SPLIT, F4>(g, e);
+        else if (g.epi == 0) ok = epilogue_two_bits<false, EW, SPLIT, F4>(g, e);
+        else if (g.epi == 1) ok = epilogue_two_bits<true, EW, SPLIT, F4>(g, e);
         else if (g.epi == 2) ok = epilogue_codes<4, 0, true, EW, SPLIT, F4>(g, e);
         else if (g.epi == 3) ok = epilogue_codes<4, 4, true, EW, SPLIT, F4>(g, e);
         else if (g.epi == 4) ok = epilogue_codes<4, 0, false, EW, SPLIT, F4>(g, e);

@@ -1,7 +1,7 @@
 """Per-CTA timeline of the tensor-core kernel (trace builds only).
 
 A library built with ``BS_EXTRA_NVCC_FLAGS=-DBS_TRACE python -m paper_2207_08820_b200.build --force`` records, for the first 148 CTAs
-of a launch with 2-bit activations and the first 48 steps of each, the SM cycle counter at the hand-offs between the kernel's roles
+of a launch with 2-bit activations and filters of at most two bits and the first 48 steps of each, the SM cycle counter at the hand-offs between the kernel's roles
 (expansion of a chunk, issue of its MMAs, epilogue of an item).  This tool runs chosen layers of a layer stack once and prints
 those timelines:
 
