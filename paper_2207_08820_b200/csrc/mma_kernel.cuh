@@ -1450,11 +1450,15 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                     const int nu = min(g.units, g.nunits - (range.beg + c) * g.units);
                     const uint32_t src = smem0 + g.off_stg + static_cast<uint32_t>(ip * g.stg_bytes);
                     const uint32_t e0 = smem0 + g.off_e + static_cast<uint32_t>(idx * g.e_bytes);
-                    for (int it = xl; it < nu << shA; it += nx) {
-                        const int u = it >> shA, i = it & (rowsA - 1);
-                        uint32_t wd[2 * A];
-                        load_row_unit<A>(src, i * g.rowA + u * 8 * A, g.swzA, wd);
-                        expand_unit<A, F4>(wd, g.a_kind, e0 + static_cast<uint32_t>(u) * (F4 ? 2u : 4u) * g16 + static_cast<uint32_t>(i) * 16u, g16, false);
+                    // two rows at a time: the second one's words are on their way while the first is expanded
+                    for (int it = xl; it < nu << shA; it += 2 * nx) {
+                        const int u0 = it >> shA, i0 = it & (rowsA - 1), u1 = (it + nx) >> shA, i1 = (it + nx) & (rowsA - 1);
+                        const bool two = it + nx < nu << shA;
+                        uint32_t wa[2 * A], wb[2 * A];
+                        load_row_unit<A>(src, i0 * g.rowA + u0 * 8 * A, g.swzA, wa);
+                        if (two) load_row_unit<A>(src, i1 * g.rowA + u1 * 8 * A, g.swzA, wb);
+                        expand_unit<A, F4>(wa, g.a_kind, e0 + static_cast<uint32_t>(u0) * (F4 ? 2u : 4u) * g16 + static_cast<uint32_t>(i0) * 16u, g16, false);
+                        if (two) expand_unit<A, F4>(wb, g.a_kind, e0 + static_cast<uint32_t>(u1) * (F4 ? 2u : 4u) * g16 + static_cast<uint32_t>(i1) * 16u, g16, false);
                     }
                     if (stream_b) {
                         const uint32_t bsrc = smem0 + g.off_bstg + static_cast<uint32_t>(ip * g.bstg_bytes);
