@@ -161,7 +161,7 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows, int sms)
 // Time model of a candidate in SM cycles: the pipeline of one CTA (expansion, MMAs, epilogue; a stage's hand-off included) over
 // its items, plus what nothing overlaps at both ends.  The constants are fitted to timed plans (B200 at 1.95 GHz): int8 to about 2500 of
 // 45 layers and products (1 to 300 pixels wide, 32 to 4608 channels, batches 1 to 64), the plan with the lowest modelled time being on
-// average 2 to 3 % and at most 16 % slower than the fastest; nibbles to 8300 of 49, on average 1.4 % and at most 19 % slower (with the
+// average 2 to 3 % and at most 16 % slower than the fastest; nibbles to 17000 of 77, on average 1.3 % and at most 19 % slower (with the
 // constants of int8: 4.5 % and 91 %, most of it from filters staged piece by piece, which cost twice what was assumed).
 struct MmaFit {
     double mma_chunk;                       // cycles per chunk beside its MMAs
@@ -169,11 +169,14 @@ struct MmaFit {
     double filt_flat, filt_staged;          // packed filters streamed, instructions per 32 rows and unit
     double x_cpi, x_chunk, x_group, x_once; // cycles per such instruction, per chunk; share by which a further group overlaps; once
     double e_res, e_codes, e_i32, e_cpi, e_once;        // epilogue, instructions per block of 32 x 32 outputs; cycles per instruction; per item
+    double e_pair;                          // of e_res and e_codes where two row tiles share a pass
+    double rows, rows_odd;                  // bytes per cycle of int32 rows, of rows that are not multiples of 16 bytes
+    double split;                           // cycles of a split item beside its sums
     double l2;                              // bytes per cycle of streamed prepared filters
     double ipc, two_first, start, filt_resident, streamed, one_stage, half;
 };
-constexpr MmaFit FIT_INT8 = {148, 102, 102, 1, 41, 20, 20, 5.34, 629, 0.83, 628, 215, 138, 94, 4.59, 997, 68.7, 3.08, 1.19, 4215, 122, 1.07, 1.11, 0.93};
-constexpr MmaFit FIT_NIBBLES = {280, 64.5, 41.6, 1, 80, 52, 129, 5.64, 513, 0.79, 693, 265, 120, 94, 4.2, 960, 68.3, 1.45, 1.21, 3208, 211, 1.05, 0.98, 0.905};
+constexpr MmaFit FIT_INT8 = {148, 102, 102, 1, 41, 20, 20, 5.34, 629, 0.83, 628, 215, 138, 94, 4.59, 997, 1, 29.6, 12.2, 2200, 68.7, 3.08, 1.19, 4215, 122, 1.07, 1.11, 0.93};
+constexpr MmaFit FIT_NIBBLES = {262, 63, 31, 1, 92.5, 64.2, 127, 5.49, 457, 0.889, 705, 247, 114, 360, 4.01, 982, 0.931, 24.3, 12.2, 4236, 98.3, 1.45, 1.226, 3484, 223, 1.076, 0.961, 0.934};
 
 double mma_cost(const MmaArgs& g, const Cand& c, int A, int WB, bool packed_out, int sms)
 {
@@ -190,12 +193,11 @@ double mma_cost(const MmaArgs& g, const Cand& c, int A, int WB, bool packed_out,
     const double units_of_work = static_cast<double>(row_groups) * c.units * c.groups / W;       // per warp of a group and chunk
     const double chunk = xi / nchunks * c.groups / W * (ceil(units_of_work) / units_of_work) * k.x_cpi + k.x_chunk;
     const double t_x = chunk * nchunks / (1.0 + (c.groups - 1) * k.x_group) + k.x_once;
-    // int32 rows leave at about 30 bytes per clock and SM
-    const double block = packed_out ? (g.has_residual ? k.e_res : k.e_codes) : k.e_i32;
+    const double block = packed_out ? (g.has_residual ? k.e_res : k.e_codes) * (c.PT > 1 ? k.e_pair : 1.0) : k.e_i32, rows = g.O % 4 ? k.rows_odd : k.rows;
     double t_e = ceil_div(c.PT * (c.TN / 32), W / 4) * block * k.e_cpi + k.e_once;
-    if (!packed_out && c.PT * 128.0 * c.TN * 4 / 29.6 > t_e) t_e = c.PT * 128.0 * c.TN * 4 / 29.6;
+    if (!packed_out && c.PT * 128.0 * c.TN * 4 / rows > t_e) t_e = c.PT * 128.0 * c.TN * 4 / rows;
     // sums through shared memory of the cluster
-    if (c.split > 1) t_e += 2200.0 + ceil_div(c.PT * (c.TN / 32), W / 4) * 200.0 * (c.split - 1);
+    if (c.split > 1) t_e += k.split + ceil_div(c.PT * (c.TN / 32), W / 4) * 200.0 * (c.split - 1);
     const double t_b = (!c.resident && !packed_b) ? share * c.TN * g.RS * g.nblk * 32 / k.l2 : 0.0;       // L2 -> shared memory
     const long long items = static_cast<long long>(g.tiles_m) * g.tiles_o * c.split;
     long long ctas = static_cast<long long>(sms) * c.cps;
