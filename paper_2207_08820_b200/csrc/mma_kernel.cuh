@@ -465,8 +465,11 @@ __device__ __forceinline__ void expand_filter_word(const uint32_t* w, int kind, 
     if constexpr (F4) {
         uint32_t n[4];
         expand_nibbles<WB>(w, kind, n);
-        const uint32_t keep = live ? 0xffffffffu : 0u;
-        mm_sts(dst, n[0] & keep, n[1] & keep, n[2] & keep, n[3] & keep);
+        if (kind == 2 && !live) {        // missing bits are no -1 (zeros as they are otherwise)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) n[k] = 0u;
+        }
+        mm_sts(dst, n[0], n[1], n[2], n[3]);
         return;
     }
     uint32_t o[8];
@@ -1422,6 +1425,8 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
         // A chunk belongs to one group of warps.  The waits, the fence and the arrival of a chunk take several hundred cycles whatever its
         // size; with several groups they overlap (see make_plan for how many).
         const int G = g.groups, nx = NXT / G, xg = xt / nx, xl = xt - xg * nx;
+        // bipolar filters of an odd number of channel words: the second half of the last K step of nibbles has to be zero, not -1
+        const bool odd_tail = F4 && g.w_kind == 2 && (g.Cw & 1);
 #ifdef BS_TRACE
         int xseq = 0;
 #endif
@@ -1468,7 +1473,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                             const int f = (i & ~31) + mma_filter_of_column(i & 31);
                             uint32_t wd[2 * WBX];
                             load_row_unit<WBX>(bsrc, f * g.rowB + u * 8 * WBX, g.swzB, wd);
-                            const bool live = w.o * g.TN + f < g.O, both = 2 * ((range.beg + c) * g.units + u) + 1 < g.Cw;
+                            const bool live = w.o * g.TN + f < g.O, both = !odd_tail || (range.beg + c) * g.units + u + 1 < g.nunits;
                             const uint32_t d = bdst + static_cast<uint32_t>(F4 ? u : 2 * u) * blk + static_cast<uint32_t>(i >> 3) * 256u + static_cast<uint32_t>(i & 7) * 16u;
                             expand_filter_word<WBX, F4>(wd, g.w_kind, live, d);
                             expand_filter_word<WBX, F4>(wd + WBX, g.w_kind, live && both, d + (F4 ? 128u : blk));
@@ -1677,7 +1682,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                         bool live = true;
                         int off;
                         if (!all_live) live = w.o * g.TN + filter_row(g, i, WBX, off) < g.O;
-                        const bool both = 2 * ((range.beg + c) * g.units + u) + 1 < g.Cw;
+                        const bool both = !odd_tail || (range.beg + c) * g.units + u + 1 < g.nunits;
                         const uint32_t d = bdst + static_cast<uint32_t>(F4 ? u : 2 * u) * blk + static_cast<uint32_t>(i >> 3) * 256u + static_cast<uint32_t>(i & 7) * 16u;
                         expand_filter_word<WBX, F4>(wd, g.w_kind, live, d);
                         expand_filter_word<WBX, F4>(wd + WBX, g.w_kind, live && both, d + (F4 ? 128u : blk));
