@@ -1395,6 +1395,10 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                 }
             }
             if (!ok) atomicOr(g.status, STATUS_TIMEOUT);
+            if (!packed_b && blockIdx.x == 0) {         // filters prepared for other widths; read last, when nothing waits for this warp
+                const uint32_t mark = reinterpret_cast<const uint32_t*>(g.wgt + blk_stride * g.Cw)[-1];
+                if ((mark == MM_NIBBLE_MARK) != F4) atomicOr(g.status, STATUS_FILTERS);
+            }
         }
         __syncwarp();
     } else if (warp == WARP_MMA) {

@@ -8,7 +8,7 @@ namespace bs {
 // the B operand block by block; nibbles: [ceil(C/64)][O/8][tap][2][8 filters][32 channels], sign and magnitude.  Within a group of 32 filters
 // the rows, and within a block of 32 channels the bytes, stand in the orders of mma_conv.h; nibble j of word m is channel 4 j + m.
 __global__ void tc_prepare_weights_kernel(const uint32_t* __restrict__ packed, int8_t* __restrict__ out, long long nvec, int O, int RS, int Cw,
-                                          int WB, int sign, int opad8, bool nibbles)
+                                          int WB, int sign, int opad8, bool nibbles, long long last)
 {
     const long long idx = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (idx >= nvec) return;
@@ -41,6 +41,10 @@ __global__ void tc_prepare_weights_kernel(const uint32_t* __restrict__ packed, i
             const unsigned byte = static_cast<unsigned>(pattern_value(pat, WB, sign)) & 0xFFu;
             vals[b >> 2] |= byte << (8 * (b & 3));
         }
+    }
+    if (nibbles && idx == nvec - 1) {       // the last vector of the tensor is this one (of channels that do not exist) or one that no layer reads
+        if (last == idx) vals[3] = MM_NIBBLE_MARK;
+        else reinterpret_cast<uint4*>(out)[last] = make_uint4(0, 0, 0, MM_NIBBLE_MARK);
     }
     reinterpret_cast<uint4*>(out)[idx] = make_uint4(vals[0], vals[1], vals[2], vals[3]);
 }
@@ -200,7 +204,8 @@ extern "C" int bs_tc_prepare_weights(const uint32_t* wgt_packed, int O, int C, i
     const long long blocks = (nvec + 255) / 256;
     if (blocks > 0x7fffffffLL) return BS_ERR_UNSUPPORTED;
     bs::tc_prepare_weights_kernel<<<static_cast<unsigned>(blocks), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        wgt_packed, out, nvec, O, R * S, C / 32, w_bits, w_sign, opad8, nibbles);
+        wgt_packed, out, nvec, O, R * S, C / 32, w_bits, w_sign, opad8, nibbles,
+        static_cast<long long>(C / 32) * opad8 * R * S * 2 * 8 - 1);
     return cudaGetLastError() == cudaSuccess ? BS_OK : BS_ERR_CUDA;
 }
 

@@ -1,0 +1,71 @@
+"""Layers of one- and two-bit codes (operands of nibbles, sums in binary32) where exactness could end: sums up to the limit of the form, all bits of
+them in use, at both sides of the reduction length from which int8 takes over; every pair of signs; odd numbers of channel words."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2207_08820_b200 import api, workloads as wl
+from gpu_util import dev
+
+pytestmark = pytest.mark.gpu
+
+LIMIT = 4000000 // 9 // 32 * 32         # longest reduction on nibbles: C * R * S * 9 below 4 million
+
+
+@pytest.mark.parametrize("K", [LIMIT, LIMIT + 32])
+@pytest.mark.parametrize("form", ["largest codes", "sums that rise and fall", "random"])
+def test_longest_reductions(K, form):
+    """Whole numbers stay exact in binary32 below 2^24, so the comparison has no tolerance."""
+    rng = np.random.default_rng(K)
+    M, N = 130, 40
+    if form == "random":
+        a, w, ws = wl.rand_codes(rng, (M, K), 2, 0), wl.rand_codes(rng, (N, K), 2, api.SIGNED), api.SIGNED
+    else:
+        a, w, ws = np.full((M, K), 3, np.int8), np.full((N, K), 3, np.int8), api.UNSIGNED
+        a[rng.random((M, K)) < 0.001] = 1
+        if form == "sums that rise and fall":
+            w[:], ws = -2, api.SIGNED
+            w[:, K // 2:] = 1
+    want = oracle.gemm_i32(a, w)
+    ap, wp = api.bs_pack_rows(dev(a), 2, 0), api.bs_pack_rows(dev(w), 2, ws)
+    got, _ = api.bitserial_gemm(ap, wp, K, w_sign=ws)
+    assert np.array_equal(got.cpu().numpy(), want)
+    wt = api.tc_prepare_weights(wp.view(N, 1, 1, -1, 2), K, ws, 2)
+    got, _ = api.bitserial_gemm_tc(ap, wt, N, K, 2, a_sign=0, w_sign=ws)
+    api.bs_check_status()
+    assert np.array_equal(got.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("a,a_sign,w,w_sign", [(1, 0, 1, 2), (1, 1, 1, 0), (1, 2, 1, 2), (1, 2, 2, 1), (1, 0, 1, 1), (2, 0, 2, 0), (2, 1, 2, 1), (2, 1, 1, 2), (2, 0, 2, 1)])
+@pytest.mark.parametrize("C,O,k,s", [(32, 40, 3, 1), (96, 33, 1, 1), (64, 64, 3, 2), (160, 130, 5, 1)])
+def test_signs(C, O, k, s, a, a_sign, w, w_sign):
+    rng = np.random.default_rng(C + a + w)
+    x, f = wl.rand_codes(rng, (2, C, 9, 12), a, a_sign), wl.rand_codes(rng, (O, C, k, k), w, w_sign)
+    pad = 0 if a_sign == api.BIPOLAR else k // 2
+    want = oracle.conv2d_i32(x, f, s, pad)
+    xa, wp = api.bitpack_activations(dev(x), 1.0, a, a_sign), api.pack_weights(dev(f), w, w_sign)
+    forms = [dict()]
+    if api.tc_supported(2, C, 9, 12, O, k, s, pad, a, a_sign, w, w_sign):
+        forms.append(dict(wgt_tc=api.tc_prepare_weights(wp, C, w_sign, a)))
+    for kw in forms:
+        acc, _ = api.bitserial_conv2d(xa, wp, C=C, stride=s, pad=pad, a_sign=a_sign, w_sign=w_sign, want_i32=True, **kw)
+        assert np.array_equal(acc.cpu().numpy(), want)
+    api.bs_check_status()
+
+
+@pytest.mark.parametrize("C", [32, 64, 96])
+@pytest.mark.parametrize("prepared,run", [(2, 3), (4, 1), (2, 1), (3, 4)])
+def test_filters_of_the_other_form_are_reported(C, prepared, run):
+    rng = np.random.default_rng(C)
+    x, f = wl.rand_codes(rng, (1, C, 8, 8), run, 0), wl.rand_codes(rng, (128, C, 3, 3), 2, api.SIGNED)
+    xa, wp = api.bitpack_activations(dev(x), 1.0, run), api.pack_weights(dev(f), 2, api.SIGNED)
+    if not api.tc_supported(1, C, 8, 8, 128, 3, 1, 1, run, 0, 2, api.SIGNED):
+        pytest.skip("records of other sizes take no prepared filters")
+    acc, _ = api.bitserial_conv2d(xa, wp, C=C, pad=1, want_i32=True, wgt_tc=api.tc_prepare_weights(wp, C, api.SIGNED, prepared))
+    if (prepared <= 2) == (run <= 2):
+        api.bs_check_status()
+        assert np.array_equal(acc.cpu().numpy(), oracle.conv2d_i32(x, f, 1, 1))
+    else:
+        with pytest.raises(api.BitserialError):
+            api.bs_check_status()
+        api.bs_check_status()               # reported once
