@@ -162,21 +162,22 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows, int sms)
 // its items, plus what nothing overlaps at both ends.  The constants are fitted to timed plans (B200 at 1.95 GHz): int8 to about 2500 of
 // 45 layers and products (1 to 300 pixels wide, 32 to 4608 channels, batches 1 to 64), the plan with the lowest modelled time being on
 // average 2 to 3 % and at most 16 % slower than the fastest; nibbles to 17000 of 77, on average 1.3 % and at most 19 % slower (with the
-// constants of int8: 4.5 % and 91 %, most of it from filters staged piece by piece, which cost twice what was assumed).
+// constants of int8: 4.5 % and 91 %, most of it from filters staged piece by piece, which cost twice what was assumed).  Their int32 in rows of
+// pixels apart, over 17 layers: 2.5 % and 11 % with 180, 4.0 % and 20 % with the 360 of rows of filters (57 x 64 x 35 x 33, 288 filters: 32.7 -> 30.2 us).
 struct MmaFit {
     double mma_chunk;                       // cycles per chunk beside its MMAs
     double unit, one_word, flat, staged;    // expansion, instructions per warp and 64-channel unit of 32 rows: arithmetic, of 32 channels only, copies by TMA, by thread
     double filt_flat, filt_staged;          // packed filters streamed, instructions per 32 rows and unit
     double x_cpi, x_chunk, x_group, x_once; // cycles per such instruction, per chunk; share by which a further group overlaps; once
-    double e_res, e_codes, e_i32, e_cpi, e_once;        // epilogue, instructions per block of 32 x 32 outputs; cycles per instruction; per item
+    double e_res, e_codes, e_i32, e_nchw, e_cpi, e_once;        // epilogue, instructions per block of 32 x 32 outputs (int32 in rows of filters or of pixels); cycles per instruction; per item
     double e_pair;                          // of e_res and e_codes where two row tiles share a pass
     double rows, rows_odd;                  // bytes per cycle of int32 rows, of rows that are not multiples of 16 bytes
     double split;                           // cycles of a split item beside its sums
     double l2;                              // bytes per cycle of streamed prepared filters
     double ipc, two_first, start, filt_resident, streamed, one_stage, half;
 };
-constexpr MmaFit FIT_INT8 = {148, 102, 102, 1, 41, 20, 20, 5.34, 629, 0.83, 628, 215, 138, 94, 4.59, 997, 1, 29.6, 12.2, 2200, 68.7, 3.08, 1.19, 4215, 122, 1.07, 1.11, 0.93};
-constexpr MmaFit FIT_NIBBLES = {262, 63, 31, 1, 92.5, 64.2, 127, 5.49, 457, 0.889, 705, 247, 114, 360, 4.01, 982, 0.931, 24.3, 12.2, 4236, 98.3, 1.45, 1.226, 3484, 223, 1.076, 0.961, 0.934};
+constexpr MmaFit FIT_INT8 = {148, 102, 102, 1, 41, 20, 20, 5.34, 629, 0.83, 628, 215, 138, 94, 94, 4.59, 997, 1, 29.6, 12.2, 2200, 68.7, 3.08, 1.19, 4215, 122, 1.07, 1.11, 0.93};
+constexpr MmaFit FIT_NIBBLES = {262, 63, 31, 1, 92.5, 64.2, 127, 5.49, 457, 0.889, 705, 247, 114, 360, 180, 4.01, 982, 0.931, 24.3, 12.2, 4236, 98.3, 1.45, 1.226, 3484, 223, 1.076, 0.961, 0.934};
 
 double mma_cost(const MmaArgs& g, const Cand& c, int A, int WB, bool packed_out, int sms)
 {
@@ -193,7 +194,7 @@ double mma_cost(const MmaArgs& g, const Cand& c, int A, int WB, bool packed_out,
     const double units_of_work = static_cast<double>(row_groups) * c.units * c.groups / W;       // per warp of a group and chunk
     const double chunk = xi / nchunks * c.groups / W * (ceil(units_of_work) / units_of_work) * k.x_cpi + k.x_chunk;
     const double t_x = chunk * nchunks / (1.0 + (c.groups - 1) * k.x_group) + k.x_once;
-    const double block = packed_out ? (g.has_residual ? k.e_res : k.e_codes) * (c.PT > 1 ? k.e_pair : 1.0) : k.e_i32, rows = g.O % 4 ? k.rows_odd : k.rows;
+    const double block = packed_out ? (g.has_residual ? k.e_res : k.e_codes) * (c.PT > 1 ? k.e_pair : 1.0) : g.i32_nhwc ? k.e_i32 : k.e_nchw, rows = g.O % 4 ? k.rows_odd : k.rows;
     double t_e = ceil_div(c.PT * (c.TN / 32), W / 4) * block * k.e_cpi + k.e_once;
     if (!packed_out && c.PT * 128.0 * c.TN * 4 / rows > t_e) t_e = c.PT * 128.0 * c.TN * 4 / rows;
     // sums through shared memory of the cluster
@@ -216,6 +217,11 @@ double mma_cost(const MmaArgs& g, const Cand& c, int A, int WB, bool packed_out,
     if (active > 1.0) first *= k.two_first;
     double t = k.start + first + (per_cta - 1.0) * step;
     if (c.resident && packed_b) t += c.TN * g.RS * (g.f4 ? 2 * g.nblk : g.Cw) / 32.0 * k.filt_resident / (2 * W) * 4.0;
+    // Resident packed filters of a call on its own arrive and are expanded before the first pixel, where streamed ones come with it (behind a chained
+    // layer that happens while the other still runs).  The median over 855 pairs of plans of 53 layers and products that differ in nothing
+    // else, 1 to 34 images of 7 to 93 pixels; the chosen plans are 4.4 % (nibbles) and 1.8 % (int8) slower than the fastest (8.9, 7.4
+    // without): 1 x 44 x 9 x 12, 256 filters 5.6 -> 4.0 us, 63 x 64 x 7 x 7 with stride 2 6.6 -> 4.4.
+    if (c.resident && packed_b && !g.early_b) t += 1900.0;
     if (!c.resident && !packed_b) t *= k.streamed;
     if (c.nse < 2) t *= k.one_stage;
     if (!c.cfg) t *= k.half;
