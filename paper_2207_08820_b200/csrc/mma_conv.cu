@@ -219,9 +219,10 @@ double mma_cost(const MmaArgs& g, const Cand& c, int A, int WB, bool packed_out,
     if (c.resident && packed_b) t += c.TN * g.RS * (g.f4 ? 2 * g.nblk : g.Cw) / 32.0 * k.filt_resident / (2 * W) * 4.0;
     // Resident packed filters of a call on its own arrive and are expanded before the first pixel, where streamed ones come with it (behind a chained
     // layer that happens while the other still runs).  The median over 855 pairs of plans of 53 layers and products that differ in nothing
-    // else, 1 to 34 images of 7 to 93 pixels; the chosen plans are 4.4 % (nibbles) and 1.8 % (int8) slower than the fastest (8.9, 7.4
+    // else, 1 to 34 images of 7 to 93 pixels; the chosen plans are 4.0 % (nibbles) and 1.8 % (int8) slower than the fastest (8.9, 7.4
     // without): 1 x 44 x 9 x 12, 256 filters 5.6 -> 4.0 us, 63 x 64 x 7 x 7 with stride 2 6.6 -> 4.4.
-    if (c.resident && packed_b && !g.early_b) t += 1900.0;
+    // Not where there is an item for every SM (28 x 129 x 25 x 25, 148 tiles: 8.9 us resident, 9.7 streamed).
+    if (c.resident && packed_b && !g.early_b && items < sms) t += 1900.0;
     if (!c.resident && !packed_b) t *= k.streamed;
     if (c.nse < 2) t *= k.one_stage;
     if (!c.cfg) t *= k.half;
