@@ -306,6 +306,8 @@ class BitserialFullNet:
     ``bs_stem_codes_f32``, or ``bs_conv2d_f32`` + ``bs_maxpool2d_f32`` + quantise and pack for shapes it does not take), the quantised body
     (:class:`BitserialNet`), floating-point head (``bs_avgpool_codes_f32`` + ``bs_fc_f32``).  Host logic only."""
 
+    MAX_CAPTURES = 16       # recorded passes whose images are kept for :attr:`stem_conv`
+
     def __init__(self, net, params: Dict[str, Dict], device="cuda", batch: Optional[int] = None, engine: str = "tc"):
         self.net = net
         self.batch = batch or net.batch
@@ -316,9 +318,15 @@ class BitserialFullNet:
         self.fc_w, self.fc_b = to(params["fc"]["w"]), to(params["fc"]["bias"])
         h1 = (net.hw + 2 * 3 - 7) // 2 + 1
         h2 = (h1 + 2 - 3) // 2 + 1
-        self._stem_conv = torch.empty(self.batch, 64, h1, h1, dtype=torch.float32, device=self.device)
-        self._stem_pool = torch.empty(self.batch, 64, h2, h2, dtype=torch.float32, device=self.device)
-        self._fused_images: Optional[torch.Tensor] = None      # images of the last pass, where it made no float tensors of the stem
+        self._stem = dict(conv=torch.empty(self.batch, 64, h1, h1, dtype=torch.float32, device=self.device),
+                          pool=torch.empty(self.batch, 64, h2, h2, dtype=torch.float32, device=self.device))
+        self._stem_held: Dict[str, weakref.ref] = {}            # what was handed out of them
+        self._stem_assigned = False                             # the caller has put tensors of their own in their place
+        self._codes_only: Optional[torch.Tensor] = None         # images of the last pass launched, where it made codes only
+        self._captures: Dict[int, torch.Tensor] = {}            # ... of the passes recorded into graphs, by number
+        self._recorded = 0
+        # number of the recorded pass that ran last where it made codes only, -1 where it made the tensors; 0 after a launched one
+        self._replayed = torch.zeros((), dtype=torch.int32, device=self.device)
         C, H, W = net.body.tensor_shapes()[net.body.out_name]
         self.pooled = torch.empty(self.batch, C, dtype=torch.float32, device=self.device)
         self.logits = torch.empty(self.batch, net.classes, dtype=torch.float32, device=self.device)
@@ -327,34 +335,93 @@ class BitserialFullNet:
 
     def run_stem(self, images: torch.Tensor) -> None:
         """The stem as layers of its own: images to ``stem_conv`` and ``stem_pool``."""
-        self._fused_images = None
-        api.conv2d_f32(images, self.stem_w, self.stem_b, stride=2, pad=3, relu=True, out=self._stem_conv)
-        api.maxpool2d_f32(self._stem_conv, 3, 2, 1, out=self._stem_pool)
+        self._stem_layers(images)
+        self._note_pass(None)
 
     def run_front(self, images: torch.Tensor) -> None:
-        """Images to the body's packed input."""
+        """Images to the body's packed input.  Codes only, where the library has the stem as one kernel and nobody holds the stem's tensors."""
         body = self.body
-        if tuple(images.shape) == (self.batch, 3, self.net.hw, self.net.hw) and api.stem_codes_f32(
+        if not self._watched() and tuple(images.shape) == (self.batch, 3, self.net.hw, self.net.hw) and api.stem_codes_f32(
                 images, self.stem_w, self.stem_b, body.act_scale, body.net.a_bits, body.bufs[body.net.in_name]):
-            self._fused_images = images
+            self._note_pass(images)
         else:
             self.run_stem(images)
-            body.pack_input(self._stem_pool)
+            body.pack_input(self._stem["pool"])
+
+    def _stem_layers(self, images: torch.Tensor) -> None:
+        api.conv2d_f32(images, self.stem_w, self.stem_b, stride=2, pad=3, relu=True, out=self._stem["conv"])
+        api.maxpool2d_f32(self._stem["conv"], 3, 2, 1, out=self._stem["pool"])
+
+    def _watched(self) -> bool:
+        return self._stem_assigned or any(r() is not None for r in self._stem_held.values())
+
+    def _note_pass(self, images: Optional[torch.Tensor]) -> None:
+        """Records that the stem's tensors follow from ``images`` from here on, or (None) that they hold what belongs to the last pass.  A pass recorded
+        into a graph records this as well: Python does not run when the graph does."""
+        if torch.cuda.is_current_stream_capturing():
+            self._recorded += 1
+            if images is not None:
+                self._captures[self._recorded] = images
+                if len(self._captures) > self.MAX_CAPTURES:
+                    del self._captures[min(self._captures)]
+            self._replayed.fill_(self._recorded if images is not None else -1)
+        else:
+            self._codes_only = images
+            if self._recorded:
+                self._replayed.zero_()
+
+    def _read_stem(self, name: str) -> torch.Tensor:
+        """The tensor ``name`` of the last pass, evaluated first where that pass made codes only."""
+        images, recording = self._codes_only, torch.cuda.is_current_stream_capturing()
+        if self._recorded and not recording:
+            k = int(self._replayed)
+            if k > 0 and k not in self._captures:
+                raise RuntimeError("the last pass was a replay of a graph recorded long ago: the images it read are not known any more")
+            if k != 0:
+                images = self._captures[k] if k > 0 else None
+        if images is not None:
+            body = self.body
+            self._stem_layers(images)
+            if not recording and not torch.equal(api.bitpack_activations(self._stem["pool"], body.act_scale, body.net.a_bits).view(-1),
+                                                 body.bufs[body.net.in_name].view(-1)):
+                raise RuntimeError("images, stem or body input have changed since the last pass, which made codes only: read stem_conv or stem_pool "
+                                   "before that, or hold one of them while passes run")
+            if not recording:
+                self._note_pass(None)
+        held = self._stem_held.get(name)
+        t = held() if held is not None else None
+        if t is None:
+            t = self._stem[name].detach()
+            self._stem_held[name] = weakref.ref(t)
+        return t
+
+    def _assign_stem(self, name: str, t: torch.Tensor) -> None:
+        self._read_stem(name)
+        self._stem[name] = t
+        self._stem_assigned = True
+        self._stem_held.pop(name, None)
+        self._note_pass(None)
 
     @property
     def stem_conv(self) -> torch.Tensor:
-        """Float output of the stem convolution.  A pass through the fused kernel does not make it: for inspection it is then evaluated from the
-        images of that pass, as they are now."""
-        if self._fused_images is not None:
-            self.run_stem(self._fused_images)
-        return self._stem_conv
+        """Float output of the stem convolution in the last pass, replays of recorded ones included.  While the tensor (or ``stem_pool``) is held, every
+        pass that is launched or recorded writes both.  Otherwise passes make codes only, and a read evaluates the tensors from the images of the
+        last pass; it raises where these have changed since.  A graph recorded while nobody held them makes codes only: after its replays a
+        held tensor is brought up to date by the next read."""
+        return self._read_stem("conv")
+
+    @stem_conv.setter
+    def stem_conv(self, t: torch.Tensor) -> None:
+        self._assign_stem("conv", t)
 
     @property
     def stem_pool(self) -> torch.Tensor:
         """Float output of the stem's pooling, like :attr:`stem_conv`."""
-        if self._fused_images is not None:
-            self.run_stem(self._fused_images)
-        return self._stem_pool
+        return self._read_stem("pool")
+
+    @stem_pool.setter
+    def stem_pool(self, t: torch.Tensor) -> None:
+        self._assign_stem("pool", t)
 
     def run_head(self) -> None:
         body = self.net.body

@@ -121,3 +121,83 @@ def test_classifier_front(hw):
     runner.stem_w = -runner.stem_w
     assert torch.equal(runner.forward(images), logits)
     api.bs_check_status()
+
+
+def classifier(hw=64, seed=8300):
+    net = wl.resnet18_full(batch=2, hw=hw)
+    images = [dev(wl.full_network_input(net, seed + k)) for k in range(3)]
+    return BitserialFullNet(net, wl.full_network_params(net, seed), batch=2), images
+
+
+def stem_layers(runner, images):
+    conv = api.conv2d_f32(images, runner.stem_w, runner.stem_b, 2, 3, True)
+    return conv, api.maxpool2d_f32(conv, 3, 2, 1)
+
+
+def record(runner, static):
+    runner.forward(static)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        runner.forward(static)
+    return graph
+
+
+def test_stem_tensors_follow_replays():
+    """Python does not run on a replay: a read between two replays must not leave the first one's tensors behind."""
+    runner, (a, b, c) = classifier()
+    static = a.clone()
+    graph = record(runner, static)
+
+    def check(images):
+        conv, pool = stem_layers(runner, images)
+        assert torch.equal(runner.stem_conv, conv) and torch.equal(runner.stem_pool, pool)
+
+    for images in (a, b, b, c):
+        static.copy_(images)
+        graph.replay()
+        check(images)
+        check(images)
+    runner.forward(a)                       # launched after replays, and replayed after a launch
+    check(a)
+    graph.replay()
+    check(c)
+    runner.run_stem(b)
+    check(b)
+    static.copy_(a)
+    graph.replay()
+    check(a)
+    kept = runner.stem_pool                 # recorded while held: the graph writes the tensors
+    second = record(runner, static)
+    static.copy_(b)
+    second.replay()
+    assert torch.equal(kept, stem_layers(runner, b)[1])
+    check(b)
+    static.copy_(c)
+    graph.replay()
+    check(c)
+
+
+def test_stem_tensors_that_are_kept_or_assigned():
+    runner, (a, b, c) = classifier()
+    logits = runner.forward(a).clone()
+    kept = runner.stem_pool
+    assert runner.stem_pool is kept
+    runner.forward(b)
+    assert torch.equal(kept, stem_layers(runner, b)[1])
+    b.zero_()                               # the pass wrote its tensors: its images may go
+    assert torch.equal(kept, runner.stem_pool)
+    assert torch.equal(runner.forward(a), logits)
+    del kept
+    runner.forward(c)
+    d = c.clone()
+    c.zero_()
+    with pytest.raises(RuntimeError):       # codes only, and their images are gone
+        runner.stem_conv
+    runner.forward(d)
+    mine = torch.zeros_like(runner.stem_pool)
+    runner.stem_pool = mine
+    assert bool((mine == 0).all())
+    runner.forward(a)
+    assert torch.equal(mine, stem_layers(runner, a)[1]) and torch.equal(runner.stem_pool, mine)
+    assert torch.equal(runner.logits, logits)
