@@ -231,8 +231,9 @@ int bitserial_gemm_noalloc(const uint32_t* a_packed, const uint32_t* w_packed, i
  *   bs_tc_weights_bytes    bytes of the prepared filter tensor (0 on bad input).
  *   bs_tc_prepare_weights  packed weights [O][R][S][Cw][w_bits] -> tiles for layers of a_bits activation bits: nibbles
  *                          [ceil(C/64)][ceil(O/128)*16][R*S][2][8][16 bytes] where a_bits and w_bits are at most 2 (the first half of the
- *                          tensor or so), int8 [C/32][ceil(O/128)*16][R*S][2][8][16] otherwise.  Use them with layers of the same widths: a layer
- *                          that meets the other form has undefined outputs, and bs_check_status then returns BS_ERR_INVALID_ARG.
+ *                          tensor or so), int8 [C/32][ceil(O/128)*16][R*S][2][8][16] otherwise.  One tensor serves layers of every a_bits; a
+ *                          layer that meets the other form converts its filters in each launch, with one warp of each SM, so prepare
+ *                          them for the widths they run with.
  */
 size_t bs_tc_weights_bytes(int O, int C, int R, int S);
 int bs_tc_prepare_weights(const uint32_t* wgt_packed, int O, int C, int R, int S, int w_bits, bs_sign_t w_sign,
@@ -339,7 +340,7 @@ int bs_fc_f32(const float* x, const float* w, const float* bias, int N, int K, i
 /*
  * bs_check_status -- synchronises `stream`, then reads and clears the device status word of the current
  * device.  Returns BS_ERR_TIMEOUT if any kernel since the last check gave up on a bounded wait (its
- * outputs are then undefined), BS_ERR_INVALID_ARG if one met filters prepared for other widths, BS_ERR_CUDA if the stream reports an error, else BS_OK.
+ * outputs are then undefined), BS_ERR_CUDA if the stream reports an error, else BS_OK.
  */
 int bs_check_status(void* stream);
 

@@ -136,8 +136,8 @@ def bitserial_gemm(a_packed: torch.Tensor, w_packed: torch.Tensor, K: int, *, a_
 
 
 def tc_prepare_weights(wgt_packed: torch.Tensor, C: int, w_sign: int, a_bits: int, stream=None) -> torch.Tensor:
-    """Packed weights [O,R,S,Cw,w_bits] -> filter tiles for the tensor-core entry points, in layers of ``a_bits`` activation bits (nibbles where
-    both widths are at most 2, int8 otherwise; a layer that meets the other form makes :func:`bs_check_status` raise)."""
+    """Packed weights [O,R,S,Cw,w_bits] -> filter tiles for the tensor-core entry points, made for layers of ``a_bits`` activation bits (nibbles where
+    both widths are at most 2, int8 otherwise; layers that need the other form take these too and convert them in each launch, more slowly)."""
     O, R, S, Cw, w_bits = wgt_packed.shape
     nbytes = lib().bs_tc_weights_bytes(O, C, R, S)
     if nbytes == 0:

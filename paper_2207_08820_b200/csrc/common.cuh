@@ -7,8 +7,8 @@
 
 namespace bs {
 
-// Device status word: kernels OR error bits into it when a bounded wait runs out or prepared filters have the wrong form.
-enum : int { STATUS_TIMEOUT = 1, STATUS_FILTERS = 2 };      // bits; FILTERS: prepared filters of another form
+// Device status word: kernels OR error bits into it when a bounded wait runs out.
+enum : int { STATUS_TIMEOUT = 1 };
 int* status_device_ptr();   // device address of the status word of the current device (host call)
 int device_sm_count();      // multiprocessors of the CURRENT device (looked up once per device ordinal; 0 on error)
 

@@ -17,6 +17,7 @@ __host__ __device__ constexpr int mma_channel_of_byte(int b) { return 8 * (b & 3
 // the signs.  Also the form of its prepared filters, so it depends only on what their preparation knows.
 constexpr bool mma_nibbles(int C, int RS, int a_bits, int w_bits) { return a_bits <= 2 && w_bits <= 2 && static_cast<long long>(C) * RS * 9 < 4000000; }
 // Prepared nibbles end with this word, four pairs of negative zeros, in room that holds no code; int8 codes (-8 .. 15) never contain its bytes.
+// A layer tells the form of its filters by it and converts them where it needs the other one.
 constexpr unsigned MM_NIBBLE_MARK = 0x88888888u;
 
 // Runs one layer.  `wgt` are filters prepared by bs_tc_prepare_weights; when it is null the packed filters `wgt_packed` are

@@ -511,6 +511,49 @@ __device__ __forceinline__ void expand_filters_resident(const MmaArgs& g, uint32
     }
 }
 
+// ----------------------------------------------------------------------------- prepared filters of the other form
+
+// Filters prepared for layers of other widths (bs_tc_prepare_weights: nibbles or int8, told apart by MM_NIBBLE_MARK) -> `nb` K steps from b0
+// on in the form of this layer, by one warp: 16-byte vectors [K step][filter / 8][tap][half][filter % 8] at `dst`.  A layer with such filters
+// is right but slow; preparing them for its widths is the remedy.
+template <bool F4>
+static __device__ __noinline__ void convert_filters(const MmaArgs& g, unsigned char* dst, int o0, int b0, int nb, int lane)
+{
+    const int per = g.TN * g.RS * 2;
+    const size_t stride = static_cast<size_t>(g.opad) * g.RS * 2;
+    const uint4* src = reinterpret_cast<const uint4*>(g.wgt) + static_cast<size_t>(o0) * g.RS * 2;
+    for (int b = 0; b < nb; ++b)
+#pragma unroll 4
+        for (int r = lane; r < per; r += 32) {
+            uint32_t o[4] = {0, 0, 0, 0};
+            if (F4) {
+                // a channel word is one vector here, two there
+                const int cw = 2 * (b0 + b) + (r >> 3 & 1);
+                if (cw < g.Cw) {
+                    const uint4 lo = src[cw * stride + (r & ~8)], hi = src[cw * stride + (r | 8)];
+                    const uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const uint32_t neg = (w[k] >> 7) & 0x01010101u, m = neg * 255u;
+                        o[k & 3] |= ((__vsub4(w[k] ^ m, m) & 0x07070707u) | neg << 3) << (k & 4);
+                    }
+                }
+            } else {
+                const int cw = b0 + b, shift = r & 8 ? 4 : 0;
+                const uint4 n = src[(cw >> 1) * stride + ((r & ~8) | (cw & 1) << 3)];
+                const uint32_t w[4] = {n.x, n.y, n.z, n.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const uint32_t v = w[k] >> shift, m = ((v >> 3) & 0x01010101u) * 255u;
+                    o[k] = __vsub4((v & 0x07070707u) ^ m, m);
+                }
+            }
+            mm_sts(smem_u32(dst) + static_cast<uint32_t>(b * per + r) * 16u, o[0], o[1], o[2], o[3]);
+        }
+    fence_proxy_async();
+    __syncwarp();
+}
+
 // ----------------------------------------------------------------------------- MMA issue
 
 // Fixed kernel sizes: the taps are unrolled, nothing but additions on uniform registers between the MMAs.
@@ -572,7 +615,7 @@ struct MmaChunks {
 };
 
 struct MmaIssue {
-    uint64_t *full_e, *empty_e, *full_acc, *empty_acc, *wgt_full;
+    uint64_t *full_e, *empty_e, *full_acc, *empty_acc, *wgt_full, *form_ok;
     uint32_t smem0, tmem;
     int items;
     bool resident;
@@ -599,6 +642,7 @@ __device__ __forceinline__ void issue_items(const MmaArgs& g, const MmaIssue& m)
     const uint32_t sf = m.tmem + static_cast<uint32_t>(g.sf_col);
     unsigned limit = 1u << 20;
     if (m.resident) mm_wait_uniform(m.wgt_full, 0, limit);
+    if (m.form_ok) mm_wait_uniform(m.form_ok, 0, limit);
     MM_TRACE((threadIdx.x & 31) == 0, TR_WGT, 0);
 #ifdef BS_TRACE
     int mseq = 0;
@@ -1301,6 +1345,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 30);
     int* fast_ok = reinterpret_cast<int*>(bars + 31);
     uint64_t* red_full = bars + 32;     // partial sums of a split item
+    uint64_t* form_ok = bars + 33;      // prepared filters are in the form of this layer, or have been brought into it
 
     constexpr bool packed_b = WB > 0;
     constexpr int WBX = WB > 0 ? WB : 1;
@@ -1319,6 +1364,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
         for (int s = 0; s < 2; ++s) { mbar_init(&full_acc[s], 1); mbar_init(&empty_acc[s], EW); }
         mbar_init(wgt_full, packed_b ? XW + EW : 1);
         mbar_init(bulk_full, 1);
+        mbar_init(form_ok, 1);
         if (SPLIT) mbar_init(red_full, (g.split - 1) * EW);
         for (int s = 0; s < MM_STAGES; ++s) { mbar_init(&full_p[s], 1); mbar_init(&empty_p[s], XW / g.groups); }
         *fast_ok = 1;
@@ -1342,14 +1388,15 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
     // a CTA with resident filters keeps its filter tile; otherwise the filter tile runs fastest over the items
     if (warp == WARP_COPY) {
         // ------------------------------------------------------------------ copy warp: prepared filters, and packed rows by TMA
-        if (lane == 0) {
+        // One lane issues the copies; with prepared filters the others follow, in case they are in the other form.
+        if (!packed_b || lane == 0) {
             bool waited = false, ok = true;
             const size_t blk_stride = static_cast<size_t>(g.opad) * g.RS * 32;
             const unsigned blk_bytes = static_cast<unsigned>(g.TN * g.RS * 32);
+            const int o0 = static_cast<int>(blockIdx.x % static_cast<unsigned>(g.tiles_o)) * g.TN;       // of resident filters
             if (!packed_b || (resident && g.bulk_b)) {
                 if (!g.early_b) { mm_pdl_wait(); waited = true; }
-                if (resident) {
-                    const int o0 = static_cast<int>(blockIdx.x % static_cast<unsigned>(g.tiles_o)) * g.TN;
+                if (resident && lane == 0) {
                     if (packed_b) {
                         // the packed tile parks in the ring of expanded pixels, which nobody uses yet
                         const int words = (g.O - o0 < g.TN ? g.O - o0 : g.TN) * g.RS * g.Cw * WBX;
@@ -1362,6 +1409,20 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                     }
                 }
             }
+            // The form is read beside the first copies, which are made as if it were the expected one: nothing waits for it that would not wait
+            // for them.  Otherwise what has landed is overwritten before the MMAs may begin.
+            uint32_t mark = 0;
+            if (!packed_b) asm volatile("ld.global.b32 %0, [%1];" : "=r"(mark) : "l"(g.wgt + blk_stride * g.Cw - 4) : "memory");
+            bool first = !packed_b, other = false;
+            auto check_form = [&](uint64_t* landed, int o, int b0, int nb) {
+                other = (mark == MM_NIBBLE_MARK) != F4;
+                if (other) {
+                    if (ok) ok = mm_wait(landed, 0);
+                    convert_filters<F4>(g, mm_smem, o, b0, nb, lane);
+                }
+                if (lane == 0) mm_arrive(form_ok);
+                first = false;
+            };
             const bool stream = stream_prepared;
             if (stream || g.tma) {
                 int ib = 0, ip = 0;
@@ -1369,41 +1430,46 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                 for (MmaWalk w(g, walk_log); w.m < g.tiles_m && ok; w.next(g)) {
                     const int8_t* src = g.wgt + static_cast<size_t>(w.o) * g.TN * g.RS * 32;
                     for (int c = range.beg; c < range.beg + range.n && ok; ++c) {
+                        const int step = F4 ? g.units : g.units * 2, b0 = c * step;
+                        const int nb = g.nblk - b0 < step ? g.nblk - b0 : step;
                         if (stream) {
                             ok = mm_wait(&empty_e[ib], pb ^ 1u);
                             if (!ok) break;
-                            const int step = F4 ? g.units : g.units * 2, b0 = c * step;
-                            const int nb = g.nblk - b0 < step ? g.nblk - b0 : step;
-                            mbar_expect_tx(&full_e[ib], blk_bytes * nb);
-                            for (int b = 0; b < nb; ++b)
-                                mm_bulk(mm_smem + static_cast<size_t>(ib) * g.b_bytes + static_cast<size_t>(b) * blk_bytes, src + (b0 + b) * blk_stride, blk_bytes, &full_e[ib]);
+                            unsigned char* dst = mm_smem + static_cast<size_t>(ib) * g.b_bytes;
+                            if (other) {
+                                convert_filters<F4>(g, dst, w.o * g.TN, b0, nb, lane);
+                                if (lane == 0) mm_arrive(&full_e[ib]);
+                            } else if (lane == 0) {
+                                mbar_expect_tx(&full_e[ib], blk_bytes * nb);
+                                for (int b = 0; b < nb; ++b) mm_bulk(dst + static_cast<size_t>(b) * blk_bytes, src + (b0 + b) * blk_stride, blk_bytes, &full_e[ib]);
+                            }
                             if (++ib == g.nse) { ib = 0; pb ^= 1u; }
                         }
                         if (g.tma) {
                             if (!waited) { mm_pdl_wait(); waited = true; }
                             ok = mm_wait(&empty_p[ip], pp ^ 1u);
                             if (!ok) break;
-                            const bool fb = packed_b && !resident;
-                            mbar_expect_tx(&full_p[ip], static_cast<unsigned>(BM * g.rowA + (fb ? g.TN * g.rowB : 0)));
-                            unsigned char* dst = mm_smem + g.off_stg + ip * g.stg_bytes;
-                            const int rows = BM < 256 ? BM : 256;
-                            for (int r = 0; r < BM; r += rows) tma_load_2d(dst + r * g.rowA, &g.tmA, &full_p[ip], c * (g.rowA >> 2), w.m * BM + r);
-                            if (fb) tma_load_2d(mm_smem + g.off_bstg + ip * g.bstg_bytes, &g.tmB, &full_p[ip], c * (g.rowB >> 2), w.o * g.TN);
+                            if (lane == 0) {
+                                const bool fb = packed_b && !resident;
+                                mbar_expect_tx(&full_p[ip], static_cast<unsigned>(BM * g.rowA + (fb ? g.TN * g.rowB : 0)));
+                                unsigned char* dst = mm_smem + g.off_stg + ip * g.stg_bytes;
+                                const int rows = BM < 256 ? BM : 256;
+                                for (int r = 0; r < BM; r += rows) tma_load_2d(dst + r * g.rowA, &g.tmA, &full_p[ip], c * (g.rowA >> 2), w.m * BM + r);
+                                if (fb) tma_load_2d(mm_smem + g.off_bstg + ip * g.bstg_bytes, &g.tmB, &full_p[ip], c * (g.rowB >> 2), w.o * g.TN);
+                            }
                             if (++ip == g.nsp) { ip = 0; pp ^= 1u; }
                         }
+                        if (first) check_form(resident ? wgt_full : &full_e[0], resident ? o0 : w.o * g.TN, resident ? 0 : b0, resident ? g.nblk : nb);
                     }
                 }
             }
-            if (!ok) atomicOr(g.status, STATUS_TIMEOUT);
-            if (!packed_b && blockIdx.x == 0) {         // filters prepared for other widths; read last, when nothing waits for this warp
-                const uint32_t mark = reinterpret_cast<const uint32_t*>(g.wgt + blk_stride * g.Cw)[-1];
-                if ((mark == MM_NIBBLE_MARK) != F4) atomicOr(g.status, STATUS_FILTERS);
-            }
+            if (first && resident && ok) check_form(wgt_full, o0, 0, g.nblk);
+            if (!ok && lane == 0) atomicOr(g.status, STATUS_TIMEOUT);
         }
         __syncwarp();
     } else if (warp == WARP_MMA) {
         // ------------------------------------------------------------------ MMA issuer (all lanes in step)
-        const MmaIssue m{full_e, empty_e, full_acc, empty_acc, wgt_full, smem0, tmem, items, resident};
+        const MmaIssue m{full_e, empty_e, full_acc, empty_acc, wgt_full, packed_b ? nullptr : form_ok, smem0, tmem, items, resident};
         if (g.R == 1) issue_items<TAPS_1, SPLIT, F4>(g, m);
         else if (g.R == 3 && g.stride == 1) issue_items<TAPS_3S1, SPLIT, F4>(g, m);
         else if (g.R == 3 && g.pad == 1) issue_items<TAPS_3S2, SPLIT, F4>(g, m);

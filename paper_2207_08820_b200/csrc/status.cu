@@ -133,7 +133,7 @@ extern "C" int bs_check_status(void* stream)
     if (h != 0) {
         int zero = 0;
         cudaMemcpyToSymbol(bs::g_status, &zero, sizeof(int));
-        return (h & bs::STATUS_TIMEOUT) ? BS_ERR_TIMEOUT : BS_ERR_INVALID_ARG;
+        return BS_ERR_TIMEOUT;
     }
     return BS_OK;
 }

@@ -2,6 +2,7 @@
 them in use, at both sides of the reduction length from which int8 takes over; every pair of signs; odd numbers of channel words."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 from paper_2207_08820_b200 import api, workloads as wl
@@ -53,19 +54,34 @@ def test_signs(C, O, k, s, a, a_sign, w, w_sign):
     api.bs_check_status()
 
 
-@pytest.mark.parametrize("C", [32, 64, 96])
-@pytest.mark.parametrize("prepared,run", [(2, 3), (4, 1), (2, 1), (3, 4)])
-def test_filters_of_the_other_form_are_reported(C, prepared, run):
+# resident and streamed filters, an odd number of channel words, rows by tensor copies, five taps a side
+@pytest.mark.parametrize("C,O,k,hw", [(32, 128, 3, 8), (64, 128, 3, 8), (96, 128, 3, 8), (64, 40, 5, 9), (512, 256, 1, 12), (1024, 300, 3, 10)])
+@pytest.mark.parametrize("prepared,run", [(2, 3), (4, 1), (2, 1), (3, 4), (3, 2), (2, 4)])
+@pytest.mark.parametrize("w,w_sign", [(2, api.SIGNED), (1, api.BIPOLAR), (2, api.UNSIGNED), (1, api.SIGNED)])
+def test_filters_prepared_for_other_widths(C, O, k, hw, prepared, run, w, w_sign):
+    """One prepared tensor serves every activation width, whatever form it has (int8 ones saved by earlier versions among them)."""
     rng = np.random.default_rng(C)
-    x, f = wl.rand_codes(rng, (1, C, 8, 8), run, 0), wl.rand_codes(rng, (128, C, 3, 3), 2, api.SIGNED)
-    xa, wp = api.bitpack_activations(dev(x), 1.0, run), api.pack_weights(dev(f), 2, api.SIGNED)
-    if not api.tc_supported(1, C, 8, 8, 128, 3, 1, 1, run, 0, 2, api.SIGNED):
+    x, f = wl.rand_codes(rng, (1, C, hw, hw), run, 0), wl.rand_codes(rng, (O, C, k, k), w, w_sign)
+    xa, wp = api.bitpack_activations(dev(x), 1.0, run), api.pack_weights(dev(f), w, w_sign)
+    if not api.tc_supported(1, C, hw, hw, O, k, 1, k // 2, run, 0, w, w_sign):
         pytest.skip("records of other sizes take no prepared filters")
-    acc, _ = api.bitserial_conv2d(xa, wp, C=C, pad=1, want_i32=True, wgt_tc=api.tc_prepare_weights(wp, C, api.SIGNED, prepared))
-    if (prepared <= 2) == (run <= 2):
+    wt = api.tc_prepare_weights(wp, C, w_sign, prepared)
+    want = oracle.conv2d_i32(x, f, 1, k // 2)
+    for chained in (False, True):
+        torch.cuda.synchronize()
+        acc, _ = api.bitserial_conv2d(xa, wp, C=C, pad=k // 2, w_sign=w_sign, want_i32=True, wgt_tc=wt, chained=chained)
         api.bs_check_status()
-        assert np.array_equal(acc.cpu().numpy(), oracle.conv2d_i32(x, f, 1, 1))
-    else:
-        with pytest.raises(api.BitserialError):
-            api.bs_check_status()
-        api.bs_check_status()               # reported once
+        assert np.array_equal(acc.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("prepared,run", [(2, 3), (4, 1)])
+@pytest.mark.parametrize("M,N,K", [(300, 70, 4032), (1000, 1024, 512), (3000, 600, 64)])
+def test_products_with_filters_prepared_for_other_widths(M, N, K, prepared, run):
+    rng = np.random.default_rng(K)
+    a, w = wl.rand_codes(rng, (M, K), run, 0), wl.rand_codes(rng, (N, K), 2, api.SIGNED)
+    wp = api.bs_pack_rows(dev(w), 2, api.SIGNED)
+    assert api.tc_supported(1, K, 1, M, N, 1, 1, 0, run, 0, 2, api.SIGNED)
+    wt = api.tc_prepare_weights(wp.view(N, 1, 1, -1, 2), K, api.SIGNED, prepared)
+    got, _ = api.bitserial_gemm_tc(api.bs_pack_rows(dev(a), run, 0), wt, N, K, 2)
+    api.bs_check_status()
+    assert np.array_equal(got.cpu().numpy(), oracle.gemm_i32(a, w))
