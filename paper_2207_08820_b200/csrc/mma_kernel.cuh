@@ -212,6 +212,11 @@ __device__ __forceinline__ void mm_landed(uint32_t (&v)[16])
     asm volatile("" : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
                       "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]));
 }
+__device__ __forceinline__ void mm_landed(uint32_t (&v)[32])
+{
+    mm_landed(*reinterpret_cast<uint32_t (*)[16]>(&v[0]));
+    mm_landed(*reinterpret_cast<uint32_t (*)[16]>(&v[16]));
+}
 __device__ __forceinline__ void mm_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void mm_st8(uint32_t taddr, uint32_t x)
 {
@@ -939,6 +944,7 @@ static __device__ __noinline__ void epilogue_formula(const MmaArgs& g, uint32_t 
     uint32_t v[32], rw[4] = {0, 0, 0, 0}, ow[4] = {0, 0, 0, 0};
     mm_ld32(addr, v);
     mm_ld_wait();
+    mm_landed(v);
     if (live) {
         for (int c = 0; c < 32; ++c) v[c] = acc_int(g.f4, v[c], bias);
         if (g.residual) load_residual(g, pix, ob, rw);
@@ -1263,6 +1269,7 @@ __device__ __forceinline__ bool epilogue_general(const MmaArgs& g, const MmaEpi&
                 uint32_t v[32];
                 mm_ld32(col, v);
                 mm_ld_wait();
+                mm_landed(v);
                 if (F4)
 #pragma unroll
                     for (int c = 0; c < 32; ++c) v[c] = acc_int(true, v[c], 0u);
