@@ -160,10 +160,10 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows, int sms)
 
 // Time model of a candidate in SM cycles: the pipeline of one CTA (expansion, MMAs, epilogue; a stage's hand-off included) over
 // its items, plus what nothing overlaps at both ends.  The constants are fitted to timed plans (B200 at 1.95 GHz): int8 to about 2500 of
-// 45 layers and products (1 to 300 pixels wide, 32 to 4608 channels, batches 1 to 64), the plan with the lowest modelled time being on
-// average 2 to 3 % and at most 16 % slower than the fastest; nibbles to 17000 of 77, on average 1.3 % and at most 19 % slower (with the
-// constants of int8: 4.5 % and 91 %, most of it from filters staged piece by piece, which cost twice what was assumed).  Their int32 in rows of
-// pixels apart, over 17 layers: 2.5 % and 11 % with 180, 4.0 % and 20 % with the 360 of rows of filters (57 x 64 x 35 x 33, 288 filters: 32.7 -> 30.2 us).
+// 45 layers and products (1 to 300 pixels wide, 32 to 4608 channels, batches 1 to 64), nibbles to 17000 of 77; then what only packed
+// filters and int32 outputs have (filt_*, resident_once, e_i32, e_nchw, rows*) to 60000 plans of 670 calls on their own, three quarters of
+// them, judged on the rest: the plan with the lowest modelled time is on average 3.8 % slower than the fastest there on either form, 4.3 and
+// 4.9 % before (a flat 1900 cycles for resident filters of less than an item per SM, int32 in rows of pixels at the rate of odd rows of filters).
 struct MmaFit {
     double mma_chunk;                       // cycles per chunk beside its MMAs
     double unit, one_word, flat, staged;    // expansion, instructions per warp and 64-channel unit of 32 rows: arithmetic, of 32 channels only, copies by TMA, by thread
@@ -174,10 +174,10 @@ struct MmaFit {
     double rows, rows_odd;                  // bytes per cycle of int32 rows, of rows that are not multiples of 16 bytes
     double split;                           // cycles of a split item beside its sums
     double l2;                              // bytes per cycle of streamed prepared filters
-    double ipc, two_first, start, filt_resident, streamed, one_stage, half;
+    double ipc, two_first, start, filt_resident, resident_once, streamed, one_stage, half;   // filt_resident, resident_once: resident packed filters, cycles per channel word of 32 rows, per launch
 };
-constexpr MmaFit FIT_INT8 = {148, 102, 102, 1, 41, 20, 20, 5.34, 629, 0.83, 628, 215, 138, 94, 94, 4.59, 997, 1, 29.6, 12.2, 2200, 68.7, 3.08, 1.19, 4215, 122, 1.07, 1.11, 0.93};
-constexpr MmaFit FIT_NIBBLES = {262, 63, 31, 1, 92.5, 64.2, 127, 5.49, 457, 0.889, 705, 247, 114, 360, 180, 4.01, 982, 0.931, 24.3, 12.2, 4236, 98.3, 1.45, 1.226, 3484, 223, 1.076, 0.961, 0.934};
+constexpr MmaFit FIT_INT8 = {148, 102, 102, 1, 41, 20, 59, 5.34, 629, 0.83, 628, 215, 138, 94, 113, 4.59, 997, 1, 17.2, 12.8, 2200, 68.7, 3.08, 1.19, 4215, 102, 910, 1.07, 1.11, 0.93};
+constexpr MmaFit FIT_NIBBLES = {262, 63, 31, 1, 92.5, 77.8, 123, 5.49, 457, 0.889, 705, 247, 114, 263, 122, 4.01, 982, 0.931, 19.2, 15, 4236, 98.3, 1.45, 1.226, 3484, 205, 1540, 1.076, 0.961, 0.934};
 
 double mma_cost(const MmaArgs& g, const Cand& c, int A, int WB, bool packed_out, int sms)
 {
@@ -194,7 +194,7 @@ double mma_cost(const MmaArgs& g, const Cand& c, int A, int WB, bool packed_out,
     const double units_of_work = static_cast<double>(row_groups) * c.units * c.groups / W;       // per warp of a group and chunk
     const double chunk = xi / nchunks * c.groups / W * (ceil(units_of_work) / units_of_work) * k.x_cpi + k.x_chunk;
     const double t_x = chunk * nchunks / (1.0 + (c.groups - 1) * k.x_group) + k.x_once;
-    const double block = packed_out ? (g.has_residual ? k.e_res : k.e_codes) * (c.PT > 1 ? k.e_pair : 1.0) : g.i32_nhwc ? k.e_i32 : k.e_nchw, rows = g.O % 4 ? k.rows_odd : k.rows;
+    const double block = packed_out ? (g.has_residual ? k.e_res : k.e_codes) * (c.PT > 1 ? k.e_pair : 1.0) : g.i32_nhwc ? k.e_i32 : k.e_nchw, rows = g.i32_nhwc && g.O % 4 ? k.rows_odd : k.rows;
     double t_e = ceil_div(c.PT * (c.TN / 32), W / 4) * block * k.e_cpi + k.e_once;
     if (!packed_out && c.PT * 128.0 * c.TN * 4 / rows > t_e) t_e = c.PT * 128.0 * c.TN * 4 / rows;
     // sums through shared memory of the cluster
@@ -217,12 +217,9 @@ double mma_cost(const MmaArgs& g, const Cand& c, int A, int WB, bool packed_out,
     if (active > 1.0) first *= k.two_first;
     double t = k.start + first + (per_cta - 1.0) * step;
     if (c.resident && packed_b) t += c.TN * g.RS * (g.f4 ? 2 * g.nblk : g.Cw) / 32.0 * k.filt_resident / (2 * W) * 4.0;
-    // Resident packed filters of a call on its own arrive and are expanded before the first pixel, where streamed ones come with it (behind a chained
-    // layer that happens while the other still runs).  The median over 855 pairs of plans of 53 layers and products that differ in nothing
-    // else, 1 to 34 images of 7 to 93 pixels; the chosen plans are 4.0 % (nibbles) and 1.8 % (int8) slower than the fastest (8.9, 7.4
-    // without): 1 x 44 x 9 x 12, 256 filters 5.6 -> 4.0 us, 63 x 64 x 7 x 7 with stride 2 6.6 -> 4.4.
-    // Not where there is an item for every SM (28 x 129 x 25 x 25, 148 tiles: 8.9 us resident, 9.7 streamed).
-    if (c.resident && packed_b && !g.early_b && items < sms) t += 1900.0;
+    // Resident packed filters of a call on its own also hold up the first pixel until every warp has expanded its share, where streamed
+    // ones come with it (behind a chained layer that happens while the other still runs).
+    if (c.resident && packed_b && !g.early_b) t += k.resident_once;
     if (!c.resident && !packed_b) t *= k.streamed;
     if (c.nse < 2) t *= k.one_stage;
     if (!c.cfg) t *= k.half;
