@@ -262,7 +262,14 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
     g.res_cw_total = ceil_div(p->res_c_total > 0 ? p->res_c_total : 1, 32);
     g.i32_nhwc = p->i32_layout == BS_NHWC;
     g.opad = up(p->O, 128);
-    g.f4 = mma_nibbles(p->C, g.RS, p->a_bits, p->w_bits);
+    // Nibbles, but int8 for packed filters where the reduction is so short that nibbles save few MMAs or none (up to 32 channels leave half of a
+    // K step empty) and the way out decides: int8 sums need no conversion to int32.  Time on nibbles over time on int8, the
+    // plans chosen for 220 layers: int32 in rows of pixels, 1x1: 32 channels 1.07, 64 and 96 1.05, 128 1.03, 160 and 192 1.02, to 288 1.00,
+    // more 0.96 (14 x 19 x 72 x 70, 125 filters: 12.1 -> 10.2 us); larger windows, up to 32 channels, 2048 outputs per SM and more: 3x3 1.01, 5x5 1.10, fewer
+    // outputs 0.98 and 0.97; codes of 5x5 windows over up to 32 channels 1.12 and 0.89 on these sides, of 3x3 windows 0.96 and 0.94.
+    const bool short_k = g.Cw == 1 && static_cast<double>(g.N) * g.P * g.Q * g.O >= 2048.0 * sms;
+    const bool pixel_rows = out_i32 && !out_packed && !g.i32_nhwc;
+    g.f4 = mma_nibbles(p->C, g.RS, p->a_bits, p->w_bits) && !(packed_b && (pixel_rows ? short_k || (g.R == 1 && g.Cw <= 6) : short_k && g.R >= 5 && !out_i32));
     const double bound = static_cast<double>(p->C) * g.RS * max_abs_of(p->a_bits, p->a_sign) * max_abs_of(p->w_bits, p->w_sign);
     g.acc_bound = static_cast<float>(bound);
     g.preset = out_packed && !out_i32 && bound < 4.0e6 && p->out_sign != BS_BIPOLAR &&

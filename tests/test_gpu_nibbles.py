@@ -85,3 +85,25 @@ def test_products_with_filters_prepared_for_other_widths(M, N, K, prepared, run)
     got, _ = api.bitserial_gemm_tc(api.bs_pack_rows(dev(a), run, 0), wt, N, K, 2)
     api.bs_check_status()
     assert np.array_equal(got.cpu().numpy(), oracle.gemm_i32(a, w))
+
+
+# both sides of the lines at which packed filters of one- and two-bit layers go to int8: channels of 1x1 layers, one channel word and more, few outputs
+# and many (a few more than 2048 for each of 148 SMs), windows of codes
+@pytest.mark.parametrize("C,O,k,N,hw,out", [(9, 33, 1, 2, 13, "acc"), (192, 40, 1, 2, 13, "acc"), (193, 40, 1, 2, 13, "acc"), (32, 66, 3, 4, 34, "acc"), (33, 66, 3, 4, 34, "acc"),
+                                            (20, 66, 5, 4, 34, "acc"), (20, 8, 5, 1, 9, "acc"), (32, 66, 5, 4, 34, "codes"), (31, 64, 5, 1, 9, "codes"), (32, 65, 7, 4, 35, "codes"),
+                                            (32, 66, 3, 4, 34, "codes")])
+@pytest.mark.parametrize("a,a_sign,w,w_sign", [(2, 0, 2, 1), (1, 0, 1, 2), (2, 1, 1, 1), (1, 0, 2, 1)])
+def test_lines_between_the_forms(C, O, k, N, hw, out, a, a_sign, w, w_sign):
+    rng = np.random.default_rng(C + O)
+    x, f = wl.rand_codes(rng, (N, C, hw, hw), a, a_sign), wl.rand_codes(rng, (O, C, k, k), w, w_sign)
+    xa, wp = api.bitpack_activations(dev(x), 1.0, a, a_sign), api.pack_weights(dev(f), w, w_sign)
+    kw = dict(C=C, stride=1, pad=k // 2, a_sign=a_sign, w_sign=w_sign)
+    want = oracle.conv2d_i32(x, f, 1, k // 2)
+    if out == "acc":
+        got, _ = api.bitserial_conv2d(xa, wp, want_i32=True, **kw)
+        assert np.array_equal(got.cpu().numpy(), want)
+    else:
+        scale, bias = np.full(O, 0.03, np.float32), np.linspace(-1.0, 2.0, O, dtype=np.float32)
+        _, got = api.bitserial_conv2d(xa, wp, scale=dev(scale), bias=dev(bias), relu=True, out_bits=2, **kw)
+        assert np.array_equal(api.bitunpack_activations(got, O, 2).cpu().numpy(), oracle.requantize(want, scale, bias, True, 2))
+    api.bs_check_status()
