@@ -324,8 +324,9 @@ int bitserial_gemm_tc(const uint32_t* a_packed, const int8_t* w_tc, int M, int N
  *                       x [N][K], w [J][K], out [N][J].
  *   bs_stem_codes_f32   bs_conv2d_f32 with ReLU, bs_maxpool2d_f32 (3, 2, 1) and the NCHW form of bitpack_activations (unsigned codes) in one
  *                       call: the same codes bit for bit, none of the float tensors in between.  Takes C = 3, O = 64, 7 x 7, stride 2,
- *                       pad 3, 2-bit codes, even W up to about 280; BS_ERR_UNSUPPORTED for anything else (use the three calls).
+ *                       pad 3, 2-bit codes, even W up to 306; BS_ERR_UNSUPPORTED for anything else (use the three calls).
  *                       x, w, out 16-byte aligned; out [N][(P + 1) / 2][(Q + 1) / 2][2][2] words.
+ *   bs_stem_codes_supported  1 where bs_stem_codes_f32 takes a layer, else 0; needs no device.
  * All asynchronous on `stream`; errors BS_ERR_INVALID_ARG / BS_ERR_ALIGNMENT / BS_ERR_UNSUPPORTED / BS_ERR_CUDA.
  */
 int bs_conv2d_f32(const float* x, const float* w, const float* bias, int N, int C, int H, int W, int O, int R, int S, int stride,
@@ -333,6 +334,7 @@ int bs_conv2d_f32(const float* x, const float* w, const float* bias, int N, int 
 int bs_maxpool2d_f32(const float* x, int N, int C, int H, int W, int k, int stride, int pad, float* out, void* stream);
 int bs_stem_codes_f32(const float* x, const float* w, const float* bias, int N, int C, int H, int W, int O, int R, int S, int stride, int pad,
                       float act_scale, int a_bits, uint32_t* out, void* stream);
+int bs_stem_codes_supported(int N, int C, int H, int W, int O, int R, int S, int stride, int pad, float act_scale, int a_bits);
 int bs_avgpool_codes_f32(const uint32_t* packed, int N, int C, int H, int W, int a_bits, bs_sign_t a_sign, float inv, float* out,
                          void* stream);
 int bs_fc_f32(const float* x, const float* w, const float* bias, int N, int K, int J, float* out, void* stream);

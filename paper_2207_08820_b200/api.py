@@ -272,6 +272,13 @@ def stem_codes_f32(x: torch.Tensor, w: torch.Tensor, bias: Optional[torch.Tensor
     return True
 
 
+def stem_codes_supported(x_shape, w_shape, act_scale: float, a_bits: int) -> bool:
+    """Whether :func:`stem_codes_f32` takes images and filters of these shapes."""
+    N, C, H, W = x_shape
+    O, C2, R, S = w_shape
+    return C == C2 and bool(lib().bs_stem_codes_supported(N, C, H, W, O, R, S, 2, 3, act_scale, a_bits))
+
+
 def avgpool_codes_f32(packed: torch.Tensor, C: int, a_sign: int, inv: float, out: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Global average pool of packed codes [N,H,W,Cw,a_bits] -> float32 [N,C] (``bs_avgpool_codes_f32``)."""
     N, H, W, Cw, a_bits = packed.shape

@@ -744,16 +744,14 @@ __global__ void __launch_bounds__(ST_THREADS, 1) stem_codes_kernel(const __grid_
 
 }  // namespace bs
 
-extern "C" int bs_stem_codes_f32(const float* x, const float* w, const float* bias, int N, int C, int H, int W, int O, int R, int S, int stride, int pad,
-                                 float act_scale, int a_bits, uint32_t* out, void* stream)
+namespace bs {
+
+// What does not depend on the tensors: sizes, shared-memory layout, bounds.  `bytes`: dynamic shared memory.
+static int stem_plan(StemArgs& g, int& bytes, int N, int C, int H, int W, int O, int R, int S, int stride, int pad, float act_scale, int a_bits)
 {
-    using namespace bs;
-    if (!x || !w || !out || N <= 0 || C <= 0 || H <= 0 || W <= 0 || O <= 0 || R <= 0 || S <= 0 || stride < 1 || pad < 0) return BS_ERR_INVALID_ARG;
+    if (N <= 0 || C <= 0 || H <= 0 || W <= 0 || O <= 0 || R <= 0 || S <= 0 || stride < 1 || pad < 0) return BS_ERR_INVALID_ARG;
     if (H + 2 * pad < R || W + 2 * pad < S || !bits_ok(a_bits, BS_UNSIGNED) || !(act_scale > 0.0f && act_scale < 3.0e38f)) return BS_ERR_INVALID_ARG;
-    if (!aligned16(x) || !aligned16(w) || !aligned16(out) || (bias && (reinterpret_cast<uintptr_t>(bias) & 3u))) return BS_ERR_ALIGNMENT;
     if (C != 3 || O != 64 || R != 7 || S != 7 || stride != 2 || pad != 3 || a_bits != 2 || W % 2 != 0) return BS_ERR_UNSUPPORTED;
-    StemArgs g{};
-    g.x = x; g.w = w; g.bias = bias; g.out = out;
     g.H = H; g.W = W;
     g.P = (H - 1) / 2 + 1; g.Q = W / 2;
     g.P2 = (g.P - 1) / 2 + 1; g.Q2 = (g.Q - 1) / 2 + 1;
@@ -761,8 +759,7 @@ extern "C" int bs_stem_codes_f32(const float* x, const float* w, const float* bi
     const int cells = ST_SLAB + 3 * g.pitch + 3;
     // the cells a thread holds, and the rows of bits the ring holds beside two slabs
     if (cells > ST_CELLS_PER_THREAD * ST_PW * 32 || 2 * ST_SLAB + 2 * g.pitch + g.Q > ST_RING) return BS_ERR_UNSUPPORTED;
-    const long long rows = static_cast<long long>(N) * g.P2;
-    if (rows > 0x7fffffffLL || static_cast<long long>(2 * g.P2 + 2) * g.pitch > 0x3ffffffLL) return BS_ERR_UNSUPPORTED;
+    if (static_cast<long long>(N) * g.P2 > 0x7fffffffLL || static_cast<long long>(2 * g.P2 + 2) * g.pitch > 0x3ffffffLL) return BS_ERR_UNSUPPORTED;
     g.d_pitch = make_div(g.pitch);
     g.d_q2 = make_div(g.Q2);
     g.d_p2 = make_div(g.P2);
@@ -777,6 +774,7 @@ extern "C" int bs_stem_codes_f32(const float* x, const float* w, const float* bi
     g.off_stat = off;   off += (static_cast<int>(sizeof(StemFilters)) + 15) / 16 * 16;
     g.off_bar = off;    off += 512;
     if (off > ST_SMEM_MAX) return BS_ERR_UNSUPPORTED;
+    bytes = off;
     float bound[15];
     if (const int rc = bs_quantiser_bounds(act_scale, a_bits, BS_UNSIGNED, bound)) return rc;
     for (int k = 0; k < 3; ++k) {
@@ -786,6 +784,30 @@ extern "C" int bs_stem_codes_f32(const float* x, const float* w, const float* bi
     }
     g.scale = act_scale;
     g.third = 1.0 / (3.0 * act_scale);
+    return BS_OK;
+}
+
+}  // namespace bs
+
+extern "C" int bs_stem_codes_supported(int N, int C, int H, int W, int O, int R, int S, int stride, int pad, float act_scale, int a_bits)
+{
+    bs::StemArgs g{};
+    int bytes = 0;
+    return bs::stem_plan(g, bytes, N, C, H, W, O, R, S, stride, pad, act_scale, a_bits) == BS_OK;
+}
+
+extern "C" int bs_stem_codes_f32(const float* x, const float* w, const float* bias, int N, int C, int H, int W, int O, int R, int S, int stride, int pad,
+                                 float act_scale, int a_bits, uint32_t* out, void* stream)
+{
+    using namespace bs;
+    if (!x || !w || !out) return BS_ERR_INVALID_ARG;
+    StemArgs g{};
+    int bytes = 0;
+    const int rc = stem_plan(g, bytes, N, C, H, W, O, R, S, stride, pad, act_scale, a_bits);
+    if (rc == BS_ERR_INVALID_ARG) return rc;
+    if (!aligned16(x) || !aligned16(w) || !aligned16(out) || (bias && (reinterpret_cast<uintptr_t>(bias) & 3u))) return BS_ERR_ALIGNMENT;
+    if (rc != BS_OK) return rc;
+    g.x = x; g.w = w; g.bias = bias; g.out = out;
     g.status = status_device_ptr();
     const int sms = device_sm_count();
     if (!g.status || sms <= 0) return BS_ERR_CUDA;
@@ -793,8 +815,9 @@ extern "C" int bs_stem_codes_f32(const float* x, const float* w, const float* bi
         cudaGetLastError();
         return BS_ERR_CUDA;
     }
+    const long long rows = static_cast<long long>(N) * g.P2;
     const unsigned grid = static_cast<unsigned>(rows < sms ? rows : sms);
     g.share = static_cast<int>(rows / grid);
     g.extra = static_cast<int>(rows % grid);
-    return launch_dependent(stem_codes_kernel, dim3(grid), dim3(ST_THREADS), static_cast<size_t>(off), static_cast<cudaStream_t>(stream), g);
+    return launch_dependent(stem_codes_kernel, dim3(grid), dim3(ST_THREADS), static_cast<size_t>(bytes), static_cast<cudaStream_t>(stream), g);
 }

@@ -331,7 +331,13 @@ class BitserialFullNet:
         self.pooled = torch.empty(self.batch, C, dtype=torch.float32, device=self.device)
         self.logits = torch.empty(self.batch, net.classes, dtype=torch.float32, device=self.device)
         self.inv = float(np.float32(np.float32(net.body_act_scale) / np.float32(H * W)))
-        self.launches_per_forward = 2 + self.body.launches_per_forward      # two more where the stem runs as layers of its own
+
+    @property
+    def launches_per_forward(self) -> int:
+        """Kernels of a pass as it would run now: two more where the stem runs as layers of its own."""
+        fused = not self._watched() and api.stem_codes_supported((self.batch, 3, self.net.hw, self.net.hw), self.stem_w.shape, self.body.act_scale,
+                                                                 self.body.net.a_bits)
+        return self.body.launches_per_forward + (2 if fused else 4)
 
     def run_stem(self, images: torch.Tensor) -> None:
         """The stem as layers of its own: images to ``stem_conv`` and ``stem_pool``."""

@@ -201,3 +201,32 @@ def test_stem_tensors_that_are_kept_or_assigned():
     runner.forward(a)
     assert torch.equal(mine, stem_layers(runner, a)[1]) and torch.equal(runner.stem_pool, mine)
     assert torch.equal(runner.logits, logits)
+
+
+@pytest.mark.parametrize("hw", [64, 308])
+def test_launches_and_layers_of_the_front(hw):
+    """``launches_per_forward`` counts what a pass launches, where the stem is one kernel, where its shape is refused and while its tensors are held."""
+    runner, (a, b, _) = classifier(hw)
+    fused = hw == 64
+
+    def launches(images):
+        before = api.launch_count
+        runner.forward(images)
+        return api.launch_count - before
+
+    for images in (a, b):
+        assert launches(images) == runner.launches_per_forward == runner.body.launches_per_forward + (2 if fused else 4)
+        conv, pool = stem_layers(runner, images)
+        assert torch.equal(runner.body.bufs[runner.net.body.in_name].view(-1), api.bitpack_activations(pool, runner.body.act_scale, 2).view(-1))
+        assert torch.equal(runner.stem_conv, conv) and torch.equal(runner.stem_pool, pool)
+    kept = runner.stem_pool
+    assert launches(a) == runner.launches_per_forward == runner.body.launches_per_forward + 4
+    assert torch.equal(kept, stem_layers(runner, a)[1])
+
+
+def test_widest_rows():
+    """Shared memory and the cells of a thread nearly full; the next even width is refused."""
+    compare(*inputs(2, 37, 306, seed=3))
+    x, w, _ = inputs(1, 16, 308)
+    assert not api.stem_codes_supported(x.shape, w.shape, 0.25, 2)
+    assert not api.stem_codes_f32(x, w, None, 0.25, 2, torch.empty(1, 4, 77, 2, 2, dtype=torch.int32, device="cuda"))
