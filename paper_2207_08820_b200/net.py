@@ -318,8 +318,8 @@ class BitserialFullNet:
         self.fc_w, self.fc_b = to(params["fc"]["w"]), to(params["fc"]["bias"])
         h1 = (net.hw + 2 * 3 - 7) // 2 + 1
         h2 = (h1 + 2 - 3) // 2 + 1
-        self._stem = dict(conv=torch.empty(self.batch, 64, h1, h1, dtype=torch.float32, device=self.device),
-                          pool=torch.empty(self.batch, 64, h2, h2, dtype=torch.float32, device=self.device))
+        self._stem_sizes = dict(conv=h1, pool=h2)
+        self._stem: Dict[str, torch.Tensor] = {}                # the stem's float tensors, from their first use on
         self._stem_held: Dict[str, weakref.ref] = {}            # what was handed out of them
         self._stem_assigned = False                             # the caller has put tensors of their own in their place
         self._codes_only: Optional[torch.Tensor] = None         # images of the last pass launched, where it made codes only
@@ -355,8 +355,16 @@ class BitserialFullNet:
             body.pack_input(self._stem["pool"])
 
     def _stem_layers(self, images: torch.Tensor) -> None:
-        api.conv2d_f32(images, self.stem_w, self.stem_b, stride=2, pad=3, relu=True, out=self._stem["conv"])
-        api.maxpool2d_f32(self._stem["conv"], 3, 2, 1, out=self._stem["pool"])
+        conv, pool = self._stem_tensor("conv"), self._stem_tensor("pool")
+        api.conv2d_f32(images, self.stem_w, self.stem_b, stride=2, pad=3, relu=True, out=conv)
+        api.maxpool2d_f32(conv, 3, 2, 1, out=pool)
+
+    def _stem_tensor(self, name: str) -> torch.Tensor:
+        t = self._stem.get(name)
+        if t is None:
+            hw = self._stem_sizes[name]
+            t = self._stem[name] = torch.empty(self.batch, 64, hw, hw, dtype=torch.float32, device=self.device)
+        return t
 
     def _watched(self) -> bool:
         return self._stem_assigned or any(r() is not None for r in self._stem_held.values())
@@ -397,7 +405,7 @@ class BitserialFullNet:
         held = self._stem_held.get(name)
         t = held() if held is not None else None
         if t is None:
-            t = self._stem[name].detach()
+            t = self._stem_tensor(name).detach()
             self._stem_held[name] = weakref.ref(t)
         return t
 

@@ -230,3 +230,13 @@ def test_widest_rows():
     x, w, _ = inputs(1, 16, 308)
     assert not api.stem_codes_supported(x.shape, w.shape, 0.25, 2)
     assert not api.stem_codes_f32(x, w, None, 0.25, 2, torch.empty(1, 4, 77, 2, 2, dtype=torch.int32, device="cuda"))
+
+
+def test_stem_tensors_take_memory_from_their_first_use_on():
+    runner, (a, _, _) = classifier()
+    runner.forward(a)
+    torch.cuda.synchronize()
+    before = torch.cuda.memory_allocated()
+    pool = runner.stem_pool
+    assert torch.cuda.memory_allocated() - before >= 4 * 2 * 64 * (32 * 32 + 16 * 16)
+    assert torch.equal(pool, stem_layers(runner, a)[1])
