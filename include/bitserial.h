@@ -229,6 +229,7 @@ int bitserial_gemm_noalloc(const uint32_t* a_packed, const uint32_t* w_packed, i
  *   1x1 stride-1 layers, N*H*W is even; res_c_offset a multiple of 32; everything else as bitserial_conv2d.  Unsupported shapes
  *   return BS_ERR_UNSUPPORTED: use bitserial_conv2d.
  *   bs_tc_weights_bytes    bytes of the prepared filter tensor (0 on bad input).
+ *   bs_tc_weights_read_bytes  bytes from its front that layers of these widths read, beside the last 16 (0 on bad input).
  *   bs_tc_prepare_weights  packed weights [O][R][S][Cw][w_bits] -> tiles for layers of a_bits activation bits: nibbles
  *                          [ceil(C/64)][ceil(O/128)*16][R*S][2][8][16 bytes] where a_bits and w_bits are at most 2 (the first half of the
  *                          tensor or so), int8 [C/32][ceil(O/128)*16][R*S][2][8][16] otherwise.  One tensor serves layers of every a_bits; a
@@ -236,6 +237,7 @@ int bitserial_gemm_noalloc(const uint32_t* a_packed, const uint32_t* w_packed, i
  *                          them for the widths they run with.
  */
 size_t bs_tc_weights_bytes(int O, int C, int R, int S);
+size_t bs_tc_weights_read_bytes(int O, int C, int R, int S, int w_bits, int a_bits);
 int bs_tc_prepare_weights(const uint32_t* wgt_packed, int O, int C, int R, int S, int w_bits, bs_sign_t w_sign,
                           int a_bits, int8_t* wgt_tc_out, void* stream);
 int bs_tc_supported(const bs_conv_params* p);

@@ -148,6 +148,13 @@ def tc_prepare_weights(wgt_packed: torch.Tensor, C: int, w_sign: int, a_bits: in
     return out
 
 
+def tc_weights_read(w_tc: torch.Tensor, wgt_shape, C: int, a_bits: int):
+    """What layers of ``a_bits`` activation bits read of filters prepared for them: a list of views."""
+    O, R, S, _, w_bits = wgt_shape
+    n = lib().bs_tc_weights_read_bytes(O, C, R, S, w_bits, a_bits)
+    return [w_tc] if n in (0, w_tc.numel()) else [w_tc[:n], w_tc[-16:]]
+
+
 def tc_supported(N, C, H, W, O, k, stride, pad, a_bits, a_sign, w_bits, w_sign) -> bool:
     p = ConvParams(N=N, C=C, H=H, W=W, O=O, R=k, S=k, stride=stride, pad=pad, a_bits=a_bits, a_sign=a_sign,
                    w_bits=w_bits, w_sign=w_sign)

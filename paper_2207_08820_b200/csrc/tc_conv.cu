@@ -191,6 +191,14 @@ extern "C" size_t bs_tc_weights_bytes(int O, int C, int R, int S)
     return static_cast<size_t>((O + 127) / 128 * 128) * R * S * C;
 }
 
+// Layers of these widths read so much from the front of the prepared tensor, and its last 16 bytes.
+extern "C" size_t bs_tc_weights_read_bytes(int O, int C, int R, int S, int w_bits, int a_bits)
+{
+    const size_t all = bs_tc_weights_bytes(O, C, R, S);
+    if (all == 0 || !bs::bits_ok(w_bits, BS_UNSIGNED) || !bs::bits_ok(a_bits, BS_UNSIGNED)) return 0;
+    return bs::mma_nibbles(C, R * S, a_bits, w_bits) ? all / (C / 32) * ((C / 32 + 1) / 2) : all;
+}
+
 extern "C" int bs_tc_prepare_weights(const uint32_t* wgt_packed, int O, int C, int R, int S, int w_bits, bs_sign_t w_sign,
                                      int a_bits, int8_t* out, void* stream)
 {

@@ -43,7 +43,7 @@ class BitserialNet:
 
     def __init__(self, net: NetSpec, params: Dict[str, Dict], act_scale: float, device="cuda", batch: Optional[int] = None,
                  engine: str = "popc", concurrent: bool = True, chains="auto"):
-        """engine: "popc" = packed filters, expanded on chip; "tc" = filters prepared as int8 tiles once for every layer that
+        """engine: "popc" = packed filters, expanded on chip; "tc" = filters prepared as operand tiles once for every layer that
         supports it (others keep packed filters).  concurrent: launch independent neighbouring layers on
         two streams (see :meth:`schedule`).  chains: True groups, with the "tc" engine, runs of consecutive same-shaped layers that the
         library accepts into units which :meth:`run_units` issues as one ``bitserial_conv2d_tc_chain`` call each; False and "auto" = a unit per
@@ -272,7 +272,8 @@ class BitserialNet:
     def prefetch_filters(self) -> None:
         """A hint before a pass whose filters have left L2: they start on their way there (a separate launch; a pass does not issue it,
         since it gains nothing while the filters are still in L2)."""
-        api.l2_prefetch([item["w_tc"] if item["w_tc"] is not None else item["w"] for item in self.layers])
+        api.l2_prefetch([t for item in self.layers for t in (
+            [item["w"]] if item["w_tc"] is None else api.tc_weights_read(item["w_tc"], item["w"].shape, item["spec"].C, self.net.a_bits))])
 
     def forward(self, x: torch.Tensor) -> torch.Tensor:
         """x: float32 [batch, C, H, W] on the device.  Returns the packed output tensor of the stack."""

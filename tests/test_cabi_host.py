@@ -209,3 +209,16 @@ def test_planner_refuses_more_input_pixels_than_it_can_count(L):
         supported = lambda N, stride: api.tc_supported(N, 32, 6000, 6000, 32, k, stride, k // 2, 4, api.UNSIGNED, 2, api.SIGNED)
         assert supported(59, 2) and supported(58, 1)                 # 2.12e9 pixels
         assert not supported(60, 2) and not supported(60, 1)         # 2.16e9
+
+
+def test_read_part_of_prepared_filters(L):
+    """Nibbles fill the front of a tensor that has room for int8."""
+    assert L.bs_tc_weights_read_bytes(200, 64, 3, 3, 2, 2) == 256 * 9 * 32
+    assert L.bs_tc_weights_read_bytes(200, 64, 3, 3, 1, 1) == 256 * 9 * 32
+    assert L.bs_tc_weights_read_bytes(200, 96, 3, 3, 2, 1) == 256 * 9 * 64
+    assert L.bs_tc_weights_read_bytes(200, 32, 3, 3, 2, 2) == L.bs_tc_weights_bytes(200, 32, 3, 3)
+    for a_bits, w_bits in ((3, 2), (2, 3), (4, 4)):
+        assert L.bs_tc_weights_read_bytes(200, 64, 3, 3, w_bits, a_bits) == L.bs_tc_weights_bytes(200, 64, 3, 3)
+    assert L.bs_tc_weights_read_bytes(64, 444416, 1, 1, 2, 2) == L.bs_tc_weights_bytes(64, 444416, 1, 1) // 2
+    assert L.bs_tc_weights_read_bytes(64, 444448, 1, 1, 2, 2) == L.bs_tc_weights_bytes(64, 444448, 1, 1)
+    assert L.bs_tc_weights_read_bytes(64, 40, 3, 3, 2, 2) == 0 and L.bs_tc_weights_read_bytes(64, 64, 3, 3, 5, 2) == 0
