@@ -1,11 +1,12 @@
-// Exact integer convolution of packed bitplanes on the tensor cores (tcgen05.mma kind::i8, accumulators in tensor memory).
+// Exact integer convolution of packed bitplanes on the tensor cores (tcgen05.mma kind::mxf4 and kind::i8, accumulators in tensor memory).
 //
-// The Section V plane-pair popcount sum equals the integer dot product of the unpacked codes, so the same int32 accumulators
-// come out of an int8 x int8 -> int32 matrix product.  Both operands stay bit-packed in memory (filters optionally as int8
-// tiles prepared once) and are expanded to int8 on chip.  A CTA walks over work items = 128 * PT accumulator rows x TN filters:
+// The Section V plane-pair popcount sum equals the integer dot product of the unpacked codes, so the same whole numbers come out of a
+// matrix product of the codes: as nibbles (codes of one and two bits on both sides, see below) or as int8.  Both operands stay
+// bit-packed in memory (filters optionally as operand tiles prepared once) and are expanded on chip.  A CTA walks over work items =
+// 128 * PT accumulator rows x TN filters:
 //
-//   expander warps   packed pixels -> int8 in the K-major core-matrix layout [16-channel group][pixel][16 bytes]
-//   one MMA warp     R*S taps x channel blocks of K = 32; a tap is only another start address of the pixel operand
+//   expander warps   packed pixels -> nibbles or int8 in the K-major core-matrix layout [channel group][pixel][16 bytes]
+//   one MMA warp     R*S taps x channel blocks of K = 64 nibbles or 32 int8; a tap is only another start address of the pixel operand
 //   epilogue warps   accumulators -> requantised, re-packed codes or int32, overlapping the MMAs of the next item
 //   one copy warp    prepared filters by bulk copies, once (resident) or chunk by chunk (streamed)
 //
@@ -17,7 +18,7 @@
 //
 // Codes of one and two bits on both sides run as tcgen05.mma kind::mxf4 (F4): two-bit codes are the small e2m1 floats 0, 0.5, 1, 1.5 with a
 // sign, so a nibble holds the code (sign and magnitude), scale factors of 2 in both operands make the products whole numbers, and
-// the sums stay exact in binary32 (below 2^22 by the plan; whole numbers up to 30188 and beyond compared).  A K = 64 step takes as long
+// the sums stay exact in binary32 (below 2^22 by mma_nibbles; compared up to 3999744 in tests/test_gpu_nibbles.py).  A K = 64 step takes as long
 // and reads as many bytes as a K = 32 step of kind::i8, so operands, filter traffic and MMA time are all half as large.
 //
 // Every wait on an mbarrier is bounded; a wait that runs out sets the device status word and the CTA drains.
@@ -46,7 +47,7 @@ inline FastDiv make_div(int d)
 struct MmaArgs {
     CUtensorMap tmA, tmB;           // flat tiles with aligned rows: packed pixels (words, rows), packed filters (words, filters)
     const uint32_t* act;
-    const int8_t* wgt;              // prepared filters [C/32][filters, padded to 128][R*S][32] in core-matrix order, or null
+    const int8_t* wgt;              // prepared filters [C/32][filters, padded to 128][R*S][32 bytes] in core-matrix order (nibbles: C/64), or null
     const uint32_t* wgt_packed;     // packed filters [O][R*S][Cw][WB], used when wgt is null
     int32_t* out_i32;
     uint32_t* out_packed;
@@ -205,8 +206,17 @@ __device__ __forceinline__ void mm_ld16(uint32_t taddr, uint32_t (&v)[16])
           "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
         : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ void mm_ld8(uint32_t taddr, uint32_t (&v)[8])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(taddr) : "memory");
+}
 __device__ __forceinline__ void mm_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // Values loaded from tensor memory may be touched only after the wait: arithmetic on them must not move above it.
+__device__ __forceinline__ void mm_landed(uint32_t (&v)[8])
+{
+    asm volatile("" : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]));
+}
 __device__ __forceinline__ void mm_landed(uint32_t (&v)[16])
 {
     asm volatile("" : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
@@ -284,7 +294,7 @@ __device__ __forceinline__ u64 f2_fma(u64 a, u64 b, u64 c) { u64 r; asm("fma.rn.
 
 __device__ __forceinline__ int fdiv(int n, const FastDiv& f) { return f.d == 1 ? n : static_cast<int>(__umulhi(static_cast<unsigned>(n), f.mul) >> f.shift); }
 
-// ----------------------------------------------------------------------------- expansion: plane words -> int8
+// ----------------------------------------------------------------------------- expansion: plane words -> int8 or nibbles
 
 // 32 codes of NB planes -> 32 bytes, byte 4 m + k = channel 8 k + m: bytes are cut out of the words with a shift and a mask, no
 // look-up (a 256-entry table in shared memory cost eight loads with bank conflicts per word).  Two planes are first merged
@@ -852,14 +862,14 @@ struct MmaEpi {
     uint64_t* red_full;      // the partial sums of the other CTAs of a split item have arrived
 };
 
-// Split items.  CTAs of rank 1 and up send their accumulators to the shared memory of rank 0 ([rank - 1][column][row], so a warp
-// stores 128 contiguous bytes), which adds them to its own in tensor memory and goes on as if it had done all the chunks.
 // Whole number of an accumulator.
 __device__ __forceinline__ uint32_t acc_int(bool f4, uint32_t v, uint32_t bias)
 {
     return f4 ? __float_as_uint(__uint_as_float(v) + 12582912.0f) - MM_PRESET : v - bias;
 }
 
+// Split items.  CTAs of rank 1 and up send their accumulators to the shared memory of rank 0 ([rank - 1][column][row], so a warp
+// stores 128 contiguous bytes), which adds them to its own in tensor memory and goes on as if it had done all the chunks.
 template <int EW, bool F4>
 __device__ __forceinline__ bool send_partials(const MmaArgs& g, const MmaEpi& e, int rank)
 {
@@ -1075,15 +1085,6 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
 // columns of each tile are computed while the next eight are on their way.
 // conv2_x of 64 images: 14.1 -> 13.5 us without, 16.4 -> 15.1 us with a residual.  (Fragments of 16 x 256 bits, whose lanes need the
 // constants of 8 filters only, made it 16.1 and 19.7: trading codes for plane words between lanes costs more than the loads.)
-__device__ __forceinline__ void mm_ld8(uint32_t taddr, uint32_t (&v)[8])
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void mm_landed8(uint32_t (&v)[8])
-{
-    asm volatile("" : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]));
-}
 // Eight columns of two tiles: codes of pair i at bits 2 i of either half of W.  z: residual codes of the pairs from bit 0 of either half on.
 template <bool RES, int NT>
 __device__ __forceinline__ void requant8(const uint32_t (&v)[NT][8], uint32_t tab, const uint32_t (&z)[NT], u64 rmul, u64 rmul4, uint32_t hi2, uint32_t (&W)[NT])
@@ -1202,7 +1203,7 @@ __device__ __forceinline__ bool epilogue_tiles(const MmaArgs& g, const MmaEpi& e
             for (int p = 0; p < 4; ++p) {
                 mm_ld_wait();
 #pragma unroll
-                for (int j = 0; j < NT; ++j) mm_landed8(v[p & 1][j]);
+                for (int j = 0; j < NT; ++j) mm_landed(v[p & 1][j]);
                 if (p < 3 || more) {
                     const uint32_t from = p < 3 ? col + 8u * (p + 1) : next;
 #pragma unroll

@@ -10,7 +10,8 @@
 //   (|bias| + |patch|_2 |filter|_2) by Cauchy and Schwarz.  An output closer to a bound than the sum of these is undecided between two codes:
 //   about 0.08 % of normalised images.  Most windows have another output that reaches the higher of the two for certain; in the others
 //   the chain itself is evaluated, tap by tap in the layer's order.  A slab whose values have no useful common scale (infinities, NaN,
-//   above 2^20) takes the chain for every output, which costs about thirty times as much as the tensor cores.
+//   above 2^20) takes the chain for every output: right, but slower than the separate layers.  64 images of 224 x 224: 1500 us where every
+//   slab is like that, 1650 where half of all outputs sit on a bound, 378 with one infinity an image, against 386 for the layers.
 //
 // What bounds it: 24 MMAs of 128 positions x (192, 128, 64) columns x 32 digits per tile, 1650 cycles alone, of which 1540 are
 // shared-memory reads of the operands, so every other access to shared memory shows: 2080 cycles a tile in the steady state, and
@@ -108,11 +109,6 @@ __device__ __forceinline__ float4 st_lds(uint32_t addr)
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
     return v;
 }
-__device__ __forceinline__ void st_ld8(uint32_t taddr, uint32_t (&v)[8])
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(taddr) : "memory");
-}
 __device__ __forceinline__ void st_st8(uint32_t taddr, const uint32_t (&v)[8])
 {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
@@ -124,10 +120,6 @@ __device__ __forceinline__ u64 st_fma_sat(u64 a, float b, float c)
     uint32_t a0, a1;
     f2_split(a, a0, a1);
     return f2_pack(__float_as_uint(__saturatef(fmaf(__uint_as_float(a0), b, c))), __float_as_uint(__saturatef(fmaf(__uint_as_float(a1), b, c))));
-}
-__device__ __forceinline__ void st_landed(uint32_t (&v)[8])
-{
-    asm volatile("" : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]));
 }
 // x in steps, rounded to a whole number (|.| <= 2^22), as three signed digits of eight bits in the low bytes + 128 each.
 __device__ __forceinline__ uint32_t st_fixed(float x, float inv) { return __float_as_uint(fmaf(x, inv, 12582912.0f)) + (0x00808080u - 0x4B400000u); }
@@ -545,7 +537,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) stem_codes_kernel(const __grid_
                 // eight filters at a time, the sums of the next eight on their way
                 uint32_t D[2][3][8];
 #pragma unroll
-                for (int d = 0; d < 3; ++d) st_ld8(acc + d * 64 + 24, D[0][d]);
+                for (int d = 0; d < 3; ++d) mm_ld8(acc + d * 64 + 24, D[0][d]);
 #pragma unroll 1
                 for (int pair = 1; pair >= 0; --pair)
 #pragma unroll
@@ -553,10 +545,10 @@ __global__ void __launch_bounds__(ST_THREADS, 1) stem_codes_kernel(const __grid_
                     const int piece = pair * 2 + odd;
                     uint32_t (&E)[3][8] = D[odd ^ 1];
                     mm_ld_wait();
-                    st_landed(E[0]); st_landed(E[1]); st_landed(E[2]);
+                    mm_landed(E[0]); mm_landed(E[1]); mm_landed(E[2]);
 #pragma unroll
                     for (int d = 0; d < 3; ++d) {
-                        if (odd || pair) st_ld8(acc + d * 64 + (piece - 1) * 8, D[odd][d]);
+                        if (odd || pair) mm_ld8(acc + d * 64 + (piece - 1) * 8, D[odd][d]);
                         st_st8(acc + d * 64 + piece * 8, preset);
                     }
                     if (!odd && !pair) {            // all is in registers: the next tile's MMAs may begin

@@ -32,7 +32,7 @@ def compare(x, w, b, scale=0.25):
     assert torch.equal(out, want)
 
 
-# one pixel pair, one pooled row, odd heights, widths whose rows end inside a tile or a slab, runs that cross images, the widest rows
+# one pixel pair, one pooled row, odd heights, widths whose rows end inside a tile or a slab, runs that cross images, wide rows (the widest: test_widest_rows)
 @pytest.mark.parametrize("N,H,W", [(5, 1, 2), (2, 8, 8), (1, 7, 34), (2, 37, 46), (3, 64, 64), (149, 20, 24), (9, 75, 126), (2, 224, 224), (1, 90, 254), (2, 256, 256), (1, 50, 278)])
 def test_sizes(N, H, W):
     compare(*inputs(N, H, W, seed=H))
@@ -240,3 +240,15 @@ def test_stem_tensors_take_memory_from_their_first_use_on():
     pool = runner.stem_pool
     assert torch.cuda.memory_allocated() - before >= 4 * 2 * 64 * (32 * 32 + 16 * 16)
     assert torch.equal(pool, stem_layers(runner, a)[1])
+
+
+def test_images_inside_a_larger_buffer():
+    x, w, b = inputs(5, 60, 64, seed=21)
+    compare(x[1:4], w, b)
+    flat = torch.cat([x.reshape(-1), x.reshape(-1)])
+    n = 2 * 3 * 60 * 64
+    compare(flat[4:4 + n].view(2, 3, 60, 64), w, b)
+    with pytest.raises(api.BitserialError):         # off a 16-byte boundary, as for the layers
+        api.stem_codes_f32(flat[1:1 + n].view(2, 3, 60, 64), w, b, 0.25, 2, torch.empty(2, 15, 16, 2, 2, dtype=torch.int32, device="cuda"))
+    with pytest.raises(api.BitserialError):
+        api.conv2d_f32(flat[1:1 + n].view(2, 3, 60, 64), w, b, 2, 3, True)
