@@ -778,7 +778,7 @@ def main():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-configs", action="store_true", help="leave out the compact measurements of the other workloads")
     ap.add_argument("--engine", default="tc", choices=["popc", "tc"],
-                    help="popc: packed filters, expanded on chip; tc: filters prepared as int8 tiles once (the same tensor-core kernel)")
+                    help="popc: packed filters, expanded on chip; tc: filters prepared as operand tiles once (the same tensor-core kernel)")
     ap.add_argument("--chains", default="auto", choices=["auto", "on", "off"], help="on: runs of same-shaped layers as one call each instead of the bound sequence; the launches are the same")
     ap.add_argument("--eager", action="store_true", help="plain stream launches instead of CUDA graphs (for per-launch profiling)")
     args = ap.parse_args()
