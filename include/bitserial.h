@@ -305,6 +305,20 @@ typedef struct {
     int join[4];
 } bs_sequence_layer;
 int bs_sequence_create(const bs_sequence_layer* layers, int nlayers, void* side_stream, bs_sequence** sequence_out);
+/*
+ * bs_sequence_create_ws -- the same with device memory in which the layers may keep, beside the packed codes, what the tensor cores read of every
+ * tensor that a later layer reads (32 channels of a position as 16 bytes of nibbles, zero padding included).  Same outputs, every packed tensor
+ * included; a layer then expands nothing.  One launch more for every tensor that is read before the layers have written all of it.
+ *   workspace             bs_sequence_workspace_bytes bytes, 16-byte aligned, ZERO before the first run, the sequence's own from then on; NULL or
+ *                         less than that: as bs_sequence_create.  May pass on to another sequence of layers of the same shapes, formats and order.
+ * bs_sequence_workspace_bytes answers 0 where the layers don't take one: layers without prepared filters, codes of more than two bits or signed ones,
+ * tensors that overlap or that are used with two shapes, rows too wide for the shared memory.  It needs no device.
+ * bs_sequence_launches: kernels that a run enqueues.
+ */
+size_t bs_sequence_workspace_bytes(const bs_sequence_layer* layers, int nlayers);
+int bs_sequence_create_ws(const bs_sequence_layer* layers, int nlayers, void* side_stream, void* workspace, size_t workspace_bytes,
+                          bs_sequence** sequence_out);
+int bs_sequence_launches(const bs_sequence* sequence);
 int bs_sequence_run(bs_sequence* sequence, void* stream);
 void bs_sequence_destroy(bs_sequence* sequence);
 int bitserial_gemm_tc(const uint32_t* a_packed, const int8_t* w_tc, int M, int N, int K, int a_bits, bs_sign_t a_sign,

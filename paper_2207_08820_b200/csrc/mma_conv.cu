@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "mma_kernel.cuh"
+#include "oper_conv.h"
 
 namespace bs {
 
@@ -511,8 +512,10 @@ struct Sequence {
     };
     std::vector<Step> steps;
     cudaStream_t side;
+    OperSequence* oper;             // the layers on operand tensors, or null: as planned in the steps
     ~Sequence()
     {
+        if (oper) oper_destroy(oper);
         for (Step& s : steps) {
             if (s.fork) cudaEventDestroy(s.fork);
             if (s.done) cudaEventDestroy(s.done);
@@ -520,18 +523,19 @@ struct Sequence {
     }
 };
 
-int mma_sequence_create(const bs_sequence_layer* layers, int n, cudaStream_t side, Sequence** out)
+int mma_sequence_create(const bs_sequence_layer* layers, int n, cudaStream_t side, void* workspace, size_t bytes, Sequence** out)
 {
     Sequence* q = new (std::nothrow) Sequence;
     if (!q) return BS_ERR_CUDA;
     q->side = side;
+    q->oper = workspace ? oper_create(layers, n, workspace, bytes) : nullptr;
     q->steps.resize(static_cast<size_t>(n));
     for (Sequence::Step& s : q->steps) s.fork = s.done = nullptr;
     for (int i = 0; i < n; ++i) {
         const bs_sequence_layer& l = layers[i];
         Sequence::Step& s = q->steps[i];
         // a layer beside its successors starts from an event, not from the kernel before it: no early filter fetch
-        int rc = bind_plan(s.plan, l.act_packed, l.wgt_tc, l.wgt_packed, &l.p, nullptr, l.out_packed, l.chained && !l.aside, false, false);
+        int rc = q->oper ? BS_OK : bind_plan(s.plan, l.act_packed, l.wgt_tc, l.wgt_packed, &l.p, nullptr, l.out_packed, l.chained && !l.aside, false, false);
         for (int k = 0; k < 4; ++k) {
             s.join[k] = l.join[k];
             if (l.join[k] >= i) rc = BS_ERR_INVALID_ARG;
@@ -547,9 +551,16 @@ int mma_sequence_create(const bs_sequence_layer* layers, int n, cudaStream_t sid
     return BS_OK;
 }
 
+int mma_sequence_launches(const Sequence* q) { return static_cast<int>(q->steps.size()) + (q->oper ? oper_imports(q->oper) : 0); }
+
 int mma_sequence_run(Sequence* q, cudaStream_t st)
 {
-    for (Sequence::Step& s : q->steps) {
+    if (q->oper) {
+        const int rc = oper_begin(q->oper, st);
+        if (rc != BS_OK) return rc;
+    }
+    for (size_t i = 0; i < q->steps.size(); ++i) {
+        Sequence::Step& s = q->steps[i];
         cudaStream_t on = st;
         for (int k = 0; k < 4 && s.join[k] >= 0; ++k)
             if (cudaStreamWaitEvent(st, q->steps[s.join[k]].done, 0) != cudaSuccess) { cudaGetLastError(); return BS_ERR_CUDA; }
@@ -557,7 +568,7 @@ int mma_sequence_run(Sequence* q, cudaStream_t st)
             if (cudaEventRecord(s.fork, st) != cudaSuccess || cudaStreamWaitEvent(q->side, s.fork, 0) != cudaSuccess) { cudaGetLastError(); return BS_ERR_CUDA; }
             on = q->side;
         }
-        const int rc = launch_plan(s.plan, on);
+        const int rc = q->oper ? oper_layer(q->oper, static_cast<int>(i), on) : launch_plan(s.plan, on);
         if (rc != BS_OK) return rc;
         if (s.done && cudaEventRecord(s.done, on) != cudaSuccess) { cudaGetLastError(); return BS_ERR_CUDA; }
     }

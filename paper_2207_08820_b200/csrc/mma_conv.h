@@ -27,8 +27,10 @@ int mma_conv_run(const uint32_t* act, const int8_t* wgt, const uint32_t* wgt_pac
                  uint32_t* out_packed, cudaStream_t st, bool chained, bool plan_only);
 
 // A sequence of layers bound to its tensors (bs_sequence_*); the layers have been validated.
+// workspace: null, or zeroed device memory of oper_workspace_bytes (oper_conv.h) bytes for layers that run on operand tensors.
 struct Sequence;
-int mma_sequence_create(const bs_sequence_layer* layers, int n, cudaStream_t side, Sequence** out);
+int mma_sequence_create(const bs_sequence_layer* layers, int n, cudaStream_t side, void* workspace, size_t bytes, Sequence** out);
+int mma_sequence_launches(const Sequence* q);
 int mma_sequence_run(Sequence* q, cudaStream_t st);
 void mma_sequence_destroy(Sequence* q);
 

@@ -531,8 +531,8 @@ __device__ __forceinline__ void expand_filters_resident(const MmaArgs& g, uint32
 // Filters prepared for layers of other widths (bs_tc_prepare_weights: nibbles or int8, told apart by MM_NIBBLE_MARK) -> `nb` K steps from b0
 // on in the form of this layer, by one warp: 16-byte vectors [K step][filter / 8][tap][half][filter % 8] at `dst`.  A layer with such filters
 // is right but slow; preparing them for its widths is the remedy.
-template <bool F4>
-static __device__ __noinline__ void convert_filters(const MmaArgs& g, unsigned char* dst, int o0, int b0, int nb, int lane)
+template <bool F4, class G>
+static __device__ __noinline__ void convert_filters(const G& g, unsigned char* dst, int o0, int b0, int nb, int lane)
 {
     const int per = g.TN * g.RS * 2;
     const size_t stride = static_cast<size_t>(g.opad) * g.RS * 2;
@@ -761,7 +761,8 @@ __device__ __forceinline__ void requant16(const uint32_t (&v)[16], uint32_t tab,
 }
 
 // The documented formula, one output at a time: any scale, bias, residual format.
-static __device__ __noinline__ void requant32_formula(const MmaArgs& g, const uint32_t* v, int ob, const uint32_t* rw, uint32_t* ow)
+template <class G>
+static __device__ __noinline__ void requant32_formula(const G& g, const uint32_t* v, int ob, const uint32_t* rw, uint32_t* ow)
 {
     int qmin, qmax;
     code_limits(g.out_bits, g.out_sign, qmin, qmax);
@@ -824,7 +825,8 @@ __device__ __forceinline__ MmaPixel mma_pixel(const MmaArgs& g, int pos)
 
 // Checks and lays out the (scale, bias) pairs of the CTA's filters: tab[16 * group + pair] = (s0, s1, b0, b1) scaled by 2^-24.
 // *ok stays 1 when the fast form takes the formula's decision for every possible accumulator.
-__device__ __forceinline__ void epilogue_tables(const MmaArgs& g, float4* tab, float2* rtab, int* ok, int o0, int t, int nt)
+template <class G>
+__device__ __forceinline__ void epilogue_tables(const G& g, float4* tab, float2* rtab, int* ok, int o0, int t, int nt)
 {
     const float res_max = g.residual ? fabsf(g.res_scale) * 15.0f : 0.0f;
     for (int e = t; e < g.TN / 2; e += nt) {
@@ -917,7 +919,8 @@ __device__ __forceinline__ bool merge_partials(const MmaArgs& g, const MmaEpi& e
     return true;
 }
 
-__device__ __forceinline__ void store_codes(const MmaArgs& g, int pix, int ob, uint32_t (&ow)[4])
+template <class G>
+__device__ __forceinline__ void store_codes(const G& g, int pix, int ob, uint32_t (&ow)[4])
 {
     if (g.O - ob < 32) {
         const uint32_t m = (1u << (g.O - ob)) - 1u;
@@ -935,7 +938,8 @@ __device__ __forceinline__ void store_codes(const MmaArgs& g, int pix, int ob, u
 }
 
 // Residual planes of (pixel, 32 filters from ob).
-__device__ __forceinline__ void load_residual(const MmaArgs& g, int pix, int ob, uint32_t (&rw)[4])
+template <class G>
+__device__ __forceinline__ void load_residual(const G& g, int pix, int ob, uint32_t (&rw)[4])
 {
     const uint32_t* rp = g.residual + (static_cast<size_t>(pix) * g.res_cw_total + ((g.res_c_off + ob) >> 5)) * g.res_bits;
     if (g.res_bits == 2) {

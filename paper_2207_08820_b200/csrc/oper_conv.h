@@ -1,0 +1,21 @@
+// Sequences of layers on operand tensors (oper_conv.cu): host interface for the sequences of mma_conv.cu.
+#pragma once
+#include <cuda_runtime.h>
+
+#include "common.cuh"
+
+namespace bs {
+
+struct OperSequence;
+
+// Bytes of zeroed device memory that the layers need to run on operand tensors; 0: they don't take them (mma_conv.cu runs them).
+size_t oper_workspace_bytes(const bs_sequence_layer* layers, int n);
+// The launches of such layers; null where oper_workspace_bytes is 0 or bytes is less.
+OperSequence* oper_create(const bs_sequence_layer* layers, int n, void* workspace, size_t bytes);
+// Launches in front of the layers, all of them on `st`; layer i on `st`.
+int oper_imports(const OperSequence* q);
+int oper_begin(const OperSequence* q, cudaStream_t st);
+int oper_layer(const OperSequence* q, int i, cudaStream_t st);
+void oper_destroy(OperSequence* q);
+
+}  // namespace bs

@@ -1,6 +1,7 @@
 // Entry points of the tensor-core formulation: validation, filter preparation, layers and chains of layers (kernel: mma_conv.cu).
 #include "common.cuh"
 #include "mma_conv.h"
+#include "oper_conv.h"
 
 namespace bs {
 
@@ -262,9 +263,9 @@ extern "C" int bitserial_gemm_tc(const uint32_t* a_packed, const int8_t* w_tc, i
     return bs::tc_conv_impl(a_packed, w_tc, &p, out_i32, out_packed, static_cast<cudaStream_t>(stream), false);
 }
 
-extern "C" int bs_sequence_create(const bs_sequence_layer* layers, int nlayers, void* side_stream, bs_sequence** out)
+static int bs_sequence_check(const bs_sequence_layer* layers, int nlayers)
 {
-    if (!layers || nlayers <= 0 || !out) return BS_ERR_INVALID_ARG;
+    if (!layers || nlayers <= 0) return BS_ERR_INVALID_ARG;
     for (int l = 0; l < nlayers; ++l) {
         const bs_sequence_layer& s = layers[l];
         if (!s.wgt_tc && !s.wgt_packed) return BS_ERR_INVALID_ARG;
@@ -272,9 +273,34 @@ extern "C" int bs_sequence_create(const bs_sequence_layer* layers, int nlayers, 
         if (rc == BS_OK && s.wgt_tc) rc = bs::tc_validate(&s.p);
         if (rc == BS_OK) rc = bs::tc_validate_outputs(s.act_packed, s.wgt_tc ? static_cast<const void*>(s.wgt_tc) : s.wgt_packed, &s.p, nullptr, s.out_packed);
         if (rc != BS_OK) return rc;
-        if (s.aside && !side_stream) return BS_ERR_INVALID_ARG;
     }
-    return bs::mma_sequence_create(layers, nlayers, static_cast<cudaStream_t>(side_stream), reinterpret_cast<bs::Sequence**>(out));
+    return BS_OK;
+}
+
+extern "C" size_t bs_sequence_workspace_bytes(const bs_sequence_layer* layers, int nlayers)
+{
+    return bs_sequence_check(layers, nlayers) == BS_OK ? bs::oper_workspace_bytes(layers, nlayers) : 0;
+}
+
+extern "C" int bs_sequence_create_ws(const bs_sequence_layer* layers, int nlayers, void* side_stream, void* workspace, size_t workspace_bytes, bs_sequence** out)
+{
+    if (!out) return BS_ERR_INVALID_ARG;
+    const int rc = bs_sequence_check(layers, nlayers);
+    if (rc != BS_OK) return rc;
+    for (int l = 0; l < nlayers; ++l)
+        if (layers[l].aside && !side_stream) return BS_ERR_INVALID_ARG;
+    if (workspace && !bs::aligned16(workspace)) return BS_ERR_ALIGNMENT;
+    return bs::mma_sequence_create(layers, nlayers, static_cast<cudaStream_t>(side_stream), workspace, workspace_bytes, reinterpret_cast<bs::Sequence**>(out));
+}
+
+extern "C" int bs_sequence_create(const bs_sequence_layer* layers, int nlayers, void* side_stream, bs_sequence** out)
+{
+    return bs_sequence_create_ws(layers, nlayers, side_stream, nullptr, 0, out);
+}
+
+extern "C" int bs_sequence_launches(const bs_sequence* sequence)
+{
+    return sequence ? bs::mma_sequence_launches(reinterpret_cast<const bs::Sequence*>(sequence)) : 0;
 }
 
 extern "C" int bs_sequence_run(bs_sequence* sequence, void* stream)

@@ -19,7 +19,7 @@ from .workloads import NetSpec
 
 class _Sequence:
     """The launches of a pass bound to what they read and write.  ``handle``: the ``bs_sequence``, None where the library does not take the
-    layers as one.  ``dicts`` name the tensors and settings of the layers; ``values`` are what was found there, kept alive because a sequence
+    layers as one; ``launches``: kernels of a run.  ``dicts`` name the tensors and settings of the layers; ``values`` are what was found there, kept alive because a sequence
     and the graphs captured from it hold the tensors' ``addresses``."""
 
     def __init__(self, units, concurrent, dicts):
@@ -28,9 +28,11 @@ class _Sequence:
         self.values = tuple(v for d in self.dicts for v in d.values())
         self.addresses = tuple(v.data_ptr() if isinstance(v, torch.Tensor) else None for v in self.values)
         self.handle = None
+        self.launches = 0
 
     def own(self, handle: int) -> None:
         self.handle = handle
+        self.launches = lib().bs_sequence_launches(handle)
         weakref.finalize(self, lib().bs_sequence_destroy, handle).atexit = False
 
     def current(self, units, concurrent) -> bool:
@@ -80,6 +82,7 @@ class BitserialNet:
         self.graph = None
         self.static_in = None
         self.launches_per_forward = 1 + len(self.layers)
+        self._workspaces: Dict[tuple, torch.Tensor] = {}
         self._sequence: Optional[_Sequence] = None
         self._captured: Optional[_Sequence] = None      # what the graph was captured from
         self._bind()
@@ -203,7 +206,7 @@ class BitserialNet:
         """All layers on the current stream, and on the side stream those that :meth:`schedule` puts there; under stream capture the
         events between them become the edges of the graph."""
         if self._bind():
-            api.run_sequence(self._sequence.handle, len(self.layers))
+            api.run_sequence(self._sequence.handle, self._sequence.launches)
         else:
             self.run_units()
 
@@ -253,10 +256,32 @@ class BitserialNet:
             q.chained, q.aside = 1, int(aside)
             q.join[:] = (join + [-1] * 4)[:4]
         handle = ctypes.c_void_p()
-        if lib().bs_sequence_create(arr, len(layers), self.side.cuda_stream, ctypes.byref(handle)) != 0:
+        ws = self._workspace(arr)
+        if lib().bs_sequence_create_ws(arr, len(layers), self.side.cuda_stream, api._ptr(ws), ws.numel() if ws is not None else 0, ctypes.byref(handle)) != 0:
             return False
         self._sequence.own(handle.value)
+        self.launches_per_forward = 1 + self._sequence.launches
         return True
+
+    def _workspace(self, arr) -> Optional[torch.Tensor]:
+        """Memory of the layers' operand tensors (``bs_sequence_create_ws``), or None.  Kept while the runner lives, for every arrangement of tensors
+        it has had: graphs that a caller recorded go on using it."""
+        nbytes = lib().bs_sequence_workspace_bytes(arr, len(arr))
+        if nbytes == 0:
+            return None
+        tensors = {}
+        at = lambda address: tensors.setdefault(address, len(tensors))
+        key = tuple((at(q.act_packed), at(q.out_packed), *(getattr(q.p, f) for f in (
+            "N", "C", "H", "W", "O", "R", "stride", "pad", "a_bits", "out_bits", "out_c_offset", "out_c_total"))) for q in arr)
+        ws = self._workspaces.get(key)
+        if ws is None and not torch.cuda.is_current_stream_capturing():     # (recorded, its clearing would belong to the graph)
+            try:
+                ws = torch.zeros(nbytes, dtype=torch.uint8, device=self.device)
+            except torch.OutOfMemoryError:
+                return None
+            torch.cuda.synchronize(self.device)
+            self._workspaces[key] = ws
+        return ws
 
     def _conv_params(self, item):
         net, L = self.net, item["spec"]

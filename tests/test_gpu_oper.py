@@ -1,0 +1,128 @@
+"""Layers of a bound sequence on operand tensors: every packed tensor of a pass equals, bit for bit, what the same layers write one call at a time
+(whose kernels read packed codes), and the oracle where that is quick.  Geometries at the edges of the position numbering: one channel
+group and odd numbers of them, readers of both strides of one tensor, windows without padding and of 5 and 7, concatenations, tensors that
+a pass only reads in part from its own layers, rows and images of one pixel."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import network as onet
+from paper_2207_08820_b200 import api, workloads as wl
+from paper_2207_08820_b200.net import BitserialNet
+from paper_2207_08820_b200.workloads import ConvSpec, NetSpec
+from gpu_util import dev
+
+pytestmark = pytest.mark.gpu
+
+L = ConvSpec
+
+
+def net(batch, in_shape, layers, a_bits=2, w_bits=2):
+    return NetSpec(name="t", batch=batch, in_name="x", in_shape=in_shape, layers=layers, a_bits=a_bits, w_bits=w_bits, out_name=layers[-1].dst)
+
+
+STACKS = {
+    "one_group": net(3, (32, 9, 12), [L("a", "x", "a", 32, 32, 3, 1, 1), L("b", "a", "b", 32, 96, 3, 2, 1), L("c", "b", "c", 96, 64, 1, 1, 0)]),
+    "odd_groups": net(2, (96, 13, 8), [L("a", "x", "a", 96, 160, 3, 1, 1), L("b", "a", "b", 160, 96, 1, 2, 0, relu=False), L("c", "b", "c", 96, 40, 3, 1, 1)]),
+    # readers of stride 1 and 2, with and without padding, of one tensor
+    "both_strides": net(5, (64, 15, 15), [L("a", "x", "a", 64, 64, 3, 1, 1), L("b", "a", "b", 64, 64, 3, 2, 1), L("c", "a", "c", 64, 64, 1, 2, 0),
+                                          L("d", "a", "d", 64, 64, 5, 1, 2), L("e", "a", "e", 64, 64, 3, 1, 0), L("f", "b", "f", 64, 64, 3, 1, 1, res="c", res_scale=0.5),
+                                          L("g", "d", "g", 64, 32, 7, 2, 3), L("h", "e", "h", 64, 32, 5, 2, 1)]),
+    "concatenation": net(2, (64, 20, 20), [L("a", "x", "cat", 64, 64, 1, 1, 0, dst_c_offset=64), L("b", "x", "b", 64, 64, 3, 1, 1),
+                                           L("c", "b", "cat", 64, 64, 3, 1, 1, res="x", res_scale=0.5), L("d", "cat", "d", 128, 256, 1, 1, 0)]),
+    "one_bit": net(3, (64, 10, 12), [L("a", "x", "a", 64, 128, 3, 1, 1), L("b", "a", "b", 128, 64, 3, 2, 1), L("c", "b", "c", 64, 64, 1, 1, 0, res="b", res_scale=0.5)], 1, 1),
+    "wide": net(1, (32, 3, 300), [L("a", "x", "a", 32, 64, 3, 1, 1), L("b", "a", "b", 64, 32, 3, 2, 1), L("c", "b", "c", 32, 32, 1, 1, 0)]),
+    "deep": net(1, (512, 7, 7), [L("a", "x", "a", 512, 256, 3, 1, 1), L("b", "a", "b", 256, 512, 1, 1, 0), L("c", "b", "c", 512, 64, 3, 2, 1)]),
+    "pixels": net(40, (64, 1, 1), [L("a", "x", "a", 64, 64, 3, 1, 1), L("b", "a", "b", 64, 64, 1, 1, 0), L("c", "b", "c", 64, 32, 3, 2, 1)]),
+}
+
+
+def runner_of(spec, seed=11):
+    params = wl.network_params(spec, seed)
+    r = BitserialNet(spec, params, 0.25, batch=spec.batch, engine="tc")
+    return r, params, wl.network_input(spec, seed, 0.25, batch=spec.batch)
+
+
+def both(r, x):
+    """Every packed tensor after a pass and after the same layers called one by one."""
+    xd, out = dev(x), []
+    for one_by_one in (False, True):
+        for b in r.bufs.values():
+            b.fill_(-1 if one_by_one else 0x5A5A5A5A)
+        r.pack_input(xd)
+        r.run_units() if one_by_one else r.run_layers()
+        api.bs_check_status()
+        out.append({k: b.clone() for k, b in r.bufs.items()})
+    return out
+
+
+@pytest.mark.parametrize("name", STACKS)
+def test_stacks(name):
+    spec = STACKS[name]
+    r, params, x = runner_of(spec)
+    assert r.launches_per_forward > 1 + len(spec.layers)             # the layers take operand tensors
+    for seed in (0, 1):
+        got, want = both(r, np.roll(x, seed, 0) if seed else x)
+        for k in want:
+            assert torch.equal(got[k], want[k]), k
+    r.forward(dev(x))
+    ref = onet.run_stack(spec, params, x, 0.25)
+    for k in ref:
+        assert np.array_equal(r.unpacked(k).cpu().numpy(), ref[k]), k
+
+
+def test_replaced_filters_scales_and_tensors():
+    """Filters prepared for other widths, scales only the formula takes, tensors that move, a graph recorded before."""
+    spec = STACKS["both_strides"]
+    r, _, x = runner_of(spec)
+    xd = dev(x)
+    graph = torch.cuda.CUDAGraph()
+    r.forward(xd)
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        r.run_layers()
+    want = {k: b.clone() for k, b in r.bufs.items()}
+    kept = [dict(item) for item in r.layers], dict(r.bufs)
+    for i, item in enumerate(r.layers):
+        if i % 2 == 0:
+            item["w_tc"] = api.tc_prepare_weights(item["w"], item["spec"].C, item["w_sign"], 4)
+        if i % 3 == 0:
+            item["scale"] = item["scale"].clone()
+            item["scale"][0] = 1e-19
+    for k in r.bufs:
+        r.bufs[k] = torch.empty_like(r.bufs[k])
+    got, one_by_one = both(r, x)
+    for k in got:
+        assert torch.equal(got[k], one_by_one[k]), k
+    for k, b in kept[1].items():
+        if k != "x":
+            b.fill_(-1)
+    graph.replay()
+    torch.cuda.synchronize()
+    for k, b in kept[1].items():
+        assert torch.equal(b, want[k]), k
+    api.bs_check_status()
+
+
+def test_sequences_that_keep_packed_tensors():
+    """Overlapping tensors and layers without prepared filters run as they did."""
+    spec = STACKS["one_group"]
+    r, _, x = runner_of(spec)
+    r.layers[1]["w_tc"] = None
+    got, want = both(r, x)
+    assert r.launches_per_forward == 1 + len(spec.layers)
+    for k in want:
+        assert torch.equal(got[k], want[k]), k
+    r, _, x = runner_of(spec)
+    whole = torch.zeros(r.bufs["a"].numel() + r.bufs["c"].numel(), dtype=torch.int32, device="cuda")
+    n = r.bufs["c"].numel()
+    r.bufs["a"] = whole[: r.bufs["a"].numel()].view_as(r.bufs["a"])
+    r.bufs["c"] = whole[4: 4 + n].view_as(r.bufs["c"])              # "a" is dead once "b" has been written
+    xd = dev(x)
+    r.forward(xd)
+    assert r.launches_per_forward == 1 + len(spec.layers)
+    have = r.bufs["c"].clone()
+    r.pack_input(xd)
+    r.run_units()
+    assert torch.equal(have, r.bufs["c"])
+    api.bs_check_status()
