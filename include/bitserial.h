@@ -313,12 +313,24 @@ int bs_sequence_create(const bs_sequence_layer* layers, int nlayers, void* side_
  *                         less than that: as bs_sequence_create.  May pass on to another sequence of layers of the same shapes, formats and order.
  * bs_sequence_workspace_bytes answers 0 where the layers don't take one: layers without prepared filters, codes of more than two bits or signed ones,
  * tensors that overlap or that are used with two shapes, rows too wide for the shared memory.  It needs no device.
- * bs_sequence_launches: kernels that a run enqueues.
+ * bs_sequence_launches: kernels that bs_sequence_run enqueues.
+ * bs_sequence_input     the operand tensor of a tensor of packed codes that the layers read before they have written all of it (it belongs to the
+ *                       sequence), NULL where there is none.  bitpack_activations_operands (fp32 NCHW, unsigned codes) and
+ *                       bs_stem_codes_operands_f32 write it beside the packed codes (NULL: these alone); their shapes, formats and output must be
+ *                       the tensor's, else BS_ERR_INVALID_ARG.  bs_sequence_run_ready then does without its launch: the caller promises that
+ *                       neither was written since.
  */
 size_t bs_sequence_workspace_bytes(const bs_sequence_layer* layers, int nlayers);
 int bs_sequence_create_ws(const bs_sequence_layer* layers, int nlayers, void* side_stream, void* workspace, size_t workspace_bytes,
                           bs_sequence** sequence_out);
 int bs_sequence_launches(const bs_sequence* sequence);
+typedef struct bs_operand_tensor bs_operand_tensor;
+const bs_operand_tensor* bs_sequence_input(const bs_sequence* sequence, const uint32_t* packed);
+int bs_sequence_run_ready(bs_sequence* sequence, const bs_operand_tensor* ready, void* stream);
+int bitpack_activations_operands(const float* x, int N, int C, int H, int W, float act_scale, int a_bits, uint32_t* packed_out,
+                                 const bs_operand_tensor* operands, void* stream);
+int bs_stem_codes_operands_f32(const float* x, const float* w, const float* bias, int N, int C, int H, int W, int O, int R, int S, int stride, int pad,
+                               float act_scale, int a_bits, uint32_t* out, const bs_operand_tensor* operands, void* stream);
 int bs_sequence_run(bs_sequence* sequence, void* stream);
 void bs_sequence_destroy(bs_sequence* sequence);
 int bitserial_gemm_tc(const uint32_t* a_packed, const int8_t* w_tc, int M, int N, int K, int a_bits, bs_sign_t a_sign,

@@ -65,6 +65,12 @@ def bitpack_activations(x: torch.Tensor, act_scale: float, a_bits: int, a_sign: 
     return out
 
 
+def bitpack_operands(x: torch.Tensor, act_scale: float, a_bits: int, out: torch.Tensor, operands: int, stream=None) -> None:
+    """:func:`bitpack_activations` of a float32 NCHW tensor to unsigned codes that writes, beside ``out``, the operand tensor ``operands`` of a bound
+    sequence (``bs_sequence_input``)."""
+    _check(native().bitpack_operands(x, act_scale, a_bits, out, operands, stream)[0], "bitpack_activations_operands")
+
+
 def bitunpack_activations(packed: torch.Tensor, C: int, a_bits: int, a_sign: int = UNSIGNED, layout: int = NCHW,
                           stream=None) -> torch.Tensor:
     N, H, W, Cw, b = packed.shape
@@ -203,10 +209,11 @@ def bitserial_conv2d_tc_chain(acts, wgts_tc, params, outs, workspace: torch.Tens
     launch_count += n - 1
 
 
-def run_sequence(sequence, launches: int, stream=None) -> None:
-    """One pass of a bound sequence of layers (``bs_sequence_run``), which enqueues ``launches`` kernels."""
+def run_sequence(sequence, launches: int, stream=None, ready: Optional[int] = None) -> None:
+    """One pass of a bound sequence of layers (``bs_sequence_run``), which enqueues ``launches`` kernels.  ``ready``: its operand tensor that is up
+    to date (``bs_sequence_run_ready``)."""
     global launch_count
-    _check(native().sequence_run(sequence, stream), "bs_sequence_run")
+    _check(native().sequence_run(sequence, stream, ready), "bs_sequence_run")
     launch_count += launches - 1
 
 
@@ -261,10 +268,10 @@ def maxpool2d_f32(x: torch.Tensor, k: int, stride: int, pad: int, out: Optional[
 
 
 def stem_codes_f32(x: torch.Tensor, w: torch.Tensor, bias: Optional[torch.Tensor], act_scale: float, a_bits: int, out: torch.Tensor,
-                   stream=None) -> bool:
+                   stream=None, operands: Optional[int] = None) -> bool:
     """Stem convolution (stride 2, pad 3) with ReLU, 3x3 stride-2 max pooling and quantise + pack in one call (``bs_stem_codes_f32``): images to the
     packed codes of :func:`conv2d_f32`, :func:`maxpool2d_f32` and :func:`bitpack_activations`.  False where the library has no such kernel for
-    the shape: nothing was launched."""
+    the shape: nothing was launched.  ``operands``: the operand tensor of ``out`` (``bs_sequence_input``), written as well."""
     N, C, H, W = x.shape
     O, C2, R, S = w.shape
     if C != C2 or x.dtype != torch.float32 or w.dtype != torch.float32:
@@ -272,7 +279,7 @@ def stem_codes_f32(x: torch.Tensor, w: torch.Tensor, bias: Optional[torch.Tensor
     P, Q = (H - 1) // 2 + 1, (W - 1) // 2 + 1
     if out.numel() != packed_act_words(N, O, (P - 1) // 2 + 1, (Q - 1) // 2 + 1, a_bits):
         raise ValueError("output of another size")
-    st = lib().bs_stem_codes_f32(_ptr(x), _ptr(w), _ptr(bias), N, C, H, W, O, R, S, 2, 3, act_scale, a_bits, _ptr(out), _stream_ptr(stream))
+    st = lib().bs_stem_codes_operands_f32(_ptr(x), _ptr(w), _ptr(bias), N, C, H, W, O, R, S, 2, 3, act_scale, a_bits, _ptr(out), operands, _stream_ptr(stream))
     if st == ERR_UNSUPPORTED:
         return False
     _check(st, "bs_stem_codes_f32")

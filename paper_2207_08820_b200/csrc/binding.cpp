@@ -218,18 +218,45 @@ PyObject* bitpack(PyObject*, PyObject* const* a, Py_ssize_t n)
     });
 }
 
-// sequence, stream
-PyObject* sequence_run(PyObject*, PyObject* const* a, Py_ssize_t n)
+// x, act_scale, a_bits, out, operands (of a sequence), stream
+PyObject* bitpack_operands(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
     return guarded([&] {
-        need(n, 2);
-        bs_sequence* s = reinterpret_cast<bs_sequence*>(PyLong_AsUnsignedLongLong(a[0]));
+        need(n, 6);
+        const at::Tensor &x = tensor(a[0]), &out = tensor(a[3]);
+        if (x.scalar_type() != at::kFloat) mismatch("x must be float32");
+        if (x.dim() != 4) mismatch("x must have four dimensions");
+        const float scale = real(a[1]);
+        const int bits = integer(a[2]);
+        const float* xp = static_cast<const float*>(pointer(x));
+        uint32_t* op = static_cast<uint32_t*>(pointer(out));
+        const bs_operand_tensor* to = reinterpret_cast<const bs_operand_tensor*>(PyLong_AsUnsignedLongLong(a[4]));
         if (PyErr_Occurred()) throw Fail();
-        void* st = stream_of(a[1]);
+        void* st = stream_of(a[5]);
         int rc;
         {
             NoGil free;
-            rc = bs_sequence_run(s, st);
+            rc = bitpack_activations_operands(xp, static_cast<int>(x.size(0)), static_cast<int>(x.size(1)), static_cast<int>(x.size(2)),
+                                              static_cast<int>(x.size(3)), scale, bits, op, to, st);
+        }
+        return result(rc, at::Tensor(), at::Tensor());
+    });
+}
+
+// sequence, stream, ready (an operand tensor of it, or None)
+PyObject* sequence_run(PyObject*, PyObject* const* a, Py_ssize_t n)
+{
+    return guarded([&] {
+        need(n, 3);
+        bs_sequence* s = reinterpret_cast<bs_sequence*>(PyLong_AsUnsignedLongLong(a[0]));
+        if (PyErr_Occurred()) throw Fail();
+        void* st = stream_of(a[1]);
+        const bs_operand_tensor* ready = a[2] == Py_None ? nullptr : reinterpret_cast<const bs_operand_tensor*>(PyLong_AsUnsignedLongLong(a[2]));
+        if (PyErr_Occurred()) throw Fail();
+        int rc;
+        {
+            NoGil free;
+            rc = bs_sequence_run_ready(s, ready, st);
         }
         return PyLong_FromLong(rc);
     });
@@ -262,7 +289,7 @@ PyObject* unchanged(PyObject*, PyObject* const* a, Py_ssize_t n)
 }
 
 #define FAST(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(name)), METH_FASTCALL, nullptr}
-PyMethodDef methods[] = {FAST(conv2d), FAST(gemm), FAST(bitpack), FAST(sequence_run), FAST(unchanged), {nullptr, nullptr, 0, nullptr}};
+PyMethodDef methods[] = {FAST(conv2d), FAST(gemm), FAST(bitpack), FAST(bitpack_operands), FAST(sequence_run), FAST(unchanged), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_binding", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace

@@ -553,10 +553,12 @@ int mma_sequence_create(const bs_sequence_layer* layers, int n, cudaStream_t sid
 
 int mma_sequence_launches(const Sequence* q) { return static_cast<int>(q->steps.size()) + (q->oper ? oper_imports(q->oper) : 0); }
 
-int mma_sequence_run(Sequence* q, cudaStream_t st)
+const OperTensor* mma_sequence_input(const Sequence* q, const uint32_t* packed) { return q->oper ? oper_input(q->oper, packed) : nullptr; }
+
+int mma_sequence_run(Sequence* q, const OperTensor* ready, cudaStream_t st)
 {
     if (q->oper) {
-        const int rc = oper_begin(q->oper, st);
+        const int rc = oper_begin(q->oper, ready, st);
         if (rc != BS_OK) return rc;
     }
     for (size_t i = 0; i < q->steps.size(); ++i) {

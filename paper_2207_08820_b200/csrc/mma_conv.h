@@ -31,7 +31,10 @@ int mma_conv_run(const uint32_t* act, const int8_t* wgt, const uint32_t* wgt_pac
 struct Sequence;
 int mma_sequence_create(const bs_sequence_layer* layers, int n, cudaStream_t side, void* workspace, size_t bytes, Sequence** out);
 int mma_sequence_launches(const Sequence* q);
-int mma_sequence_run(Sequence* q, cudaStream_t st);
+// ready: one of its input tensors whose operand forms are up to date, or null.
+struct OperTensor;
+const OperTensor* mma_sequence_input(const Sequence* q, const uint32_t* packed);
+int mma_sequence_run(Sequence* q, const OperTensor* ready, cudaStream_t st);
 void mma_sequence_destroy(Sequence* q);
 
 }  // namespace bs

@@ -25,24 +25,11 @@
 #pragma once
 #include "conv_kernel.cuh"
 #include "mma_conv.h"
+#include "oper_tensor.cuh"
 
 namespace bs {
 
 constexpr int MM_STAGES = 8;         // most stages of packed words in front of the expanders
-
-struct FastDiv { unsigned mul, shift; int d; };      // quotient of 0 <= n < 2^31 by d as umulhi(n, mul) >> shift
-inline FastDiv make_div(int d)
-{
-    FastDiv f{0, 0, d};
-    if (d > 1) {
-        int l = 0;
-        while ((1LL << l) < d) ++l;                       // ceil(log2 d)
-        const unsigned long long p = 31 + l;
-        f.mul = static_cast<unsigned>(((1ULL << p) + d - 1) / d);
-        f.shift = static_cast<unsigned>(p - 32);
-    }
-    return f;
-}
 
 struct MmaArgs {
     CUtensorMap tmA, tmB;           // flat tiles with aligned rows: packed pixels (words, rows), packed filters (words, filters)
@@ -291,8 +278,6 @@ __device__ __forceinline__ u64 f2_pack(uint32_t lo, uint32_t hi) { u64 r; asm("m
 __device__ __forceinline__ void f2_split(u64 v, uint32_t& lo, uint32_t& hi) { asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(v)); }
 __device__ __forceinline__ u64 f2_add(u64 a, u64 b) { u64 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 __device__ __forceinline__ u64 f2_fma(u64 a, u64 b, u64 c) { u64 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
-
-__device__ __forceinline__ int fdiv(int n, const FastDiv& f) { return f.d == 1 ? n : static_cast<int>(__umulhi(static_cast<unsigned>(n), f.mul) >> f.shift); }
 
 // ----------------------------------------------------------------------------- expansion: plane words -> int8 or nibbles
 

@@ -13,38 +13,25 @@ namespace bs {
 
 // ----------------------------------------------------------------------------- packed codes -> operand tensors
 
-struct ImportArgs {
-    const uint32_t* src;            // [pixels][Cw][bits]
-    OperDst dst1, dst2;
-    int pixels, W, Cw, bits;
-    FastDiv d_img, d_row;
-};
-
 // A lane per pixel and channel word: a warp reads the words of 32 pixels (whole sectors over its channel words, which a block shares) and writes runs
 // of 512 bytes.
-static __global__ void __launch_bounds__(256) oper_import_kernel(const __grid_constant__ ImportArgs g)
+static __global__ void __launch_bounds__(256) oper_import_kernel(const __grid_constant__ OperTensor g)
 {
-    const uint32_t* src = dependent_begin(g.src);
-    const int lane = threadIdx.x & 31, warps = static_cast<int>(gridDim.x) * 8, runs = (g.pixels + 31) / 32;
+    const uint32_t* src = dependent_begin(g.packed);
+    const int lane = threadIdx.x & 31, warps = static_cast<int>(gridDim.x) * 8, pixels = g.N * g.d_img.d, runs = (pixels + 31) / 32;
     for (long long w = blockIdx.x * 8 + (threadIdx.x >> 5); w < static_cast<long long>(runs) * g.Cw; w += warps) {
         const int run = static_cast<int>(w / g.Cw), cw = static_cast<int>(w - static_cast<long long>(run) * g.Cw), pix = run * 32 + lane;
-        if (pix >= g.pixels) continue;
+        if (pix >= pixels) continue;
         const uint32_t* p = src + (static_cast<size_t>(pix) * g.Cw + cw) * g.bits;
-        uint32_t v[4];
+        uint32_t e, d;
         if (g.bits == 2) {
             const uint2 t = *reinterpret_cast<const uint2*>(p);
-            const uint32_t two[2] = {t.x, t.y};
-            expand_nibbles<2>(two, 0, v);
+            oper_pairs(t.x, t.y, e, d);
         } else {
-            const uint32_t one[2] = {p[0], 0u};
-            expand_nibbles<1>(one, 0, v);
+            oper_pairs(p[0], 0u, e, d);
         }
         const int n = fdiv(pix, g.d_img), rem = pix - n * g.d_img.d, y = fdiv(rem, g.d_row), x = rem - y * g.W;
-        const uint4 out = make_uint4(v[0], v[1], v[2], v[3]);
-        if (g.dst1.base) *reinterpret_cast<uint4*>(g.dst1.base + cw * g.dst1.group + static_cast<long long>(n * g.dst1.img + y * g.dst1.pitch + x) * 16) = out;
-        if (g.dst2.base)
-            *reinterpret_cast<uint4*>(g.dst2.base + cw * g.dst2.group +
-                                      static_cast<long long>(n * g.dst2.img + (y >> 1) * g.dst2.pitch + (x >> 1) + (2 * (y & 1) + (x & 1)) * g.dst2.plane) * 16) = out;
+        oper_put(g.dst1, g.dst2, cw, oper_at1(g.dst1, n, y, x), oper_at2(g.dst2, n, y, x), e, d);
     }
 }
 
@@ -244,7 +231,7 @@ double cost_of(const OperArgs& g, const Cand& c, int sms)
 
 struct OperSequence {
     struct Step { OperArgs g; unsigned grid; int smem; };
-    struct Import { ImportArgs g; unsigned grid; };
+    struct Import { OperTensor g; unsigned grid; };
     std::vector<Step> steps;
     std::vector<Import> imports;
 };
@@ -340,14 +327,13 @@ static bool build(const bs_sequence_layer* layers, int n, unsigned char* ws, Ope
     for (const Tensor& t : lay.tensors) {
         if (!t.read || !t.import) continue;
         OperSequence::Import m{};
-        m.g.src = t.ptr;
+        m.g.packed = t.ptr;
         m.g.dst1 = dst_of(t, 0, ws, 0);
         m.g.dst2 = dst_of(t, 1, ws, 0);
-        m.g.pixels = t.N * t.H * t.W;
-        m.g.W = t.W; m.g.Cw = t.Cw; m.g.bits = t.bits;
+        m.g.N = t.N; m.g.H = t.H; m.g.W = t.W; m.g.Cw = t.Cw; m.g.bits = t.bits;
         m.g.d_img = make_div(t.H * t.W);
         m.g.d_row = make_div(t.W);
-        const long long blocks = (ceil_div_ll(m.g.pixels, 32) * t.Cw + 7) / 8;
+        const long long blocks = (ceil_div_ll(static_cast<long long>(t.N) * t.H * t.W, 32) * t.Cw + 7) / 8;
         m.grid = static_cast<unsigned>(blocks < 8LL * sms ? blocks : 8LL * sms);
         q.imports.push_back(m);
     }
@@ -376,9 +362,17 @@ OperSequence* oper_create(const bs_sequence_layer* layers, int n, void* workspac
 
 int oper_imports(const OperSequence* q) { return static_cast<int>(q->imports.size()); }
 
-int oper_begin(const OperSequence* q, cudaStream_t st)
+const OperTensor* oper_input(const OperSequence* q, const uint32_t* packed)
+{
+    for (const OperSequence::Import& m : q->imports)
+        if (m.g.packed == packed) return &m.g;
+    return nullptr;
+}
+
+int oper_begin(const OperSequence* q, const OperTensor* ready, cudaStream_t st)
 {
     for (const OperSequence::Import& m : q->imports) {
+        if (&m.g == ready) continue;
         const int rc = launch_dependent(oper_import_kernel, dim3(m.grid), dim3(256), 0, st, m.g);
         if (rc != BS_OK) return rc;
     }

@@ -7,14 +7,17 @@
 namespace bs {
 
 struct OperSequence;
+struct OperTensor;
 
 // Bytes of zeroed device memory that the layers need to run on operand tensors; 0: they don't take them (mma_conv.cu runs them).
 size_t oper_workspace_bytes(const bs_sequence_layer* layers, int n);
 // The launches of such layers; null where oper_workspace_bytes is 0 or bytes is less.
 OperSequence* oper_create(const bs_sequence_layer* layers, int n, void* workspace, size_t bytes);
-// Launches in front of the layers, all of them on `st`; layer i on `st`.
+// The forms of a tensor that the layers read from its packed codes, which launches in front of the layers bring into them; null: no such tensor.
 int oper_imports(const OperSequence* q);
-int oper_begin(const OperSequence* q, cudaStream_t st);
+const OperTensor* oper_input(const OperSequence* q, const uint32_t* packed);
+// These launches but the one of `ready`, whose forms are up to date (or null), and layer i, on `st`.
+int oper_begin(const OperSequence* q, const OperTensor* ready, cudaStream_t st);
 int oper_layer(const OperSequence* q, int i, cudaStream_t st);
 void oper_destroy(OperSequence* q);
 

@@ -17,14 +17,6 @@ namespace bs {
 
 constexpr int OP_STAGES = 8, OP_EW = 8, OP_THREADS = (OP_EW + 2) * 32;
 
-// A tensor as the epilogue writes it: byte address of position 0 of the first group written, or null.  Stride 2: position (y / 2, x / 2) of plane
-// 2 (y & 1) + (x & 1).
-struct OperDst {
-    unsigned char* base;
-    long long group;                // bytes between channel groups
-    int plane, pitch, img;          // positions of a parity plane, a row, an image
-};
-
 struct OperArgs {
     const unsigned char* src;       // operand tensor of the input, at the first halo position of tile 0 (of plane 0, group 0)
     long long src_group, src_plane; // bytes between channel groups, parity planes
@@ -64,8 +56,8 @@ __device__ __forceinline__ OperPos oper_position(const OperArgs& g, int pos)
     OperPos o;
     const int n = fdiv(pos, g.d_img), rem = pos - n * g.d_img.d, y = fdiv(rem, g.d_pitch), x = rem - y * g.d_pitch.d;
     o.pix = pos < g.total && y < g.P && x < g.Q ? (n * g.P + y) * g.Q + x : -1;
-    o.at1 = n * g.dst1.img + y * g.dst1.pitch + x;
-    o.at2 = n * g.dst2.img + (y >> 1) * g.dst2.pitch + (x >> 1) + (2 * (y & 1) + (x & 1)) * g.dst2.plane;
+    o.at1 = oper_at1(g.dst1, n, y, x);
+    o.at2 = oper_at2(g.dst2, n, y, x);
     return o;
 }
 
@@ -74,9 +66,7 @@ __device__ __forceinline__ void oper_store(const OperArgs& g, const OperPos& o, 
 {
     uint32_t ow[4] = {(e & 0x55555555u) | ((d << 1) & 0xAAAAAAAAu), ((e >> 1) & 0x55555555u) | (d & 0xAAAAAAAAu), 0u, 0u};
     store_codes(g, o.pix, ob, ow);
-    const uint4 v = make_uint4(e & 0x33333333u, d & 0x33333333u, (e >> 2) & 0x33333333u, (d >> 2) & 0x33333333u);
-    if (g.dst1.base) *reinterpret_cast<uint4*>(g.dst1.base + (ob >> 5) * g.dst1.group + static_cast<long long>(o.at1) * 16) = v;
-    if (g.dst2.base) *reinterpret_cast<uint4*>(g.dst2.base + (ob >> 5) * g.dst2.group + static_cast<long long>(o.at2) * 16) = v;
+    oper_put(g.dst1, g.dst2, ob >> 5, o.at1, o.at2, e, d);
 }
 
 // An item through the documented formula, one output at a time (scales and biases outside the range of the fast form).
@@ -95,7 +85,9 @@ static __device__ __noinline__ void oper_item_formula(const OperArgs& g, uint32_
             for (int c = 0; c < 32; ++c) v[c] = acc_int(true, v[c], 0u);
             if (g.residual) load_residual(g, px.pix, ob, rw);
             requant32_formula(g, v, ob, rw, ow);
-            oper_store(g, px, ob, (ow[0] & 0x55555555u) | ((ow[1] << 1) & 0xAAAAAAAAu), ((ow[0] >> 1) & 0x55555555u) | (ow[1] & 0xAAAAAAAAu));
+            uint32_t even, odd;
+            oper_pairs(ow[0], ow[1], even, odd);
+            oper_store(g, px, ob, even, odd);
         }
         __syncwarp();
     }

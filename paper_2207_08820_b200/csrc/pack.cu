@@ -2,8 +2,10 @@
 // unpack, and the offline plane split of weights / matrix rows.
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "common.cuh"
+#include "oper_tensor.cuh"
 
 namespace bs {
 
@@ -170,10 +172,13 @@ __device__ __forceinline__ uint32_t warp_transpose32(uint32_t x, int lane)
 constexpr int FAST_THREADS = 128;
 constexpr int FAST_WARPS = FAST_THREADS / 32;
 
-template <int BITS, bool LEVELS>
+// OPER: the codes also go to the operand tensors of the layers that read them (o), 16 bytes a lane in runs of 512, where a pass over the packed codes
+// would follow.
+struct NoOper {};
+template <int BITS, bool LEVELS, typename Oper = NoOper>
 __global__ void __launch_bounds__(FAST_THREADS, 8)
 bitpack_nchw_f32_kernel(const float* __restrict__ x_in, uint32_t* __restrict__ out, int C, int HW, int Cw, long long nunits,
-                        int units_per_img, const __grid_constant__ QuantParams q)
+                        int units_per_img, const __grid_constant__ QuantParams q, const __grid_constant__ Oper o)
 {
     __shared__ float s_below[16];
     load_levels<LEVELS>(s_below, q);
@@ -213,6 +218,12 @@ bitpack_nchw_f32_kernel(const float* __restrict__ x_in, uint32_t* __restrict__ o
     // pattern = (qmin + count) mod 2^BITS: two's-complement codes (qmin = -2^(BITS-1)) flip the top plane only
     if (q.sign == BS_SIGNED) planes.w[BITS - 1] ^= fl;
     store_planes<BITS>(out + ((static_cast<size_t>(n) * HW + hw0 + lane) * Cw + cw) * BITS, planes.w);
+    if constexpr (!std::is_same<Oper, NoOper>::value) {
+        const int y = fdiv(hw0 + lane, o.d_row), x = hw0 + lane - y * o.W;
+        uint32_t even, odd;
+        oper_pairs(planes.w[0], BITS > 1 ? planes.w[BITS - 1] : 0u, even, odd);
+        oper_put(o.dst1, o.dst2, cw, oper_at1(o.dst1, static_cast<int>(n), y, x), oper_at2(o.dst2, static_cast<int>(n), y, x), even, odd);
+    }
 }
 
 // fp32 NHWC input, comparison form at any width.  Work unit of a warp = 32 consecutive pixels x one 32-channel word, lane
@@ -715,7 +726,7 @@ template <int BITS, bool LEVELS>
 static int launch_f32(bool nhwc, const void* x, uint32_t* out, int N, int C, int HW, const QuantParams& q, cudaStream_t st)
 {
     return nhwc ? launch_units(bitpack_nhwc_f32_kernel<BITS, LEVELS>, x, out, N, C, HW, 32, st, q)
-                : launch_units(bitpack_nchw_f32_kernel<BITS, LEVELS>, x, out, N, C, HW, 32, st, q);
+                : launch_units(bitpack_nchw_f32_kernel<BITS, LEVELS>, x, out, N, C, HW, 32, st, q, NoOper{});
 }
 
 static int launch_bitpack_f32(bool nhwc, const void* x, uint32_t* out, int N, int C, int HW, const QuantParams& q, cudaStream_t st)
@@ -728,6 +739,32 @@ static int launch_bitpack_f32(bool nhwc, const void* x, uint32_t* out, int N, in
     }
 }
 
+// The bisection of the bounds takes several microseconds: a thread keeps the last one it made.
+static const QuantParams& quant_params(float act_scale, int bits, int sign)
+{
+    static thread_local QuantParams q;
+    static thread_local float q_scale = 0.0f;
+    if (q_scale != act_scale || q.bits != bits || q.sign != sign) {
+        q = make_quant_params(act_scale, bits, sign);
+        q_scale = act_scale;
+    }
+    return q;
+}
+
+extern "C" int bitpack_activations_operands(const float* x, int N, int C, int H, int W, float act_scale, int a_bits, uint32_t* packed_out,
+                                            const bs_operand_tensor* operands, void* stream)
+{
+    const OperTensor* o = reinterpret_cast<const OperTensor*>(operands);
+    if (!o) return bitpack_activations(x, 1, BS_NCHW, N, C, H, W, act_scale, a_bits, BS_UNSIGNED, packed_out, stream);
+    if (!x || !packed_out || packed_out != o->packed || N != o->N || C != o->Cw * 32 || H != o->H || W != o->W || a_bits != o->bits) return BS_ERR_INVALID_ARG;
+    if (!(act_scale > 0.0f && act_scale < 3.0e38f)) return BS_ERR_INVALID_ARG;
+    if (!aligned16(x) || !aligned16(packed_out)) return BS_ERR_ALIGNMENT;
+    const QuantParams& q = quant_params(act_scale, a_bits, BS_UNSIGNED);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    return a_bits == 1 ? launch_units(bitpack_nchw_f32_kernel<1, false, OperTensor>, x, packed_out, N, C, H * W, 32, st, q, *o)
+                       : launch_units(bitpack_nchw_f32_kernel<2, false, OperTensor>, x, packed_out, N, C, H * W, 32, st, q, *o);
+}
+
 extern "C" int bitpack_activations(const void* x, int x_is_fp32, bs_layout_t layout, int N, int C, int H, int W,
                                    float act_scale, int a_bits, bs_sign_t a_sign, uint32_t* packed_out, void* stream)
 {
@@ -738,16 +775,7 @@ extern "C" int bitpack_activations(const void* x, int x_is_fp32, bs_layout_t lay
     if (static_cast<long long>(H) * W > 0x7fffffffLL) return BS_ERR_UNSUPPORTED;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int HW = H * W;
-    if (x_is_fp32) {
-        // the bisection of the bounds takes several microseconds: a thread keeps the last one it made
-        static thread_local QuantParams q;
-        static thread_local float q_scale = 0.0f;
-        if (q_scale != act_scale || q.bits != a_bits || q.sign != a_sign) {
-            q = make_quant_params(act_scale, a_bits, a_sign);
-            q_scale = act_scale;
-        }
-        return launch_bitpack_f32(layout == BS_NHWC, x, packed_out, N, C, HW, q, st);
-    }
+    if (x_is_fp32) return launch_bitpack_f32(layout == BS_NHWC, x, packed_out, N, C, HW, quant_params(act_scale, a_bits, a_sign), st);
     return layout == BS_NHWC ? launch_bitpack_i8<true>(x, packed_out, N, C, HW, a_bits, a_sign == BS_BIPOLAR, st)
                              : launch_bitpack_i8<false>(x, packed_out, N, C, HW, a_bits, a_sign == BS_BIPOLAR, st);
 }

@@ -48,6 +48,7 @@ struct StemArgs {
     const float* w;
     const float* bias;
     uint32_t* out;
+    OperDst dst1, dst2;             // the codes as operand tensors of the layers that read them, or null
     int* status;
     int H, W, P, Q, P2, Q2;
     int share, extra;           // pooled rows of a CTA, CTAs with one more
@@ -630,7 +631,13 @@ __global__ void __launch_bounds__(ST_THREADS, 1) stem_codes_kernel(const __grid_
                         }
                     // an undecided output matters where none is certain to reach the code it may have
                     uint32_t und = (u0 & ~o1) | (u1 & ~o2) | (u2 & ~o3);
-                    *reinterpret_cast<uint2*>(out + i * 2) = make_uint2(((o1 & ~o2) | o3) & ~und, o2 & ~und);
+                    const uint32_t c0 = ((o1 & ~o2) | o3) & ~und, c1 = o2 & ~und;
+                    *reinterpret_cast<uint2*>(out + i * 2) = make_uint2(c0, c1);
+                    if (a.dst1.base || a.dst2.base) {
+                        uint32_t even, odd;
+                        oper_pairs(c0, c1, even, odd);
+                        oper_put(a.dst1, a.dst2, i & 1, oper_at1(a.dst1, w.n, w.y0 + r, x), oper_at2(a.dst2, w.n, w.y0 + r, x), even, odd);
+                    }
                     while (und) {
                         const unsigned f = static_cast<unsigned>(__ffs(und)) - 1;
                         und &= und - 1;
@@ -679,7 +686,13 @@ __global__ void __launch_bounds__(ST_THREADS, 1) stem_codes_kernel(const __grid_
                             const float v = stem_chain_eight(image, ws + filter * ST_TAPS, bias, a.H, a.W, p0 + m / 3, q0 + m % 3, l, live, own);
                             if (live && v > below) { ++top; members = 0; }
                         }
-                        if (k < n && l < 2 && (top >> l & 1u)) atomicOr(out + i * 2 + l, 1u << f);
+                        if (k < n && l < 2 && (top >> l & 1u)) {
+                            atomicOr(out + i * 2 + l, 1u << f);
+                            const int y = w.y0 + r, x = (i >> 1) - r * a.Q2;
+                            const uint32_t bit = 1u << (4 * (f >> 2) + l);          // nibble f / 4 of word f % 4
+                            if (a.dst1.base) atomicOr(oper_words(a.dst1, i & 1, oper_at1(a.dst1, w.n, y, x)) + (f & 3), bit);
+                            if (a.dst2.base) atomicOr(oper_words(a.dst2, i & 1, oper_at2(a.dst2, w.n, y, x)) + (f & 3), bit);
+                        }
                     }
                 } else {
                     resolve(2 * done * a.pitch, 2 * ready * a.pitch + a.Q);         // too many for the list: all of these rows, then once more
@@ -791,6 +804,12 @@ extern "C" int bs_stem_codes_supported(int N, int C, int H, int W, int O, int R,
 extern "C" int bs_stem_codes_f32(const float* x, const float* w, const float* bias, int N, int C, int H, int W, int O, int R, int S, int stride, int pad,
                                  float act_scale, int a_bits, uint32_t* out, void* stream)
 {
+    return bs_stem_codes_operands_f32(x, w, bias, N, C, H, W, O, R, S, stride, pad, act_scale, a_bits, out, nullptr, stream);
+}
+
+extern "C" int bs_stem_codes_operands_f32(const float* x, const float* w, const float* bias, int N, int C, int H, int W, int O, int R, int S, int stride, int pad,
+                                          float act_scale, int a_bits, uint32_t* out, const bs_operand_tensor* operands, void* stream)
+{
     using namespace bs;
     if (!x || !w || !out) return BS_ERR_INVALID_ARG;
     StemArgs g{};
@@ -799,6 +818,11 @@ extern "C" int bs_stem_codes_f32(const float* x, const float* w, const float* bi
     if (rc == BS_ERR_INVALID_ARG) return rc;
     if (!aligned16(x) || !aligned16(w) || !aligned16(out) || (bias && (reinterpret_cast<uintptr_t>(bias) & 3u))) return BS_ERR_ALIGNMENT;
     if (rc != BS_OK) return rc;
+    if (const OperTensor* o = reinterpret_cast<const OperTensor*>(operands)) {
+        if (out != o->packed || N != o->N || O != o->Cw * 32 || g.P2 != o->H || g.Q2 != o->W || a_bits != o->bits) return BS_ERR_INVALID_ARG;
+        g.dst1 = o->dst1;
+        g.dst2 = o->dst2;
+    }
     g.x = x; g.w = w; g.bias = bias; g.out = out;
     g.status = status_device_ptr();
     const int sms = device_sm_count();

@@ -303,9 +303,17 @@ extern "C" int bs_sequence_launches(const bs_sequence* sequence)
     return sequence ? bs::mma_sequence_launches(reinterpret_cast<const bs::Sequence*>(sequence)) : 0;
 }
 
-extern "C" int bs_sequence_run(bs_sequence* sequence, void* stream)
+extern "C" int bs_sequence_run(bs_sequence* sequence, void* stream) { return bs_sequence_run_ready(sequence, nullptr, stream); }
+
+extern "C" const bs_operand_tensor* bs_sequence_input(const bs_sequence* sequence, const uint32_t* packed)
 {
-    return sequence ? bs::mma_sequence_run(reinterpret_cast<bs::Sequence*>(sequence), static_cast<cudaStream_t>(stream)) : BS_ERR_INVALID_ARG;
+    return sequence ? reinterpret_cast<const bs_operand_tensor*>(bs::mma_sequence_input(reinterpret_cast<const bs::Sequence*>(sequence), packed)) : nullptr;
+}
+
+extern "C" int bs_sequence_run_ready(bs_sequence* sequence, const bs_operand_tensor* ready, void* stream)
+{
+    return sequence ? bs::mma_sequence_run(reinterpret_cast<bs::Sequence*>(sequence), reinterpret_cast<const bs::OperTensor*>(ready), static_cast<cudaStream_t>(stream))
+                    : BS_ERR_INVALID_ARG;
 }
 
 extern "C" void bs_sequence_destroy(bs_sequence* sequence) { bs::mma_sequence_destroy(reinterpret_cast<bs::Sequence*>(sequence)); }

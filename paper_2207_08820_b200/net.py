@@ -29,10 +29,12 @@ class _Sequence:
         self.addresses = tuple(v.data_ptr() if isinstance(v, torch.Tensor) else None for v in self.values)
         self.handle = None
         self.launches = 0
+        self.input: Optional[int] = None        # operand tensor of the network's input
 
-    def own(self, handle: int) -> None:
+    def own(self, handle: int, packed: int) -> None:
         self.handle = handle
         self.launches = lib().bs_sequence_launches(handle)
+        self.input = lib().bs_sequence_input(handle, packed)
         weakref.finalize(self, lib().bs_sequence_destroy, handle).atexit = False
 
     def current(self, units, concurrent) -> bool:
@@ -128,9 +130,20 @@ class BitserialNet:
         return units
 
     def _run(self, x: torch.Tensor) -> torch.Tensor:
-        self.pack_input(x)
-        self.run_layers()
+        self._run_layers(self._pack(x, self._ready()))
         return self.bufs[self.net.out_name]
+
+    def _ready(self) -> Optional[int]:
+        """The operand tensor of the packed input (``bs_sequence_input``) that a producer of the input may write as well, or None."""
+        return self._sequence.input if self._bind() else None
+
+    def _pack(self, x: torch.Tensor, ready: Optional[int]) -> Optional[int]:
+        """:meth:`pack_input`, to ``ready`` as well where ``x`` is the whole input; returns what is ready then."""
+        if ready is not None and x.dtype == torch.float32 and tuple(x.shape) == (self.batch, *self.net.in_shape):
+            api.bitpack_operands(x, self.act_scale, self.net.a_bits, self.bufs[self.net.in_name], ready)
+            return ready
+        self.pack_input(x)
+        return None
 
     def pack_input(self, x: torch.Tensor) -> None:
         """Quantise + bitplane-pack the fp32 input on the current stream."""
@@ -205,8 +218,13 @@ class BitserialNet:
     def run_layers(self) -> None:
         """All layers on the current stream, and on the side stream those that :meth:`schedule` puts there; under stream capture the
         events between them become the edges of the graph."""
+        self._run_layers(None)
+
+    def _run_layers(self, ready: Optional[int]) -> None:
         if self._bind():
-            api.run_sequence(self._sequence.handle, self._sequence.launches)
+            q = self._sequence
+            ready = ready if ready == q.input else None
+            api.run_sequence(q.handle, q.launches - (ready is not None), ready=ready)
         else:
             self.run_units()
 
@@ -259,8 +277,8 @@ class BitserialNet:
         ws = self._workspace(arr)
         if lib().bs_sequence_create_ws(arr, len(layers), self.side.cuda_stream, api._ptr(ws), ws.numel() if ws is not None else 0, ctypes.byref(handle)) != 0:
             return False
-        self._sequence.own(handle.value)
-        self.launches_per_forward = 1 + self._sequence.launches
+        self._sequence.own(handle.value, api._ptr(self.bufs[self.net.in_name]))
+        self.launches_per_forward = 1 + self._sequence.launches - (self._sequence.input is not None)
         return True
 
     def _workspace(self, arr) -> Optional[torch.Tensor]:
@@ -376,15 +394,15 @@ class BitserialFullNet:
         self._front(images)
         self._join_note()
 
-    def _front(self, images: torch.Tensor) -> None:
+    def _front(self, images: torch.Tensor, ready: Optional[int] = None) -> Optional[int]:
         body = self.body
         if not self._watched() and tuple(images.shape) == (self.batch, 3, self.net.hw, self.net.hw) and api.stem_codes_f32(
-                images, self.stem_w, self.stem_b, body.act_scale, body.net.a_bits, body.bufs[body.net.in_name]):
+                images, self.stem_w, self.stem_b, body.act_scale, body.net.a_bits, body.bufs[body.net.in_name], operands=ready):
             self._note_pass(images)
-        else:
-            self._stem_layers(images)
-            self._note_pass(None)
-            body.pack_input(self._stem["pool"])
+            return ready
+        self._stem_layers(images)
+        self._note_pass(None)
+        return body._pack(self._stem["pool"], ready)
 
     def _stem_layers(self, images: torch.Tensor) -> None:
         conv, pool = self._stem_tensor("conv"), self._stem_tensor("pool")
@@ -485,8 +503,7 @@ class BitserialFullNet:
 
     def forward(self, images: torch.Tensor) -> torch.Tensor:
         """images: float32 [batch, 3, hw, hw] on the device.  Returns the logits [batch, classes]."""
-        self._front(images)
-        self.body.run_layers()
+        self.body._run_layers(self._front(images, self.body._ready()))
         self.run_head()
         self._join_note()
         return self.logits

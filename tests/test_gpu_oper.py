@@ -60,7 +60,7 @@ def both(r, x):
 def test_stacks(name):
     spec = STACKS[name]
     r, params, x = runner_of(spec)
-    assert r.launches_per_forward > 1 + len(spec.layers)             # the layers take operand tensors
+    assert r._sequence.launches == len(spec.layers) + 1             # the layers take operand tensors, of the input by a launch of its own
     for seed in (0, 1):
         got, want = both(r, np.roll(x, seed, 0) if seed else x)
         for k in want:
@@ -69,6 +69,32 @@ def test_stacks(name):
     ref = onet.run_stack(spec, params, x, 0.25)
     for k in ref:
         assert np.array_equal(r.unpacked(k).cpu().numpy(), ref[k]), k
+
+
+@pytest.mark.parametrize("name", ["one_group", "both_strides", "one_bit"])
+def test_packing_writes_the_operand_tensor(name):
+    """A pass from floats writes the operand tensor of the input with its codes, without the launch of its own; layers alone follow codes that
+    were written since, and inputs of another shape or type go the general way."""
+    spec = STACKS[name]
+    r, _, x = runner_of(spec)
+    xd = dev(x)
+    assert r.launches_per_forward == 1 + len(spec.layers)
+    before = api.launch_count
+    got = r.forward(xd).clone()
+    assert api.launch_count - before == r.launches_per_forward
+    codes = r.bufs["x"].clone()
+    assert torch.equal(codes.view(-1), api.bitpack_activations(xd, 0.25, spec.a_bits).view(-1))
+    r.bufs["x"].copy_(codes.roll(1, 0))                              # codes that no float input of a pass had
+    r.run_layers()
+    want = r.bufs[spec.out_name].clone()
+    r.run_units()
+    assert torch.equal(r.bufs[spec.out_name], want) and (spec.batch == 1 or torch.equal(want, got.roll(1, 0)))
+    assert torch.equal(r.forward(xd), got)
+    with pytest.raises(ValueError):
+        r.forward(xd.transpose(2, 3))
+    with pytest.raises(ValueError):
+        r.forward(xd.cpu())
+    api.bs_check_status()
 
 
 def test_replaced_filters_scales_and_tensors():
