@@ -102,7 +102,8 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows, int sms)
     const int rel_bytes = g.flat ? 0 : up(g.NI * 4 * (1 + (c.units == 1 ? g.nsp + c.groups : 0)), 16);      // relative rows; located pixels of each group, one table more than stages
     const int pix_bytes = rel_bytes + (fb && !g.tma && c.units == 1 ? up(c.TN * g.RS * 4, 16) : 0);
     const int cap = c.cfg ? 222 * 1024 : 111 * 1024;
-    const int fixed = c.TN * 8 + 64 + 320 + red_bytes + (g.tma ? 1024 : 0) + (int_rows ? EW * 4096 : 0) + 256 + pix_bytes;
+    const int tab = c.TN * (g.f4 && A == 3 ? 12 : 8) + 64;            // scales, biases, residual multipliers, sums of filters
+    const int fixed = tab + 320 + red_bytes + (g.tma ? 1024 : 0) + (int_rows ? EW * 4096 : 0) + 256 + pix_bytes;
     const long long filters = c.resident ? static_cast<long long>(g.nblk) * c.TN * g.RS * 32 : 0;
     const long long rest = fixed + static_cast<long long>(g.nsp) * (g.stg_bytes + g.bstg_bytes) + filters;
     c.nsb = 0;
@@ -149,7 +150,7 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows, int sms)
     off += pix_bytes;
     off = (off + 127) / 128 * 128;
     g.off_out = static_cast<int>(off);              if (int_rows) off += EW * 4096;
-    g.off_tab = static_cast<int>(off);              off += c.TN * 8 + 64;
+    g.off_tab = static_cast<int>(off);              off += tab;
     off = (off + 15) / 16 * 16;
     g.off_bar = static_cast<int>(off);              off += 320;
     g.off_red = static_cast<int>(off);              off += red_bytes;
@@ -270,7 +271,7 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
     // outputs 0.98 and 0.97; codes of 5x5 windows over up to 32 channels 1.12 and 0.89 on these sides, of 3x3 windows 0.96 and 0.94.
     const bool short_k = g.Cw == 1 && static_cast<double>(g.N) * g.P * g.Q * g.O >= 2048.0 * sms;
     const bool pixel_rows = out_i32 && !out_packed && !g.i32_nhwc;
-    g.f4 = mma_nibbles(p->C, g.RS, p->a_bits, p->w_bits) && !(packed_b && (pixel_rows ? short_k || (g.R == 1 && g.Cw <= 6) : short_k && g.R >= 5 && !out_i32));
+    g.f4 = mma_nibbles(p->C, g.RS, p->a_bits, p->w_bits, p->w_sign) && !(packed_b && (pixel_rows ? short_k || (g.R == 1 && g.Cw <= 6) : short_k && g.R >= 5 && !out_i32));
     const double bound = static_cast<double>(p->C) * g.RS * max_abs_of(p->a_bits, p->a_sign) * max_abs_of(p->w_bits, p->w_sign);
     g.acc_bound = static_cast<float>(bound);
     g.preset = out_packed && !out_i32 && bound < 4.0e6 && p->out_sign != BS_BIPOLAR &&
@@ -357,7 +358,7 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
     else if (grid > items) grid = items;
     const int wb = packed_b ? p->w_bits : 0;
     const bool half = !best.cfg, split = best.split > 1;
-    plan.kern = g.f4 ? (A == 1 ? mma_kernel_f1(wb, half, split) : mma_kernel_f2(wb, half, split)) : A == 1 ? mma_kernel_a1(wb, half, split) : A == 2 ? mma_kernel_a2(wb, half, split) : A == 3 ? mma_kernel_a3(wb, half, split) : mma_kernel_a4(wb, half, split);
+    plan.kern = g.f4 ? (A == 1 ? mma_kernel_f1(wb, half, split) : A == 2 ? mma_kernel_f2(wb, half, split) : mma_kernel_f3(wb, half, split)) : A == 1 ? mma_kernel_a1(wb, half, split) : A == 2 ? mma_kernel_a2(wb, half, split) : A == 3 ? mma_kernel_a3(wb, half, split) : mma_kernel_a4(wb, half, split);
     plan.grid = static_cast<unsigned>(grid);
     plan.block = best.cfg ? MmaShape<false>::THREADS : MmaShape<true>::THREADS;
     plan.smem = static_cast<int>(best.smem);

@@ -21,6 +21,10 @@
 // the sums stay exact in binary32 (below 2^22 by mma_nibbles; compared up to 3999744 in tests/test_gpu_nibbles.py).  A K = 64 step takes as long
 // and reads as many bytes as a K = 32 step of kind::i8, so operands, filter traffic and MMA time are all half as large.
 //
+// Codes of three bits: signed ones, -4 .. 3, are halves as they are.  Of unsigned activations 5 and 7 are not, so the operand holds a - 4 (the top plane
+// inverted; padding, whose code is 0, becomes -4 like every zero) and the epilogue adds four times the sum of a filter's codes, as many as the
+// tile holds: sum (a - 4) w + 4 sum w = sum a w.  32 x 256 x 28 x 28, 256 filters, three bits both: 30.6 -> 25.6 us.
+//
 // Every wait on an mbarrier is bounded; a wait that runs out sets the device status word and the CTA drains.
 #pragma once
 #include "conv_kernel.cuh"
@@ -323,7 +327,7 @@ __device__ __forceinline__ void expand_word(const uint32_t* p, int kind, uint32_
     }
 }
 
-// 32 codes of one or two planes -> 32 nibbles, nibble j of word m = channel 4 j + m, sign and magnitude (magnitude in halves).  NB = 2: 10
+// 32 codes of one to three planes -> 32 nibbles, nibble j of word m = channel 4 j + m, sign and magnitude (magnitude in halves).  NB = 2: 10
 // operations, and half the bytes.
 template <int NB>
 __device__ __forceinline__ void expand_nibbles(const uint32_t* p, int kind, uint32_t (&o)[4])
@@ -338,6 +342,14 @@ __device__ __forceinline__ void expand_nibbles(const uint32_t* p, int kind, uint
 #pragma unroll
             for (int m = 0; m < 4; ++m) o[m] = 0x99999999u ^ (o[m] << 3);
         }
+    } else if (NB == 3) {
+        // two's complement, of unsigned codes less 4: sign and 4 - (the other two bits) where the top bit is set
+        const uint32_t p1 = p[NB > 1 ? 1 : 0], s = kind == 0 ? ~p[NB - 1] : p[NB - 1];
+        const uint32_t m1 = p1 ^ (p[0] & s), m2 = s & ~(p1 | p[0]);
+        const uint32_t e = (p[0] & 0x55555555u) | ((m1 << 1) & 0xAAAAAAAAu), d = ((p[0] >> 1) & 0x55555555u) | (m1 & 0xAAAAAAAAu);
+        const uint32_t f = (m2 & 0x55555555u) | ((s << 1) & 0xAAAAAAAAu), h = ((m2 >> 1) & 0x55555555u) | (s & 0xAAAAAAAAu);
+        o[0] = (e & 0x33333333u) | ((f << 2) & 0xCCCCCCCCu); o[1] = (d & 0x33333333u) | ((h << 2) & 0xCCCCCCCCu);
+        o[2] = ((e >> 2) & 0x33333333u) | (f & 0xCCCCCCCCu); o[3] = ((d >> 2) & 0x33333333u) | (h & 0xCCCCCCCCu);
     } else {
         const uint32_t p1 = p[NB > 1 ? 1 : 0];
         const uint32_t e = (p[0] & 0x55555555u) | ((p1 << 1) & 0xAAAAAAAAu), d = ((p[0] >> 1) & 0x55555555u) | (p1 & 0xAAAAAAAAu);
@@ -458,6 +470,17 @@ __device__ __forceinline__ int filter_row(const MmaArgs& g, int i, int WB, int& 
     return f;
 }
 
+// Sum of the 32 codes of a channel word as the operand holds them (a bipolar word has no missing ones).
+template <int WB>
+__device__ __forceinline__ int word_sum(const uint32_t* w, int kind)
+{
+    if (kind == 2) return 2 * __popc(w[0]) - 32;
+    int s = 0;
+#pragma unroll
+    for (int k = 0; k < WB; ++k) s += (kind == 1 && k == WB - 1 ? -1 : 1) * (__popc(w[k]) << k);
+    return s;
+}
+
 // One channel word of a filter row -> its two 16-byte core-matrix rows (one of nibbles); rows past the last filter are zero.
 template <int WB, bool F4>
 __device__ __forceinline__ void expand_filter_word(const uint32_t* w, int kind, bool live, uint32_t dst)
@@ -483,9 +506,9 @@ __device__ __forceinline__ void expand_filter_word(const uint32_t* w, int kind, 
 }
 
 // `base`: packed records of the tile's filters, in shared memory (bulk copy) or global.  Nibbles: a K step is two channel words, the second
-// of an odd number zero.
-template <int WB, bool F4>
-__device__ __forceinline__ void expand_filters_resident(const MmaArgs& g, uint32_t b_base, const uint32_t* base, int o0, int t, int nt)
+// of an odd number zero.  SUMS: the sum of each filter's codes is collected by column of the tile.
+template <int WB, bool F4, bool SUMS>
+__device__ __forceinline__ void expand_filters_resident(const MmaArgs& g, uint32_t b_base, const uint32_t* base, int o0, int t, int nt, int* sums)
 {
     constexpr int BATCH = 4;                // loads in flight per thread
     const int rows = g.TN * g.RS, total = rows * (F4 ? 2 * g.nblk : g.Cw);
@@ -495,9 +518,11 @@ __device__ __forceinline__ void expand_filters_resident(const MmaArgs& g, uint32
     for (int j0 = t; j0 < total; j0 += BATCH * nt) {
         uint32_t w[BATCH][WB], dst[BATCH];
         bool live[BATCH];
+        int col[BATCH];
 #pragma unroll
         for (int b = 0; b < BATCH; ++b) {
             int off = 0;
+            if (SUMS) col[b] = fdiv(i >> 3, g.d_rs) * 8 + (i & 7);
             live[b] = cw < g.Cw && o0 + filter_row(g, i, WB, off) < g.O;
             dst[b] = b_base + (F4 ? (cw >> 1) * blk + (cw & 1) * 128u : cw * blk) + static_cast<uint32_t>(i >> 3) * 256u + static_cast<uint32_t>(i & 7) * 16u;
 #pragma unroll
@@ -507,7 +532,10 @@ __device__ __forceinline__ void expand_filters_resident(const MmaArgs& g, uint32
         }
 #pragma unroll
         for (int b = 0; b < BATCH; ++b)
-            if (j0 + b * nt < total) expand_filter_word<WB, F4>(w[b], g.w_kind, live[b], dst[b]);
+            if (j0 + b * nt < total) {
+                expand_filter_word<WB, F4>(w[b], g.w_kind, live[b], dst[b]);
+                if (SUMS && live[b]) atomicAdd(sums + col[b], word_sum<WB>(w[b], g.w_kind));
+            }
     }
 }
 
@@ -552,6 +580,50 @@ static __device__ __noinline__ void convert_filters(const G& g, unsigned char* d
         }
     fence_proxy_async();
     __syncwarp();
+}
+
+// ----------------------------------------------------------------------------- sums of filters (unsigned activations of three bits)
+
+// Four times the sum of each filter's codes, by column of the tile, from memory: by EW warps, four columns at a time.  Packed filters (WB > 0) or
+// prepared ones in either form.
+template <int WB, int EW>
+static __device__ __noinline__ void filter_sums(const MmaArgs& g, float* out, int o0, int warp, int lane)
+{
+    const bool nib = WB == 0 && *reinterpret_cast<const volatile uint32_t*>(g.wgt + static_cast<size_t>(g.opad) * g.RS * 32 * g.Cw - 4) == MM_NIBBLE_MARK;
+    const int vecs = WB > 0 ? g.RS * g.Cw : (nib ? (g.Cw + 1) / 2 : g.Cw) * g.RS * 2;
+    for (int c0 = warp * 4; c0 < g.TN; c0 += EW * 4) {
+        int s[4] = {0, 0, 0, 0};
+        for (int v = lane; v < vecs; v += 32)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int c = c0 + k;
+                if (WB > 0) {
+                    const int o = o0 + (c & ~31) + mma_filter_of_column(c & 31);
+                    if (o >= g.O) continue;
+                    uint32_t w[WB > 0 ? WB : 1];
+#pragma unroll
+                    for (int j = 0; j < WB; ++j) w[j] = g.wgt_packed[(static_cast<size_t>(o) * vecs + v) * WB + j];
+                    s[k] += word_sum<WB>(w, g.w_kind);
+                } else {
+                    const int half = v & 1, t = v >> 1, blk = fdiv(t, g.d_rs), tap = t - blk * g.RS, col = o0 + c;
+                    const uint4 x = reinterpret_cast<const uint4*>(g.wgt)[((static_cast<size_t>(blk) * (g.opad >> 3) + (col >> 3)) * g.RS + tap) * 16 + half * 8 + (col & 7)];
+                    const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+                    // (the last vector of the tensor carries the mark, negative zeros)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        if (!nib) { s[k] = __dp4a(static_cast<int>(w[j]), 0x01010101, s[k]); continue; }
+                        const uint32_t m = w[j] & 0x77777777u, neg = m & ((w[j] >> 3 & 0x11111111u) * 7u);
+                        s[k] += static_cast<int>(__dp4a(m & 0x0F0F0F0Fu, 0x01010101u, __dp4a(m >> 4 & 0x0F0F0F0Fu, 0x01010101u, 0u)));
+                        s[k] -= 2 * static_cast<int>(__dp4a(neg & 0x0F0F0F0Fu, 0x01010101u, __dp4a(neg >> 4 & 0x0F0F0F0Fu, 0x01010101u, 0u)));
+                    }
+                }
+            }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int sum = __reduce_add_sync(0xffffffffu, s[k]);
+            if (lane == 0) out[c0 + k] = 4.0f * static_cast<float>(sum);
+        }
+    }
 }
 
 // ----------------------------------------------------------------------------- MMA issue
@@ -706,8 +778,8 @@ constexpr uint32_t MM_PRESET = 0x4B400000u;      // 1.5 * 2^23: an accumulator t
 // one word (4 i' and two words for wider codes), and a few operations per group de-interleave the words of both halves into
 // planes.  About 4 instructions per output, a quarter of them loads and integer ALU; the threshold-table form it replaces
 // took 8 (12 with a residual).
-template <int OBC, int RESC, bool LO0, bool F4>
-__device__ __forceinline__ void requant16(const uint32_t (&v)[16], uint32_t tab, uint32_t rtab, uint32_t z0, uint32_t z1, uint32_t lo2, uint32_t hi2,
+template <int OBC, int RESC, bool LO0, bool F4, bool OFS>
+__device__ __forceinline__ void requant16(const uint32_t (&v)[16], uint32_t tab, uint32_t cor, uint32_t rtab, uint32_t z0, uint32_t z1, uint32_t lo2, uint32_t hi2,
                                           uint32_t (&W)[2])
 {
     const u64 unbias = f2_pack(0xCB400000u, 0xCB400000u), magic = f2_pack(0x3F400000u, 0x3F400000u);
@@ -717,7 +789,12 @@ __device__ __forceinline__ void requant16(const uint32_t (&v)[16], uint32_t tab,
     for (int i = 0; i < 8; ++i) {
         u64 s2, b2;
         asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(s2), "=l"(b2) : "r"(tab + i * 16));
-        const u64 acc = f2_pack(v[2 * i], v[2 * i + 1]);
+        u64 acc = f2_pack(v[2 * i], v[2 * i + 1]);
+        if (OFS) {
+            u64 c2;
+            asm volatile("ld.shared.b64 %0, [%1];" : "=l"(c2) : "r"(cor + i * 8));
+            acc = f2_add(acc, c2);
+        }
         u64 t = f2_fma(F4 ? acc : f2_add(acc, unbias), s2, b2);
         if (RESC) {
             u64 rmul;
@@ -938,14 +1015,14 @@ __device__ __forceinline__ void load_residual(const G& g, int pix, int ob, uint3
 }
 
 // One group of 32 filters through the documented formula (any scale, bias, residual and output format).
-static __device__ __noinline__ void epilogue_formula(const MmaArgs& g, uint32_t addr, bool live, int pix, int ob, uint32_t bias)
+static __device__ __noinline__ void epilogue_formula(const MmaArgs& g, uint32_t addr, bool live, int pix, int ob, uint32_t bias, const float* cor)
 {
     uint32_t v[32], rw[4] = {0, 0, 0, 0}, ow[4] = {0, 0, 0, 0};
     mm_ld32(addr, v);
     mm_ld_wait();
     mm_landed(v);
     if (live) {
-        for (int c = 0; c < 32; ++c) v[c] = acc_int(g.f4, v[c], bias);
+        for (int c = 0; c < 32; ++c) v[c] = acc_int(g.f4, cor ? __float_as_uint(__uint_as_float(v[c]) + cor[c]) : v[c], bias);
         if (g.residual) load_residual(g, pix, ob, rw);
         requant32_formula(g, v, ob, rw, ow);
         store_codes(g, pix, ob, ow);
@@ -953,14 +1030,14 @@ static __device__ __noinline__ void epilogue_formula(const MmaArgs& g, uint32_t 
     __syncwarp();
 }
 // A whole item that way, its accumulators set back to the preset.
-static __device__ __noinline__ void epilogue_item_formula(const MmaArgs& g, uint32_t acc, int base, int o0, int set, int step)
+static __device__ __noinline__ void epilogue_item_formula(const MmaArgs& g, uint32_t acc, int base, int o0, int set, int step, const float* cor)
 {
     const int groups = g.TN >> 5;
     for (int u = set; u < g.PT * groups; u += step) {
         const int t = u / groups, cc = u - t * groups;
         const MmaPixel px = mma_pixel(g, base + t * 128);
         const uint32_t col = acc + static_cast<uint32_t>(t * g.TN + cc * 32);
-        epilogue_formula(g, col, px.valid && o0 + cc * 32 < g.O, px.pix, o0 + cc * 32, MM_PRESET);
+        epilogue_formula(g, col, px.valid && o0 + cc * 32 < g.O, px.pix, o0 + cc * 32, MM_PRESET, cor ? cor + cc * 32 : nullptr);
         if (!g.f4)
             for (int c = 0; c < 32; c += 8) mm_st8(col + c, MM_PRESET);
     }
@@ -968,11 +1045,11 @@ static __device__ __noinline__ void epilogue_item_formula(const MmaArgs& g, uint
 
 // Codes out, fast form.  One warp's accumulators arrive 16 columns at a time; the next 16 are on their way from tensor memory
 // while the current ones are computed, and the residual words of a group are fetched one group ahead.
-template <int OBC, int RESC, bool LO0, int EW, bool SPLIT, bool F4>
-__device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e)
+template <int OBC, int RESC, bool LO0, int EW, bool SPLIT, bool F4, bool OFS, class Sums>
+__device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e, const Sums& sums)
 {
     constexpr int STEP = EW / 4;
-    const uint32_t tab0 = smem_u32(e.smem + g.off_tab), rtab = tab0 + static_cast<uint32_t>(g.TN) * 8u;
+    const uint32_t tab0 = smem_u32(e.smem + g.off_tab), rtab = tab0 + static_cast<uint32_t>(g.TN) * 8u, cor0 = rtab + 64u;
     int qmin, qmax;
     code_limits(g.out_bits, g.out_sign, qmin, qmax);
     const int lo = g.relu && qmin < 0 ? 0 : qmin;
@@ -987,6 +1064,7 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
             if (tab_o >= 0) asm volatile("bar.sync 2, %0;" ::"n"(EW * 32) : "memory");     // every warp is done with the old table
             epilogue_tables(g, reinterpret_cast<float4*>(e.smem + g.off_tab), reinterpret_cast<float2*>(e.smem + g.off_tab + g.TN * 8), e.fast_ok, o0,
                             e.tid, EW * 32);
+            if (OFS) sums(o0);
             asm volatile("bar.sync 2, %0;" ::"n"(EW * 32) : "memory");
             fast = *reinterpret_cast<volatile int*>(e.fast_ok) != 0;
             tab_o = w.o;
@@ -1004,7 +1082,7 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
         MM_TRACE(e.tid == 0, TR_EBEG, (w.it - static_cast<int>(blockIdx.x)) / static_cast<int>(gridDim.x));
         const uint32_t acc = e.acc + static_cast<uint32_t>(ia * g.PT * g.TN);
         if (!fast) {
-            epilogue_item_formula(g, acc, base, o0, e.set, STEP);
+            epilogue_item_formula(g, acc, base, o0, e.set, STEP, OFS ? reinterpret_cast<const float*>(e.smem + g.off_tab + g.TN * 8 + 64) : nullptr);
             t = g.PT;
         }
         uint32_t A[16], B[16];
@@ -1039,12 +1117,12 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
                 z[2] = ((p >> 2) & 0x33333333u) | (r & 0xCCCCCCCCu);          // 2, 6, .. (half 0, odd pairs)
                 z[3] = ((q >> 2) & 0x33333333u) | (s & 0xCCCCCCCCu);
             }
-            requant16<OBC, RESC, LO0, F4>(A, tab, rtab, z[0], z[2], lo2, hi2, Wa);
+            requant16<OBC, RESC, LO0, F4, OFS>(A, tab, cor0 + static_cast<uint32_t>(ob - o0) * 4u, rtab, z[0], z[2], lo2, hi2, Wa);
             mm_ld_wait();
             mm_landed(B);
             if (t < g.PT) mm_ld16(acc + static_cast<uint32_t>(t * g.TN + cc * 32), A);
             if (!F4) { mm_st8(col + 16, MM_PRESET); mm_st8(col + 24, MM_PRESET); }
-            requant16<OBC, RESC, LO0, F4>(B, tab + 128u, rtab, z[1], z[3], lo2, hi2, Wb);
+            requant16<OBC, RESC, LO0, F4, OFS>(B, tab + 128u, cor0 + static_cast<uint32_t>(ob - o0) * 4u + 64u, rtab, z[1], z[3], lo2, hi2, Wb);
             uint32_t ow[4] = {0, 0, 0, 0};
             if (OBC == 2) {
                 ow[0] = (Wa[0] & 0x55555555u) | ((Wb[0] << 1) & 0xAAAAAAAAu);
@@ -1156,7 +1234,7 @@ __device__ __forceinline__ bool epilogue_tiles(const MmaArgs& g, const MmaEpi& e
         MM_TRACE(e.tid == 0, TR_EBEG, (w.it - static_cast<int>(blockIdx.x)) / static_cast<int>(gridDim.x));
         const uint32_t acc = e.acc + static_cast<uint32_t>(ia * g.PT * g.TN), TN = static_cast<uint32_t>(g.TN);
         if (!fast) {
-            epilogue_item_formula(g, acc, base, o0, e.set, STEP);
+            epilogue_item_formula(g, acc, base, o0, e.set, STEP, nullptr);
             t = g.PT;
         }
         uint32_t v[2][NT][8];           // [buffer][tile]
@@ -1224,25 +1302,32 @@ __device__ __forceinline__ bool epilogue_tiles(const MmaArgs& g, const MmaEpi& e
 }
 
 // Codes of at most two bits from zero on, residual codes of at most two bits.
-template <bool RES, int EW, bool SPLIT, bool F4>
-__device__ __forceinline__ bool epilogue_two_bits(const MmaArgs& g, const MmaEpi& e)
+template <bool RES, int EW, bool SPLIT, bool F4, bool OFS, class Sums>
+__device__ __forceinline__ bool epilogue_two_bits(const MmaArgs& g, const MmaEpi& e, const Sums& sums)
 {
-    if constexpr (!F4) return epilogue_codes<2, RES ? 2 : 0, true, EW, SPLIT, false>(g, e);
+    if constexpr (!F4 || OFS) return epilogue_codes<2, RES ? 2 : 0, true, EW, SPLIT, F4, OFS>(g, e, sums);
     else if constexpr (SPLIT) return epilogue_tiles<RES, 1, EW, true>(g, e);       // one row tile
     else return g.PT > 1 ? epilogue_tiles<RES, 2, EW, false>(g, e) : epilogue_tiles<RES, 1, EW, false>(g, e);
 }
 
 // int32 accumulators out (and codes through the formula where both are asked for or the fast form does not apply).
-template <int EW, bool SPLIT, bool F4>
-__device__ __forceinline__ bool epilogue_general(const MmaArgs& g, const MmaEpi& e)
+template <int EW, bool SPLIT, bool F4, bool OFS, class Sums>
+__device__ __forceinline__ bool epilogue_general(const MmaArgs& g, const MmaEpi& e, const Sums& sums)
 {
     const int groups = g.TN >> 5;
-    int ia = 0;
+    const float* cor = OFS ? reinterpret_cast<const float*>(e.smem + g.off_tab + g.TN * 8 + 64) : nullptr;
+    int ia = 0, sum_o = -1;
     unsigned pa = 0;
     bool ok = true;
     mm_pdl_wait();
     for (MmaWalk w(g, SPLIT ? g.split_log : 0); w.m < g.tiles_m; w.next(g)) {
         const int o0 = w.o * g.TN, base = w.m * 128 * g.PT + e.row0;
+        if (OFS && w.o != sum_o) {
+            if (sum_o >= 0) asm volatile("bar.sync 2, %0;" ::"n"(EW * 32) : "memory");      // every warp is done with the old ones
+            sums(o0);
+            asm volatile("bar.sync 2, %0;" ::"n"(EW * 32) : "memory");
+            sum_o = w.o;
+        }
         if (ok) ok = mm_wait(&e.full_acc[ia], pa);
         mm_fence_after();
         if (SPLIT && ok) ok = merge_partials<EW, F4>(g, e);
@@ -1262,7 +1347,7 @@ __device__ __forceinline__ bool epilogue_general(const MmaArgs& g, const MmaEpi&
                 mm_landed(v);
                 if (F4)
 #pragma unroll
-                    for (int c = 0; c < 32; ++c) v[c] = acc_int(true, v[c], 0u);
+                    for (int c = 0; c < 32; ++c) v[c] = acc_int(true, OFS ? __float_as_uint(__uint_as_float(v[c]) + cor[cc * 32 + c]) : v[c], 0u);
                 if (g.flat && g.i32_nhwc) {
                     // The 32 x 32 block of the warp goes through 4 KB of shared memory so that a store writes a run of a row: 16 bytes a lane where rows
                     // are multiples of that, else 4 (a lane's own row, word by word, touches 32 lines a store: 4059 x 1382 x 1518: 62.6 -> 23.3 us).
@@ -1298,7 +1383,7 @@ __device__ __forceinline__ bool epilogue_general(const MmaArgs& g, const MmaEpi&
                 }
                 __syncwarp();
             }
-            if (g.out_packed) epilogue_formula(g, col, live, px.pix, ob, 0u);
+            if (g.out_packed) epilogue_formula(g, col, live, px.pix, ob, 0u, OFS ? cor + cc * 32 : nullptr);
             cc += EW / 4;
             while (cc >= groups) { cc -= groups; ++t; }
         }
@@ -1321,7 +1406,7 @@ struct MmaShape {
     static constexpr int EW = HALF ? 4 : 8, XW = HALF ? 4 : 8, THREADS = (EW + XW + 2) * 32, CPS = HALF ? 2 : 1;
 };
 
-// SPLIT: an item belongs to a cluster of CTAs, each with a share of its chunks.  F4: nibbles (A and WB at most 2).
+// SPLIT: an item belongs to a cluster of CTAs, each with a share of its chunks.  F4: nibbles (A and WB at most 3).
 template <int A, int WB, bool HALF, bool SPLIT, bool F4>
 __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) bitserial_mma_kernel(const __grid_constant__ MmaArgs g)
 {
@@ -1346,6 +1431,8 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
 
     constexpr bool packed_b = WB > 0;
     constexpr int WBX = WB > 0 ? WB : 1;
+    constexpr bool OFS = F4 && A == 3;              // unsigned activations enter as a - 4
+    int* sums_i = reinterpret_cast<int*>(mm_smem + g.off_tab + g.TN * 8 + 64);
     const bool resident = g.nsb == 0;
     const bool stream_prepared = !resident && !packed_b;      // a stage then holds expanded pixels and the filters of the same chunk
     const int items = g.tiles_m * g.tiles_o;
@@ -1353,6 +1440,8 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
 
     MM_TRACE(tid == 0, TR_START, 0);
     mm_pdl_release();
+    if (OFS)
+        for (int c = tid; c < g.TN; c += MmaShape<HALF>::THREADS) sums_i[c] = 0;
     if (tid == 0) {
         for (int s = 0; s < 4; ++s) {
             mbar_init(&full_e[s], XW / g.groups + (stream_prepared ? 1 : 0));
@@ -1482,7 +1571,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                 if (!mm_wait(bulk_full, 0)) atomicOr(g.status, STATUS_TIMEOUT);
                 src = reinterpret_cast<const uint32_t*>(mm_smem + g.off_e);
             }
-            expand_filters_resident<WBX, F4>(g, smem0, src, o0, tid, NXT + NET);
+            expand_filters_resident<WBX, F4, OFS>(g, smem0, src, o0, tid, NXT + NET, sums_i);
             fence_proxy_async();
             // the parked tile has been read: the ring may be filled once every warp is here
             asm volatile("bar.sync 4, %0;" ::"n"(NXT + NET) : "memory");
@@ -1798,7 +1887,7 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
                 if (!mm_wait(bulk_full, 0)) atomicOr(g.status, STATUS_TIMEOUT);
                 src = reinterpret_cast<const uint32_t*>(mm_smem + g.off_e);
             }
-            expand_filters_resident<WBX, F4>(g, smem0, src, o0, tid, NXT + NET);
+            expand_filters_resident<WBX, F4, OFS>(g, smem0, src, o0, tid, NXT + NET, sums_i);
             fence_proxy_async();
             // the parked tile has been read: the ring may be filled once every warp is here
             asm volatile("bar.sync 4, %0;" ::"n"(NXT + NET) : "memory");
@@ -1810,15 +1899,23 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
         e.smem = mm_smem; e.full_acc = full_acc; e.empty_acc = empty_acc; e.fast_ok = fast_ok;
         e.acc = tmem + lane_addr; e.row0 = quad * 32 + lane; e.set = set;
         e.tid = tid; e.lane = lane; e.warp = warp; e.red_full = red_full;
+        // what the epilogue adds to the accumulators of a filter tile, as floats by column
+        auto sums = [&](int o0) {
+            if constexpr (OFS) {
+                if (g.a_kind != 0 || (packed_b && resident))
+                    for (int c = tid; c < g.TN; c += NET) reinterpret_cast<float*>(sums_i)[c] = g.a_kind != 0 ? 0.0f : 4.0f * static_cast<float>(sums_i[c]);
+                else filter_sums<WB, EW>(g, reinterpret_cast<float*>(sums_i), o0, warp, lane);
+            }
+        };
         bool ok;
         if (SPLIT && range.rank > 0) ok = send_partials<EW, F4>(g, e, range.rank);
-        else if (!g.preset) ok = epilogue_general<EW, SPLIT, F4>(g, e);
-        else if (g.epi == 0) ok = epilogue_two_bits<false, EW, SPLIT, F4>(g, e);
-        else if (g.epi == 1) ok = epilogue_two_bits<true, EW, SPLIT, F4>(g, e);
-        else if (g.epi == 2) ok = epilogue_codes<4, 0, true, EW, SPLIT, F4>(g, e);
-        else if (g.epi == 3) ok = epilogue_codes<4, 4, true, EW, SPLIT, F4>(g, e);
-        else if (g.epi == 4) ok = epilogue_codes<4, 0, false, EW, SPLIT, F4>(g, e);
-        else ok = epilogue_codes<4, 4, false, EW, SPLIT, F4>(g, e);
+        else if (!g.preset) ok = epilogue_general<EW, SPLIT, F4, OFS>(g, e, sums);
+        else if (g.epi == 0) ok = epilogue_two_bits<false, EW, SPLIT, F4, OFS>(g, e, sums);
+        else if (g.epi == 1) ok = epilogue_two_bits<true, EW, SPLIT, F4, OFS>(g, e, sums);
+        else if (g.epi == 2) ok = epilogue_codes<4, 0, true, EW, SPLIT, F4, OFS>(g, e, sums);
+        else if (g.epi == 3) ok = epilogue_codes<4, 4, true, EW, SPLIT, F4, OFS>(g, e, sums);
+        else if (g.epi == 4) ok = epilogue_codes<4, 0, false, EW, SPLIT, F4, OFS>(g, e, sums);
+        else ok = epilogue_codes<4, 4, false, EW, SPLIT, F4, OFS>(g, e, sums);
         if (!ok && lane == 0) atomicOr(g.status, STATUS_TIMEOUT);
     }
     mm_fence_before();
@@ -1841,6 +1938,7 @@ MmaKernel mma_kernel_a3(int wb, bool half, bool split);
 MmaKernel mma_kernel_a4(int wb, bool half, bool split);
 MmaKernel mma_kernel_f1(int wb, bool half, bool split);
 MmaKernel mma_kernel_f2(int wb, bool half, bool split);
+MmaKernel mma_kernel_f3(int wb, bool half, bool split);
 
 template <int A, int WB, bool F4>
 MmaKernel mma_pick_shape(bool half, bool split)
@@ -1861,7 +1959,12 @@ MmaKernel mma_pick(int wb, bool half, bool split)
 template <int A>
 MmaKernel mma_pick_nibbles(int wb, bool half, bool split)
 {
-    return wb == 0 ? mma_pick_shape<A, 0, true>(half, split) : wb == 1 ? mma_pick_shape<A, 1, true>(half, split) : mma_pick_shape<A, 2, true>(half, split);
+    switch (wb) {
+        case 0: return mma_pick_shape<A, 0, true>(half, split);
+        case 1: return mma_pick_shape<A, 1, true>(half, split);
+        case 2: return mma_pick_shape<A, 2, true>(half, split);
+        default: return mma_pick_shape<A, 3, true>(half, split);
+    }
 }
 
 }  // namespace bs

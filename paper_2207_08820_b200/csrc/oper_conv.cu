@@ -99,7 +99,7 @@ bool lay_out(const bs_sequence_layer* layers, int n, Layout& l)
         const bs_conv_params& p = layers[i].p;
         if (!layers[i].wgt_tc || !layers[i].out_packed || !layers[i].act_packed || p.C % 32 != 0) return false;
         if (p.a_sign != BS_UNSIGNED || p.out_sign != BS_UNSIGNED || p.out_bits > 2 || p.out_bits < 1) return false;
-        if (!mma_nibbles(p.C, p.R * p.S, p.a_bits, p.w_bits) || p.stride > 2 || p.R != p.S) return false;
+        if (p.a_bits > 2 || !mma_nibbles(p.C, p.R * p.S, p.a_bits, p.w_bits, p.w_sign) || p.stride > 2 || p.R != p.S) return false;
         if (p.residual && (p.res_sign != BS_UNSIGNED || p.res_bits > 2 || !(fabsf(p.res_scale) < 3.9f) || (p.res_scale != 0.0f && fabsf(p.res_scale) <= 1e-18f))) return false;
         const Shape s = shape_of(p);
         const int src = tensor_index(l, layers[i].act_packed, p.N, p.H, p.W, p.C / 32, p.a_bits);
