@@ -39,7 +39,7 @@ static __global__ void __launch_bounds__(256) oper_import_kernel(const __grid_co
 
 namespace {
 
-constexpr int OP_SMEM_MAX = 112 * 1024, OP_MAX_ROWS = 1024;
+constexpr int OP_SMEM_MAX = 224 * 1024, OP_MAX_ROWS = 1024;         // of a CTA that has an SM to itself; half of it otherwise
 
 int up(int v, int m) { return (v + m - 1) / m * m; }
 
@@ -159,11 +159,12 @@ OperDst dst_of(const Tensor& t, int k, unsigned char* ws, int word)
     return d;
 }
 
-struct Cand { int TN, PT, units, cps, resident, nse, nacc; size_t smem; long long grid; double cost; };
+struct Cand { int TN, PT, units, cps, full, resident, nse, nacc; size_t smem; long long grid; double cost; };
 
 // Shared memory of a candidate; false when it does not fit.
 bool layout_cand(OperArgs& g, Cand& c, int sms)
 {
+    const int smem_max = c.full ? OP_SMEM_MAX : OP_SMEM_MAX / 2;
     const int rmax = g.stride == 1 ? g.R - 1 - g.pad : (g.R - 1 - g.pad) >> 1, BM = 128 * c.PT;
     g.TN = c.TN; g.PT = c.PT; g.units = c.units; g.resident = c.resident;
     g.HL = BM + (rmax - g.rmin) * g.pitch + (rmax - g.smin);
@@ -175,22 +176,24 @@ bool layout_cand(OperArgs& g, Cand& c, int sms)
     if (g.tiles_o > sms) return false;
     const long long run = static_cast<long long>(g.NI) * 16 * g.halves;
     const long long blk = static_cast<long long>(c.TN) * g.RS * 32, filters = c.resident ? blk * g.nunits : 0;
-    if (filters > OP_SMEM_MAX || blk > OP_SMEM_MAX || run * c.units > OP_SMEM_MAX) return false;
+    if (filters > smem_max || blk > smem_max || run * c.units > smem_max) return false;
     g.a_bytes = up(static_cast<int>(run) * c.units, 128);
     g.stage_bytes = g.a_bytes + (c.resident ? 0 : static_cast<int>(blk) * c.units);
     const int fixed = up(c.TN * 8 + 64, 128) + 256;
-    const long long room = OP_SMEM_MAX - fixed - filters;
+    const long long room = smem_max - fixed - filters;
     int most = static_cast<int>(room > 0 ? room / g.stage_bytes : 0);
     const int slots = sms * c.cps / g.tiles_o, waves = ceil_div(g.tiles_m, slots);
     if (most > OP_STAGES) most = OP_STAGES;
     if (most > waves * g.nchunks) most = waves * g.nchunks;        // (less shared memory for the next launch to wait for)
     if (most < 1) return false;
     c.nse = g.nse = most;
-    const int cols = 256 - MM_SF_COLS;
+    const int cols = (c.full ? 512 : 256) - MM_SF_COLS;
     if (c.PT * c.TN > cols) return false;
     c.nacc = cols / (c.PT * c.TN);
     if (c.nacc > 4) c.nacc = 4;
     if (c.nacc > waves) c.nacc = waves;
+    // (with one buffer a team of epilogue warps could take the end of its last item for that of its next: the other team's lies between)
+    if (c.full && c.nacc < 2) return false;
     g.nacc = c.nacc;
     g.sf_col = c.nacc * c.PT * c.TN;
     int tc = 32;
@@ -206,31 +209,44 @@ bool layout_cand(OperArgs& g, Cand& c, int sms)
     return true;
 }
 
-// Time model in SM cycles: the items of a CTA one after the other, CTAs of an SM sharing what they share.
+// Time model of a candidate in SM cycles: a CTA's items one after the other (ring of stages, MMAs, epilogue), and what the CTAs of an SM share.  Fitted
+// to about 4000 timed plans of 135 layers (1 to 64 images, 7 to 300 pixels wide, 32 to 2048 channels, chained launches, B200 at 1.92 GHz):
+// the plan with the lowest modelled time is on average 1.3 % (6 % with the constants first guessed) slower than the fastest.
+struct OperFit {
+    double start, full_start;       // of a launch; more where a CTA takes a whole SM and cannot begin beside the launch before
+    double lat, rate, fill;         // a chunk's copies: cycles, bytes per cycle of one chunk; share of the first one that nothing hides
+    double issue, m32, m64, m128;   // cycles per MMA: between two of one CTA, of the tensor core for 32, 64, 128 filters
+    double chunk;                   // cycles per chunk beside its MMAs
+    double e_codes, e_res, e_pair;  // two blocks of 32 x 32 outputs side by side, with a residual; factor where row tiles share the scales
+    double e_once, teams;           // per item; share of an epilogue's time that two teams take
+    double s_codes, s_res, l2;      // of the SM: a quarter block, with a residual; bytes per cycle
+};
+constexpr OperFit OPER_FIT = {1256, 1888, 278, 177, 1.42, 48.6, 42, 20.6, 26.6, 443, 920, 1548, 0.904, 1568, 0.447, 77.6, 33.1, 103.7};
+
 double cost_of(const OperArgs& g, const Cand& c, int sms)
 {
-    const double mma = c.TN == 32 ? 42 : c.TN == 64 ? 49 : 65;
-    const double t_m = c.PT * g.RS * g.nunits * mma + 120.0 * g.nchunks;
-    const int blocks = c.PT * (c.TN / 32);
-    const double t_e = ceil_div(blocks, 2) * (g.residual ? 330.0 : 270.0) + 500.0, use_e = blocks * 4.0 * (g.residual ? 42.0 : 34.0);
-    const double bytes = static_cast<double>(g.NI) * 16 * g.halves * g.nunits + (c.resident ? 0.0 : static_cast<double>(c.TN) * g.RS * 32 * g.nunits);
-    const double t_b = bytes / 50.0;
-    const int waves = ceil_div(g.tiles_m, g.step_m);
+    const OperFit& k = OPER_FIT;
+    const double mma = c.TN == 32 ? k.m32 : c.TN == 64 ? k.m64 : k.m128, n = static_cast<double>(c.PT) * g.RS * g.nunits;
+    const double t_m = n * (mma > k.issue ? mma : k.issue) + k.chunk * g.nchunks;
+    const int blocks = c.PT * (c.TN / 32), waves = ceil_div(g.tiles_m, g.step_m);
+    const double pair = c.PT > 1 && blocks >= 4 ? k.e_pair : 1.0;
+    const double t_e = ceil_div(blocks, 2) * (g.residual ? k.e_res : k.e_codes) * pair + k.e_once;
     const double active = static_cast<double>(ceil_div_ll(c.grid, sms));
-    const double t_mb = t_m > t_b ? t_m : t_b;
-    double step = c.nacc > 1 ? (t_mb > t_e ? t_mb : t_e) : t_mb + t_e;
-    if (c.nse < 2) step += t_b;
-    if (active * t_m > step) step = active * t_m;
-    if (active * t_b > step) step = active * t_b;
-    if (active * use_e > step) step = active * use_e;
-    const double first = 1200.0 + (c.resident ? 0.0 : 0.3 * t_b) + active * t_mb + t_e;
-    return 3000.0 + first + (waves - 1) * step;
+    const double bytes = (static_cast<double>(g.NI) * 16 * g.halves + (c.resident ? 0.0 : c.TN * g.RS * 32.0)) * g.nunits;
+    const double load = k.lat + bytes / g.nchunks / k.rate;
+    const double ring = g.nchunks * (load + t_m / g.nchunks) / c.nse;
+    const double t_mb = t_m > ring ? t_m : ring;
+    auto most = [](double a, double b) { return a > b ? a : b; };
+    const double shared_m = most(active * n * mma, active * bytes / k.l2), shared_e = active * blocks * 4.0 * (g.residual ? k.s_res : k.s_codes) * pair;
+    const double e_rate = c.full ? t_e * k.teams : t_e;
+    const double step = most(most(c.nacc > 1 ? most(t_mb, e_rate) : t_mb + t_e, shared_m), shared_e);
+    return k.start + (c.full ? k.full_start : 0.0) + load * k.fill + most(t_mb, shared_m) + most(t_e, shared_e) + (waves - 1) * step;
 }
 
 }  // namespace
 
 struct OperSequence {
-    struct Step { OperArgs g; unsigned grid; int smem; };
+    struct Step { OperArgs g; unsigned grid; int smem, full; };
     struct Import { OperTensor g; unsigned grid; };
     std::vector<Step> steps;
     std::vector<Import> imports;
@@ -287,11 +303,11 @@ static bool plan_layer(OperSequence::Step& s, int sms)
         for (int PT = 1; PT <= 4; PT *= 2)
             for (int units = 1; units <= 4; units *= 2) {
                 if (units > 1 && (units > s.g.nunits || s.g.R > 1)) continue;
-                for (int v = 0; v < 4; ++v) {
+                for (int v = 0; v < 6; ++v) {
                     Cand c{};
-                    c.TN = TN; c.PT = PT; c.units = units; c.cps = 1 + (v & 1); c.resident = v >> 1;
+                    c.TN = TN; c.PT = PT; c.units = units; c.resident = v & 1; c.full = v >> 1 == 2; c.cps = c.full ? 1 : 1 + (v >> 1);
 #ifdef BS_TUNING
-                    if ((ov[0] && TN != ov[0]) || (ov[1] && PT != ov[1]) || (ov[2] && units != ov[2]) || (ov[3] && c.cps != ov[3]) || (ov[4] >= 0 && c.resident != ov[4])) continue;
+                    if ((ov[0] && TN != ov[0]) || (ov[1] && PT != ov[1]) || (ov[2] && units != ov[2]) || (ov[3] && c.cps + 2 * c.full != ov[3]) || (ov[4] >= 0 && c.resident != ov[4])) continue;
 #endif
                     OperArgs t = s.g;
                     if (!layout_cand(t, c, sms)) continue;
@@ -303,13 +319,14 @@ static bool plan_layer(OperSequence::Step& s, int sms)
     if (!found || !layout_cand(s.g, best, sms)) return false;
 #ifdef BS_TUNING
     if (getenv("BS_OP_VERBOSE"))
-        fprintf(stderr, "oper plan: N%d C%d %dx%d O%d k%d s%d res%d -> TN %d PT %d units %d cps %d resident %d stages %d nacc %d HL %d tiles %d x %d grid %lld smem %zu cost %.0f\n", s.g.N, s.g.Cw * 32,
-                s.g.P, s.g.Q, s.g.O, s.g.R, s.g.stride, s.g.residual ? 1 : 0, best.TN, best.PT, best.units, best.cps, best.resident, best.nse, best.nacc, s.g.HL, s.g.tiles_m, s.g.tiles_o, best.grid, best.smem, best.cost);
+        fprintf(stderr, "oper plan: N%d C%d %dx%d O%d k%d s%d res%d -> TN %d PT %d units %d cps %d full %d resident %d stages %d nacc %d HL %d tiles %d x %d grid %lld smem %zu cost %.0f\n", s.g.N, s.g.Cw * 32,
+                s.g.P, s.g.Q, s.g.O, s.g.R, s.g.stride, s.g.residual ? 1 : 0, best.TN, best.PT, best.units, best.cps, best.full, best.resident, best.nse, best.nacc, s.g.HL, s.g.tiles_m, s.g.tiles_o, best.grid, best.smem, best.cost);
 #endif
     // float += e2m1 x e2m1 with ue8m0 scale factors; TN columns, 128 rows
     s.g.idesc = (1u << 7) | (1u << 10) | (1u << 23) | (static_cast<unsigned>(s.g.TN >> 3) << 17) | (static_cast<unsigned>(128 >> 4) << 24);
     s.grid = static_cast<unsigned>(best.grid);
     s.smem = static_cast<int>(best.smem);
+    s.full = best.full;
     return true;
 }
 
@@ -353,7 +370,8 @@ OperSequence* oper_create(const bs_sequence_layer* layers, int n, void* workspac
     OperSequence* q = new (std::nothrow) OperSequence;
     size_t need = 0;
     if (q && workspace && build(layers, n, static_cast<unsigned char*>(workspace), *q, need) && need <= bytes && status_device_ptr() &&
-        cudaFuncSetAttribute(bitserial_oper_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, OP_SMEM_MAX + 512) == cudaSuccess)
+        cudaFuncSetAttribute(bitserial_oper_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, OP_SMEM_MAX / 2) == cudaSuccess &&
+        cudaFuncSetAttribute(bitserial_oper_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, OP_SMEM_MAX) == cudaSuccess)
         return q;
     cudaGetLastError();
     delete q;
@@ -382,7 +400,7 @@ int oper_begin(const OperSequence* q, const OperTensor* ready, cudaStream_t st)
 int oper_layer(const OperSequence* q, int i, cudaStream_t st)
 {
     const OperSequence::Step& s = q->steps[static_cast<size_t>(i)];
-    return launch_dependent(bitserial_oper_kernel, dim3(s.grid), dim3(OP_THREADS), static_cast<size_t>(s.smem), st, s.g);
+    return launch_dependent(s.full ? bitserial_oper_kernel<true> : bitserial_oper_kernel<false>, dim3(s.grid), dim3(oper_threads(s.full)), static_cast<size_t>(s.smem), st, s.g);
 }
 
 void oper_destroy(OperSequence* q) { delete q; }

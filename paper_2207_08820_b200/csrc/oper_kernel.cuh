@@ -15,7 +15,9 @@
 
 namespace bs {
 
-constexpr int OP_STAGES = 8, OP_EW = 8, OP_THREADS = (OP_EW + 2) * 32;
+constexpr int OP_STAGES = 8, OP_EW = 8;         // stages at most; epilogue warps of an item
+// FULL: one CTA per SM with all its tensor memory, 16 epilogue warps, of which eight take every other item.
+constexpr int oper_threads(bool full) { return ((full ? 2 : 1) * OP_EW + 2) * 32; }
 
 struct OperArgs {
     const unsigned char* src;       // operand tensor of the input, at the first halo position of tile 0 (of plane 0, group 0)
@@ -94,27 +96,29 @@ static __device__ __noinline__ void oper_item_formula(const OperArgs& g, uint32_
 }
 
 // As epilogue_tiles (mma_kernel.cuh): NT row tiles share the loads of scales and biases, eight columns of each on their way while eight are computed.
-template <bool RES, int NT>
+template <bool RES, int NT, bool FULL>
 __device__ __forceinline__ bool oper_epilogue(const OperArgs& g, const MmaEpi& e)
 {
-    constexpr int STEP = OP_EW / 4;
+    constexpr int STEP = OP_EW / 4, TEAMS = FULL ? 2 : 1, EPI_THREADS = TEAMS * OP_EW * 32;
     const uint32_t tab0 = smem_u32(e.smem + g.off_tab);
     const uint32_t hi2 = ((1u << g.out_bits) - 1u) * 0x10001u;
     // a residual code in the low bits of a word is the denormal code * 2^-149; everything is scaled by 2^-24
     const uint32_t rm = __float_as_uint(g.res_scale * __uint_as_float(252u << 23)), rm4 = __float_as_uint(g.res_scale * __uint_as_float(250u << 23));
     const u64 rmul = f2_pack(rm, rm), rmul4 = f2_pack(rm4, rm4);
     const int groups = g.TN >> 5, o0 = static_cast<int>(blockIdx.x % static_cast<unsigned>(g.tiles_o)) * g.TN;
-    epilogue_tables(g, reinterpret_cast<float4*>(e.smem + g.off_tab), reinterpret_cast<float2*>(e.smem + g.off_tab + g.TN * 8), e.fast_ok, o0, e.tid, OP_EW * 32);
-    asm volatile("bar.sync 2, %0;" ::"n"(OP_EW * 32) : "memory");
+    epilogue_tables(g, reinterpret_cast<float4*>(e.smem + g.off_tab), reinterpret_cast<float2*>(e.smem + g.off_tab + g.TN * 8), e.fast_ok, o0, e.tid, EPI_THREADS);
+    asm volatile("bar.sync 2, %0;" ::"n"(EPI_THREADS) : "memory");
     const bool fast = *reinterpret_cast<volatile int*>(e.fast_ok) != 0;
     if (g.early_b) mm_pdl_wait();
-    int ia = 0;
+    const int team = FULL ? e.warp / OP_EW : 0;
+    int ia = team;
     unsigned pa = 0;
+    if (ia >= g.nacc) { ia -= g.nacc; pa ^= 1u; }
     bool ok = true;
 #ifdef BS_TRACE
     int seq = 0;
 #endif
-    for (int m = static_cast<int>(blockIdx.x / static_cast<unsigned>(g.tiles_o)); m < g.tiles_m; m += g.step_m) {
+    for (int m = static_cast<int>(blockIdx.x / static_cast<unsigned>(g.tiles_o)) + team * g.step_m; m < g.tiles_m; m += TEAMS * g.step_m) {
         const int base = m * 128 * g.PT + e.row0;
         // units (NT tiles, group), group fastest
         int t = 0, cc = e.set;
@@ -212,7 +216,7 @@ __device__ __forceinline__ bool oper_epilogue(const OperArgs& g, const MmaEpi& e
 #ifdef BS_TRACE
         ++seq;
 #endif
-        if (++ia == g.nacc) { ia = 0; pa ^= 1u; }
+        for (ia += TEAMS; ia >= g.nacc; ia -= g.nacc) pa ^= 1u;
     }
     return ok;
 }
@@ -224,13 +228,44 @@ struct OperIssue {
     uint32_t smem0, tmem;
 };
 
+// The nine taps of a K step under one elect.sync, in one asm statement: OFF advances the pixel operand to the next tap.
+#define OP_MMA(A, B, P) "@p tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], " A ", " B ", %3, [%5], [%5], " P ";\n\t"
+#define OP_STEP(OFF) "add.s64 a, a, " OFF ";\n\tadd.s64 b, b, 16;\n\t" OP_MMA("a", "b", "t")
+template <int ST>
+__device__ __forceinline__ void oper_taps(uint32_t d, uint32_t a, uint32_t a_hi, uint32_t b, uint32_t b_hi, uint32_t idesc, uint32_t acc, uint32_t pitch, uint32_t HL, uint32_t sf)
+{
+    const uint64_t da = (static_cast<uint64_t>(a_hi) << 32) | a, db = (static_cast<uint64_t>(b_hi) << 32) | b;
+    if (ST == 1) {
+        const uint64_t row = pitch - 2u;        // from the last tap of a row to the first of the next
+        asm volatile(
+            "{\n\t.reg .pred p, q, t;\n\t.reg .b64 a, b;\n\t"
+            "elect.sync _|p, 0xffffffff;\n\t"
+            "setp.ne.b32 q, %4, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
+            "mov.b64 a, %1;\n\tmov.b64 b, %2;\n\t"
+            OP_MMA("a", "b", "q") OP_STEP("1") OP_STEP("1") OP_STEP("%6") OP_STEP("1") OP_STEP("1") OP_STEP("%6") OP_STEP("1") OP_STEP("1")
+            "}"
+            ::"r"(d), "l"(da), "l"(db), "r"(idesc), "r"(acc), "r"(sf), "l"(row) : "memory");
+    } else {
+        // offsets of the taps (issue_taps): 3 HL, 2 HL + 1, 3 HL + 1; HL, 1, HL + 1 and 3 HL, 2 HL + 1, 3 HL + 1, these a row on
+        const uint64_t back = 1ull - HL, fwd = HL, r1 = static_cast<uint64_t>(pitch) - 2ull * HL - 1ull, r2 = 2ull * HL - 1ull;
+        asm volatile(
+            "{\n\t.reg .pred p, q, t;\n\t.reg .b64 a, b;\n\t"
+            "elect.sync _|p, 0xffffffff;\n\t"
+            "setp.ne.b32 q, %4, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
+            "mov.b64 a, %1;\n\tmov.b64 b, %2;\n\t"
+            OP_MMA("a", "b", "q") OP_STEP("%6") OP_STEP("%7") OP_STEP("%8") OP_STEP("%6") OP_STEP("%7") OP_STEP("%9") OP_STEP("%6") OP_STEP("%7")
+            "}"
+            ::"r"(d), "l"(da + 3u * HL), "l"(db), "r"(idesc), "r"(acc), "r"(sf), "l"(back), "l"(fwd), "l"(r1), "l"(r2) : "memory");
+    }
+}
+
 template <int TAPS>
 __device__ __forceinline__ void oper_block(const OperArgs& g, uint32_t d, uint32_t a, uint32_t a_hi, uint32_t b, uint32_t b_hi, uint32_t acc, uint32_t sf)
 {
     const uint32_t pitch = static_cast<uint32_t>(g.pitch), HL = static_cast<uint32_t>(g.HL), idesc = g.idesc;
     if (TAPS == TAPS_1) issue_mma<true>(d, a, a_hi, b, b_hi, idesc, acc, sf);
-    else if (TAPS == TAPS_3S1) issue_taps<3, 1, true>(d, a, a_hi, b, b_hi, idesc, acc, pitch, HL, sf);
-    else if (TAPS == TAPS_3S2) issue_taps<3, 2, true>(d, a, a_hi, b, b_hi, idesc, acc, pitch, HL, sf);
+    else if (TAPS == TAPS_3S1) oper_taps<1>(d, a, a_hi, b, b_hi, idesc, acc, pitch, HL, sf);
+    else if (TAPS == TAPS_3S2) oper_taps<2>(d, a, a_hi, b, b_hi, idesc, acc, pitch, HL, sf);
     else
         for (int r = 0; r < g.R; ++r)
             for (int s = 0; s < g.R; ++s) {
@@ -304,7 +339,8 @@ __device__ __forceinline__ void oper_issue(const OperArgs& g, const OperIssue& m
 
 // ----------------------------------------------------------------------------- the kernel
 
-static __global__ void __launch_bounds__(OP_THREADS, 2) bitserial_oper_kernel(const __grid_constant__ OperArgs g)
+template <bool FULL>
+__global__ void __launch_bounds__(oper_threads(FULL), FULL ? 1 : 2) bitserial_oper_kernel(const __grid_constant__ OperArgs g)
 {
     extern __shared__ __align__(1024) unsigned char op_smem[];
     const int tid = threadIdx.x, lane = tid & 31;
@@ -319,7 +355,7 @@ static __global__ void __launch_bounds__(OP_THREADS, 2) bitserial_oper_kernel(co
     uint64_t* form_ok = wgt_full + 1;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(form_ok + 1);
     int* fast_ok = reinterpret_cast<int*>(form_ok + 2);
-    constexpr int WARP_COPY = OP_EW, WARP_MMA = OP_EW + 1;
+    constexpr int WARP_COPY = (FULL ? 2 : 1) * OP_EW, WARP_MMA = WARP_COPY + 1;
 
     MM_TRACE(tid == 0, TR_START, 0);
     if (tid == 0) {
@@ -407,15 +443,17 @@ static __global__ void __launch_bounds__(OP_THREADS, 2) bitserial_oper_kernel(co
         else if (g.R == 3 && g.pad == 1) oper_issue<TAPS_3S2>(g, m);
         else oper_issue<TAPS_ANY>(g, m);
     } else {
-        const int quad = warp & 3, set = warp >> 2;
+        const int quad = warp & 3, set = (warp >> 2) & 1;
         const uint32_t lane_addr = static_cast<uint32_t>(quad * 32) << 16;
         // scale factors of 2 for every row, column and block
+        if (warp < OP_EW) {
         for (int c = set * 8; c < MM_SF_COLS; c += 8 * (OP_EW / 4)) mm_st8(tmem + lane_addr + static_cast<uint32_t>(g.sf_col + c), 0x80808080u);
         mm_st_wait();
         mm_fence_before();
         __syncwarp();
         if (lane == 0)
             for (int s = 0; s < g.nacc; ++s) mm_arrive(&empty_acc[s]);
+        }
         if (!g.early_b) mm_pdl_wait();
         MmaEpi e;
         e.smem = op_smem; e.full_acc = full_acc; e.empty_acc = empty_acc; e.fast_ok = fast_ok;
@@ -424,8 +462,8 @@ static __global__ void __launch_bounds__(OP_THREADS, 2) bitserial_oper_kernel(co
         // (pairs of row tiles where that leaves both warps of a lane quadrant some)
         const bool pair = g.PT > 1 && g.PT * (g.TN >> 5) >= 4;
         bool ok;
-        if (g.residual) ok = pair ? oper_epilogue<true, 2>(g, e) : oper_epilogue<true, 1>(g, e);
-        else ok = pair ? oper_epilogue<false, 2>(g, e) : oper_epilogue<false, 1>(g, e);
+        if (g.residual) ok = pair ? oper_epilogue<true, 2, FULL>(g, e) : oper_epilogue<true, 1, FULL>(g, e);
+        else ok = pair ? oper_epilogue<false, 2, FULL>(g, e) : oper_epilogue<false, 1, FULL>(g, e);
         if (!ok && lane == 0) atomicOr(g.status, STATUS_TIMEOUT);
     }
     mm_fence_before();

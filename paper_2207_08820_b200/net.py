@@ -130,25 +130,23 @@ class BitserialNet:
         return units
 
     def _run(self, x: torch.Tensor) -> torch.Tensor:
-        self._run_layers(self._pack(x, self._ready()))
+        self.run_layers(self.pack_input(x, operands=True))
         return self.bufs[self.net.out_name]
 
-    def _ready(self) -> Optional[int]:
-        """The operand tensor of the packed input (``bs_sequence_input``) that a producer of the input may write as well, or None."""
+    def input_operands(self) -> Optional[int]:
+        """The operand tensor of the packed input (``bs_sequence_input``), which a producer of the input may write as well, or None."""
         return self._sequence.input if self._bind() else None
 
-    def _pack(self, x: torch.Tensor, ready: Optional[int]) -> Optional[int]:
-        """:meth:`pack_input`, to ``ready`` as well where ``x`` is the whole input; returns what is ready then."""
-        if ready is not None and x.dtype == torch.float32 and tuple(x.shape) == (self.batch, *self.net.in_shape):
-            api.bitpack_operands(x, self.act_scale, self.net.a_bits, self.bufs[self.net.in_name], ready)
-            return ready
-        self.pack_input(x)
-        return None
-
-    def pack_input(self, x: torch.Tensor) -> None:
-        """Quantise + bitplane-pack the fp32 input on the current stream."""
-        net = self.net
-        api.bitpack_activations(x, self.act_scale, net.a_bits, api.UNSIGNED, api.NCHW, out=self.bufs[net.in_name].view(-1))
+    def pack_input(self, x: torch.Tensor, operands: bool = False) -> Optional[int]:
+        """Quantise + bitplane-pack the fp32 input on the current stream.  operands: its operand tensor too, where the layers have one and ``x`` is
+        the whole input; :meth:`run_layers` takes what is returned then, as long as neither is written in between."""
+        net, buf = self.net, self.bufs[self.net.in_name]
+        ready = self.input_operands() if operands and x.dtype == torch.float32 and tuple(x.shape) == (self.batch, *net.in_shape) else None
+        if ready is not None:
+            api.bitpack_operands(x, self.act_scale, net.a_bits, buf, ready)
+        else:
+            api.bitpack_activations(x, self.act_scale, net.a_bits, api.UNSIGNED, api.NCHW, out=buf.view(-1))
+        return ready
 
     def run_layer(self, item, chained: bool = True) -> None:
         """One conv layer through the C ABI on the current stream."""
@@ -215,12 +213,9 @@ class BitserialNet:
             out.append((unit, aside, join))
         return out
 
-    def run_layers(self) -> None:
+    def run_layers(self, ready: Optional[int] = None) -> None:
         """All layers on the current stream, and on the side stream those that :meth:`schedule` puts there; under stream capture the
-        events between them become the edges of the graph."""
-        self._run_layers(None)
-
-    def _run_layers(self, ready: Optional[int]) -> None:
+        events between them become the edges of the graph.  ready: the operand tensor of the input, where it holds what the packed input holds."""
         if self._bind():
             q = self._sequence
             ready = ready if ready == q.input else None
@@ -402,7 +397,7 @@ class BitserialFullNet:
             return ready
         self._stem_layers(images)
         self._note_pass(None)
-        return body._pack(self._stem["pool"], ready)
+        return body.pack_input(self._stem["pool"], operands=ready is not None)
 
     def _stem_layers(self, images: torch.Tensor) -> None:
         conv, pool = self._stem_tensor("conv"), self._stem_tensor("pool")
@@ -503,7 +498,7 @@ class BitserialFullNet:
 
     def forward(self, images: torch.Tensor) -> torch.Tensor:
         """images: float32 [batch, 3, hw, hw] on the device.  Returns the logits [batch, classes]."""
-        self.body._run_layers(self._front(images, self.body._ready()))
+        self.body.run_layers(self._front(images, self.body.input_operands()))
         self.run_head()
         self._join_note()
         return self.logits
