@@ -24,7 +24,7 @@ int up(int v, int m) { return (v + m - 1) / m * m; }
 int max_abs_of(int bits, int sign) { return sign == BS_BIPOLAR ? 1 : (sign == BS_SIGNED ? 1 << (bits - 1) : (1 << bits) - 1); }
 
 struct Cand {
-    int TN, PT, units, cfg, cps, ns, resident, groups, split, nse, nsb, nacc;
+    int TN, PT, units, cfg, cps, ns, resident, groups, split, nse, nsb, nacc, f4;
     size_t smem;
     double cost;
 };
@@ -271,7 +271,10 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
     // outputs 0.98 and 0.97; codes of 5x5 windows over up to 32 channels 1.12 and 0.89 on these sides, of 3x3 windows 0.96 and 0.94.
     const bool short_k = g.Cw == 1 && static_cast<double>(g.N) * g.P * g.Q * g.O >= 2048.0 * sms;
     const bool pixel_rows = out_i32 && !out_packed && !g.i32_nhwc;
-    g.f4 = mma_nibbles(p->C, g.RS, p->a_bits, p->w_bits, p->w_sign) && !(packed_b && (pixel_rows ? short_k || (g.R == 1 && g.Cw <= 6) : short_k && g.R >= 5 && !out_i32));
+    g.f4 = (mma_nibbles(p->C, g.RS, p->a_bits, p->w_bits, p->w_sign) || (packed_b && mma_nibbles_a3(p->C, g.RS, p->a_bits, p->w_bits, p->w_sign))) &&
+           !(packed_b && (pixel_rows ? short_k || (g.R == 1 && g.Cw <= 6) : short_k && g.R >= 5 && !out_i32));
+    // Unsigned activations of three bits need the filters' sums, which only resident filters give: such plans on nibbles against all on int8, by their time.
+    const bool offset = g.f4 && A == 3 && p->a_sign == BS_UNSIGNED;
     const double bound = static_cast<double>(p->C) * g.RS * max_abs_of(p->a_bits, p->a_sign) * max_abs_of(p->w_bits, p->w_sign);
     g.acc_bound = static_cast<float>(bound);
     g.preset = out_packed && !out_i32 && bound < 4.0e6 && p->out_sign != BS_BIPOLAR &&
@@ -295,6 +298,10 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
         MmaArgs t = g;
         if (!mma_layout(t, c, A, packed_b ? p->w_bits : 0, int_rows, sms)) return;
         c.cost = mma_cost(t, c, A, packed_b ? p->w_bits : 0, out_packed, sms);
+        c.f4 = g.f4;
+        // (the model takes nibbles of three bits for about 5 % faster than they are: 1024 x 1024 x 2304 modelled 0.99 of int8, timed 1.05; the layer of
+        // 32 x 256 x 28 x 28 and 256 filters 0.90 and 0.84)
+        if (offset && g.f4) c.cost *= 1.06;
         if (c.cost < best.cost) { best = c; found = true; }
     };
     int ns_list[12], nns = 0;
@@ -310,6 +317,7 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
     int ov[8] = {0, 0, 0, -1, 0, -1, 0, 0};    // TN, PT, units, config, strips, resident, groups, split; 0 / -1: free
     if (const char* e = getenv("BS_MM")) sscanf(e, "%d,%d,%d,%d,%d,%d,%d,%d", ov, ov + 1, ov + 2, ov + 3, ov + 4, ov + 5, ov + 6, ov + 7);
 #endif
+    for (int form = 0; form < (offset ? 2 : 1); ++form, g.f4 = 0)
     for (int TN = 32; TN <= 256; TN *= 2) {
         if (TN > 32 && TN / 2 >= up(p->O, 32)) continue;
         if (TN == 256 && !packed_b && g.opad % 256 != 0) continue;
@@ -320,7 +328,7 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
                         if (units > 1 && units > (g.Cw + 1) / 2) continue;
                         for (int v = 0; v < 18; ++v) {
                             const int res = v & 1, groups = 1 << ((v >> 1) % 3), split = 1 << (v / 6);
-                            if (groups > 2 && cfg != 1) continue;
+                            if ((groups > 2 && cfg != 1) || (offset && form == 0 && !res)) continue;
                             // Splits only for calls on their own: between the layers of a stack the change to another kernel costs what
                             // the split gains (18- and 50-layer stacks of batch 1 to 17: 2 % faster to 3 % slower).
                             // 32 filters wide: wider tiles expand more filters per CTA, and 32 without a split then beats them
@@ -338,6 +346,7 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
                     }
     }
     if (!found) return BS_ERR_UNSUPPORTED;
+    g.f4 = best.f4;
     if (!mma_layout(g, best, A, packed_b ? p->w_bits : 0, int_rows, sms)) return BS_ERR_UNSUPPORTED;
 #ifdef BS_TUNING
     if (getenv("BS_MM_VERBOSE"))

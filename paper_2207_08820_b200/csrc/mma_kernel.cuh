@@ -23,7 +23,8 @@
 //
 // Codes of three bits: signed ones, -4 .. 3, are halves as they are.  Of unsigned activations 5 and 7 are not, so the operand holds a - 4 (the top plane
 // inverted; padding, whose code is 0, becomes -4 like every zero) and the epilogue adds four times the sum of a filter's codes, as many as the
-// tile holds: sum (a - 4) w + 4 sum w = sum a w.  32 x 256 x 28 x 28, 256 filters, three bits both: 30.6 -> 25.6 us.
+// tile holds: sum (a - 4) w + 4 sum w = sum a w.  The sums are collected where resident packed filters are expanded; other plans of such
+// layers are int8.  32 x 256 x 28 x 28, 256 filters, three bits both: 30.6 -> 25.6 us.
 //
 // Every wait on an mbarrier is bounded; a wait that runs out sets the device status word and the CTA drains.
 #pragma once
@@ -582,50 +583,6 @@ static __device__ __noinline__ void convert_filters(const G& g, unsigned char* d
     __syncwarp();
 }
 
-// ----------------------------------------------------------------------------- sums of filters (unsigned activations of three bits)
-
-// Four times the sum of each filter's codes, by column of the tile, from memory: by EW warps, four columns at a time.  Packed filters (WB > 0) or
-// prepared ones in either form.
-template <int WB, int EW>
-static __device__ __noinline__ void filter_sums(const MmaArgs& g, float* out, int o0, int warp, int lane)
-{
-    const bool nib = WB == 0 && *reinterpret_cast<const volatile uint32_t*>(g.wgt + static_cast<size_t>(g.opad) * g.RS * 32 * g.Cw - 4) == MM_NIBBLE_MARK;
-    const int vecs = WB > 0 ? g.RS * g.Cw : (nib ? (g.Cw + 1) / 2 : g.Cw) * g.RS * 2;
-    for (int c0 = warp * 4; c0 < g.TN; c0 += EW * 4) {
-        int s[4] = {0, 0, 0, 0};
-        for (int v = lane; v < vecs; v += 32)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int c = c0 + k;
-                if (WB > 0) {
-                    const int o = o0 + (c & ~31) + mma_filter_of_column(c & 31);
-                    if (o >= g.O) continue;
-                    uint32_t w[WB > 0 ? WB : 1];
-#pragma unroll
-                    for (int j = 0; j < WB; ++j) w[j] = g.wgt_packed[(static_cast<size_t>(o) * vecs + v) * WB + j];
-                    s[k] += word_sum<WB>(w, g.w_kind);
-                } else {
-                    const int half = v & 1, t = v >> 1, blk = fdiv(t, g.d_rs), tap = t - blk * g.RS, col = o0 + c;
-                    const uint4 x = reinterpret_cast<const uint4*>(g.wgt)[((static_cast<size_t>(blk) * (g.opad >> 3) + (col >> 3)) * g.RS + tap) * 16 + half * 8 + (col & 7)];
-                    const uint32_t w[4] = {x.x, x.y, x.z, x.w};
-                    // (the last vector of the tensor carries the mark, negative zeros)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        if (!nib) { s[k] = __dp4a(static_cast<int>(w[j]), 0x01010101, s[k]); continue; }
-                        const uint32_t m = w[j] & 0x77777777u, neg = m & ((w[j] >> 3 & 0x11111111u) * 7u);
-                        s[k] += static_cast<int>(__dp4a(m & 0x0F0F0F0Fu, 0x01010101u, __dp4a(m >> 4 & 0x0F0F0F0Fu, 0x01010101u, 0u)));
-                        s[k] -= 2 * static_cast<int>(__dp4a(neg & 0x0F0F0F0Fu, 0x01010101u, __dp4a(neg >> 4 & 0x0F0F0F0Fu, 0x01010101u, 0u)));
-                    }
-                }
-            }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int sum = __reduce_add_sync(0xffffffffu, s[k]);
-            if (lane == 0) out[c0 + k] = 4.0f * static_cast<float>(sum);
-        }
-    }
-}
-
 // ----------------------------------------------------------------------------- MMA issue
 
 // Fixed kernel sizes: the taps are unrolled, nothing but additions on uniform registers between the MMAs.
@@ -1064,7 +1021,7 @@ __device__ __forceinline__ bool epilogue_codes(const MmaArgs& g, const MmaEpi& e
             if (tab_o >= 0) asm volatile("bar.sync 2, %0;" ::"n"(EW * 32) : "memory");     // every warp is done with the old table
             epilogue_tables(g, reinterpret_cast<float4*>(e.smem + g.off_tab), reinterpret_cast<float2*>(e.smem + g.off_tab + g.TN * 8), e.fast_ok, o0,
                             e.tid, EW * 32);
-            if (OFS) sums(o0);
+            if (OFS) sums();
             asm volatile("bar.sync 2, %0;" ::"n"(EW * 32) : "memory");
             fast = *reinterpret_cast<volatile int*>(e.fast_ok) != 0;
             tab_o = w.o;
@@ -1324,7 +1281,7 @@ __device__ __forceinline__ bool epilogue_general(const MmaArgs& g, const MmaEpi&
         const int o0 = w.o * g.TN, base = w.m * 128 * g.PT + e.row0;
         if (OFS && w.o != sum_o) {
             if (sum_o >= 0) asm volatile("bar.sync 2, %0;" ::"n"(EW * 32) : "memory");      // every warp is done with the old ones
-            sums(o0);
+            sums();
             asm volatile("bar.sync 2, %0;" ::"n"(EW * 32) : "memory");
             sum_o = w.o;
         }
@@ -1899,13 +1856,10 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
         e.smem = mm_smem; e.full_acc = full_acc; e.empty_acc = empty_acc; e.fast_ok = fast_ok;
         e.acc = tmem + lane_addr; e.row0 = quad * 32 + lane; e.set = set;
         e.tid = tid; e.lane = lane; e.warp = warp; e.red_full = red_full;
-        // what the epilogue adds to the accumulators of a filter tile, as floats by column
-        auto sums = [&](int o0) {
-            if constexpr (OFS) {
-                if (g.a_kind != 0 || (packed_b && resident))
-                    for (int c = tid; c < g.TN; c += NET) reinterpret_cast<float*>(sums_i)[c] = g.a_kind != 0 ? 0.0f : 4.0f * static_cast<float>(sums_i[c]);
-                else filter_sums<WB, EW>(g, reinterpret_cast<float*>(sums_i), o0, warp, lane);
-            }
+        // what the epilogue adds to the accumulators of a filter: four times the sum of its codes (only plans with resident filters take unsigned codes)
+        auto sums = [&]() {
+            if constexpr (OFS)
+                for (int c = tid; c < g.TN; c += NET) reinterpret_cast<float*>(sums_i)[c] = g.a_kind != 0 ? 0.0f : 4.0f * static_cast<float>(sums_i[c]);
         };
         bool ok;
         if (SPLIT && range.rank > 0) ok = send_partials<EW, F4>(g, e, range.rank);
@@ -1960,7 +1914,7 @@ template <int A>
 MmaKernel mma_pick_nibbles(int wb, bool half, bool split)
 {
     switch (wb) {
-        case 0: return mma_pick_shape<A, 0, true>(half, split);
+        case 0: if constexpr (A <= 2) return mma_pick_shape<A, 0, true>(half, split); else return nullptr;        // prepared filters are int8 there
         case 1: return mma_pick_shape<A, 1, true>(half, split);
         case 2: return mma_pick_shape<A, 2, true>(half, split);
         default: return mma_pick_shape<A, 3, true>(half, split);

@@ -198,7 +198,7 @@ extern "C" size_t bs_tc_weights_read_bytes(int O, int C, int R, int S, int w_bit
     const size_t all = bs_tc_weights_bytes(O, C, R, S);
     if (all == 0 || !bs::bits_ok(w_bits, BS_UNSIGNED) || !bs::bits_ok(a_bits, BS_UNSIGNED)) return 0;
     // (three bits: it depends on the sign of the filters)
-    return a_bits <= 2 && w_bits <= 2 && bs::mma_nibbles(C, R * S, a_bits, w_bits, BS_SIGNED) ? all / (C / 32) * ((C / 32 + 1) / 2) : all;
+    return w_bits <= 2 && bs::mma_nibbles(C, R * S, a_bits, w_bits, BS_SIGNED) ? all / (C / 32) * ((C / 32 + 1) / 2) : all;
 }
 
 extern "C" int bs_tc_prepare_weights(const uint32_t* wgt_packed, int O, int C, int R, int S, int w_bits, bs_sign_t w_sign,
