@@ -308,10 +308,11 @@ int bs_sequence_create(const bs_sequence_layer* layers, int nlayers, void* side_
 /*
  * bs_sequence_create_ws -- the same with device memory in which the layers may keep, beside the packed codes, what the tensor cores read of every
  * tensor that a later layer reads (32 channels of a position as 16 bytes of nibbles, zero padding included).  Same outputs, every packed tensor
- * included; a layer then expands nothing.  One launch more for every tensor that is read before the layers have written all of it.
+ * included; a layer then expands nothing.  One launch more for every tensor that is read before the layers have written all of it, and one
+ * that prepares filters, of a third of the layers and 16 at most, which came packed.
  *   workspace             bs_sequence_workspace_bytes bytes, 16-byte aligned, ZERO before the first run, the sequence's own from then on; NULL or
  *                         less than that: as bs_sequence_create.  May pass on to another sequence of layers of the same shapes, formats and order.
- * bs_sequence_workspace_bytes answers 0 where the layers don't take one: layers without prepared filters, codes of more than two bits or signed ones,
+ * bs_sequence_workspace_bytes answers 0 where the layers don't take one: too many layers without prepared filters, codes of more than two bits or signed ones,
  * tensors that overlap or that are used with two shapes, rows too wide for the shared memory.  It needs no device.
  * bs_sequence_launches: kernels that bs_sequence_run enqueues.
  * bs_sequence_input     the operand tensor of a tensor of packed codes that the layers read before they have written all of it (it belongs to the

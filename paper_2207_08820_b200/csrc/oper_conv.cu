@@ -35,6 +35,44 @@ static __global__ void __launch_bounds__(256) oper_import_kernel(const __grid_co
     }
 }
 
+// ----------------------------------------------------------------------------- packed filters -> prepared ones, of several layers in a launch
+
+constexpr int OP_FILTERS = 16;              // layers whose filters a pass prepares, at most
+
+struct FilterSet {
+    struct Layer {
+        const uint32_t* packed;             // [O][R*S][Cw][bits]
+        uint4* out;                         // as bs_tc_prepare_weights lays out nibbles, [C/64][O/8][tap][2][8 filters], the mark in the last vector
+        int O, RS, Cw, bits, kind, groups, vecs;        // groups of eight filters, vectors written
+        long long last;
+    } layer[OP_FILTERS];
+};
+
+static __global__ void __launch_bounds__(256) oper_filters_kernel(const __grid_constant__ FilterSet set)
+{
+    const FilterSet::Layer& f = set.layer[blockIdx.y];
+    const uint32_t* packed = dependent_begin(f.packed);
+    for (int idx = blockIdx.x * 256 + threadIdx.x; idx < f.vecs; idx += gridDim.x * 256) {
+        int t = idx >> 4;
+        const int half = idx >> 3 & 1, tap = t % f.RS;
+        t /= f.RS;
+        const int og = t % f.groups, cw = t / f.groups * 2 + half, col = og * 8 + (idx & 7), o = (col & ~31) + mma_filter_of_column(col & 31);
+        uint32_t v[4] = {0, 0, 0, 0};
+        if (o < f.O && cw < f.Cw) {
+            const uint32_t* p = packed + ((static_cast<size_t>(o) * f.RS + tap) * f.Cw + cw) * f.bits;
+            uint32_t w[3] = {p[0], f.bits > 1 ? p[1] : 0u, f.bits > 2 ? p[2] : 0u};
+            if (f.bits == 1) expand_nibbles<1>(w, f.kind, v);
+            else if (f.bits == 2) expand_nibbles<2>(w, f.kind, v);
+            else expand_nibbles<3>(w, f.kind, v);
+        }
+        if (idx == f.vecs - 1) {
+            if (f.last == idx) v[3] = MM_NIBBLE_MARK;
+            else f.out[f.last] = make_uint4(0, 0, 0, MM_NIBBLE_MARK);
+        }
+        f.out[idx] = make_uint4(v[0], v[1], v[2], v[3]);
+    }
+}
+
 // ----------------------------------------------------------------------------- tensors of a sequence
 
 namespace {
@@ -75,6 +113,7 @@ Shape shape_of(const bs_conv_params& p)
 struct Layout {
     std::vector<Tensor> tensors;
     std::vector<int> src, dst;      // of each layer
+    std::vector<size_t> filters;    // where its filters are prepared in front of the layers, 0: they came prepared
     size_t bytes;
 };
 
@@ -95,11 +134,16 @@ int tensor_index(Layout& l, const uint32_t* ptr, int N, int H, int W, int Cw, in
 // used with two shapes.
 bool lay_out(const bs_sequence_layer* layers, int n, Layout& l)
 {
+    // Layers whose records the prepared-filter entry points refuse come with packed filters; one launch prepares them in every pass, where each such
+    // layer gains a microsecond or more.
+    int unprepared = 0;
+    for (int i = 0; i < n; ++i) unprepared += !layers[i].wgt_tc;
+    if (unprepared > n / 3 || unprepared > OP_FILTERS) return false;
     for (int i = 0; i < n; ++i) {
         const bs_conv_params& p = layers[i].p;
-        if (!layers[i].wgt_tc || !layers[i].out_packed || !layers[i].act_packed || p.C % 32 != 0) return false;
+        if (!layers[i].out_packed || !layers[i].act_packed || p.C % 32 != 0) return false;
         if (p.a_sign != BS_UNSIGNED || p.out_sign != BS_UNSIGNED || p.out_bits > 2 || p.out_bits < 1) return false;
-        if (p.a_bits > 2 || !mma_nibbles(p.C, p.R * p.S, p.a_bits, p.w_bits, p.w_sign) || p.stride > 2 || p.R != p.S) return false;
+        if (!mma_nibbles(p.C, p.R * p.S, p.a_bits, p.w_bits, p.w_sign) || p.stride > 2 || p.R != p.S) return false;
         if (p.residual && (p.res_sign != BS_UNSIGNED || p.res_bits > 2 || !(fabsf(p.res_scale) < 3.9f) || (p.res_scale != 0.0f && fabsf(p.res_scale) <= 1e-18f))) return false;
         const Shape s = shape_of(p);
         const int src = tensor_index(l, layers[i].act_packed, p.N, p.H, p.W, p.C / 32, p.a_bits);
@@ -142,6 +186,13 @@ bool lay_out(const bs_sequence_layer* layers, int n, Layout& l)
             f.offset = (off + edge + 255) / 256 * 256;
             off = f.offset + f.group * static_cast<size_t>(t.Cw) + edge + static_cast<size_t>(OP_MAX_ROWS) * 16;
         }
+    for (int i = 0; i < n; ++i) {
+        const bs_conv_params& p = layers[i].p;
+        l.filters.push_back(0);
+        if (layers[i].wgt_tc) continue;
+        l.filters.back() = (off + 255) / 256 * 256;
+        off = l.filters.back() + bs_tc_weights_bytes(p.O, p.C, p.R, p.S);
+    }
     l.bytes = off;
     return true;
 }
@@ -250,6 +301,8 @@ struct OperSequence {
     struct Import { OperTensor g; unsigned grid; };
     std::vector<Step> steps;
     std::vector<Import> imports;
+    FilterSet filters;
+    int nfilters, filter_blocks;
 };
 
 // Arguments of layer i but its tiling.
@@ -272,7 +325,7 @@ static bool fill(OperArgs& g, const bs_sequence_layer& l, const Layout& lay, int
     g.src = ws + f.offset + (static_cast<long long>(s.rmin) * f.pitch + s.rmin) * 16;
     g.src_group = static_cast<long long>(f.group);
     g.src_plane = static_cast<long long>(f.plane);
-    g.wgt = l.wgt_tc;
+    g.wgt = l.wgt_tc ? l.wgt_tc : reinterpret_cast<int8_t*>(ws + lay.filters[i]);
     g.out_packed = l.out_packed;
     const int word = p.out_c_offset / 32;
     g.dst1 = dst_of(out, 0, ws, word);
@@ -284,7 +337,7 @@ static bool fill(OperArgs& g, const bs_sequence_layer& l, const Layout& lay, int
     g.out_cw_off = word; g.out_cw_total = out.Cw;
     g.res_bits = p.res_bits; g.res_sign = p.res_sign; g.res_c_off = p.res_c_offset;
     g.res_cw_total = ceil_div(p.res_c_total > 0 ? p.res_c_total : 1, 32);
-    g.early_b = l.chained && !l.aside;
+    g.early_b = l.chained && !l.aside && l.wgt_tc;
     g.status = status_device_ptr();
     return true;
 }
@@ -337,9 +390,21 @@ static bool build(const bs_sequence_layer* layers, int n, unsigned char* ws, Ope
     int sms = device_sm_count();
     if (sms <= 0) sms = 148;
     q.steps.resize(static_cast<size_t>(n));
+    q.nfilters = q.filter_blocks = 0;
     for (int i = 0; i < n; ++i) {
         memset(static_cast<void*>(&q.steps[i]), 0, sizeof q.steps[i]);
         if (!fill(q.steps[i].g, layers[i], lay, i, ws) || !plan_layer(q.steps[i], sms)) return false;
+        const bs_conv_params& p = layers[i].p;
+        if (!layers[i].wgt_tc) {
+            FilterSet::Layer& f = q.filters.layer[q.nfilters++];
+            const int groups = up(p.O, 128) / 8, RS = p.R * p.S, Cw = p.C / 32;
+            const long long vecs = static_cast<long long>((Cw + 1) / 2) * groups * RS * 16;
+            if (vecs > 0x7fffff00LL) return false;
+            f = {layers[i].wgt_packed, reinterpret_cast<uint4*>(ws + lay.filters[i]), p.O, RS, Cw, p.w_bits, p.w_sign == BS_SIGNED ? 1 : p.w_sign == BS_BIPOLAR ? 2 : 0, groups,
+                 static_cast<int>(vecs), static_cast<long long>(Cw) * groups * RS * 16 - 1};
+            const int blocks = static_cast<int>((vecs + 255) / 256);
+            if (blocks > q.filter_blocks) q.filter_blocks = blocks < 4 * sms ? blocks : 4 * sms;
+        }
     }
     for (const Tensor& t : lay.tensors) {
         if (!t.read || !t.import) continue;
@@ -378,7 +443,7 @@ OperSequence* oper_create(const bs_sequence_layer* layers, int n, void* workspac
     return nullptr;
 }
 
-int oper_imports(const OperSequence* q) { return static_cast<int>(q->imports.size()); }
+int oper_imports(const OperSequence* q) { return static_cast<int>(q->imports.size()) + (q->nfilters > 0); }
 
 const OperTensor* oper_input(const OperSequence* q, const uint32_t* packed)
 {
@@ -389,6 +454,10 @@ const OperTensor* oper_input(const OperSequence* q, const uint32_t* packed)
 
 int oper_begin(const OperSequence* q, const OperTensor* ready, cudaStream_t st)
 {
+    if (q->nfilters > 0) {
+        const int rc = launch_dependent(oper_filters_kernel, dim3(static_cast<unsigned>(q->filter_blocks), static_cast<unsigned>(q->nfilters)), dim3(256), 0, st, q->filters);
+        if (rc != BS_OK) return rc;
+    }
     for (const OperSequence::Import& m : q->imports) {
         if (&m.g == ready) continue;
         const int rc = launch_dependent(oper_import_kernel, dim3(m.grid), dim3(256), 0, st, m.g);

@@ -13,7 +13,7 @@ struct OperTensor;
 size_t oper_workspace_bytes(const bs_sequence_layer* layers, int n);
 // The launches of such layers; null where oper_workspace_bytes is 0 or bytes is less.
 OperSequence* oper_create(const bs_sequence_layer* layers, int n, void* workspace, size_t bytes);
-// The forms of a tensor that the layers read from its packed codes, which launches in front of the layers bring into them; null: no such tensor.
+// Launches in front of the layers: filters to prepare, forms of tensors that the layers read from their packed codes; those of one tensor, or null.
 int oper_imports(const OperSequence* q);
 const OperTensor* oper_input(const OperSequence* q, const uint32_t* packed);
 // These launches but the one of `ready`, whose forms are up to date (or null), and layer i, on `st`.

@@ -176,7 +176,7 @@ class BitserialNet:
         block) runs ``aside`` on a second stream when it does not fill the GPU by itself: at most one 128 x 128 block of outputs per
         multiprocessor (a measure of its size; the plans cut their own tiles).  ``join``: positions of the calls that must be waited for first.
 
-        Layers of a pass as a graph, us, never aside / by this line / always where the data allow (B200):
+        Layers of a pass as a graph, each expanding packed codes, us, never aside / by this line / always where the data allow (B200):
         18-layer stack, batch 1: 100.4 / 92.5 / 92.5, 8: 127.2 / 124.5 / 124.7, 16: 137.9 / 139.4 / 139.6, 64: 226.5 / 226.2 / 227.6;
         50-layer stack, 1: 252.3 / 237.1 / 238.6, 8: 339.0 / 337.7 / 336.3, 32: 515.8 / 516.2 / 522.2;
         detection stack (160 px), 1: 126.6 / 117.6 / 117.6, 4: 143.7 / 137.4 / 140.2, 16: 176.2 / 177.9 / 180.0, 32: 219.0 / 221.5 / 224.1.
@@ -224,7 +224,7 @@ class BitserialNet:
             self.run_units()
 
     def run_units(self) -> None:
-        """The same launches one call per unit: what :meth:`run_layers` does where the library does not take the layers as one sequence."""
+        """The same layers one call per unit, on packed codes: what :meth:`run_layers` does where the library does not take them as one sequence."""
         main = torch.cuda.current_stream(self.device)
         done: Dict[int, torch.cuda.Event] = {}
         for i, (unit, aside, join) in enumerate(self.schedule()):

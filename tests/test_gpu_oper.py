@@ -33,6 +33,11 @@ STACKS = {
     "one_bit": net(3, (64, 10, 12), [L("a", "x", "a", 64, 128, 3, 1, 1), L("b", "a", "b", 128, 64, 3, 2, 1), L("c", "b", "c", 64, 64, 1, 1, 0, res="b", res_scale=0.5)], 1, 1),
     "wide": net(1, (32, 3, 300), [L("a", "x", "a", 32, 64, 3, 1, 1), L("b", "a", "b", 64, 32, 3, 2, 1), L("c", "b", "c", 32, 32, 1, 1, 0)]),
     "deep": net(1, (512, 7, 7), [L("a", "x", "a", 512, 256, 3, 1, 1), L("b", "a", "b", 256, 512, 1, 1, 0), L("c", "b", "c", 512, 64, 3, 2, 1)]),
+    # records that no prepared filters are taken for: the pass prepares them
+    "odd_records": net(2, (32, 9, 11), [L("a", "x", "a", 32, 64, 3, 2, 1), L("b", "a", "b", 64, 32, 1, 1, 0), L("c", "b", "c", 32, 32, 3, 1, 1, res="b", res_scale=0.5),
+                                        L("d", "c", "d", 32, 128, 1, 1, 0), L("e", "d", "e", 128, 64, 3, 1, 1), L("f", "e", "f", 64, 64, 3, 1, 1), L("g", "f", "g", 64, 64, 1, 1, 0),
+                                        L("h", "g", "h", 64, 64, 3, 1, 1), L("i", "h", "i", 64, 64, 3, 1, 1)]),
+    "odd_one_bit": net(3, (64, 9, 13), [L("a", "x", "a", 64, 96, 3, 1, 1), L("b", "a", "b", 96, 64, 3, 2, 1)] + [L(f"l{i}", f"l{i - 1}" if i else "b", f"l{i}", 64 if i == 0 else 128, 128, 1, 1, 0) for i in range(7)], 1, 1),
     "pixels": net(40, (64, 1, 1), [L("a", "x", "a", 64, 64, 3, 1, 1), L("b", "a", "b", 64, 64, 1, 1, 0), L("c", "b", "c", 64, 32, 3, 2, 1)]),
 }
 
@@ -60,7 +65,9 @@ def both(r, x):
 def test_stacks(name):
     spec = STACKS[name]
     r, params, x = runner_of(spec)
-    assert r._sequence.launches == len(spec.layers) + 1             # the layers take operand tensors, of the input by a launch of its own
+    # the layers take operand tensors, of the input by a launch of its own
+    assert r._sequence.launches == len(spec.layers) + 1 + any(item["w_tc"] is None for item in r.layers)
+    assert (name in ("odd_records", "odd_one_bit")) == any(item["w_tc"] is None for item in r.layers)
     for seed in (0, 1):
         got, want = both(r, np.roll(x, seed, 0) if seed else x)
         for k in want:
@@ -130,11 +137,26 @@ def test_replaced_filters_scales_and_tensors():
     api.bs_check_status()
 
 
+def test_filters_prepared_in_the_pass_follow_the_packed_ones():
+    spec = STACKS["odd_records"]
+    (a, _, x), (b, _, _) = runner_of(spec), runner_of(spec, seed=12)
+    xd = dev(x)
+    want = b.forward(xd).clone()
+    assert not torch.equal(a.forward(xd), want)
+    for mine, theirs in zip(a.layers, b.layers):
+        for key in ("w", "w_tc", "scale", "bias"):
+            if theirs[key] is not None:
+                mine[key].copy_(theirs[key])                         # in place: nothing is bound again
+    assert torch.equal(a.forward(xd), want)
+    api.bs_check_status()
+
+
 def test_sequences_that_keep_packed_tensors():
-    """Overlapping tensors and layers without prepared filters run as they did."""
+    """Overlapping tensors, and stacks in which most layers have no prepared filters, run as they did."""
     spec = STACKS["one_group"]
     r, _, x = runner_of(spec)
-    r.layers[1]["w_tc"] = None
+    for item in r.layers[:2]:
+        item["w_tc"] = None
     got, want = both(r, x)
     assert r.launches_per_forward == 1 + len(spec.layers)
     for k in want:
