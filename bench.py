@@ -106,7 +106,7 @@ def captured_traffic(net_name: str, batch: int):
     import hashlib
     import re
     path = os.path.join(ROOT, "profiles", f"bitserial_conv_tc_kernels_{net_name}_dram_traffic.md")
-    src = os.path.join(ROOT, "paper_2207_08820_b200", "csrc", "mma_kernel.cuh")
+    src = os.path.join(ROOT, "paper_2207_08820_b200", "csrc", "oper_kernel.cuh")
     if not (os.path.exists(path) and os.path.exists(src)):
         return None, None
     text = open(path).read()
@@ -346,7 +346,7 @@ def measure_other_configs(torch, api, stream, args):
       detection_backbone            the detection-shaped stack at batch 16 on the tensor-core engine: conv time per pass under a
                                     CUDA graph, images/s, and sum(roofline time) / measured time over its layers;
       layer_chains   the residual stack's conv layers at batch 16 and 64, the bound sequence (one call) against a call per unit, runs of
-                     same-shaped layers among them as one (bitserial_conv2d_tc_chain); the launches are the same;
+                     same-shaped layers among them as one (bitserial_conv2d_tc_chain); the former runs on operand tensors;
       pack_large     the pack kernels on inputs larger than L2 (fp32 NCHW and NHWC, 2 and 3 bits)."""
     from paper_2207_08820_b200.net import BitserialNet
     dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
@@ -697,7 +697,7 @@ def run_ours(args):
         def tensor_roofline(t_ms, engine):
             a = 2.0 * macs / (t_ms * 1e-3) / 1e12
             _, sums = layer_roofline(net, engine, peaks)
-            traffic = tc_traffic if engine == "tc" else None
+            traffic = tc_traffic if engine == "tc" and whole else None
             return {"bound": "tensor", "kernel": "bitserial_oper_kernel" if engine == "tc" and whole else "bitserial_mma_kernel", "achieved": a, "peak": burst,
                     "unit": "TOP/s", "frac": a / burst, "peak_burst": burst, "peak_sustained": sustained,
                     "frac_sustained": a / sustained,
@@ -726,7 +726,7 @@ def run_ours(args):
             "roofline": roof,
             "pack": {"bound": "hbm", "ms": t_pack, "achieved": pack_bytes / (t_pack * 1e-3) / 1e9, "peak": peaks["hbm_gbs"],
                      "unit": "GB/s", "frac": pack_bytes / (t_pack * 1e-3) / 1e9 / peaks["hbm_gbs"],
-                     "note": "54.6 MB input: a 12 us kernel, ramp and tail dominate; pack_large has the inputs larger than L2"},
+                     "note": "51 MB input: a 12 us kernel, ramp and tail dominate, which also writes the layers' operand tensor (6.7 MB, not counted); pack_large has the inputs larger than L2"},
             "e2e": {"value": 2.0 * macs * world / (t_e2e * 1e-3) / 1e9, "unit": UNIT, "ms_per_step": t_e2e, "overlap": "h2d of step k+1 beside the kernels of step k (two input buffers); L2 flush inside",
                     "h2d_bytes_per_step": in_bytes, "d2h_bytes_per_step": out_host.numel() * 4},
             "gpu_launches": (runner.launches_per_forward if whole else 1 + len(net.layers)) * nsteps,

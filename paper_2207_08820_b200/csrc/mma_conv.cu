@@ -300,7 +300,7 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
         c.cost = mma_cost(t, c, A, packed_b ? p->w_bits : 0, out_packed, sms);
         c.f4 = g.f4;
         // (the model takes nibbles of three bits for about 5 % faster than they are: 1024 x 1024 x 2304 modelled 0.99 of int8, timed 1.05; the layer of
-        // 32 x 256 x 28 x 28 and 256 filters 0.90 and 0.84)
+        // 32 x 256 x 28 x 28 and 256 filters 0.90 and 0.75)
         if (offset && g.f4) c.cost *= 1.06;
         if (c.cost < best.cost) { best = c; found = true; }
     };

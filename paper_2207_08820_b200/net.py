@@ -51,7 +51,7 @@ class BitserialNet:
         supports it (others keep packed filters).  concurrent: launch independent neighbouring layers on
         two streams (see :meth:`schedule`).  chains: True groups, with the "tc" engine, runs of consecutive same-shaped layers that the
         library accepts into units which :meth:`run_units` issues as one ``bitserial_conv2d_tc_chain`` call each; False and "auto" = a unit per
-        layer.  A pass is one call of a bound sequence whatever the units are; the launches are the same on either way."""
+        layer.  A pass is one call of a bound sequence whatever the units are."""
         self.net = net
         self.engine = engine
         self.act_scale = float(act_scale)
