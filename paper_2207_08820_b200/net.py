@@ -176,11 +176,11 @@ class BitserialNet:
         block) runs ``aside`` on a second stream when it does not fill the GPU by itself: at most one 128 x 128 block of outputs per
         multiprocessor (a measure of its size; the plans cut their own tiles).  ``join``: positions of the calls that must be waited for first.
 
-        Layers of a pass as a graph, each expanding packed codes, us, never aside / by this line / always where the data allow (B200):
-        18-layer stack, batch 1: 100.4 / 92.5 / 92.5, 8: 127.2 / 124.5 / 124.7, 16: 137.9 / 139.4 / 139.6, 64: 226.5 / 226.2 / 227.6;
-        50-layer stack, 1: 252.3 / 237.1 / 238.6, 8: 339.0 / 337.7 / 336.3, 32: 515.8 / 516.2 / 522.2;
-        detection stack (160 px), 1: 126.6 / 117.6 / 117.6, 4: 143.7 / 137.4 / 140.2, 16: 176.2 / 177.9 / 180.0, 32: 219.0 / 221.5 / 224.1.
-        Up to 7 % gained while a layer leaves room, about 1 % lost near the line, 2 % where both neighbours fill the GPU."""
+        Layers of a pass as a graph, us, never aside / by this line / always where the data allow (B200, operand tensors):
+        18-layer stack, batch 1: 62.0 / 59.9 / 59.9, 8: 74.6 / 73.6 / 73.9, 16: 85.0 / 85.4 / 84.6, 64: 143.7 / 143.9 / 145.5;
+        50-layer stack, 1: 173.2 / 169.4 / 169.2, 8: 231.1 / 231.6 / 232.1, 32: 382.3 / 382.6 / 386.8;
+        detection stack (160 px), 1: 82.3 / 77.6 / 78.0, 4: 90.6 / 88.4 / 89.0, 16: 118.5 / 117.2 / 121.3, 32: 145.8 / 147.9 / 152.0.
+        Up to 6 % gained while a layer leaves room, about 1 % lost near the line, up to 4 % where both neighbours fill the GPU."""
         out, pending = [], {}
         n = len(self.units)
 
