@@ -1396,7 +1396,6 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
     const int BM = 128 * g.PT;
 
     MM_TRACE(tid == 0, TR_START, 0);
-    mm_pdl_release();
     if (OFS)
         for (int c = tid; c < g.TN; c += MmaShape<HALF>::THREADS) sums_i[c] = 0;
     if (tid == 0) {
@@ -1422,6 +1421,9 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
     mm_fence_before();
     __syncthreads();
     mm_fence_after();
+    // Only now: a CTA of a later launch may take tensor memory as soon as it runs, and keeps it until every launch before it has ended.  Released while
+    // this CTA still waits for its columns, the two could wait for each other.
+    mm_pdl_release();
     if (SPLIT) mm_cluster_sync();      // the barriers of rank 0 are initialised
     const MmaChunks range(g, SPLIT);
     const int walk_log = SPLIT ? g.split_log : 0;
