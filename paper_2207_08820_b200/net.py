@@ -284,7 +284,8 @@ class BitserialNet:
             return None
         tensors = {}
         at = lambda address: tensors.setdefault(address, len(tensors))
-        key = tuple((at(q.act_packed), at(q.out_packed), *(getattr(q.p, f) for f in (
+        # (filters that a pass prepares lie there as well)
+        key = nbytes, *((at(q.act_packed), at(q.out_packed), bool(q.wgt_tc), *(getattr(q.p, f) for f in (
             "N", "C", "H", "W", "O", "R", "stride", "pad", "a_bits", "out_bits", "out_c_offset", "out_c_total"))) for q in arr)
         ws = self._workspaces.get(key)
         if ws is None and not torch.cuda.is_current_stream_capturing():     # (recorded, its clearing would belong to the graph)

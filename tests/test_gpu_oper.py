@@ -174,3 +174,19 @@ def test_sequences_that_keep_packed_tensors():
     r.run_units()
     assert torch.equal(have, r.bufs["c"])
     api.bs_check_status()
+
+
+def test_filters_taken_away_from_a_bound_runner():
+    """A layer that loses its prepared filters changes what the workspace holds, not whether the stack runs on operand tensors."""
+    spec = STACKS["one_group"]
+    r, _, x = runner_of(spec)
+    n = len(spec.layers)
+    assert r._sequence.launches == n + 1
+    for i in range(n):
+        kept, r.layers[i]["w_tc"] = r.layers[i]["w_tc"], None
+        got, want = both(r, x)
+        assert r._sequence.launches == n + 2, i                      # the input's import, and one launch that prepares the filters
+        for k in want:
+            assert torch.equal(got[k], want[k]), k
+        r.layers[i]["w_tc"] = kept
+    api.bs_check_status()
