@@ -30,6 +30,7 @@ class _Sequence:
         self.handle = None
         self.launches = 0
         self.input: Optional[int] = None        # operand tensor of the network's input
+        self.workspace: Optional[_Workspace] = None
 
     def own(self, handle: int, packed: int) -> None:
         self.handle = handle
@@ -42,8 +43,17 @@ class _Sequence:
         return units is self.units and concurrent == self.concurrent and native().unchanged(self.dicts, self.values, self.addresses)
 
 
+class _Workspace:
+    """Memory of the operand tensors of sequences of one ``geometry``, the last of which had its tensors at ``addresses``.  ``recorded``: a pass that
+    uses it went into a graph, which may be replayed beside passes over other tensors."""
+
+    def __init__(self, geometry, addresses, memory: torch.Tensor):
+        self.geometry, self.addresses, self.memory, self.recorded = geometry, addresses, memory, False
+
+
 class BitserialNet:
     MAX_CHAIN = 4
+    MAX_WORKSPACES = 4      # arrangements of tensors that have memory for operand tensors; passes over further ones run on packed codes
 
     def __init__(self, net: NetSpec, params: Dict[str, Dict], act_scale: float, device="cuda", batch: Optional[int] = None,
                  engine: str = "popc", concurrent: bool = True, chains="auto"):
@@ -84,7 +94,7 @@ class BitserialNet:
         self.graph = None
         self.static_in = None
         self.launches_per_forward = 1 + len(self.layers)
-        self._workspaces: Dict[tuple, torch.Tensor] = {}
+        self._workspaces: List[_Workspace] = []
         self._sequence: Optional[_Sequence] = None
         self._captured: Optional[_Sequence] = None      # what the graph was captured from
         self._bind()
@@ -244,12 +254,14 @@ class BitserialNet:
     def _bind(self) -> bool:
         """Binds the layers as one sequence to the tensors and settings they have now, again when one was replaced; False where the library does
         not take them as one."""
-        q = self._sequence
+        q, recording = self._sequence, torch.cuda.is_current_stream_capturing()
         if q is not None and q.current(self.units, self.concurrent):
+            if recording and q.workspace is not None:
+                q.workspace.recorded = True
             return q.handle is not None
         items = [item for unit in self.units for item in unit["items"]]
         self._sequence = _Sequence(self.units, self.concurrent, [self.bufs, *items, *(vars(item["spec"]) for item in items)])
-        if q is not None and not torch.cuda.is_current_stream_capturing():
+        if q is not None and not recording:
             torch.cuda.synchronize(self.device)     # as at set-up: what replaced a filter, scale or bias has to be final
         steps = self.schedule()
         at, layers = {}, []                          # position of a launch among the layers
@@ -269,33 +281,48 @@ class BitserialNet:
             q.chained, q.aside = 1, int(aside)
             q.join[:] = (join + [-1] * 4)[:4]
         handle = ctypes.c_void_p()
-        ws = self._workspace(arr)
-        if lib().bs_sequence_create_ws(arr, len(layers), self.side.cuda_stream, api._ptr(ws), ws.numel() if ws is not None else 0, ctypes.byref(handle)) != 0:
+        ws = self._sequence.workspace = self._workspace(arr, recording)
+        memory, nbytes = (api._ptr(ws.memory), ws.memory.numel()) if ws is not None else (None, 0)
+        if lib().bs_sequence_create_ws(arr, len(layers), self.side.cuda_stream, memory, nbytes, ctypes.byref(handle)) != 0:
             return False
+        if recording and ws is not None:
+            ws.recorded = True
         self._sequence.own(handle.value, api._ptr(self.bufs[self.net.in_name]))
         self.launches_per_forward = 1 + self._sequence.launches - (self._sequence.input is not None)
         return True
 
-    def _workspace(self, arr) -> Optional[torch.Tensor]:
-        """Memory of the layers' operand tensors (``bs_sequence_create_ws``), or None.  Kept while the runner lives, for every arrangement of tensors
-        it has had: graphs that a caller recorded go on using it."""
+    def _workspace(self, arr, recording: bool) -> Optional[_Workspace]:
+        """Memory of the layers' operand tensors (``bs_sequence_create_ws``), or None.  What a graph was recorded with stays with its tensors while the
+        runner lives; otherwise it passes on to the next arrangement of the same geometry, whose passes begin on an idle device."""
         nbytes = lib().bs_sequence_workspace_bytes(arr, len(arr))
         if nbytes == 0:
             return None
         tensors = {}
         at = lambda address: tensors.setdefault(address, len(tensors))
         # (filters that a pass prepares lie there as well)
-        key = nbytes, *((at(q.act_packed), at(q.out_packed), bool(q.wgt_tc), *(getattr(q.p, f) for f in (
-            "N", "C", "H", "W", "O", "R", "stride", "pad", "a_bits", "out_bits", "out_c_offset", "out_c_total"))) for q in arr)
-        ws = self._workspaces.get(key)
-        if ws is None and not torch.cuda.is_current_stream_capturing():     # (recorded, its clearing would belong to the graph)
-            try:
-                ws = torch.zeros(nbytes, dtype=torch.uint8, device=self.device)
-            except torch.OutOfMemoryError:
-                return None
-            torch.cuda.synchronize(self.device)
-            self._workspaces[key] = ws
-        return ws
+        geometry = (nbytes, *((at(q.act_packed), at(q.out_packed), bool(q.wgt_tc), *(getattr(q.p, f) for f in (
+            "N", "C", "H", "W", "O", "R", "stride", "pad", "a_bits", "out_bits", "out_c_offset", "out_c_total"))) for q in arr))
+        addresses = tuple(tensors)
+        alike = [w for w in self._workspaces if w.geometry == geometry]
+        for w in alike:
+            if w.addresses == addresses:
+                return w
+        if recording:                           # (its clearing would belong to the graph, and nobody has waited for passes under way)
+            return None
+        for w in alike:
+            if not w.recorded:
+                w.addresses = addresses
+                return w
+        self._workspaces = [w for w in self._workspaces if w.recorded]
+        if len(self._workspaces) >= self.MAX_WORKSPACES:
+            return None
+        try:
+            memory = torch.zeros(nbytes, dtype=torch.uint8, device=self.device)
+        except torch.OutOfMemoryError:
+            return None
+        torch.cuda.synchronize(self.device)
+        self._workspaces.append(_Workspace(geometry, addresses, memory))
+        return self._workspaces[-1]
 
     def _conv_params(self, item):
         net, L = self.net, item["spec"]

@@ -190,3 +190,41 @@ def test_filters_taken_away_from_a_bound_runner():
             assert torch.equal(got[k], want[k]), k
         r.layers[i]["w_tc"] = kept
     api.bs_check_status()
+
+
+def test_recorded_passes_keep_their_workspace():
+    """A graph that reads tensors of its own shares no memory with passes over others: the two may run side by side.  Without a graph the workspace
+    passes on, and the number of those that graphs hold is bounded."""
+    spec = STACKS["both_strides"]
+    r, _, x = runner_of(spec)
+    xd = dev(x)
+    r.forward(xd)
+    first = r._sequence.workspace
+
+    def move():
+        for k in r.bufs:
+            r.bufs[k] = torch.empty_like(r.bufs[k])
+        torch.cuda.synchronize()
+
+    old = dict(r.bufs)
+    move()
+    want = r.forward(xd).clone()
+    assert r._sequence.workspace is first and len(r._workspaces) == 1
+    graphs, tensors = [], []
+    for i in range(r.MAX_WORKSPACES + 1):
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            r.run_layers()
+        graphs.append(graph)
+        tensors.append(dict(r.bufs))
+        move()
+        r.pack_input(xd)
+        r.run_layers()
+        live, recorded = r._sequence.workspace, [w for w in r._workspaces if w.recorded]
+        assert (live is None) == (i + 1 >= r.MAX_WORKSPACES) and len(recorded) == min(i + 1, r.MAX_WORKSPACES) and live not in recorded
+        assert torch.equal(r.bufs[spec.out_name], want)
+    for graph, bufs in zip(graphs, tensors):
+        bufs[spec.out_name].fill_(-1)
+        graph.replay()
+        assert torch.equal(bufs[spec.out_name], want)
+    api.bs_check_status()
