@@ -271,7 +271,7 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
     // outputs 0.98 and 0.97; codes of 5x5 windows over up to 32 channels 1.12 and 0.89 on these sides, of 3x3 windows 0.96 and 0.94.
     const bool short_k = g.Cw == 1 && static_cast<double>(g.N) * g.P * g.Q * g.O >= 2048.0 * sms;
     const bool pixel_rows = out_i32 && !out_packed && !g.i32_nhwc;
-    g.f4 = (mma_nibbles(p->C, g.RS, p->a_bits, p->w_bits, p->w_sign) || (packed_b && mma_nibbles_a3(p->C, g.RS, p->a_bits, p->w_bits, p->w_sign))) &&
+    g.f4 = (packed_b ? mma_nibbles_packed(p->C, g.RS, p->a_bits, p->w_bits, p->w_sign) : mma_nibbles(p->C, g.RS, p->a_bits, p->w_bits)) &&
            !(packed_b && (pixel_rows ? short_k || (g.R == 1 && g.Cw <= 6) : short_k && g.R >= 5 && !out_i32));
     // Unsigned activations of three bits need the filters' sums, which only resident filters give: such plans on nibbles against all on int8, by their time.
     const bool offset = g.f4 && A == 3 && p->a_sign == BS_UNSIGNED;

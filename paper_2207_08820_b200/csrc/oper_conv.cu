@@ -60,10 +60,9 @@ static __global__ void __launch_bounds__(256) oper_filters_kernel(const __grid_c
         uint32_t v[4] = {0, 0, 0, 0};
         if (o < f.O && cw < f.Cw) {
             const uint32_t* p = packed + ((static_cast<size_t>(o) * f.RS + tap) * f.Cw + cw) * f.bits;
-            uint32_t w[3] = {p[0], f.bits > 1 ? p[1] : 0u, f.bits > 2 ? p[2] : 0u};
+            uint32_t w[2] = {p[0], f.bits > 1 ? p[1] : 0u};
             if (f.bits == 1) expand_nibbles<1>(w, f.kind, v);
-            else if (f.bits == 2) expand_nibbles<2>(w, f.kind, v);
-            else expand_nibbles<3>(w, f.kind, v);
+            else expand_nibbles<2>(w, f.kind, v);
         }
         if (idx == f.vecs - 1) {
             if (f.last == idx) v[3] = MM_NIBBLE_MARK;
@@ -143,7 +142,7 @@ bool lay_out(const bs_sequence_layer* layers, int n, Layout& l)
         const bs_conv_params& p = layers[i].p;
         if (!layers[i].out_packed || !layers[i].act_packed || p.C % 32 != 0) return false;
         if (p.a_sign != BS_UNSIGNED || p.out_sign != BS_UNSIGNED || p.out_bits > 2 || p.out_bits < 1) return false;
-        if (!mma_nibbles(p.C, p.R * p.S, p.a_bits, p.w_bits, p.w_sign) || p.stride > 2 || p.R != p.S) return false;
+        if (!mma_nibbles(p.C, p.R * p.S, p.a_bits, p.w_bits) || p.stride > 2 || p.R != p.S) return false;
         if (p.residual && (p.res_sign != BS_UNSIGNED || p.res_bits > 2 || !(fabsf(p.res_scale) < 3.9f) || (p.res_scale != 0.0f && fabsf(p.res_scale) <= 1e-18f))) return false;
         const Shape s = shape_of(p);
         const int src = tensor_index(l, layers[i].act_packed, p.N, p.H, p.W, p.C / 32, p.a_bits);

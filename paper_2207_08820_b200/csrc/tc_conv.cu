@@ -197,8 +197,7 @@ extern "C" size_t bs_tc_weights_read_bytes(int O, int C, int R, int S, int w_bit
 {
     const size_t all = bs_tc_weights_bytes(O, C, R, S);
     if (all == 0 || !bs::bits_ok(w_bits, BS_UNSIGNED) || !bs::bits_ok(a_bits, BS_UNSIGNED)) return 0;
-    // (three bits: it depends on the sign of the filters)
-    return w_bits <= 2 && bs::mma_nibbles(C, R * S, a_bits, w_bits, BS_SIGNED) ? all / (C / 32) * ((C / 32 + 1) / 2) : all;
+    return bs::mma_nibbles(C, R * S, a_bits, w_bits) ? all / (C / 32) * ((C / 32 + 1) / 2) : all;
 }
 
 extern "C" int bs_tc_prepare_weights(const uint32_t* wgt_packed, int O, int C, int R, int S, int w_bits, bs_sign_t w_sign,
@@ -209,7 +208,7 @@ extern "C" int bs_tc_prepare_weights(const uint32_t* wgt_packed, int O, int C, i
     if (!bs::aligned16(wgt_packed) || !bs::aligned16(out)) return BS_ERR_ALIGNMENT;
     if (C % 32 != 0) return BS_ERR_UNSUPPORTED;
     const int opad8 = (O + 127) / 128 * 16;
-    const bool nibbles = bs::mma_nibbles(C, R * S, a_bits, w_bits, w_sign);
+    const bool nibbles = bs::mma_nibbles(C, R * S, a_bits, w_bits);
     const long long nvec = static_cast<long long>(nibbles ? (C / 32 + 1) / 2 : C / 32) * opad8 * R * S * 2 * 8;
     const long long blocks = (nvec + 255) / 256;
     if (blocks > 0x7fffffffLL) return BS_ERR_UNSUPPORTED;

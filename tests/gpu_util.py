@@ -3,7 +3,8 @@ through the binding, bring results back as numpy for element-by-element comparis
 import numpy as np
 import torch
 
-from paper_2207_08820_b200 import api
+from paper_2207_08820_b200 import api, workloads as wl
+from paper_2207_08820_b200._lib import ConvParams, SequenceLayer
 
 
 def dev(a: np.ndarray) -> torch.Tensor:
@@ -87,3 +88,25 @@ def gpu_conv(case, want_i32=True, want_packed=True, i32_layout=api.NCHW, residua
     api.bs_check_status()
     guard.check()
     return (acc.cpu().numpy() if acc is not None else None), (words(packed) if packed is not None else None)
+
+
+def layer_array(spec, w_sign=None):
+    """The layers of a stack as ``bs_sequence_layer`` records over addresses that nothing is at: what the host side of the library (planner, workspace
+    size) is asked with, without a device."""
+    sign = wl.weight_sign(spec.w_bits) if w_sign is None else w_sign
+    shapes, at, end = spec.tensor_shapes(), {}, 1 << 20
+    for name, (C, H, W) in shapes.items():
+        at[name] = end
+        end += -(-spec.batch * H * W * -(-C // 32) * spec.a_bits * 4 // 4096) * 4096
+    arr = (SequenceLayer * len(spec.layers))()
+    for q, l in zip(arr, spec.layers):
+        C, H, W = shapes[l.src]
+        prepared = api.tc_supported(spec.batch, l.C, H, W, l.O, l.k, l.stride, l.pad, spec.a_bits, api.UNSIGNED, spec.w_bits, sign)
+        q.act_packed, q.out_packed, q.wgt_packed, q.wgt_tc = at[l.src], at[l.dst], 4096, 8192 if prepared else None
+        q.p = ConvParams(N=spec.batch, C=l.C, H=H, W=W, O=l.O, R=l.k, S=l.k, stride=l.stride, pad=l.pad, a_bits=spec.a_bits, a_sign=api.UNSIGNED, w_bits=spec.w_bits,
+                         w_sign=sign, scale=4096, bias=4096, relu=int(l.relu), out_bits=spec.a_bits, out_sign=api.UNSIGNED, residual=at[l.res] if l.res else None,
+                         res_scale=l.res_scale if l.res else 0.0, res_bits=spec.a_bits if l.res else 0, res_sign=api.UNSIGNED, res_c_offset=0,
+                         res_c_total=shapes[l.res][0] if l.res else l.O, out_c_offset=l.dst_c_offset, out_c_total=shapes[l.dst][0])
+        q.chained = 1
+        q.join[:] = [-1] * 4
+    return arr

@@ -82,3 +82,14 @@ def test_residual_of_three_bits():
                                   out_bits=3, residual=api.bitpack_activations(dev(r), 1.0, 3), res_scale=0.5, res_bits=3)
     assert np.array_equal(api.bitunpack_activations(got, O, 3).cpu().numpy(), oracle.requantize(want, scale, bias, True, 3, 0, r, 0.5))
     api.bs_check_status()
+
+
+@pytest.mark.parametrize("w_sign", [api.SIGNED, api.UNSIGNED])
+def test_prepared_filters_serve_every_width(w_sign):
+    """Three-bit filters are prepared alike for activations of every width, so that no layer converts them."""
+    rng = np.random.default_rng(3)
+    wp = api.pack_weights(dev(wl.rand_codes(rng, (70, 96, 3, 3), 3, w_sign)), 3, w_sign)
+    first = api.tc_prepare_weights(wp, 96, w_sign, 1)
+    for a in (2, 3, 4):
+        assert torch.equal(api.tc_prepare_weights(wp, 96, w_sign, a), first)
+    api.bs_check_status()
