@@ -102,7 +102,7 @@ bool mma_layout(MmaArgs& g, Cand& c, int A, int WB, bool int_rows, int sms)
     const int rel_bytes = g.flat ? 0 : up(g.NI * 4 * (1 + (c.units == 1 ? g.nsp + c.groups : 0)), 16);      // relative rows; located pixels of each group, one table more than stages
     const int pix_bytes = rel_bytes + (fb && !g.tma && c.units == 1 ? up(c.TN * g.RS * 4, 16) : 0);
     const int cap = c.cfg ? 222 * 1024 : 111 * 1024;
-    const int tab = c.TN * (g.f4 && A == 3 ? 12 : 8) + 64;            // scales, biases, residual multipliers, sums of filters
+    const int tab = c.TN * (g.f4 && A == 3 && g.a_kind == 0 ? 12 : 8) + 64;          // scales, biases, residual multipliers, sums of filters
     const int fixed = tab + 320 + red_bytes + (g.tma ? 1024 : 0) + (int_rows ? EW * 4096 : 0) + 256 + pix_bytes;
     const long long filters = c.resident ? static_cast<long long>(g.nblk) * c.TN * g.RS * 32 : 0;
     const long long rest = fixed + static_cast<long long>(g.nsp) * (g.stg_bytes + g.bstg_bytes) + filters;
@@ -367,7 +367,7 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
     else if (grid > items) grid = items;
     const int wb = packed_b ? p->w_bits : 0;
     const bool half = !best.cfg, split = best.split > 1;
-    plan.kern = g.f4 ? (A == 1 ? mma_kernel_f1(wb, half, split) : A == 2 ? mma_kernel_f2(wb, half, split) : mma_kernel_f3(wb, half, split)) : A == 1 ? mma_kernel_a1(wb, half, split) : A == 2 ? mma_kernel_a2(wb, half, split) : A == 3 ? mma_kernel_a3(wb, half, split) : mma_kernel_a4(wb, half, split);
+    plan.kern = g.f4 ? (A == 1 ? mma_kernel_f1(wb, half, split) : A == 2 ? mma_kernel_f2(wb, half, split) : mma_kernel_f3(wb, half, split, offset)) : A == 1 ? mma_kernel_a1(wb, half, split) : A == 2 ? mma_kernel_a2(wb, half, split) : A == 3 ? mma_kernel_a3(wb, half, split) : mma_kernel_a4(wb, half, split);
     plan.grid = static_cast<unsigned>(grid);
     plan.block = best.cfg ? MmaShape<false>::THREADS : MmaShape<true>::THREADS;
     plan.smem = static_cast<int>(best.smem);

@@ -1363,8 +1363,9 @@ struct MmaShape {
     static constexpr int EW = HALF ? 4 : 8, XW = HALF ? 4 : 8, THREADS = (EW + XW + 2) * 32, CPS = HALF ? 2 : 1;
 };
 
-// SPLIT: an item belongs to a cluster of CTAs, each with a share of its chunks.  F4: nibbles (A and WB at most 3).
-template <int A, int WB, bool HALF, bool SPLIT, bool F4>
+// SPLIT: an item belongs to a cluster of CTAs, each with a share of its chunks.  F4: nibbles (A and WB at most 3).  OFS: unsigned activations of three bits
+// on nibbles enter as a - 4, the filters (packed, resident) give their sums.
+template <int A, int WB, bool HALF, bool SPLIT, bool F4, bool OFS>
 __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) bitserial_mma_kernel(const __grid_constant__ MmaArgs g)
 {
     extern __shared__ __align__(1024) unsigned char mm_smem[];
@@ -1388,7 +1389,6 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
 
     constexpr bool packed_b = WB > 0;
     constexpr int WBX = WB > 0 ? WB : 1;
-    constexpr bool OFS = F4 && A == 3;              // unsigned activations enter as a - 4
     int* sums_i = reinterpret_cast<int*>(mm_smem + g.off_tab + g.TN * 8 + 64);
     const bool resident = g.nsb == 0;
     const bool stream_prepared = !resident && !packed_b;      // a stage then holds expanded pixels and the filters of the same chunk
@@ -1858,10 +1858,10 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
         e.smem = mm_smem; e.full_acc = full_acc; e.empty_acc = empty_acc; e.fast_ok = fast_ok;
         e.acc = tmem + lane_addr; e.row0 = quad * 32 + lane; e.set = set;
         e.tid = tid; e.lane = lane; e.warp = warp; e.red_full = red_full;
-        // what the epilogue adds to the accumulators of a filter: four times the sum of its codes (only plans with resident filters take unsigned codes)
+        // what the epilogue adds to the accumulators of a filter: four times the sum of its codes
         auto sums = [&]() {
             if constexpr (OFS)
-                for (int c = tid; c < g.TN; c += NET) reinterpret_cast<float*>(sums_i)[c] = g.a_kind != 0 ? 0.0f : 4.0f * static_cast<float>(sums_i[c]);
+                for (int c = tid; c < g.TN; c += NET) reinterpret_cast<float*>(sums_i)[c] = 4.0f * static_cast<float>(sums_i[c]);
         };
         bool ok;
         if (SPLIT && range.rank > 0) ok = send_partials<EW, F4>(g, e, range.rank);
@@ -1887,20 +1887,24 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
 typedef void (*MmaKernel)(MmaArgs);
 
 // The instantiations for A activation bits, a translation unit each (mma_inst_a*.cu; nibbles: mma_inst_f*.cu): filters prepared (wb = 0)
-// or packed in wb bits, half an SM or a whole one per CTA, a whole one with the item split over a cluster.
+// or packed in wb bits, half an SM or a whole one per CTA, a whole one with the item split over a cluster; offset: unsigned activations of three bits.
 MmaKernel mma_kernel_a1(int wb, bool half, bool split);
 MmaKernel mma_kernel_a2(int wb, bool half, bool split);
 MmaKernel mma_kernel_a3(int wb, bool half, bool split);
 MmaKernel mma_kernel_a4(int wb, bool half, bool split);
 MmaKernel mma_kernel_f1(int wb, bool half, bool split);
 MmaKernel mma_kernel_f2(int wb, bool half, bool split);
-MmaKernel mma_kernel_f3(int wb, bool half, bool split);
+MmaKernel mma_kernel_f3(int wb, bool half, bool split, bool offset);
 
 template <int A, int WB, bool F4>
 MmaKernel mma_pick_shape(bool half, bool split)
 {
-    return split ? bitserial_mma_kernel<A, WB, false, true, F4> : half ? bitserial_mma_kernel<A, WB, true, false, F4> : bitserial_mma_kernel<A, WB, false, false, F4>;
+    return split ? bitserial_mma_kernel<A, WB, false, true, F4, false> : half ? bitserial_mma_kernel<A, WB, true, false, F4, false>
+                                                                              : bitserial_mma_kernel<A, WB, false, false, F4, false>;
 }
+// (resident filters are not split)
+template <int WB>
+MmaKernel mma_pick_offset(bool half) { return half ? bitserial_mma_kernel<3, WB, true, false, true, true> : bitserial_mma_kernel<3, WB, false, false, true, true>; }
 template <int A>
 MmaKernel mma_pick(int wb, bool half, bool split)
 {
