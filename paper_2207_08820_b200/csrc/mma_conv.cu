@@ -273,7 +273,14 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
     const bool pixel_rows = out_i32 && !out_packed && !g.i32_nhwc;
     g.f4 = (packed_b ? mma_nibbles_packed(p->C, g.RS, p->a_bits, p->w_bits, p->w_sign) : mma_nibbles(p->C, g.RS, p->a_bits, p->w_bits)) &&
            !(packed_b && (pixel_rows ? short_k || (g.R == 1 && g.Cw <= 6) : short_k && g.R >= 5 && !out_i32));
-    // Unsigned activations of three bits need the filters' sums, which only resident filters give: such plans on nibbles against all on int8, by their time.
+    // Unsigned activations of three bits need the filters' sums, which only resident filters give: such plans on nibbles against all on int8, by their
+    // modelled time, with 6 % for int8.  Of 135 layers with larger windows, timed on both forms, 6 go to nibbles, which take 0.36 to 0.83 of int8's time.
+    // Without the 6 % 14 would, the others 0.67 to 0.92, but of 90 more layers one then loses (59 x 37 x 68 x 68, 448 filters, stride 2: 50.7 -> 55.0 us),
+    // and with 11 % for nibbles 39 would, four of them slower.  1x1 stays on int8: what the 6 % leave of 169 products and layers takes 0.82 to 1.19
+    // of int8's time (111 x 3428 x 2688: 11.7 -> 14.0 us; 7 x 239 x 88 x 88, 64 filters: 7.6 -> 8.4), and the model does not tell them apart.
+    // Signed ones are nibbles: 0.92 of int8's time over 103 products and 1x1 layers (at most 1.02), 0.88 over 348 layers with larger windows, of which 12
+    // lose more than 2 %, 12 at most, and the model does not tell them from the others.
+    if (A == 3 && p->a_sign == BS_UNSIGNED && g.R == 1) g.f4 = 0;
     const bool offset = g.f4 && A == 3 && p->a_sign == BS_UNSIGNED;
     const double bound = static_cast<double>(p->C) * g.RS * max_abs_of(p->a_bits, p->a_sign) * max_abs_of(p->w_bits, p->w_sign);
     g.acc_bound = static_cast<float>(bound);
@@ -299,8 +306,6 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
         if (!mma_layout(t, c, A, packed_b ? p->w_bits : 0, int_rows, sms)) return;
         c.cost = mma_cost(t, c, A, packed_b ? p->w_bits : 0, out_packed, sms);
         c.f4 = g.f4;
-        // (the model takes nibbles of three bits for about 5 % faster than they are: 1024 x 1024 x 2304 modelled 0.99 of int8, timed 1.05; the layer of
-        // 32 x 256 x 28 x 28 and 256 filters 0.90 and 0.75)
         if (offset && g.f4) c.cost *= 1.06;
         if (c.cost < best.cost) { best = c; found = true; }
     };
