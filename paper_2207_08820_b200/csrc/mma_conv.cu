@@ -278,10 +278,13 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
     // Without the 6 % 14 would, the others 0.67 to 0.92, but of 90 more layers one then loses (59 x 37 x 68 x 68, 448 filters, stride 2: 50.7 -> 55.0 us),
     // and with 11 % for nibbles 39 would, four of them slower.  1x1 stays on int8: what the 6 % leave of 169 products and layers takes 0.82 to 1.19
     // of int8's time (111 x 3428 x 2688: 11.7 -> 14.0 us; 7 x 239 x 88 x 88, 64 filters: 7.6 -> 8.4), and the model does not tell them apart.
-    // Signed ones are nibbles: 0.92 of int8's time over 103 products and 1x1 layers (at most 1.02), 0.88 over 348 layers with larger windows, of which 12
-    // lose more than 2 %, 12 at most, and the model does not tell them from the others.
     if (A == 3 && p->a_sign == BS_UNSIGNED && g.R == 1) g.f4 = 0;
     const bool offset = g.f4 && A == 3 && p->a_sign == BS_UNSIGNED;
+    // Signed activations of three bits, filters of three bits under narrower ones: nibbles for larger windows, which take 0.88 of int8's time over 348
+    // layers of the former, 0.89 over 177 of the latter, and up to 1.2 in one of 25, which the model does not tell from the others.  1x1: both forms
+    // by their modelled time, with 10 % for nibbles.  316 calls timed on both: 0.93 of int8's time; on nibbles alone 7 lose more than 3 %, large products a
+    // quarter (2049 x 2620 x 4182: 92.6 -> 117.7 us); without the 10 % 55 lose more than 3 % against nibbles, with them 16, at most 12 %.
+    const bool either = g.f4 && g.R == 1 && (A == 3 || p->w_bits == 3);
     const double bound = static_cast<double>(p->C) * g.RS * max_abs_of(p->a_bits, p->a_sign) * max_abs_of(p->w_bits, p->w_sign);
     g.acc_bound = static_cast<float>(bound);
     g.preset = out_packed && !out_i32 && bound < 4.0e6 && p->out_sign != BS_BIPOLAR &&
@@ -306,7 +309,7 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
         if (!mma_layout(t, c, A, packed_b ? p->w_bits : 0, int_rows, sms)) return;
         c.cost = mma_cost(t, c, A, packed_b ? p->w_bits : 0, out_packed, sms);
         c.f4 = g.f4;
-        if (offset && g.f4) c.cost *= 1.06;
+        if (g.f4) c.cost *= offset ? 1.06 : either ? 0.9 : 1.0;
         if (c.cost < best.cost) { best = c; found = true; }
     };
     int ns_list[12], nns = 0;
@@ -322,7 +325,7 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
     int ov[8] = {0, 0, 0, -1, 0, -1, 0, 0};    // TN, PT, units, config, strips, resident, groups, split; 0 / -1: free
     if (const char* e = getenv("BS_MM")) sscanf(e, "%d,%d,%d,%d,%d,%d,%d,%d", ov, ov + 1, ov + 2, ov + 3, ov + 4, ov + 5, ov + 6, ov + 7);
 #endif
-    for (int form = 0; form < (offset ? 2 : 1); ++form, g.f4 = 0)
+    for (int form = 0; form < (offset || either ? 2 : 1); ++form, g.f4 = 0)
     for (int TN = 32; TN <= 256; TN *= 2) {
         if (TN > 32 && TN / 2 >= up(p->O, 32)) continue;
         if (TN == 256 && !packed_b && g.opad % 256 != 0) continue;
