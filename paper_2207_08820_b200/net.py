@@ -140,7 +140,8 @@ class BitserialNet:
         return units
 
     def _run(self, x: torch.Tensor) -> torch.Tensor:
-        self.run_layers(self.pack_input(x, operands=True))
+        bound = self._bind()
+        self._layers(self._pack(x, self._sequence.input if bound else None), bound)
         return self.bufs[self.net.out_name]
 
     def input_operands(self) -> Optional[int]:
@@ -150,13 +151,15 @@ class BitserialNet:
     def pack_input(self, x: torch.Tensor, operands: bool = False) -> Optional[int]:
         """Quantise + bitplane-pack the fp32 input on the current stream.  operands: its operand tensor too, where the layers have one and ``x`` is
         the whole input; :meth:`run_layers` takes what is returned then, as long as neither is written in between."""
+        return self._pack(x, self.input_operands() if operands else None)
+
+    def _pack(self, x: torch.Tensor, operands: Optional[int]) -> Optional[int]:
         net, buf = self.net, self.bufs[self.net.in_name]
-        ready = self.input_operands() if operands and x.dtype == torch.float32 and tuple(x.shape) == (self.batch, *net.in_shape) else None
-        if ready is not None:
-            api.bitpack_operands(x, self.act_scale, net.a_bits, buf, ready)
-        else:
-            api.bitpack_activations(x, self.act_scale, net.a_bits, api.UNSIGNED, api.NCHW, out=buf.view(-1))
-        return ready
+        if operands is not None and x.dtype == torch.float32 and tuple(x.shape) == (self.batch, *net.in_shape):
+            api.bitpack_operands(x, self.act_scale, net.a_bits, buf, operands)
+            return operands
+        api.bitpack_activations(x, self.act_scale, net.a_bits, api.UNSIGNED, api.NCHW, out=buf.view(-1))
+        return None
 
     def run_layer(self, item, chained: bool = True) -> None:
         """One conv layer through the C ABI on the current stream."""
@@ -226,7 +229,11 @@ class BitserialNet:
     def run_layers(self, ready: Optional[int] = None) -> None:
         """All layers on the current stream, and on the side stream those that :meth:`schedule` puts there; under stream capture the
         events between them become the edges of the graph.  ready: the operand tensor of the input, where it holds what the packed input holds."""
-        if self._bind():
+        self._layers(ready, self._bind())
+
+    def _layers(self, ready: Optional[int], bound: bool) -> None:
+        """:meth:`run_layers` behind a look at the tensors: a pass takes one, in front of what writes its input."""
+        if bound:
             q = self._sequence
             ready = ready if ready == q.input else None
             api.run_sequence(q.handle, q.launches - (ready is not None), ready=ready)
@@ -425,7 +432,7 @@ class BitserialFullNet:
             return ready
         self._stem_layers(images)
         self._note_pass(None)
-        return body.pack_input(self._stem["pool"], operands=ready is not None)
+        return body._pack(self._stem["pool"], ready)
 
     def _stem_layers(self, images: torch.Tensor) -> None:
         conv, pool = self._stem_tensor("conv"), self._stem_tensor("pool")
@@ -526,7 +533,9 @@ class BitserialFullNet:
 
     def forward(self, images: torch.Tensor) -> torch.Tensor:
         """images: float32 [batch, 3, hw, hw] on the device.  Returns the logits [batch, classes]."""
-        self.body.run_layers(self._front(images, self.body.input_operands()))
+        body = self.body
+        bound = body._bind()
+        body._layers(self._front(images, body._sequence.input if bound else None), bound)
         self.run_head()
         self._join_note()
         return self.logits

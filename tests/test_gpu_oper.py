@@ -8,7 +8,7 @@ import torch
 
 from oracle import network as onet
 from paper_2207_08820_b200 import api, workloads as wl
-from paper_2207_08820_b200.net import BitserialNet
+from paper_2207_08820_b200.net import BitserialFullNet, BitserialNet
 from paper_2207_08820_b200.workloads import ConvSpec, NetSpec
 from gpu_util import dev
 
@@ -227,4 +227,26 @@ def test_recorded_passes_keep_their_workspace():
         bufs[spec.out_name].fill_(-1)
         graph.replay()
         assert torch.equal(bufs[spec.out_name], want)
+    api.bs_check_status()
+
+
+@pytest.mark.parametrize("whole", [False, True])
+def test_a_pass_looks_at_its_tensors_once(whole, monkeypatch):
+    """Whether an entry was replaced costs host time, which passes of few images are made of."""
+    if whole:
+        spec = wl.resnet18_full(2, 64)
+        params = wl.full_network_params(spec, 5)
+        r, x = BitserialFullNet(spec, params, batch=2), torch.randn(2, 3, 64, 64, device="cuda")
+        body = r.body
+    else:
+        r, _, x = runner_of(STACKS["both_strides"])
+        x, body = dev(x), r
+    r.forward(x)
+    looks = []
+    monkeypatch.setattr(type(body._sequence), "current", lambda self, *a, current=type(body._sequence).current: looks.append(1) or current(self, *a))
+    want = r.forward(x).clone()
+    assert len(looks) == 1
+    for k in body.bufs:
+        body.bufs[k] = torch.empty_like(body.bufs[k])
+    assert torch.equal(r.forward(x), want) and len(looks) == 2
     api.bs_check_status()
