@@ -314,6 +314,8 @@ int bs_sequence_create(const bs_sequence_layer* layers, int nlayers, void* side_
  *                         less than that: as bs_sequence_create.  May pass on to another sequence of layers of the same shapes, formats and order.
  * bs_sequence_workspace_bytes answers 0 where the layers don't take one: too many layers without prepared filters, codes of more than two bits or signed ones,
  * tensors that overlap or that are used with two shapes, rows too wide for the shared memory.  It needs no device.
+ * bs_sequence_layer_plan  how layer `layer` runs on operand tensors; BS_ERR_UNSUPPORTED where bs_sequence_workspace_bytes is 0.  Needs no device either:
+ *                       without one it answers for 148 multiprocessors.
  * bs_sequence_launches: kernels that bs_sequence_run enqueues.
  * bs_sequence_input     the operand tensor of a tensor of packed codes that the layers read before they have written all of it (it belongs to the
  *                       sequence), NULL where there is none.  bitpack_activations_operands (fp32 NCHW, unsigned codes) and
@@ -324,6 +326,15 @@ int bs_sequence_create(const bs_sequence_layer* layers, int nlayers, void* side_
 size_t bs_sequence_workspace_bytes(const bs_sequence_layer* layers, int nlayers);
 int bs_sequence_create_ws(const bs_sequence_layer* layers, int nlayers, void* side_stream, void* workspace, size_t workspace_bytes,
                           bs_sequence** sequence_out);
+typedef struct {
+    int filters, row_tiles;     /* of a work item: filters, tiles of 128 positions */
+    int channels;               /* 64-channel steps that a stage holds */
+    int resident;               /* filters stay in shared memory; else they come with the pixels */
+    int stages, accumulators;   /* buffers of pixels, of sums */
+    int teams;                  /* 2: a block has a multiprocessor to itself and two teams of epilogue warps */
+    int blocks, items;          /* thread blocks; work items of the one that has most */
+} bs_layer_plan;
+int bs_sequence_layer_plan(const bs_sequence_layer* layers, int nlayers, int layer, bs_layer_plan* plan_out);
 int bs_sequence_launches(const bs_sequence* sequence);
 typedef struct bs_operand_tensor bs_operand_tensor;
 const bs_operand_tensor* bs_sequence_input(const bs_sequence* sequence, const uint32_t* packed);

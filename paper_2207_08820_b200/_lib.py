@@ -42,6 +42,11 @@ class SequenceLayer(ctypes.Structure):
                 ("p", ConvParams), ("chained", ctypes.c_int), ("aside", ctypes.c_int), ("join", ctypes.c_int * 4)]
 
 
+class LayerPlan(ctypes.Structure):
+    """Mirror of ``bs_layer_plan`` (include/bitserial.h)."""
+    _fields_ = [(f, ctypes.c_int) for f in ("filters", "row_tiles", "channels", "resident", "stages", "accumulators", "teams", "blocks", "items")]
+
+
 def native():
     """The compiled binding (csrc/binding.cpp), linked against the library beside it."""
     global _native
@@ -124,6 +129,8 @@ def lib() -> ctypes.CDLL:
     L.bs_sequence_workspace_bytes.argtypes = [ctypes.POINTER(SequenceLayer), i]
     L.bs_sequence_create_ws.restype = i
     L.bs_sequence_create_ws.argtypes = [ctypes.POINTER(SequenceLayer), i, vp, vp, ctypes.c_size_t, ctypes.POINTER(vp)]
+    L.bs_sequence_layer_plan.restype = i
+    L.bs_sequence_layer_plan.argtypes = [ctypes.POINTER(SequenceLayer), i, i, ctypes.POINTER(LayerPlan)]
     L.bs_sequence_launches.restype = i
     L.bs_sequence_launches.argtypes = [vp]
     L.bs_sequence_input.restype = vp
@@ -172,6 +179,6 @@ EXPORTED = ("bs_packed_act_bytes", "bs_packed_wgt_bytes", "bs_packed_rows_bytes"
             "bitunpack_activations", "pack_weights", "bs_pack_rows", "bitserial_conv2d", "bitserial_gemm",
             "bitserial_conv2d_ws", "bitserial_gemm_ws", "bs_conv_workspace_bytes", "bs_gemm_workspace_bytes",
             "bitserial_gemm_noalloc", "bs_gemm_noalloc_max_scratch_bytes", "bs_selftest_dirty_noalloc_scratch",
-            "bs_tc_weights_bytes", "bs_tc_weights_read_bytes", "bs_tc_prepare_weights", "bs_tc_supported", "bitserial_conv2d_tc", "bitserial_conv2d_tc_chained", "bs_tc_chain_workspace_bytes", "bitserial_conv2d_tc_chain", "bitserial_gemm_tc", "bs_sequence_create", "bs_sequence_create_ws", "bs_sequence_workspace_bytes", "bs_sequence_launches", "bs_sequence_input", "bs_sequence_run_ready", "bitpack_activations_operands", "bs_stem_codes_operands_f32", "bs_sequence_run", "bs_sequence_destroy", "bs_l2_prefetch",
+            "bs_tc_weights_bytes", "bs_tc_weights_read_bytes", "bs_tc_prepare_weights", "bs_tc_supported", "bitserial_conv2d_tc", "bitserial_conv2d_tc_chained", "bs_tc_chain_workspace_bytes", "bitserial_conv2d_tc_chain", "bitserial_gemm_tc", "bs_sequence_create", "bs_sequence_create_ws", "bs_sequence_workspace_bytes", "bs_sequence_launches", "bs_sequence_layer_plan", "bs_sequence_input", "bs_sequence_run_ready", "bitpack_activations_operands", "bs_stem_codes_operands_f32", "bs_sequence_run", "bs_sequence_destroy", "bs_l2_prefetch",
             "bs_conv2d_f32", "bs_maxpool2d_f32", "bs_stem_codes_f32", "bs_stem_codes_supported", "bs_avgpool_codes_f32", "bs_fc_f32",
             "bs_check_status", "bs_quantiser_bounds", "bs_requant_bounds", "bs_selftest_wait_timeout", "bs_popc_rate", "bs_status_string")

@@ -429,6 +429,16 @@ size_t oper_workspace_bytes(const bs_sequence_layer* layers, int n)
     return build(layers, n, nullptr, q, bytes) ? bytes : 0;
 }
 
+int oper_layer_plan(const bs_sequence_layer* layers, int n, int i, bs_layer_plan* out)
+{
+    OperSequence q;
+    size_t bytes = 0;
+    if (!build(layers, n, nullptr, q, bytes)) return BS_ERR_UNSUPPORTED;
+    const OperSequence::Step& s = q.steps[static_cast<size_t>(i)];
+    *out = {s.g.TN, s.g.PT, s.g.units, s.g.resident, s.g.nse, s.g.nacc, s.full ? 2 : 1, static_cast<int>(s.grid), ceil_div(s.g.tiles_m, s.g.step_m)};
+    return BS_OK;
+}
+
 OperSequence* oper_create(const bs_sequence_layer* layers, int n, void* workspace, size_t bytes)
 {
     OperSequence* q = new (std::nothrow) OperSequence;

@@ -11,6 +11,8 @@ struct OperTensor;
 
 // Bytes of zeroed device memory that the layers need to run on operand tensors; 0: they don't take them (mma_conv.cu runs them).
 size_t oper_workspace_bytes(const bs_sequence_layer* layers, int n);
+// How layer i runs then; BS_ERR_UNSUPPORTED where they don't.
+int oper_layer_plan(const bs_sequence_layer* layers, int n, int i, bs_layer_plan* out);
 // The launches of such layers; null where oper_workspace_bytes is 0 or bytes is less.
 OperSequence* oper_create(const bs_sequence_layer* layers, int n, void* workspace, size_t bytes);
 // Launches in front of the layers: filters to prepare, forms of tensors that the layers read from their packed codes; those of one tensor, or null.

@@ -282,6 +282,13 @@ extern "C" size_t bs_sequence_workspace_bytes(const bs_sequence_layer* layers, i
     return bs_sequence_check(layers, nlayers) == BS_OK ? bs::oper_workspace_bytes(layers, nlayers) : 0;
 }
 
+extern "C" int bs_sequence_layer_plan(const bs_sequence_layer* layers, int nlayers, int layer, bs_layer_plan* out)
+{
+    if (!out || layer < 0 || layer >= nlayers) return BS_ERR_INVALID_ARG;
+    const int rc = bs_sequence_check(layers, nlayers);
+    return rc == BS_OK ? bs::oper_layer_plan(layers, nlayers, layer, out) : rc;
+}
+
 extern "C" int bs_sequence_create_ws(const bs_sequence_layer* layers, int nlayers, void* side_stream, void* workspace, size_t workspace_bytes, bs_sequence** out)
 {
     if (!out) return BS_ERR_INVALID_ARG;

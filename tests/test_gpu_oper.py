@@ -1,7 +1,9 @@
 """Layers of a bound sequence on operand tensors: every packed tensor of a pass equals, bit for bit, what the same layers write one call at a time
 (whose kernels read packed codes), and the oracle where that is quick.  Geometries at the edges of the position numbering: one channel
 group and odd numbers of them, readers of both strides of one tensor, windows without padding and of 5 and 7, concatenations, tensors that
-a pass only reads in part from its own layers, rows and images of one pixel."""
+a pass only reads in part from its own layers, rows and images of one pixel.  All of them with few images, whose plans are the simplest, and with many."""
+from dataclasses import replace
+
 import numpy as np
 import pytest
 import torch
@@ -42,6 +44,12 @@ STACKS = {
 }
 
 
+# The same geometries with so many images that the plans are those of large batches: tiles of 64 and 128 filters, pairs of row tiles and four of them,
+# several items a block, one to four accumulators, streamed filters, two teams (tests/test_host_sequence.py asserts that each is met).
+MANY = {name: replace(STACKS[name], batch=batch) for name, batch in dict(one_group=3000, odd_groups=1500, both_strides=1500, concatenation=900, one_bit=2000,
+                                                                        wide=300, deep=400, odd_records=1500, odd_one_bit=1500, pixels=100000).items()}
+
+
 def runner_of(spec, seed=11):
     params = wl.network_params(spec, seed)
     r = BitserialNet(spec, params, 0.25, batch=spec.batch, engine="tc")
@@ -49,12 +57,15 @@ def runner_of(spec, seed=11):
 
 
 def both(r, x):
-    """Every packed tensor after a pass and after the same layers called one by one."""
-    xd, out = dev(x), []
+    """Every packed tensor after a pass and after the same layers called one by one.  x: float input, or the packed one."""
+    xd, out = dev(x) if isinstance(x, np.ndarray) else x, []
     for one_by_one in (False, True):
         for b in r.bufs.values():
             b.fill_(-1 if one_by_one else 0x5A5A5A5A)
-        r.pack_input(xd)
+        if xd.dtype == torch.int32:
+            r.bufs[r.net.in_name].copy_(xd)
+        else:
+            r.pack_input(xd)
         r.run_units() if one_by_one else r.run_layers()
         api.bs_check_status()
         out.append({k: b.clone() for k, b in r.bufs.items()})
@@ -76,6 +87,40 @@ def test_stacks(name):
     ref = onet.run_stack(spec, params, x, 0.25)
     for k in ref:
         assert np.array_equal(r.unpacked(k).cpu().numpy(), ref[k]), k
+
+
+def packed_input(r, seed):
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    return torch.randint(-2**31, 2**31, r.bufs[r.net.in_name].shape, generator=gen, device="cuda").to(torch.int32)      # (whole channel words)
+
+
+@pytest.mark.parametrize("name", MANY)
+def test_many_images(name):
+    spec = MANY[name]
+    r = BitserialNet(spec, wl.network_params(spec, 13), 0.25, batch=spec.batch, engine="tc")
+    assert r._sequence.launches > len(spec.layers)
+    for seed in (0, 1):
+        got, want = both(r, packed_input(r, seed))
+        for k in want:
+            assert torch.equal(got[k], want[k]), k
+
+
+@pytest.mark.parametrize("name", ["one_group", "odd_groups", "both_strides", "concatenation", "deep", "pixels"])
+def test_many_images_by_the_slow_ways(name):
+    """Filters of the other form, resident and streamed, and scales that only the formula takes, with every plan of large batches."""
+    spec = MANY[name]
+    r = BitserialNet(spec, wl.network_params(spec, 14), 0.25, batch=spec.batch, engine="tc")
+    for step in (0, 1):
+        for item in r.layers:
+            if step == 0:
+                item["w_tc"] = api.tc_prepare_weights(item["w"], item["spec"].C, item["w_sign"], 4)
+            else:
+                item["scale"] = item["scale"].clone()
+                item["scale"][-1] = 1e-19
+        got, want = both(r, packed_input(r, step))
+        assert r._sequence.launches > len(spec.layers)
+        for k in want:
+            assert torch.equal(got[k], want[k]), k
 
 
 @pytest.mark.parametrize("name", ["one_group", "both_strides", "one_bit"])
