@@ -56,12 +56,16 @@ class BitserialNet:
     MAX_WORKSPACES = 4      # arrangements of tensors that have memory for operand tensors; passes over further ones run on packed codes
 
     def __init__(self, net: NetSpec, params: Dict[str, Dict], act_scale: float, device="cuda", batch: Optional[int] = None,
-                 engine: str = "popc", concurrent: bool = True, chains="auto"):
+                 engine: str = "popc", concurrent: bool = True, chains="auto", operand_tensors: bool = True):
         """engine: "popc" = packed filters, expanded on chip; "tc" = filters prepared as operand tiles once for every layer that
         supports it (others keep packed filters).  concurrent: launch independent neighbouring layers on
         two streams (see :meth:`schedule`).  chains: True groups, with the "tc" engine, runs of consecutive same-shaped layers that the
         library accepts into units which :meth:`run_units` issues as one ``bitserial_conv2d_tc_chain`` call each; False and "auto" = a unit per
-        layer.  A pass is one call of a bound sequence whatever the units are."""
+        layer.  A pass is one call of a bound sequence whatever the units are.
+        operand_tensors: with filters prepared as nibbles a pass keeps what the tensor cores read of every tensor between its layers in device memory of
+        its own (``bs_sequence_create_ws``), about twice the packed tensors together: 59 MB for the 18-layer stack at 64 images, 139 MB for
+        the detection stack at 16, 169 MB for the 50-layer one at 32, held while the runner lives (:attr:`operand_bytes`), once more for every
+        set of tensors that a graph was recorded with.  False: no such memory, layers expand packed codes, 1.2 to 1.5 times the time."""
         self.net = net
         self.engine = engine
         self.act_scale = float(act_scale)
@@ -94,6 +98,7 @@ class BitserialNet:
         self.graph = None
         self.static_in = None
         self.launches_per_forward = 1 + len(self.layers)
+        self.operand_tensors = operand_tensors
         self._workspaces: List[_Workspace] = []
         self._sequence: Optional[_Sequence] = None
         self._captured: Optional[_Sequence] = None      # what the graph was captured from
@@ -143,6 +148,11 @@ class BitserialNet:
         bound = self._bind()
         self._layers(self._pack(x, self._sequence.input if bound else None), bound)
         return self.bufs[self.net.out_name]
+
+    @property
+    def operand_bytes(self) -> int:
+        """Device memory of the operand tensors (see the constructor)."""
+        return sum(w.memory.numel() for w in self._workspaces)
 
     def input_operands(self) -> Optional[int]:
         """The operand tensor of the packed input (``bs_sequence_input``), which a producer of the input may write as well, or None."""
@@ -301,7 +311,7 @@ class BitserialNet:
     def _workspace(self, arr, recording: bool) -> Optional[_Workspace]:
         """Memory of the layers' operand tensors (``bs_sequence_create_ws``), or None.  What a graph was recorded with stays with its tensors while the
         runner lives; otherwise it passes on to the next arrangement of the same geometry, whose passes begin on an idle device."""
-        nbytes = lib().bs_sequence_workspace_bytes(arr, len(arr))
+        nbytes = lib().bs_sequence_workspace_bytes(arr, len(arr)) if self.operand_tensors else 0
         if nbytes == 0:
             return None
         tensors = {}
@@ -382,11 +392,11 @@ class BitserialFullNet:
 
     MAX_CAPTURES = 16       # recorded passes whose images are kept for :attr:`stem_conv`
 
-    def __init__(self, net, params: Dict[str, Dict], device="cuda", batch: Optional[int] = None, engine: str = "tc"):
+    def __init__(self, net, params: Dict[str, Dict], device="cuda", batch: Optional[int] = None, engine: str = "tc", operand_tensors: bool = True):
         self.net = net
         self.batch = batch or net.batch
         self.device = torch.device(device)
-        self.body = BitserialNet(net.body, params, net.stem_act_scale, device=device, batch=self.batch, engine=engine)
+        self.body = BitserialNet(net.body, params, net.stem_act_scale, device=device, batch=self.batch, engine=engine, operand_tensors=operand_tensors)
         to = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(self.device)
         self.stem_w, self.stem_b = to(params["stem"]["w"]), to(params["stem"]["bias"])
         self.fc_w, self.fc_b = to(params["fc"]["w"]), to(params["fc"]["bias"])

@@ -295,3 +295,13 @@ def test_a_pass_looks_at_its_tensors_once(whole, monkeypatch):
         body.bufs[k] = torch.empty_like(body.bufs[k])
     assert torch.equal(r.forward(x), want) and len(looks) == 2
     api.bs_check_status()
+
+
+def test_operand_tensors_can_be_declined():
+    spec = STACKS["both_strides"]
+    r, params, x = runner_of(spec)
+    plain, xd = BitserialNet(spec, params, 0.25, batch=spec.batch, engine="tc", operand_tensors=False), dev(x)
+    assert r.operand_bytes == r._sequence.workspace.memory.numel() > 0 and plain.operand_bytes == 0
+    assert plain._sequence.launches == len(spec.layers) and plain.input_operands() is None
+    assert torch.equal(r.forward(xd), plain.forward(xd))
+    api.bs_check_status()
