@@ -27,6 +27,34 @@ constexpr bool mma_nibbles_packed(int C, int RS, int a_bits, int w_bits, int w_s
 // A layer tells the form of its filters by it and converts them where it needs the other one.
 constexpr unsigned MM_NIBBLE_MARK = 0x88888888u;
 
+#ifdef __CUDACC__
+// What vector idx of prepared filters holds, [step][groups of eight filters][taps][2][8 filters][16 bytes]: nibbles of channel word 2 step + half, or 16 int8
+// codes of channel word `step`.
+struct FilterVector { int o, tap, half, step; };
+template <class I>
+__device__ __forceinline__ FilterVector filter_vector(I idx, int groups, int RS)
+{
+    FilterVector f;
+    I t = idx / 16;
+    f.half = static_cast<int>(idx / 8 % 2);
+    f.tap = static_cast<int>(t % RS);       t /= RS;
+    const int col = static_cast<int>(t % groups) * 8 + static_cast<int>(idx % 8);
+    f.step = static_cast<int>(t / groups);
+    f.o = (col & ~31) + mma_filter_of_column(col & 31);
+    return f;
+}
+// Vector idx of n vectors of nibbles; the mark ends the tensor, in vector `last`: this one (of channels that do not exist) or one that no layer reads.
+template <class I>
+__device__ __forceinline__ void put_nibbles(uint4* out, I idx, I n, long long last, uint4 v)
+{
+    if (idx == n - 1) {
+        if (last == idx) v.w = MM_NIBBLE_MARK;
+        else out[last] = make_uint4(0, 0, 0, MM_NIBBLE_MARK);
+    }
+    out[idx] = v;
+}
+#endif
+
 // Runs one layer.  `wgt` are filters prepared by bs_tc_prepare_weights; when it is null the packed filters `wgt_packed` are
 // expanded inside the kernel.  chained: the caller promises that filters, scale and bias were final before the preceding
 // kernel of the stream was launched.  plan_only: validate and plan, launch nothing.

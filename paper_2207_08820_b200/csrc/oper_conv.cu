@@ -53,22 +53,16 @@ static __global__ void __launch_bounds__(256) oper_filters_kernel(const __grid_c
     const FilterSet::Layer& f = set.layer[blockIdx.y];
     const uint32_t* packed = dependent_begin(f.packed);
     for (int idx = blockIdx.x * 256 + threadIdx.x; idx < f.vecs; idx += gridDim.x * 256) {
-        int t = idx >> 4;
-        const int half = idx >> 3 & 1, tap = t % f.RS;
-        t /= f.RS;
-        const int og = t % f.groups, cw = t / f.groups * 2 + half, col = og * 8 + (idx & 7), o = (col & ~31) + mma_filter_of_column(col & 31);
+        const FilterVector at = filter_vector(static_cast<unsigned>(idx), f.groups, f.RS);
+        const int cw = at.step * 2 + at.half;
         uint32_t v[4] = {0, 0, 0, 0};
-        if (o < f.O && cw < f.Cw) {
-            const uint32_t* p = packed + ((static_cast<size_t>(o) * f.RS + tap) * f.Cw + cw) * f.bits;
+        if (at.o < f.O && cw < f.Cw) {
+            const uint32_t* p = packed + ((static_cast<size_t>(at.o) * f.RS + at.tap) * f.Cw + cw) * f.bits;
             uint32_t w[2] = {p[0], f.bits > 1 ? p[1] : 0u};
             if (f.bits == 1) expand_nibbles<1>(w, f.kind, v);
             else expand_nibbles<2>(w, f.kind, v);
         }
-        if (idx == f.vecs - 1) {
-            if (f.last == idx) v[3] = MM_NIBBLE_MARK;
-            else f.out[f.last] = make_uint4(0, 0, 0, MM_NIBBLE_MARK);
-        }
-        f.out[idx] = make_uint4(v[0], v[1], v[2], v[3]);
+        put_nibbles(f.out, idx, f.vecs, f.last, make_uint4(v[0], v[1], v[2], v[3]));
     }
 }
 

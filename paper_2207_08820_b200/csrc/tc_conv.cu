@@ -13,14 +13,8 @@ __global__ void tc_prepare_weights_kernel(const uint32_t* __restrict__ packed, i
 {
     const long long idx = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (idx >= nvec) return;
-    long long t = idx;
-    const int row = static_cast<int>(t % 8);        t /= 8;
-    const int half = static_cast<int>(t % 2);       t /= 2;
-    const int tap = static_cast<int>(t % RS);       t /= RS;
-    const int og = static_cast<int>(t % opad8);     t /= opad8;
-    const int blk = static_cast<int>(t);
-    const int col = og * 8 + row;
-    const int o = (col & ~31) + mma_filter_of_column(col & 31);
+    const FilterVector f = filter_vector(idx, opad8, RS);
+    const int o = f.o, tap = f.tap, half = f.half, blk = f.step;
     uint32_t vals[4] = {0, 0, 0, 0};
     if (nibbles) {
         const int cw = blk * 2 + half;
@@ -43,11 +37,9 @@ __global__ void tc_prepare_weights_kernel(const uint32_t* __restrict__ packed, i
             vals[b >> 2] |= byte << (8 * (b & 3));
         }
     }
-    if (nibbles && idx == nvec - 1) {       // the last vector of the tensor is this one (of channels that do not exist) or one that no layer reads
-        if (last == idx) vals[3] = MM_NIBBLE_MARK;
-        else reinterpret_cast<uint4*>(out)[last] = make_uint4(0, 0, 0, MM_NIBBLE_MARK);
-    }
-    reinterpret_cast<uint4*>(out)[idx] = make_uint4(vals[0], vals[1], vals[2], vals[3]);
+    const uint4 v = make_uint4(vals[0], vals[1], vals[2], vals[3]);
+    if (nibbles) put_nibbles(reinterpret_cast<uint4*>(out), idx, nvec, last, v);
+    else reinterpret_cast<uint4*>(out)[idx] = v;
 }
 
 static int tc_max_abs(int bits, int sign)
