@@ -101,13 +101,14 @@ def layer_roofline(net, engine: str, peaks: dict):
 
 def captured_traffic(net_name: str, batch: int):
     """dram__bytes_read + dram__bytes_write of one pass of the conv launches, from the tracked ncu summary of that capture
-    under profiles/.  The summary names the SHA-256 of the kernel source it was taken on; a different source gives None
-    (the counters are stale once the kernel has changed)."""
+    under profiles/.  The summary names the SHA-256 of the sources it was taken on, one after the other; different ones give None
+    (the counters are stale once the kernel or its plans have changed)."""
     import hashlib
     import re
     path = os.path.join(ROOT, "profiles", f"bitserial_conv_tc_kernels_{net_name}_dram_traffic.md")
-    src = os.path.join(ROOT, "paper_2207_08820_b200", "csrc", "oper_kernel.cuh")
-    if not (os.path.exists(path) and os.path.exists(src)):
+    # the kernel, what it shares with the others, and where its tiles and the layout of its tensors are decided
+    sources = [os.path.join(ROOT, "paper_2207_08820_b200", "csrc", f) for f in ("oper_kernel.cuh", "oper_conv.cu", "oper_tensor.cuh", "mma_kernel.cuh")]
+    if not all(os.path.exists(p) for p in (path, *sources)):
         return None, None
     text = open(path).read()
     m_bytes = re.search(r"traffic_bytes_per_pass:\s*([0-9.eE+]+)", text)
@@ -115,7 +116,7 @@ def captured_traffic(net_name: str, batch: int):
     m_sha = re.search(r"kernel_source_sha256:\s*([0-9a-f]{64})", text)
     if not (m_bytes and m_sha and m_batch) or int(m_batch.group(1)) != batch:
         return None, os.path.basename(path)
-    if hashlib.sha256(open(src, "rb").read()).hexdigest() != m_sha.group(1):
+    if hashlib.sha256(b"".join(open(p, "rb").read() for p in sources)).hexdigest() != m_sha.group(1):
         return None, os.path.basename(path) + " (stale: the kernel source changed after the capture)"
     return float(m_bytes.group(1)), os.path.basename(path)
 

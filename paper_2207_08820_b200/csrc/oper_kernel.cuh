@@ -6,10 +6,12 @@
 // per parity).  The pixels of any tile and their halo are then one run of memory per channel group, so a layer has nothing to expand, no pixel
 // to locate and no thread that copies: one warp fetches runs by bulk copies, one warp issues MMAs, eight warps requantise.
 //
-// What bounds it: the epilogue and the start of a launch.  Half an SM's shared memory and tensor memory per CTA, so that two CTAs overlap each
-// other's MMAs and epilogues, or the next layer's CTA sets up and fetches its filters beside the last one of this layer.
-// Layers one after the other, expanding packed codes -> on operand tensors, us: 64 images, 64 channels of 56 x 56, 3 x 3: 12.6 -> 8.3, with a residual
-// 14.2 -> 10.0; 256 of 14 x 14: 8.6 -> 6.4; one image of the former 3.0 -> 2.4; 512 of 7 x 7: 6.2 -> 4.6.
+// What bounds it: the turn of MMAs and epilogue, and the start of a launch (a 56 x 56 layer of 64 images: 1000 cycles of MMA issue and 1800 to 2500 of
+// epilogue an item, three items, 4000 cycles from a CTA's start to its first MMA; without its stores 5 %, without reads of scales 7 % faster).
+// Half an SM's shared memory and tensor memory per CTA, so that two CTAs overlap each other's MMAs and epilogues, or the next layer's CTA sets up
+// and fetches its filters beside the last one of this layer.
+// Layers one after the other, calls on packed codes -> on operand tensors, us: 64 images, 64 channels of 56 x 56, 3 x 3: 13.4 -> 8.8, with a residual
+// 15.1 -> 10.1; 256 of 14 x 14: 9.2 -> 6.3; one image of the former 3.7 -> 2.5; 512 of 7 x 7: 6.9 -> 4.6.
 #pragma once
 #include "mma_kernel.cuh"
 
