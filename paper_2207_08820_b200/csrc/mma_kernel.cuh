@@ -1417,13 +1417,13 @@ __global__ void __launch_bounds__(MmaShape<HALF>::THREADS, MmaShape<HALF>::CPS) 
     if (warp == WARP_MMA) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(g.tmem_cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        // Only now: a CTA of a later launch may take tensor memory as soon as it runs, and keeps it until every launch before it has ended.  Released
+        // while this CTA still waits for its columns, the two could wait for each other.
+        mm_pdl_release();
     }
     mm_fence_before();
     __syncthreads();
     mm_fence_after();
-    // Only now: a CTA of a later launch may take tensor memory as soon as it runs, and keeps it until every launch before it has ended.  Released while
-    // this CTA still waits for its columns, the two could wait for each other.
-    mm_pdl_release();
     if (SPLIT) mm_cluster_sync();      // the barriers of rank 0 are initialised
     const MmaChunks range(g, SPLIT);
     const int walk_log = SPLIT ? g.split_log : 0;
