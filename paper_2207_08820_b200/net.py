@@ -65,7 +65,7 @@ class BitserialNet:
         operand_tensors: with filters prepared as nibbles a pass keeps what the tensor cores read of every tensor between its layers in device memory of
         its own (``bs_sequence_create_ws``), about twice the packed tensors together: 59 MB for the 18-layer stack at 64 images, 139 MB for
         the detection stack at 16, 169 MB for the 50-layer one at 32, held while the runner lives (:attr:`operand_bytes`), once more for every
-        set of tensors that a graph was recorded with.  False: no such memory, layers expand packed codes, 1.2 to 1.5 times the time."""
+        set of tensors that a graph was recorded with.  False: no such memory, layers expand packed codes, 1.1 to 1.5 times the time."""
         self.net = net
         self.engine = engine
         self.act_scale = float(act_scale)
