@@ -155,12 +155,13 @@ class BitserialNet:
         return sum(w.memory.numel() for w in self._workspaces)
 
     def input_operands(self) -> Optional[int]:
-        """The operand tensor of the packed input (``bs_sequence_input``), which a producer of the input may write as well, or None."""
+        """The operand tensor of the packed input (``bs_sequence_input``), which a producer of the input may write as well, or None.  It is
+        the bound sequence's: valid until an entry of the layers is replaced."""
         return self._sequence.input if self._bind() else None
 
     def pack_input(self, x: torch.Tensor, operands: bool = False) -> Optional[int]:
         """Quantise + bitplane-pack the fp32 input on the current stream.  operands: its operand tensor too, where the layers have one and ``x`` is
-        the whole input; :meth:`run_layers` takes what is returned then, as long as neither is written in between."""
+        the whole input; :meth:`run_layers` takes the object that is returned then, as long as neither is written in between."""
         return self._pack(x, self.input_operands() if operands else None)
 
     def _pack(self, x: torch.Tensor, operands: Optional[int]) -> Optional[int]:
@@ -245,7 +246,7 @@ class BitserialNet:
         """:meth:`run_layers` behind a look at the tensors: a pass takes one, in front of what writes its input."""
         if bound:
             q = self._sequence
-            ready = ready if ready == q.input else None
+            ready = ready if ready is q.input else None         # (an address may come back with another sequence, the object does not)
             api.run_sequence(q.handle, q.launches - (ready is not None), ready=ready)
         else:
             self.run_units()

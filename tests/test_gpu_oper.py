@@ -305,3 +305,23 @@ def test_operand_tensors_can_be_declined():
     assert plain._sequence.launches == len(spec.layers) and plain.input_operands() is None
     assert torch.equal(r.forward(xd), plain.forward(xd))
     api.bs_check_status()
+
+
+def test_an_address_that_comes_back_is_not_a_packed_input():
+    """Sequences of a runner follow each other, and the next may lie where the last one lay: what was written for one is not taken for the other's."""
+    spec = STACKS["both_strides"]
+    r, _, x = runner_of(spec)
+    xd = dev(x)
+    r.forward(xd)
+    r.bufs["x"].copy_(r.bufs["x"].roll(1, 0))
+    r.run_layers(ready=int(str(r.input_operands())))
+    got = r.bufs[spec.out_name].clone()
+    r.run_units()
+    assert torch.equal(got, r.bufs[spec.out_name])
+    ready = r.pack_input(xd, operands=True)
+    r.layers[0]["w_tc"] = None                                       # binds again, to another workspace
+    r.run_layers(ready=ready)
+    got = r.bufs[spec.out_name].clone()
+    r.run_units()
+    assert torch.equal(got, r.bufs[spec.out_name])
+    api.bs_check_status()
