@@ -53,7 +53,9 @@ typedef enum {
     BS_ERR_TIMEOUT = 5      /* a bounded device-side wait ran out (reported by bs_check_status)       */
 } bs_status;
 
-typedef enum { BS_UNSIGNED = 0, BS_SIGNED = 1, BS_BIPOLAR = 2 } bs_sign_t;
+typedef enum { BS_UNSIGNED = 0, BS_SIGNED = 1, BS_BIPOLAR = 2,
+               BS_SIGNED_NIBBLES = 3    /* BS_SIGNED filters of three bits, prepared as nibbles (bs_tc_prepare_weights); nowhere else */
+} bs_sign_t;
 typedef enum { BS_NCHW = 0, BS_NHWC = 1 } bs_layout_t; /* for weights: OIHW = BS_NCHW, OHWI = BS_NHWC */
 
 /* Bytes of a packed activation tensor / packed weight tensor / packed row matrix (0 on bad input). */
@@ -234,7 +236,9 @@ int bitserial_gemm_noalloc(const uint32_t* a_packed, const uint32_t* w_packed, i
  *                          [ceil(C/64)][ceil(O/128)*16][R*S][2][8][16 bytes] where a_bits and w_bits are at most 2 (the first half of the
  *                          tensor or so), int8 [C/32][ceil(O/128)*16][R*S][2][8][16] otherwise.  One tensor serves layers of every a_bits; a
  *                          layer that meets the other form converts its filters in each launch, with one warp of each SM, so prepare
- *                          them for the widths they run with.
+ *                          them for the widths they run with.  Signed filters of three bits are int8 as BS_SIGNED, which layers of every a_bits read as
+ *                          they are; with w_sign BS_SIGNED_NIBBLES, here and in the layer, they are nibbles for a_bits of at most 2, which take
+ *                          0.67 to 0.95 of the time (BS_ERR_UNSUPPORTED for wider activations and reductions of C * R * S >= 142858).
  */
 size_t bs_tc_weights_bytes(int O, int C, int R, int S);
 size_t bs_tc_weights_read_bytes(int O, int C, int R, int S, int w_bits, int a_bits);

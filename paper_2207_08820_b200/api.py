@@ -14,6 +14,7 @@ import torch
 from ._lib import BitserialError, ConvParams, lib, native
 
 UNSIGNED, SIGNED, BIPOLAR = 0, 1, 2
+SIGNED_NIBBLES = 3      # signed filters of three bits prepared as nibbles; only where prepared filters are
 NCHW, NHWC = 0, 1
 ERR_UNSUPPORTED = 2
 
@@ -143,21 +144,38 @@ def bitserial_gemm(a_packed: torch.Tensor, w_packed: torch.Tensor, K: int, *, a_
 
 def tc_prepare_weights(wgt_packed: torch.Tensor, C: int, w_sign: int, a_bits: int, stream=None) -> torch.Tensor:
     """Packed weights [O,R,S,Cw,w_bits] -> filter tiles for the tensor-core entry points, made for layers of ``a_bits`` activation bits (nibbles where
-    both widths are at most 2, int8 otherwise; layers that need the other form take these too and convert them in each launch, more slowly)."""
+    both widths are at most 2, int8 otherwise; layers that need the other form take these too and convert them in each launch, more slowly).
+    Signed filters of three bits for one or two bits are both, int8 and then nibbles, in a tensor of twice the size: layers of every width read
+    their form as it is."""
     O, R, S, Cw, w_bits = wgt_packed.shape
     nbytes = lib().bs_tc_weights_bytes(O, C, R, S)
     if nbytes == 0:
         raise BitserialError(2, "bs_tc_weights_bytes")
-    out = torch.empty(nbytes, dtype=torch.int8, device=wgt_packed.device)
-    st = lib().bs_tc_prepare_weights(_ptr(wgt_packed), O, C, R, S, w_bits, w_sign, a_bits, _ptr(out), _stream_ptr(stream))
-    _check(st, "bs_tc_prepare_weights")
+    signs = [w_sign, SIGNED_NIBBLES] if w_bits == 3 and w_sign == SIGNED and a_bits <= 2 and C * R * S * 28 < 4000000 else [w_sign]
+    out = torch.empty(nbytes * len(signs), dtype=torch.int8, device=wgt_packed.device)
+    for k, sign in enumerate(signs):
+        st = lib().bs_tc_prepare_weights(_ptr(wgt_packed), O, C, R, S, w_bits, sign, a_bits, _ptr(out[k * nbytes:(k + 1) * nbytes]), _stream_ptr(stream))
+        _check(st, "bs_tc_prepare_weights")
     return out
+
+
+def tc_weights_form(w_tc: Optional[torch.Tensor], wgt_shape, C: int, w_sign: int, a_bits: int):
+    """(part of ``w_tc`` that layers of ``a_bits`` activation bits read, ``bs_sign_t`` that goes with it)."""
+    O, R, S, _, w_bits = wgt_shape
+    if w_tc is not None and w_bits == 3 and w_sign == SIGNED and a_bits <= 2:
+        n = lib().bs_tc_weights_bytes(O, C, R, S)
+        if w_tc.numel() * w_tc.element_size() == 2 * n:
+            return w_tc.view(-1)[w_tc.numel() // 2:], SIGNED_NIBBLES
+    return w_tc, w_sign
 
 
 def tc_weights_read(w_tc: torch.Tensor, wgt_shape, C: int, a_bits: int):
     """What layers of ``a_bits`` activation bits read of filters prepared for them: a list of views."""
     O, R, S, _, w_bits = wgt_shape
-    n = lib().bs_tc_weights_read_bytes(O, C, R, S, w_bits, a_bits)
+    w_tc, sign = tc_weights_form(w_tc, wgt_shape, C, SIGNED, a_bits)
+    n = lib().bs_tc_weights_read_bytes(O, C, R, S, 2 if sign == SIGNED_NIBBLES else w_bits, a_bits)     # (nibbles are laid out as those of two bits)
+    if w_bits == 3 and n:
+        w_tc = w_tc[:lib().bs_tc_weights_bytes(O, C, R, S)]
     return [w_tc] if n in (0, w_tc.numel()) else [w_tc[:n], w_tc[-16:]]
 
 

@@ -80,6 +80,18 @@ PyObject* guarded(F f)
     return nullptr;
 }
 
+// Prepared filters of three bits for narrow activations hold both forms, int8 and nibbles (tc_prepare_weights in api.py): the nibbles where they are
+// wanted, with the sign that says so.
+const int8_t* prepared(const at::Tensor& t, int O, int C, int R, int S, int w_bits, int a_bits, int& w_sign)
+{
+    const int8_t* p = static_cast<const int8_t*>(pointer(t));
+    if (w_bits != 3 || a_bits > 2 || w_sign != BS_SIGNED) return p;
+    const size_t bytes = bs_tc_weights_bytes(O, C, R, S);
+    if (bytes == 0 || t.nbytes() != 2 * bytes) return p;
+    w_sign = BS_SIGNED_NIBBLES;
+    return p + bytes;
+}
+
 void mismatch(const char* what) { PyErr_SetString(PyExc_ValueError, what); throw Fail(); }
 
 // act, wgt, C, stride, pad, a_sign, w_sign, scale, bias, relu, out_bits, out_sign, residual, res_scale, res_bits, res_sign, res_c_offset,
@@ -111,7 +123,7 @@ PyObject* conv2d(PyObject*, PyObject* const* a, Py_ssize_t n)
         auto fdiv = [](int x, int y) { return x / y - (x % y != 0 && (x < 0) != (y < 0)); };
         const int64_t P = fdiv(p.H + 2 * p.pad - p.R, p.stride) + 1, Q = fdiv(p.W + 2 * p.pad - p.S, p.stride) + 1;
         const uint32_t* ap = static_cast<const uint32_t*>(pointer(act));
-        const int8_t* tc = static_cast<const int8_t*>(pointer_or_null(a[25]));
+        const int8_t* tc = a[25] == Py_None ? nullptr : prepared(tensor(a[25]), p.O, p.C, p.R, p.S, p.w_bits, p.a_bits, p.w_sign);
         const uint32_t* wp = tc ? nullptr : static_cast<const uint32_t*>(pointer(wgt));
         at::Tensor i32, packed;
         if (a[18] != Py_None) i32 = tensor(a[18]);
@@ -160,11 +172,12 @@ PyObject* gemm(PyObject*, PyObject* const* a, Py_ssize_t n)
             if (x.size(1) != w.size(1) || x.size(1) != (static_cast<int64_t>(K) + 31) / 32) mismatch("reduction words of the operands disagree");
             N = static_cast<int>(w.size(0)); w_bits = static_cast<int>(w.size(2));
         }
-        const int a_sign = integer(a[5]), w_sign = integer(a[6]);
+        const int a_sign = integer(a[5]);
+        int w_sign = integer(a[6]);
         const float *scale = static_cast<const float*>(pointer_or_null(a[7])), *bias = static_cast<const float*>(pointer_or_null(a[8]));
         const int relu = PyObject_IsTrue(a[9]), out_bits = integer(a[10]), out_sign = integer(a[11]);
         const uint32_t* xp = static_cast<const uint32_t*>(pointer(x));
-        const void* wp = pointer(w);
+        const void* wp = tc ? prepared(w, N, K, 1, 1, w_bits, a_bits, w_sign) : pointer(w);
         at::Tensor i32, packed;
         if (a[12] != Py_None) i32 = tensor(a[12]);
         else if (PyObject_IsTrue(a[13])) i32 = words({M, N}, x);

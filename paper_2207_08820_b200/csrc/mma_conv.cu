@@ -21,7 +21,7 @@ constexpr int MM_SMEM_MAX = 224 * 1024;
 
 int up(int v, int m) { return (v + m - 1) / m * m; }
 
-int max_abs_of(int bits, int sign) { return sign == BS_BIPOLAR ? 1 : (sign == BS_SIGNED ? 1 << (bits - 1) : (1 << bits) - 1); }
+int max_abs_of(int bits, int sign) { return sign == BS_BIPOLAR ? 1 : (sign == BS_UNSIGNED ? (1 << bits) - 1 : 1 << (bits - 1)); }
 
 struct Cand {
     int TN, PT, units, cfg, cps, ns, resident, groups, split, nse, nsb, nacc, f4;
@@ -256,7 +256,7 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
     g.P = (p->H + 2 * p->pad - p->R) / p->stride + 1;
     g.Q = (p->W + 2 * p->pad - p->S) / p->stride + 1;
     g.Cw = ceil_div(p->C, 32);
-    auto kind = [](int sign) { return sign == BS_SIGNED ? 1 : sign == BS_BIPOLAR ? 2 : 0; };
+    auto kind = [](int sign) { return sign == BS_UNSIGNED ? 0 : sign == BS_BIPOLAR ? 2 : 1; };
     g.a_kind = kind(p->a_sign); g.w_kind = kind(p->w_sign);
     g.relu = p->relu; g.out_bits = p->out_bits; g.out_sign = p->out_sign;
     g.out_cw_off = p->out_c_offset / 32; g.out_cw_total = ceil_div(p->out_c_total > 0 ? p->out_c_total : 1, 32);
@@ -271,7 +271,7 @@ static int make_plan(MmaPlan& plan, const bs_conv_params* p, int flags, int sms)
     // outputs 0.98 and 0.97; codes of 5x5 windows over up to 32 channels 1.12 and 0.89 on these sides, of 3x3 windows 0.96 and 0.94.
     const bool short_k = g.Cw == 1 && static_cast<double>(g.N) * g.P * g.Q * g.O >= 2048.0 * sms;
     const bool pixel_rows = out_i32 && !out_packed && !g.i32_nhwc;
-    g.f4 = (packed_b ? mma_nibbles_packed(p->C, g.RS, p->a_bits, p->w_bits, p->w_sign) : mma_nibbles(p->C, g.RS, p->a_bits, p->w_bits)) &&
+    g.f4 = (packed_b ? mma_nibbles_packed(p->C, g.RS, p->a_bits, p->w_bits, p->w_sign) : mma_nibbles(p->C, g.RS, p->a_bits, p->w_bits, p->w_sign)) &&
            !(packed_b && (pixel_rows ? short_k || (g.R == 1 && g.Cw <= 6) : short_k && g.R >= 5 && !out_i32));
     // Unsigned activations of three bits need the filters' sums, which only resident filters give: such plans on nibbles against all on int8, by their
     // modelled time, with 6 % for int8.  Of 135 layers with larger windows, timed on both forms, 6 go to nibbles, which take 0.36 to 0.83 of int8's time.

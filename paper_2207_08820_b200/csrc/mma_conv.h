@@ -14,14 +14,19 @@ __host__ __device__ constexpr int mma_column_of_filter(int f) { return 16 * (f &
 __host__ __device__ constexpr int mma_channel_of_byte(int b) { return 8 * (b & 3) + (b >> 2); }
 
 // Whether a layer runs on nibbles (kind::mxf4, see mma_kernel.cuh): codes of at most two bits on both sides whose sums stay below 2^22 whatever
-// the signs.  Also the form of its prepared filters, so it depends only on what their preparation knows.  Prepared filters of three bits are int8 for
-// activations of every width: on nibbles a layer of two by three bits takes 0.67 to 0.95 of the time, but a tensor in the other form is converted
-// in each launch, 2 to 20 times the time (4096 x 4096 x 4608, two by three bits: 94 us on int8, 64 on nibbles, 1496 on int8 filters converted).
-constexpr bool mma_nibbles(int C, int RS, int a_bits, int w_bits) { return a_bits <= 2 && w_bits <= 2 && static_cast<long long>(C) * RS * 9 < 4000000; }
+// the signs.  Also the form of its prepared filters, so it depends only on what their preparation knows.  Signed filters of three bits say by their
+// sign what they were prepared as: a tensor in the other form is converted in each launch, 2 to 20 times the time (4096 x 4096 x 4608, two by three
+// bits: 94 us on int8, 64 on nibbles, 1496 on int8 filters converted), so those of callers who don't say are int8 for activations of every width.
+constexpr bool mma_nibbles(int C, int RS, int a_bits, int w_bits, int w_sign)
+{
+    return a_bits <= 2 && (w_sign == BS_SIGNED_NIBBLES ? w_bits == 3 && static_cast<long long>(C) * RS * 28 < 4000000
+                                                       : w_bits <= 2 && static_cast<long long>(C) * RS * 9 < 4000000);
+}
 // Packed filters run on nibbles with three bits a side as well (unsigned filters of three bits have no exact form).
 constexpr bool mma_nibbles_packed(int C, int RS, int a_bits, int w_bits, int w_sign)
 {
-    return mma_nibbles(C, RS, a_bits, w_bits) || (a_bits <= 3 && (w_bits <= 2 ? a_bits == 3 : w_bits == 3 && w_sign == BS_SIGNED) && static_cast<long long>(C) * RS * 28 < 4000000);
+    return mma_nibbles(C, RS, a_bits, w_bits, w_sign) ||
+           (a_bits <= 3 && (w_bits <= 2 ? a_bits == 3 : w_bits == 3 && w_sign == BS_SIGNED) && static_cast<long long>(C) * RS * 28 < 4000000);
 }
 // Prepared nibbles end with this word, four pairs of negative zeros, in room that holds no code; int8 codes (-8 .. 15) never contain its bytes.
 // A layer tells the form of its filters by it and converts them where it needs the other one.

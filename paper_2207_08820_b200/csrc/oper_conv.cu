@@ -136,7 +136,7 @@ bool lay_out(const bs_sequence_layer* layers, int n, Layout& l)
         const bs_conv_params& p = layers[i].p;
         if (!layers[i].out_packed || !layers[i].act_packed || p.C % 32 != 0) return false;
         if (p.a_sign != BS_UNSIGNED || p.out_sign != BS_UNSIGNED || p.out_bits > 2 || p.out_bits < 1) return false;
-        if (!mma_nibbles(p.C, p.R * p.S, p.a_bits, p.w_bits) || p.stride > 2 || p.R != p.S) return false;
+        if (!mma_nibbles(p.C, p.R * p.S, p.a_bits, p.w_bits, p.w_sign) || p.stride > 2 || p.R != p.S) return false;
         if (p.residual && (p.res_sign != BS_UNSIGNED || p.res_bits > 2 || !(fabsf(p.res_scale) < 3.9f) || (p.res_scale != 0.0f && fabsf(p.res_scale) <= 1e-18f))) return false;
         const Shape s = shape_of(p);
         const int src = tensor_index(l, layers[i].act_packed, p.N, p.H, p.W, p.C / 32, p.a_bits);
@@ -325,7 +325,7 @@ static bool fill(OperArgs& g, const bs_sequence_layer& l, const Layout& lay, int
     g.dst2 = dst_of(out, 1, ws, word);
     if ((out.form[0].used || out.form[1].used) && p.O % 32 != 0) return false;
     g.scale = p.scale; g.bias = p.bias; g.residual = p.residual; g.res_scale = p.res_scale;
-    g.acc_bound = static_cast<float>(static_cast<double>(p.C) * g.RS * ((1 << p.a_bits) - 1) * (p.w_sign == BS_BIPOLAR ? 1 : p.w_sign == BS_SIGNED ? 1 << (p.w_bits - 1) : (1 << p.w_bits) - 1));
+    g.acc_bound = static_cast<float>(static_cast<double>(p.C) * g.RS * ((1 << p.a_bits) - 1) * (p.w_sign == BS_BIPOLAR ? 1 : p.w_sign == BS_UNSIGNED ? (1 << p.w_bits) - 1 : 1 << (p.w_bits - 1)));
     g.relu = p.relu; g.out_bits = p.out_bits; g.out_sign = p.out_sign;
     g.out_cw_off = word; g.out_cw_total = out.Cw;
     g.res_bits = p.res_bits; g.res_sign = p.res_sign; g.res_c_off = p.res_c_offset;

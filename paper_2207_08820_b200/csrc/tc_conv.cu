@@ -71,9 +71,12 @@ static int tc_validate_shape(const bs_conv_params* p)
 // kernels themselves take any record).
 static int tc_validate(const bs_conv_params* p)
 {
-    const int rc = tc_validate_shape(p);
+    if (!p) return BS_ERR_INVALID_ARG;
+    bs_conv_params q = *p;
+    if (p->w_sign == BS_SIGNED_NIBBLES) q.w_sign = BS_SIGNED;
+    const int rc = tc_validate_shape(&q);
     if (rc != BS_OK) return rc;
-    if (p->C % 32 != 0) return BS_ERR_UNSUPPORTED;
+    if (p->C % 32 != 0 || (p->w_sign == BS_SIGNED_NIBBLES && !mma_nibbles(p->C, p->R * p->S, p->a_bits, p->w_bits, p->w_sign))) return BS_ERR_UNSUPPORTED;
     const int rec = p->C / 32 * p->a_bits;
     if (rec % 4 != 0) {
         if (rec % 2 != 0 || (p->W * rec) % 4 != 0) return BS_ERR_UNSUPPORTED;
@@ -189,23 +192,25 @@ extern "C" size_t bs_tc_weights_read_bytes(int O, int C, int R, int S, int w_bit
 {
     const size_t all = bs_tc_weights_bytes(O, C, R, S);
     if (all == 0 || !bs::bits_ok(w_bits, BS_UNSIGNED) || !bs::bits_ok(a_bits, BS_UNSIGNED)) return 0;
-    return bs::mma_nibbles(C, R * S, a_bits, w_bits) ? all / (C / 32) * ((C / 32 + 1) / 2) : all;
+    return bs::mma_nibbles(C, R * S, a_bits, w_bits, BS_UNSIGNED) ? all / (C / 32) * ((C / 32 + 1) / 2) : all;
 }
 
 extern "C" int bs_tc_prepare_weights(const uint32_t* wgt_packed, int O, int C, int R, int S, int w_bits, bs_sign_t w_sign,
                                      int a_bits, int8_t* out, void* stream)
 {
     if (!wgt_packed || !out || O <= 0 || C <= 0 || R <= 0 || S <= 0) return BS_ERR_INVALID_ARG;
-    if (!bs::bits_ok(w_bits, w_sign) || a_bits < 1 || a_bits > 4) return BS_ERR_INVALID_ARG;
+    const bs_sign_t sign = w_sign == BS_SIGNED_NIBBLES ? BS_SIGNED : w_sign;
+    if (!bs::bits_ok(w_bits, sign) || a_bits < 1 || a_bits > 4) return BS_ERR_INVALID_ARG;
     if (!bs::aligned16(wgt_packed) || !bs::aligned16(out)) return BS_ERR_ALIGNMENT;
     if (C % 32 != 0) return BS_ERR_UNSUPPORTED;
     const int opad8 = (O + 127) / 128 * 16;
-    const bool nibbles = bs::mma_nibbles(C, R * S, a_bits, w_bits);
+    const bool nibbles = bs::mma_nibbles(C, R * S, a_bits, w_bits, w_sign);
+    if (w_sign == BS_SIGNED_NIBBLES && !nibbles) return BS_ERR_UNSUPPORTED;
     const long long nvec = static_cast<long long>(nibbles ? (C / 32 + 1) / 2 : C / 32) * opad8 * R * S * 2 * 8;
     const long long blocks = (nvec + 255) / 256;
     if (blocks > 0x7fffffffLL) return BS_ERR_UNSUPPORTED;
     bs::tc_prepare_weights_kernel<<<static_cast<unsigned>(blocks), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        wgt_packed, out, nvec, O, R * S, C / 32, w_bits, w_sign, opad8, nibbles,
+        wgt_packed, out, nvec, O, R * S, C / 32, w_bits, sign, opad8, nibbles,
         static_cast<long long>(C / 32) * opad8 * R * S * 2 * 8 - 1);
     return cudaGetLastError() == cudaSuccess ? BS_OK : BS_ERR_CUDA;
 }
@@ -261,8 +266,7 @@ static int bs_sequence_check(const bs_sequence_layer* layers, int nlayers)
     for (int l = 0; l < nlayers; ++l) {
         const bs_sequence_layer& s = layers[l];
         if (!s.wgt_tc && !s.wgt_packed) return BS_ERR_INVALID_ARG;
-        int rc = bs::tc_validate_shape(&s.p);
-        if (rc == BS_OK && s.wgt_tc) rc = bs::tc_validate(&s.p);
+        int rc = s.wgt_tc ? bs::tc_validate(&s.p) : bs::tc_validate_shape(&s.p);
         if (rc == BS_OK) rc = bs::tc_validate_outputs(s.act_packed, s.wgt_tc ? static_cast<const void*>(s.wgt_tc) : s.wgt_packed, &s.p, nullptr, s.out_packed);
         if (rc != BS_OK) return rc;
     }

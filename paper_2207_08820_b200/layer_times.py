@@ -35,13 +35,14 @@ class BoundLayer:
         codes = torch.zeros(32, C, 1, 1, dtype=torch.int8, device=out.device)
         w, rest = api.pack_weights(codes, runner.net.w_bits, item["w_sign"]), torch.zeros(*out.shape[:3], 1, runner.net.a_bits, dtype=torch.int32, device=out.device)
         scale = torch.ones(32, dtype=torch.float32, device=out.device)
-        w_tc = api.tc_prepare_weights(w, C, item["w_sign"], runner.net.a_bits)
-        self.keep += [w, w_tc, rest, scale]
+        both = api.tc_prepare_weights(w, C, item["w_sign"], runner.net.a_bits)
+        w_tc, sign = api.tc_weights_form(both, w.shape, C, item["w_sign"], runner.net.a_bits)
+        self.keep += [w, both, rest, scale]
         self.layers = (SequenceLayer * (reps + 1))()
         for k, q in enumerate(self.layers):
             q.act_packed, q.out_packed = (runner.bufs[item["spec"].src].data_ptr(), out.data_ptr()) if k else (out.data_ptr(), rest.data_ptr())
-            q.wgt_packed, q.wgt_tc = (item["w"].data_ptr(), item["w_tc"].data_ptr()) if k else (w.data_ptr(), w_tc.data_ptr())
-            q.p = runner._conv_params(item) if k else api.conv_params(out.shape, w.shape, C=C, w_sign=item["w_sign"], scale=scale, bias=scale, out_bits=runner.net.a_bits)
+            q.wgt_packed, q.wgt_tc = (item["w"].data_ptr(), runner._filters(item)[0].data_ptr()) if k else (w.data_ptr(), w_tc.data_ptr())
+            q.p = runner._conv_params(item) if k else api.conv_params(out.shape, w.shape, C=C, w_sign=sign, scale=scale, bias=scale, out_bits=runner.net.a_bits)
             q.chained = 1
             q.join[:] = [-1] * 4
         nbytes = lib().bs_sequence_workspace_bytes(self.layers, reps + 1)

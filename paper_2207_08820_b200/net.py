@@ -191,7 +191,7 @@ class BitserialNet:
             return
         items = unit["items"]
         params = [self._layer_params(it) for it in items]       # pointers of the buffers as they are now (tests swap them)
-        api.bitserial_conv2d_tc_chain([self.bufs[it["spec"].src] for it in items], [it["w_tc"] for it in items], params,
+        api.bitserial_conv2d_tc_chain([self.bufs[it["spec"].src] for it in items], [self._filters(it)[0] for it in items], params,
                                       [self.bufs[it["spec"].dst] for it in items], unit["workspace"], chained=chained)
 
     def schedule(self):
@@ -294,7 +294,7 @@ class BitserialNet:
         for q, (item, aside, join) in zip(arr, layers):
             L = item["spec"]
             q.act_packed, q.out_packed = api._ptr(self.bufs[L.src]), api._ptr(self.bufs[L.dst])
-            q.wgt_packed, q.wgt_tc = api._ptr(item["w"]), api._ptr(item["w_tc"])
+            q.wgt_packed, q.wgt_tc = api._ptr(item["w"]), api._ptr(self._filters(item)[0])
             q.p = self._conv_params(item)
             q.chained, q.aside = 1, int(aside)
             q.join[:] = (join + [-1] * 4)[:4]
@@ -342,10 +342,14 @@ class BitserialNet:
         self._workspaces.append(_Workspace(geometry, addresses, memory))
         return self._workspaces[-1]
 
+    def _filters(self, item):
+        """Prepared filters of a layer, or None, and the sign that goes with them."""
+        return api.tc_weights_form(item["w_tc"], item["w"].shape, item["spec"].C, item["w_sign"], self.net.a_bits)
+
     def _conv_params(self, item):
         net, L = self.net, item["spec"]
         q = api.conv_params(
-            self.bufs[L.src].shape, item["w"].shape, C=L.C, stride=L.stride, pad=L.pad, a_sign=api.UNSIGNED, w_sign=item["w_sign"],
+            self.bufs[L.src].shape, item["w"].shape, C=L.C, stride=L.stride, pad=L.pad, a_sign=api.UNSIGNED, w_sign=self._filters(item)[1],
             scale=item["scale"], bias=item["bias"], relu=L.relu, out_bits=net.a_bits, out_sign=api.UNSIGNED,
             residual=self.bufs[L.res] if L.res else None, res_scale=L.res_scale, res_bits=net.a_bits if L.res else 0,
             res_sign=api.UNSIGNED)

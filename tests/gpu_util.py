@@ -90,9 +90,9 @@ def gpu_conv(case, want_i32=True, want_packed=True, i32_layout=api.NCHW, residua
     return (acc.cpu().numpy() if acc is not None else None), (words(packed) if packed is not None else None)
 
 
-def layer_array(spec, w_sign=None):
+def layer_array(spec, w_sign=None, prepared_sign=None):
     """The layers of a stack as ``bs_sequence_layer`` records over addresses that nothing is at: what the host side of the library (planner, workspace
-    size) is asked with, without a device."""
+    size) is asked with, without a device.  prepared_sign: the sign of layers with prepared filters, where it is another."""
     sign = wl.weight_sign(spec.w_bits) if w_sign is None else w_sign
     shapes, at, end = spec.tensor_shapes(), {}, 1 << 20
     for name, (C, H, W) in shapes.items():
@@ -104,7 +104,7 @@ def layer_array(spec, w_sign=None):
         prepared = api.tc_supported(spec.batch, l.C, H, W, l.O, l.k, l.stride, l.pad, spec.a_bits, api.UNSIGNED, spec.w_bits, sign)
         q.act_packed, q.out_packed, q.wgt_packed, q.wgt_tc = at[l.src], at[l.dst], 4096, 8192 if prepared else None
         q.p = ConvParams(N=spec.batch, C=l.C, H=H, W=W, O=l.O, R=l.k, S=l.k, stride=l.stride, pad=l.pad, a_bits=spec.a_bits, a_sign=api.UNSIGNED, w_bits=spec.w_bits,
-                         w_sign=sign, scale=4096, bias=4096, relu=int(l.relu), out_bits=spec.a_bits, out_sign=api.UNSIGNED, residual=at[l.res] if l.res else None,
+                         w_sign=prepared_sign if prepared and prepared_sign is not None else sign, scale=4096, bias=4096, relu=int(l.relu), out_bits=spec.a_bits, out_sign=api.UNSIGNED, residual=at[l.res] if l.res else None,
                          res_scale=l.res_scale if l.res else 0.0, res_bits=spec.a_bits if l.res else 0, res_sign=api.UNSIGNED, res_c_offset=0,
                          res_c_total=shapes[l.res][0] if l.res else l.O, out_c_offset=l.dst_c_offset, out_c_total=shapes[l.dst][0])
         q.chained = 1

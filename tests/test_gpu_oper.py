@@ -33,6 +33,7 @@ STACKS = {
     "concatenation": net(2, (64, 20, 20), [L("a", "x", "cat", 64, 64, 1, 1, 0, dst_c_offset=64), L("b", "x", "b", 64, 64, 3, 1, 1),
                                            L("c", "b", "cat", 64, 64, 3, 1, 1, res="x", res_scale=0.5), L("d", "cat", "d", 128, 256, 1, 1, 0)]),
     "one_bit": net(3, (64, 10, 12), [L("a", "x", "a", 64, 128, 3, 1, 1), L("b", "a", "b", 128, 64, 3, 2, 1), L("c", "b", "c", 64, 64, 1, 1, 0, res="b", res_scale=0.5)], 1, 1),
+    "three_bit_filters": net(3, (96, 11, 12), [L("a", "x", "a", 96, 128, 3, 1, 1), L("b", "a", "b", 128, 64, 3, 2, 1), L("c", "b", "c", 64, 64, 1, 1, 0, res="b", res_scale=0.5)], 2, 3),
     "wide": net(1, (32, 3, 300), [L("a", "x", "a", 32, 64, 3, 1, 1), L("b", "a", "b", 64, 32, 3, 2, 1), L("c", "b", "c", 32, 32, 1, 1, 0)]),
     "deep": net(1, (512, 7, 7), [L("a", "x", "a", 512, 256, 3, 1, 1), L("b", "a", "b", 256, 512, 1, 1, 0), L("c", "b", "c", 512, 64, 3, 2, 1)]),
     # records that no prepared filters are taken for: the pass prepares them
@@ -46,7 +47,7 @@ STACKS = {
 
 # The same geometries with so many images that the plans are those of large batches: tiles of 64 and 128 filters, pairs of row tiles and four of them,
 # several items a block, one to four accumulators, streamed filters, two teams (tests/test_host_sequence.py asserts that each is met).
-MANY = {name: replace(STACKS[name], batch=batch) for name, batch in dict(one_group=3000, odd_groups=1500, both_strides=1500, concatenation=900, one_bit=2000,
+MANY = {name: replace(STACKS[name], batch=batch) for name, batch in dict(one_group=3000, odd_groups=1500, three_bit_filters=1500, both_strides=1500, concatenation=900, one_bit=2000,
                                                                         wide=300, deep=400, odd_records=1500, odd_one_bit=1500, pixels=100000).items()}
 
 

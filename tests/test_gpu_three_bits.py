@@ -86,10 +86,22 @@ def test_residual_of_three_bits():
 
 @pytest.mark.parametrize("w_sign", [api.SIGNED, api.UNSIGNED])
 def test_prepared_filters_serve_every_width(w_sign):
-    """Three-bit filters are prepared alike for activations of every width, so that no layer converts them."""
+    """Whatever width three-bit filters were prepared for, no layer converts them: their int8 form is in front, nibbles behind it where such layers take them."""
     rng = np.random.default_rng(3)
-    wp = api.pack_weights(dev(wl.rand_codes(rng, (70, 96, 3, 3), 3, w_sign)), 3, w_sign)
-    first = api.tc_prepare_weights(wp, 96, w_sign, 1)
-    for a in (2, 3, 4):
-        assert torch.equal(api.tc_prepare_weights(wp, 96, w_sign, a), first)
+    w = wl.rand_codes(rng, (70, 128, 3, 3), 3, w_sign)
+    wp = api.pack_weights(dev(w), 3, w_sign)
+    made = [api.tc_prepare_weights(wp, 128, w_sign, a) for a in (1, 2, 3, 4)]
+    int8 = made[3]
+    assert all(torch.equal(t[:int8.numel()], int8) for t in made) and made[2].numel() == int8.numel()
+    assert all(t.numel() == (2 if w_sign == api.SIGNED else 1) * int8.numel() for t in made[:2])
+    for a in (1, 2, 3, 4):
+        x = wl.rand_codes(rng, (2, 128, 8, 8), a, 0)
+        want, xa = oracle.conv2d_i32(x, w, 1, 1), api.bitpack_activations(dev(x), 1.0, a)
+        for t in made:
+            part, sign = api.tc_weights_form(t, wp.shape, 128, w_sign, a)
+            assert (sign == api.SIGNED_NIBBLES) == (a <= 2 and t.numel() > int8.numel())
+            assert int(part[-4:].view(torch.int32)) == -0x77777778 if sign == api.SIGNED_NIBBLES else torch.equal(part[:int8.numel()], int8)
+            assert sum(v.numel() for v in api.tc_weights_read(t, wp.shape, 128, a)) == (2 * 128 * 9 * 32 + 16 if sign == api.SIGNED_NIBBLES else int8.numel())
+            acc, _ = api.bitserial_conv2d(xa, wp, C=128, pad=1, w_sign=w_sign, want_i32=True, wgt_tc=t)
+            assert np.array_equal(acc.cpu().numpy(), want)
     api.bs_check_status()

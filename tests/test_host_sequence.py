@@ -3,8 +3,8 @@ import ctypes
 
 import pytest
 
-from paper_2207_08820_b200 import workloads as wl
-from paper_2207_08820_b200._lib import LayerPlan, lib
+from paper_2207_08820_b200 import api, workloads as wl
+from paper_2207_08820_b200._lib import ConvParams, LayerPlan, lib
 from gpu_util import layer_array
 from test_gpu_oper import MANY, STACKS
 
@@ -22,9 +22,33 @@ def test_filters_that_are_prepared_as_nibbles(w_bits, w_sign, takes):
     assert (workspace(spec, w_sign=w_sign) > 0) == takes
 
 
+@pytest.mark.parametrize("a_bits,w_bits,takes", [(2, 3, True), (1, 3, True), (3, 3, False), (2, 2, False), (2, 4, False)])
+def test_three_bit_filters_prepared_as_nibbles(a_bits, w_bits, takes):
+    spec = wl.resnet18_body(2, 28)
+    spec.a_bits, spec.w_bits = a_bits, w_bits
+    assert (workspace(spec, w_sign=wl.SIGNED, prepared_sign=api.SIGNED_NIBBLES) > 0) == takes
+
+
+def test_the_sign_of_nibbles_is_for_prepared_filters_only():
+    p = ConvParams(N=1, C=64, H=8, W=8, O=64, R=3, S=3, stride=1, pad=1, a_bits=2, w_bits=3, w_sign=api.SIGNED_NIBBLES)
+    assert lib().bs_tc_supported(ctypes.byref(p)) == 1
+    assert lib().bitserial_conv2d(4096, 4096, ctypes.byref(p), 4096, None, None) == 1
+    assert lib().bs_conv_workspace_bytes(ctypes.byref(p)) == 0
+    assert lib().pack_weights(4096, 0, 64, 64, 3, 3, 3, api.SIGNED_NIBBLES, 4096, None) == 1
+    assert lib().bs_tc_prepare_weights(4096, 64, 64, 3, 3, 3, api.SIGNED_NIBBLES, 3, 4096, None) == 2
+    assert lib().bs_tc_prepare_weights(4096, 64, 64, 3, 3, 2, api.SIGNED_NIBBLES, 2, 4096, None) == 2
+    arr = layer_array(STACKS["one_group"])
+    arr[0].wgt_tc, arr[0].p.w_sign, arr[0].p.w_bits = None, api.SIGNED_NIBBLES, 3
+    assert lib().bs_sequence_layer_plan(arr, len(arr), 0, ctypes.byref(LayerPlan())) == 1
+    for field, value in (("a_bits", 3), ("a_bits", 4), ("w_bits", 2), ("a_sign", api.SIGNED_NIBBLES)):
+        q = ConvParams.from_buffer_copy(p)
+        setattr(q, field, value)
+        assert lib().bs_tc_supported(ctypes.byref(q)) == 0
+
+
 def plans(spec):
     """(layer, its plan) of every layer of a stack."""
-    arr = layer_array(spec)
+    arr = layer_array(spec, prepared_sign=api.SIGNED_NIBBLES if spec.w_bits == 3 else None)
     for i, layer in enumerate(spec.layers):
         plan = LayerPlan()
         assert lib().bs_sequence_layer_plan(arr, len(arr), i, ctypes.byref(plan)) == 0
