@@ -154,7 +154,7 @@ def tc_prepare_weights(wgt_packed: torch.Tensor, C: int, w_sign: int, a_bits: in
     signs = [w_sign, SIGNED_NIBBLES] if w_bits == 3 and w_sign == SIGNED and a_bits <= 2 and C * R * S * 28 < 4000000 else [w_sign]
     out = torch.empty(nbytes * len(signs), dtype=torch.int8, device=wgt_packed.device)
     for k, sign in enumerate(signs):
-        st = lib().bs_tc_prepare_weights(_ptr(wgt_packed), O, C, R, S, w_bits, sign, a_bits, _ptr(out[k * nbytes:(k + 1) * nbytes]), _stream_ptr(stream))
+        st = lib().bs_tc_prepare_weights(_ptr(wgt_packed), O, C, R, S, w_bits, sign, a_bits, _ptr(out) + k * nbytes, _stream_ptr(stream))
         _check(st, "bs_tc_prepare_weights")
     return out
 
